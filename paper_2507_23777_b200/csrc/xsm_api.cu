@@ -1,7 +1,7 @@
 // Host side of the C ABI declared in include/xsm.h: argument checks, workspace layout, phase tables,
 // launches.  No device memory is allocated here; everything lives in the caller's workspace.
 #include "../../include/xsm.h"
-#include "xsm_internal.h"
+#include "xsm_host.h"
 
 #include <cuda.h>
 
@@ -33,6 +33,7 @@ struct Layout {
     size_t h, rope_cs;
     size_t xchg_begin, hpub, qkv, attn, qc, cattn, act, y, logits0, hlogits, part, cpart, candx, header, done, sspub, qh, hattn, gpub,
         hpart, treex, xchg_end;
+    size_t rp, xa, qp, aa, actp, yp, hq, ha, ss, apart, acount;      // launch chain
     size_t stage_cond, stage_kv, stage_tok, trace, ckv_pool, hckv_pool, kv_pool;
     int n_pages = 0, max_blocks = 0, cpages = 0, tok_ld = 0, n_phases = 0, n_jobs = 0;
     size_t page_bytes = 0;
@@ -82,7 +83,7 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.step_n_new = take(cur, 4 * B);
     L.prompt = take(cur, 4 * B * (c.max_seq_len + 1));
     L.script = take(cur, 4 * B * L.tok_ld);
-    L.h = take(cur, 4 * M * d);
+    L.h = take(cur, 4 * (size_t)kMaxTokens * d);
     L.rope_cs = take(cur, 8 * (size_t)(c.max_seq_len + K1 + 1) * (dh / 2));
     // tagged exchange buffers, cleared together at every xsm_prefill
     L.xchg_begin = cur;
@@ -109,6 +110,20 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.hpart = take(cur, 4 * nh * part_items * K1 * (dh + 2));
     L.treex = take(cur, 4 * B * (c.n_draft > 0 ? c.n_draft : 1) * 8 * 2);
     L.xchg_end = cur;
+    if (c.dtype == 1) {      // launch chain: planes of at most kMaxTokens token rows, twice (hi, lo), two bytes an element
+        const size_t row = 4 * (size_t)kMaxTokens;
+        L.rp = take(cur, sizeof(RunParams) + 64);
+        L.xa = take(cur, row * d);
+        L.qp = take(cur, row * d);
+        L.aa = take(cur, row * d);
+        L.actp = take(cur, row * f);
+        L.yp = take(cur, row * d * c.n_draft);
+        L.hq = take(cur, row * d * nh);
+        L.ha = take(cur, row * d * nh);
+        L.ss = take(cur, 4 * (size_t)kMaxTokens * 160);
+        L.apart = take(cur, 4 * (size_t)kSizingGrid * kMaxTokens * (dh + 2));      // (split items: at most 9/8 of the SMs)
+        L.acount = take(cur, 4 * kSizingGrid);
+    }
     L.stage_cond = take(cur, esize(c) * B * c.n_cond * c.d_cond);
     L.stage_kv = take(cur, 4 * 2 * (size_t)kKvStagePositions * d);
     L.stage_tok = take(cur, 4 * B * (c.max_seq_len + 1));
@@ -165,12 +180,6 @@ const char *check_config(const xsm_model_config &c) {
     return nullptr;
 }
 
-struct WeightOffsets {
-    size_t E, gf, W0;
-    std::vector<size_t> g1, wq, wo, g2, wqc, wkc, wvc, woc, g3, wgate, wup, wdown, W1, Wout, hq, hk, hv, ho;
-    size_t total;
-};
-
 WeightOffsets weight_offsets(const xsm_model_config &c) {
     WeightOffsets w;
     const size_t d = c.d_model, f = c.d_ff, V = c.vocab, dc = c.d_cond, hd = c.head_hidden;
@@ -223,14 +232,18 @@ struct xsm_ctx {
     int grid, sm_count, smem_bytes, phase_launch, prefilled, batch;
     uint32_t serial;          // decoding steps launched since the last xsm_prefill
     int static_steps;         // the latest step kept its attention partials in the library's own scratch array
-    uint64_t launches;
+    unsigned long long launches;
     std::string err;
     Tables h_tab;
     std::vector<CUtensorMap> h_tmaps;   // tcgen05 path: host copies of the jobs' tensor maps (uploaded by xsm_prefill)
     int n_stages;             // stages of one decoding step
+    Chain chain;              // bf16 models: the launch chain
+    bool use_chain;
+    RunParams run;
+    int request;              // number of the latest xsm_prefill
     void *encode_tiled;       // cuTensorMapEncodeTiled of the driver (null: the tcgen05 path is not used)
     int *pinned;              // [4] n_active, status
-    cudaEvent_t ev0, ev1;
+    cudaEvent_t ev0, ev1, step_ev[2];
     double last_wall_ms;
 };
 
@@ -241,6 +254,7 @@ xsm_status fail(xsm_ctx *ctx, xsm_status st, const std::string &msg) {
     return st;
 }
 xsm_status cuda_fail(xsm_ctx *ctx, cudaError_t e, const char *what) {
+    (void)cudaGetLastError();      // reported here: the next call starts clean
     return fail(ctx, XSM_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 #define XSM_CUDA(ctx, call)                                             \
@@ -481,6 +495,14 @@ xsm_status check_device_status(xsm_ctx *ctx) {
 
 // n_steps decoding steps on the stream
 xsm_status run_steps(xsm_ctx *ctx, int n_steps, bool static_scratch = false) {
+    if (ctx->use_chain) {
+        // a recording is replayed unless single launches were asked for, a timeline is taken (the recording has none), or
+        // the call must not make the driver allocate anything
+        const bool graph = !ctx->phase_launch && !static_scratch && ctx->dev.trace == nullptr;
+        for (int t = 0; t < n_steps; ++t)
+            XSM_CUDA(ctx, ctx->chain.step(ctx->dev, ctx->stream, graph, !ctx->phase_launch, &ctx->launches));
+        return XSM_OK;
+    }
     const int np = ctx->n_stages;
     if (!static_scratch && ctx->static_steps) {
         // The steps since the workspace partials were last written went through the library's scratch array, so the
@@ -504,6 +526,53 @@ xsm_status run_steps(xsm_ctx *ctx, int n_steps, bool static_scratch = false) {
             ctx->serial += 1u;
         }
     }
+    return XSM_OK;
+}
+
+// the request's parameters in device memory, if they are not there already
+xsm_status set_run(xsm_ctx *ctx, const RunParams &r) {
+    if (memcmp(&r, &ctx->run, sizeof(r)) == 0) return XSM_OK;
+    ctx->run = r;
+    XSM_CUDA(ctx, launch_set_run(ctx->dev, r, ctx->stream));
+    ctx->launches += 1;
+    return XSM_OK;
+}
+xsm_status set_max_new(xsm_ctx *ctx, int max_new) {
+    ctx->dev.max_new = max_new;
+    if (!ctx->use_chain) return XSM_OK;
+    RunParams r = ctx->run;
+    r.max_new = max_new;
+    return set_run(ctx, r);
+}
+
+// Algorithm 1 line 1 on the launch chain: state, the condition's keys and values, the prompt, the first window
+xsm_status chain_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_t *d_prompt, int prompt_len, const xsm_decode_config *dc) {
+    const xsm_model_config &c = ctx->cfg;
+    Dev &D = ctx->dev;
+    D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8;
+    if (!ctx->chain.select(D)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
+    ctx->n_stages = ctx->chain.n_ops();
+    RunParams &r = ctx->run;
+    memset(&r, 0, sizeof(r));
+    r.verify_mode = dc->verify_mode; r.k_accept = dc->k_accept; r.delta = dc->delta;
+    r.sample_mode = dc->sample_mode; r.k_sample = dc->k_sample; r.temperature = dc->temperature;
+    r.key0 = (uint32_t)dc->seed; r.key1 = (uint32_t)(dc->seed >> 32);
+    r.max_new = INT_MAX; r.prompt_len = prompt_len;
+    r.request = ++ctx->request;
+    if ((const void *)d_prompt != (const void *)D.prompt)
+        XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
+    XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
+    XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off), at<size_t>(ctx, ctx->lay.wvc_off), d_cond,
+                                  D.ckv_pool, D.L, ctx->stream));
+    if (c.head_kind == 1 && D.K > 0) {
+        XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off), at<size_t>(ctx, ctx->lay.hv_off), d_cond,
+                                      D.hckv_pool, D.K, ctx->stream));
+        ctx->launches += 1;
+    }
+    ctx->launches += 3;
+    if (prompt_len > 1) XSM_CUDA(ctx, ctx->chain.ingest(D, prompt_len - 1, ctx->stream, &ctx->launches));
+    XSM_CUDA(ctx, launch_embed_rows(D, D.K1, D.Mp, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
+    ctx->prefilled = 1;
     return XSM_OK;
 }
 
@@ -546,12 +615,16 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     ctx->stream = (cudaStream_t)cuda_stream;
     ctx->phase_launch = 0; ctx->prefilled = 0; ctx->batch = 0; ctx->launches = 0; ctx->last_wall_ms = 0; ctx->serial = 0;
     ctx->static_steps = 0;
-    ctx->pinned = nullptr; ctx->ev0 = ctx->ev1 = nullptr;
+    ctx->request = 0; ctx->use_chain = false;
+    memset(&ctx->run, 0, sizeof(ctx->run));
+    ctx->pinned = nullptr; ctx->ev0 = ctx->ev1 = ctx->step_ev[0] = ctx->step_ev[1] = nullptr;
     auto bail = [&](cudaError_t e, const char *what) {
         g_create_error = std::string(what) + ": " + cudaGetErrorString(e);
         if (ctx->pinned) cudaFreeHost(ctx->pinned);
         if (ctx->ev0) cudaEventDestroy(ctx->ev0);
         if (ctx->ev1) cudaEventDestroy(ctx->ev1);
+        for (cudaEvent_t ev : ctx->step_ev)
+            if (ev) cudaEventDestroy(ev);
         delete ctx;
         return XSM_ERR_CUDA;
     };
@@ -582,6 +655,9 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     }
     if ((e = cudaEventCreate(&ctx->ev0)) != cudaSuccess) return bail(e, "cudaEventCreate");
     if ((e = cudaEventCreate(&ctx->ev1)) != cudaSuccess) return bail(e, "cudaEventCreate");
+    for (cudaEvent_t &ev : ctx->step_ev)
+        if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "cudaEventCreate");
+    memset(ctx->pinned, 0, 64);
 
     // constant tables
     // cos and sin of position * theta^(-2i/dh) for every position a window row can take
@@ -646,6 +722,16 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     D.qh = at<float>(ctx, L.qh); D.hattn = at<float>(ctx, L.hattn); D.gpub = at<float>(ctx, L.gpub); D.hpart = at<float>(ctx, L.hpart);
     D.hckv_pool = ctx->ws + L.hckv_pool;
     D.treex = at<uint32_t>(ctx, L.treex);
+    if (cfg->dtype == 1) {
+        ctx->use_chain = ctx->chain.init(*cfg, ctx->wo, ctx->weights, ctx->sm_count);
+        D.rp = at<RunParams>(ctx, L.rp);
+        D.stage_word = reinterpret_cast<int *>(ctx->ws + L.rp + sizeof(RunParams) + 32);
+        D.host_done = ctx->pinned + 8;
+        D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
+        D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
+        D.apart = at<float>(ctx, L.apart); D.acount = at<int>(ctx, L.acount);
+        D.tail_row_bytes = 160 * 1024;
+    }
     *out = ctx;
     return XSM_OK;
 }
@@ -672,6 +758,13 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     if ((long long)batch * ctx->lay.max_blocks > ctx->lay.n_pages)
         return fail(ctx, XSM_ERR_CAPACITY, "the page pool cannot hold `batch` sequences of max_seq_len positions");
     Dev &D = ctx->dev;
+    ctx->dc = *dc;
+    ctx->batch = batch;
+    {
+        const int bh = batch * D.H, s_max = ctx->grid / bh;
+        D.S_max = s_max < 1 ? 1 : (s_max > 64 ? 64 : s_max);
+    }
+    if (ctx->use_chain) return chain_prefill(ctx, batch, d_cond, d_prompt, prompt_len, dc);
     int smem_bytes = 0;
     D.umma = (umma_shape(c, batch) && ctx->encode_tiled != nullptr) ? 1 : 0;
     if (const char *m = plan_smem(c, batch, D, smem_bytes, ctx->grid)) return fail(ctx, XSM_ERR_CAPACITY, m);
@@ -692,17 +785,12 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
         XSM_CUDA(ctx, step_kernel_setup(probe, c.dtype, smem_bytes, &resident));
         if (resident < ctx->grid) return fail(ctx, XSM_ERR_CUDA, "the step kernel does not fit on this device");
     }
-    ctx->dc = *dc;
-    ctx->batch = batch;
     D.B = batch; D.M = batch * D.K1;
     D.inv_m = ((1 << 20) + D.M - 1) / D.M;
     D.verify_mode = dc->verify_mode; D.k_accept = dc->k_accept; D.delta = dc->delta;
     D.sample_mode = dc->sample_mode; D.k_sample = dc->k_sample; D.temperature = dc->temperature;
     D.key0 = (uint32_t)dc->seed; D.key1 = (uint32_t)(dc->seed >> 32);
     D.max_new = INT_MAX; D.prompt_len = prompt_len;
-    const int bh = batch * D.H;
-    int s_max = ctx->grid / bh;
-    D.S_max = s_max < 1 ? 1 : (s_max > 64 ? 64 : s_max);
     // the condition's keys and values of one head: one item while that is at most 96 KB, else split over CTAs
     int s_cross = 1;
     if ((long long)D.cpages * 2 * D.tile_bytes > 96 * 1024) {
@@ -752,8 +840,8 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
 xsm_status xsm_spec_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_spec_step before xsm_prefill");
-    ctx->dev.max_new = INT_MAX;
-    xsm_status st = run_steps(ctx, 1);
+    xsm_status st = set_max_new(ctx, INT_MAX);
+    if (st == XSM_OK) st = run_steps(ctx, 1);
     if (st != XSM_OK) return st;
     const Dev &D = ctx->dev;
     if (d_new_tokens)
@@ -783,6 +871,16 @@ xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_
         return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch need " +
                                                std::to_string(n_sets * half) + " bytes, the built-in scratch holds " +
                                                std::to_string(kStaticScratchBytes));
+    if (ctx->use_chain) {      // the key splits meet in distributed shared memory: no scratch, and no recording either
+        xsm_status st = set_max_new(ctx, INT_MAX);
+        if (st == XSM_OK) st = run_steps(ctx, 1, true);
+        if (st != XSM_OK) return st;
+        if (d_new_tokens)
+            XSM_CUDA(ctx, cudaMemcpyAsync(d_new_tokens, D.step_tokens, sizeof(int32_t) * D.M, cudaMemcpyDeviceToDevice, ctx->stream));
+        if (d_n_new)
+            XSM_CUDA(ctx, cudaMemcpyAsync(d_n_new, D.step_n_new, sizeof(int32_t) * D.B, cudaMemcpyDeviceToDevice, ctx->stream));
+        return XSM_OK;
+    }
     int dev = 0;
     XSM_CUDA(ctx, cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return fail(ctx, XSM_ERR_INVALID_ARG, "device ordinal out of range");
@@ -817,9 +915,24 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     if (max_new_tokens < 1 || max_new_tokens > ctx->cfg.max_seq_len)
         return fail(ctx, XSM_ERR_INVALID_ARG, "max_new_tokens must be in [1, max_seq_len]");
     Dev &D = ctx->dev;
-    D.max_new = max_new_tokens;
+    xsm_status set = set_max_new(ctx, max_new_tokens);
+    if (set != XSM_OK) return set;
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     long long budget = (long long)max_new_tokens + 2;   // every step commits at least one token per live sequence
+    if (ctx->use_chain) {
+        // one step ahead of the device: the next is on its way while one runs, and the one too many at the end finds
+        // every sequence ended and does nothing
+        volatile int *const done = ctx->pinned + 8;
+        for (long long i = 0; i < budget && *done != ctx->request; ++i) {
+            xsm_status st = run_steps(ctx, 1);
+            if (st != XSM_OK) return st;
+            XSM_CUDA(ctx, cudaEventRecord(ctx->step_ev[i & 1], ctx->stream));
+            if (i > 0) XSM_CUDA(ctx, cudaEventSynchronize(ctx->step_ev[(i - 1) & 1]));
+        }
+        budget = 0;
+        xsm_status st = check_device_status(ctx);
+        if (st != XSM_OK) return st;
+    }
     while (budget > 0) {
         const int n = (int)(budget < kChunkSteps ? budget : kChunkSteps);
         xsm_status st = run_steps(ctx, n);
@@ -889,6 +1002,8 @@ xsm_status xsm_destroy(xsm_ctx *ctx) {
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
+    for (cudaEvent_t ev : ctx->step_ev)
+        if (ev) cudaEventDestroy(ev);
     delete ctx;
     return XSM_OK;
 }
@@ -911,11 +1026,11 @@ xsm_status xsm_debug_get_logits(xsm_ctx *ctx, float *h_logits0, float *h_head_lo
     if (st != XSM_OK) return st;
     if (h_logits0) {
         XSM_CUDA(ctx, cudaMemcpy(h_logits0, D.logits0, sizeof(float) * (size_t)D.M * D.V, cudaMemcpyDeviceToHost));
-        strip_tags(h_logits0, (size_t)D.M * D.V);
+        if (!ctx->use_chain) strip_tags(h_logits0, (size_t)D.M * D.V);
     }
     if (h_head_logits && D.K > 0) {
         XSM_CUDA(ctx, cudaMemcpy(h_head_logits, D.hlogits, sizeof(float) * (size_t)D.K * D.M * D.V, cudaMemcpyDeviceToHost));
-        strip_tags(h_head_logits, (size_t)D.K * D.M * D.V);
+        if (!ctx->use_chain) strip_tags(h_head_logits, (size_t)D.K * D.M * D.V);
     }
     return XSM_OK;
 }
@@ -953,6 +1068,10 @@ xsm_status xsm_debug_set_drafts(xsm_ctx *ctx, const int32_t *h_drafts) {
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy2D(D.window + 1, sizeof(int32_t) * D.K1, h_drafts, sizeof(int32_t) * D.K,
                                sizeof(int32_t) * D.K, D.B, cudaMemcpyHostToDevice));
+    if (ctx->use_chain) {
+        XSM_CUDA(ctx, launch_embed_rows(D, D.K1, D.Mp, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
+        return XSM_OK;
+    }
     XSM_CUDA(ctx, launch_embed(D, ctx->cfg.dtype, ctx->serial, ctx->stream));
     ctx->launches += 1;
     return XSM_OK;
@@ -978,20 +1097,22 @@ xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t capacity
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_trace_step before xsm_prefill");
     if (ctx->phase_launch) return fail(ctx, XSM_ERR_STATE, "the timeline is taken from the persistent kernel");
     const int rows = 1 + 2 * ctx->n_stages;
-    const size_t words = (size_t)rows * ctx->grid;
+    const int ctas = ctx->use_chain ? kTraceCtas : ctx->grid;
+    const size_t words = (size_t)rows * ctas;
     if (capacity < words) return fail(ctx, XSM_ERR_CAPACITY, "h_times is too small");
     unsigned long long *d_trace = at<unsigned long long>(ctx, ctx->lay.trace);
     XSM_CUDA(ctx, cudaMemsetAsync(d_trace, 0, 8 * words, ctx->stream));
+    xsm_status st = set_max_new(ctx, INT_MAX);
+    if (st != XSM_OK) return st;
     ctx->dev.trace = d_trace;
-    ctx->dev.max_new = INT_MAX;
-    xsm_status st = run_steps(ctx, 1);
+    st = run_steps(ctx, 1);
     ctx->dev.trace = nullptr;
     if (st != XSM_OK) return st;
     st = check_device_status(ctx);
     if (st != XSM_OK) return st;
     XSM_CUDA(ctx, cudaMemcpy(h_times, d_trace, 8 * words, cudaMemcpyDeviceToHost));
     *n_rows = rows;
-    *n_ctas = ctx->grid;
+    *n_ctas = ctas;
     return XSM_OK;
 }
 
@@ -999,7 +1120,11 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_set_script before xsm_prefill");
     Dev &D = ctx->dev;
-    if (h_tokens == nullptr || n <= 0) { D.script = nullptr; D.script_n = 0; D.script_acc = 0; return XSM_OK; }
+    RunParams r = ctx->run;
+    if (h_tokens == nullptr || n <= 0) {
+        D.script = r.script = nullptr; D.script_n = r.script_n = 0; D.script_acc = r.script_acc = 0;
+        return ctx->use_chain ? set_run(ctx, r) : XSM_OK;
+    }
     if (n > ctx->lay.tok_ld) return fail(ctx, XSM_ERR_INVALID_ARG, "script longer than max_seq_len + n_draft + 1");
     if (!(mean_accept >= 0.f) || mean_accept > (float)D.K) return fail(ctx, XSM_ERR_INVALID_ARG, "mean_accept must be in [0, n_draft]");
     for (long long i = 0; i < (long long)D.B * n; ++i)
@@ -1008,13 +1133,18 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy(d_script, h_tokens, sizeof(int32_t) * (size_t)D.B * n, cudaMemcpyHostToDevice));
     D.script = d_script; D.script_n = n; D.script_acc = (int)lrintf(mean_accept * 1024.f);
-    return XSM_OK;
+    r.script = d_script; r.script_n = n; r.script_acc = D.script_acc;
+    return ctx->use_chain ? set_run(ctx, r) : XSM_OK;
 }
 
 xsm_status xsm_debug_set_wait_limits(xsm_ctx *ctx, uint32_t polls, uint32_t barrier_tries) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     ctx->dev.spin_limit = polls ? polls : kSpinLimit;
     ctx->dev.mbar_limit = barrier_tries ? barrier_tries : kMbarSpinLimit;
+    if (ctx->use_chain && ctx->prefilled) {      // the limits are part of the recordings
+        ctx->chain.forget();
+        if (!ctx->chain.select(ctx->dev)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
+    }
     return XSM_OK;
 }
 
@@ -1022,6 +1152,13 @@ xsm_status xsm_debug_launch_stage(xsm_ctx *ctx, int stage) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_launch_stage before xsm_prefill");
     if (stage < 0 || stage >= ctx->n_stages) return fail(ctx, XSM_ERR_INVALID_ARG, "no such stage");
+    if (ctx->use_chain) {
+        XSM_CUDA(ctx, launch_stage_gate(ctx->dev, stage, ctx->stream));
+        XSM_CUDA(ctx, ctx->chain.run_op(ctx->dev, stage, ctx->stream, &ctx->launches));
+        XSM_CUDA(ctx, launch_stage_mark(ctx->dev, (stage + 1) % ctx->n_stages, ctx->stream));
+        ctx->launches += 2;
+        return XSM_OK;
+    }
     XSM_CUDA(ctx, launch_step(ctx->dev, ctx->cfg.dtype, stage, stage + 1, 1, ctx->serial, ctx->grid, ctx->smem_bytes, ctx->stream));
     ctx->launches += 1;
     return XSM_OK;

@@ -1,0 +1,433 @@
+// Attention of bf16 models over the paged fp16 caches, as a kernel of the launch chain.
+//
+// Up to S CTAs serve one (sequence, head): they cut the keys by pages, a producer warp streams (page, head) tiles of
+// keys and values through a ring in shared memory, eight warps attend with mma.sync over 32 keys at a time (a unit).  How
+// many of the S take part depends on the context of the step (one up to 640 keys: a merge costs as much as four units);
+// they leave partial results in global memory and the last one to finish merges them, in the order of the keys.  (A
+// cluster that merges through distributed shared memory took 3 us longer: two cluster barriers with eight CTAs.)
+// The keys and values of the rows themselves have been written to the cache by the projection before, so self-attention
+// is the same walk with a causal limit per row.  Pages that the step does not write (and the condition's) are fetched
+// before the kernel waits for its predecessor.
+//
+// Few rows (at most eight, every step of a batch of any size with up to seven heads): the product is transposed,
+// S^T = K Q^T and O^T = V^T P^T, so that the 16 keys of a product sit on its M side and the rows on its 8-wide N side;
+// all eight warps take different keys.  More rows (chunks of a prompt, many heads): tiles of 16 rows on the M side; the
+// warps are divided over the row tiles first and over the keys with what is left.
+#include "xsm_proj.cuh"
+
+namespace xsm {
+
+constexpr int kAttnWarps = 8, kAttnThreads = kAttnWarps * 32 + 32;
+constexpr int kAttnSlots = 16;
+
+// ------------------------------------------------------------------- 32 keys against at most eight rows
+
+template <int DH> struct FewState {
+    float o[DH / 16][4];          // rows 16 dp + g (0, 1) and + 8 (2, 3) of O^T; columns 2t (0, 2) and 2t + 1 (1, 3)
+    float m[2], l[2];             // rows 2t, 2t + 1; l: this thread's keys only until the state is parked
+};
+
+// lim: last key of the unit that row 2t (2t + 1) sees
+template <int DH>
+__device__ __forceinline__ void few_unit(const unsigned (&qh)[DH / 8], const unsigned (&ql)[DH / 8], uint32_t k_tile, uint32_t v_tile, int key0,
+                                         int lim0, int lim1, FewState<DH> &ws) {
+    constexpr int RB = DH * 2;
+    const int lane = threadIdx.x & 31, g = lane >> 2;
+    float s[2][4];
+#pragma unroll
+    for (int kt = 0; kt < 2; ++kt) s[kt][0] = s[kt][1] = s[kt][2] = s[kt][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < DH / 16; ++ks) {
+#pragma unroll
+        for (int kt = 0; kt < 2; ++kt) {
+            const int row = key0 + kt * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);
+            const int chunk = 2 * ks + (lane >> 4);
+            unsigned ka[4];
+            ldmatrix_x4(ka, k_tile + (uint32_t)row * RB + (uint32_t)swz(row, chunk, RB) * 16u);
+            mma16816_f16(s[kt], ka[0], ka[1], ka[2], ka[3], qh[2 * ks], qh[2 * ks + 1]);
+            mma16816_f16(s[kt], ka[0], ka[1], ka[2], ka[3], ql[2 * ks], ql[2 * ks + 1]);
+        }
+    }
+    float mx0 = kNegBig, mx1 = kNegBig;
+#pragma unroll
+    for (int kt = 0; kt < 2; ++kt) {
+        const int r0 = kt * 16 + g, r1 = r0 + 8;
+        if (r0 > lim0) s[kt][0] = -INFINITY;
+        if (r0 > lim1) s[kt][1] = -INFINITY;
+        if (r1 > lim0) s[kt][2] = -INFINITY;
+        if (r1 > lim1) s[kt][3] = -INFINITY;
+        mx0 = fmaxf(mx0, fmaxf(s[kt][0], s[kt][2]));
+        mx1 = fmaxf(mx1, fmaxf(s[kt][1], s[kt][3]));
+    }
+#pragma unroll
+    for (int o = 4; o <= 16; o <<= 1) {
+        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+    }
+    const float m0 = fmaxf(ws.m[0], mx0), m1 = fmaxf(ws.m[1], mx1);
+    const float c0 = ex2(ws.m[0] - m0), c1 = ex2(ws.m[1] - m1);
+    ws.m[0] = m0; ws.m[1] = m1;
+    float l0 = 0.f, l1 = 0.f;
+    unsigned pb[2][2];             // P^T as B fragments of the 16-key steps (fp16: weights in [0, 1])
+#pragma unroll
+    for (int kt = 0; kt < 2; ++kt) {
+        const float p0 = ex2(s[kt][0] - m0), p1 = ex2(s[kt][1] - m1);
+        const float p2 = ex2(s[kt][2] - m0), p3 = ex2(s[kt][3] - m1);
+        l0 += p0 + p2; l1 += p1 + p3;
+        pb[kt][0] = movmatrix_trans(pack_f16x2(p0, p1));      // keys 0..7 of the step
+        pb[kt][1] = movmatrix_trans(pack_f16x2(p2, p3));      // keys 8..15
+    }
+    ws.l[0] = ws.l[0] * c0 + l0;
+    ws.l[1] = ws.l[1] * c1 + l1;
+    if (__any_sync(0xffffffffu, c0 != 1.f || c1 != 1.f)) {     // a new maximum somewhere in the warp's columns
+#pragma unroll
+        for (int dp = 0; dp < DH / 16; ++dp) { ws.o[dp][0] *= c0; ws.o[dp][1] *= c1; ws.o[dp][2] *= c0; ws.o[dp][3] *= c1; }
+    }
+#pragma unroll
+    for (int kt = 0; kt < 2; ++kt) {
+#pragma unroll
+        for (int dp = 0; dp < DH / 16; ++dp) {   // value columns 16dp .. 16dp+15 (chunks 2dp, 2dp+1) are rows of O^T
+            const int row = key0 + kt * 16 + (lane & 7) + ((lane >> 4) << 3);
+            const int chunk = 2 * dp + ((lane >> 3) & 1);
+            unsigned va[4];
+            ldmatrix_x4_trans(va, v_tile + (uint32_t)row * RB + (uint32_t)swz(row, chunk, RB) * 16u);
+            mma16816_f16(ws.o[dp], va[0], va[1], va[2], va[3], pb[kt][0], pb[kt][1]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------ 32 keys against sixteen rows
+
+template <int DH> struct RowsState {
+    float o[DH / 8][4];
+    float m[2], l[2];             // rows g, g + 8
+};
+
+template <int DH>
+__device__ __forceinline__ void rows_unit(const unsigned (&qh)[DH / 16][4], const unsigned (&ql)[DH / 16][4], uint32_t k_tile, uint32_t v_tile,
+                                          int key0, int lim0, int lim1, RowsState<DH> &ws) {
+    constexpr int RB = DH * 2;
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    float s[4][4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < DH / 16; ++ks) {
+#pragma unroll
+        for (int np = 0; np < 2; ++np) {      // key tiles 2np, 2np+1 (8 keys each)
+            const int row = key0 + np * 16 + (lane & 7) + ((lane >> 4) << 3);
+            const int chunk = 2 * ks + ((lane >> 3) & 1);
+            unsigned kb[4];
+            ldmatrix_x4(kb, k_tile + (uint32_t)row * RB + (uint32_t)swz(row, chunk, RB) * 16u);
+            mma16816_f16(s[2 * np], qh[ks][0], qh[ks][1], qh[ks][2], qh[ks][3], kb[0], kb[1]);
+            mma16816_f16(s[2 * np], ql[ks][0], ql[ks][1], ql[ks][2], ql[ks][3], kb[0], kb[1]);
+            mma16816_f16(s[2 * np + 1], qh[ks][0], qh[ks][1], qh[ks][2], qh[ks][3], kb[2], kb[3]);
+            mma16816_f16(s[2 * np + 1], ql[ks][0], ql[ks][1], ql[ks][2], ql[ks][3], kb[2], kb[3]);
+        }
+    }
+    float mx0 = kNegBig, mx1 = kNegBig;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const int k0 = nt * 8 + 2 * t;
+        if (k0 > lim0) s[nt][0] = -INFINITY;
+        if (k0 + 1 > lim0) s[nt][1] = -INFINITY;
+        if (k0 > lim1) s[nt][2] = -INFINITY;
+        if (k0 + 1 > lim1) s[nt][3] = -INFINITY;
+        mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]));
+        mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]));
+    }
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)); mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
+    const float m0 = fmaxf(ws.m[0], mx0), m1 = fmaxf(ws.m[1], mx1);
+    const float c0 = ex2(ws.m[0] - m0), c1 = ex2(ws.m[1] - m1);
+    ws.m[0] = m0; ws.m[1] = m1;
+    float l0 = 0.f, l1 = 0.f;
+    unsigned ph[2][4];             // P as A fragments of the two 16-key steps (fp16: weights in [0, 1])
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const float p0 = ex2(s[nt][0] - m0), p1 = ex2(s[nt][1] - m0);
+        const float p2 = ex2(s[nt][2] - m1), p3 = ex2(s[nt][3] - m1);
+        l0 += p0 + p1; l1 += p2 + p3;
+        const int kk = nt >> 1, hi2 = (nt & 1) * 2;     // a0,a1 from the even key tile, a2,a3 from the odd one
+        ph[kk][hi2] = pack_f16x2(p0, p1); ph[kk][hi2 + 1] = pack_f16x2(p2, p3);
+    }
+    ws.l[0] = ws.l[0] * c0 + l0;
+    ws.l[1] = ws.l[1] * c1 + l1;
+    if (__any_sync(0xffffffffu, c0 != 1.f || c1 != 1.f)) {     // a new maximum somewhere in the warp's rows
+#pragma unroll
+        for (int dn = 0; dn < DH / 8; ++dn) { ws.o[dn][0] *= c0; ws.o[dn][1] *= c0; ws.o[dn][2] *= c1; ws.o[dn][3] *= c1; }
+    }
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+#pragma unroll
+        for (int dp = 0; dp < DH / 16; ++dp) {   // value columns 16dp .. 16dp+15 (chunks 2dp, 2dp+1)
+            const int row = key0 + kk * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);
+            const int chunk = 2 * dp + (lane >> 4);
+            unsigned vb[4];
+            ldmatrix_x4_trans(vb, v_tile + (uint32_t)row * RB + (uint32_t)swz(row, chunk, RB) * 16u);
+            mma16816_f16(ws.o[2 * dp], ph[kk][0], ph[kk][1], ph[kk][2], ph[kk][3], vb[0], vb[1]);
+            mma16816_f16(ws.o[2 * dp + 1], ph[kk][0], ph[kk][1], ph[kk][2], ph[kk][3], vb[2], vb[3]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------- kernel
+
+__device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(reinterpret_cast<const unsigned *>(p)); }
+
+template <int DH, bool FEW>
+__global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_kernel(const Dev D, const AttnArgs A) {
+    extern __shared__ __align__(128) char smem[];
+    __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z % D.B, set = blockIdx.z / D.B;
+    const int P = D.P, upp = P >> 5, slots = A.slots;
+    const bool cross = A.cross != 0;
+    const int start = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);      // (the state was written by an earlier step)
+    const int n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + A.t, A.pos_end) : start + A.t;
+    const int S = min(A.S, (n_keys + A.split - 1) / A.split);                    // CTAs that take part
+    if (rank >= S) return;
+    // few rows: a warp looks only at the pages whose units it owns when the units of 1, 2 or 4 pages fill a round of the
+    // warps (the ring is a whole number of rounds, so a warp meets every fill of its slots)
+    const bool owned = FEW && (upp == 1 || upp == 2 || upp == 4);
+    if (tid == 0) {
+        for (int i = 0; i < slots; ++i) {
+            mbar_init(smem_u32(&full[i]), 1u);
+            mbar_init(smem_u32(&empty[i]), owned ? (uint32_t)upp : (uint32_t)kAttnWarps);
+        }
+        mbar_init_fence();
+    }
+    __syncthreads();
+    chain_go();
+    const bool dead = A.pos0 < 0 && __ldcg(D.finished + b) != 0;
+    if (dead) {
+        chain_wait();
+        return;
+    }
+    const int np = page_of(D, n_keys + P - 1), p_lo = rank * np / S, p_hi = (rank + 1) * np / S;
+    const uint32_t tile_bytes = (uint32_t)P * DH * 2u, ring = smem_u32(smem);
+    const int qt_n = FEW ? 1 : (A.t + 15) >> 4;                       // row tiles
+    int wq = 1;                                                       // warps that share the keys between them: kAttnWarps / wq
+    if (!FEW)
+        while (wq < qt_n) wq <<= 1;
+    const int kg_n = kAttnWarps / wq;
+    // parked states of the warps [kAttnWarps][rows][DH + 2]; they reuse the ring
+    constexpr int LD = DH + 2;
+    const int srows = FEW ? A.t : 16;
+    float *st = reinterpret_cast<float *>(smem);
+
+    if (warp == kAttnWarps) {
+        if (lane == 0) {
+            const int n_old = cross ? np : page_of(D, start);         // pages that nobody writes in this step
+            bool waited = false;
+            for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
+                if (!waited && pg >= n_old) {
+                    chain_wait();
+                    fence_proxy_async();
+                    waited = true;
+                }
+                const int sl = i % slots;
+                if (i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
+                const int page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
+                const int pool_pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
+                const __half *kt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 0, page, h);
+                const __half *vt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 1, page, h);
+                const uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
+                mbar_arrive_expect_tx(f, 2u * tile_bytes);
+                bulk_g2s(dst, kt, tile_bytes, f);
+                bulk_g2s(dst + tile_bytes, vt, tile_bytes, f);
+            }
+        }
+        __syncwarp();
+        chain_wait();
+        __syncthreads();                 // (1) every page has been consumed
+    } else {
+        const int g = lane >> 2, t4 = lane & 3;
+        const __half *qhi = A.q + (size_t)set * 2 * A.Mp * D.d + (size_t)(b * A.t) * D.d + h * DH, *qlo = qhi + (size_t)A.Mp * D.d;
+        chain_wait();
+        trace_mark(D, 1 + 2 * A.stage);
+        if (FEW) {
+            unsigned qh[DH / 8], ql[DH / 8];
+#pragma unroll
+            for (int c = 0; c < DH / 8; ++c) {
+                const size_t o = (size_t)g * D.d + 8 * c + 2 * t4;
+                qh[c] = g < A.t ? ldcg_u32(qhi + o) : 0u;
+                ql[c] = g < A.t ? ldcg_u32(qlo + o) : 0u;
+            }
+            FewState<DH> ws;
+#pragma unroll
+            for (int i = 0; i < DH / 16; ++i) ws.o[i][0] = ws.o[i][1] = ws.o[i][2] = ws.o[i][3] = 0.f;
+            ws.m[0] = ws.m[1] = kNegBig;
+            ws.l[0] = ws.l[1] = 0.f;
+            const int row_lim0 = cross ? D.C - 1 : start + 2 * t4, row_lim1 = cross ? D.C - 1 : row_lim0 + 1;
+            const int stride = owned ? kAttnWarps / upp : 1;
+            for (int i = owned ? warp / upp : 0; i < p_hi - p_lo; i += stride) {
+                const int sl = i % slots;
+                mbar_wait(smem_u32(&full[sl]), (uint32_t)((i / slots) & 1), D.mbar_limit, D.status);
+                const uint32_t kt = ring + (uint32_t)sl * 2u * tile_bytes;
+                for (int uu = owned ? warp % upp : 0; uu < upp; uu += owned ? upp : 1) {
+                    if (!owned && ((i * upp + uu) & (kAttnWarps - 1)) != warp) continue;
+                    const int base = (p_lo + i) * P + uu * 32;
+                    if (base < n_keys) few_unit<DH>(qh, ql, kt, kt + tile_bytes, uu * 32, row_lim0 - base, row_lim1 - base, ws);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
+            }
+            __syncthreads();             // (1)
+#pragma unroll
+            for (int o = 4; o <= 16; o <<= 1) {
+                ws.l[0] += __shfl_xor_sync(0xffffffffu, ws.l[0], o);
+                ws.l[1] += __shfl_xor_sync(0xffffffffu, ws.l[1], o);
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int r = 2 * t4 + c;
+                if (r < A.t) {
+                    float *dst = st + (warp * srows + r) * LD;
+#pragma unroll
+                    for (int dp = 0; dp < DH / 16; ++dp) {
+                        dst[16 * dp + g] = ws.o[dp][c];
+                        dst[16 * dp + g + 8] = ws.o[dp][2 + c];
+                    }
+                    if (g == 0) { dst[DH] = ws.m[c]; dst[DH + 1] = ws.l[c]; }
+                }
+            }
+        } else {
+            const int qt = warp & (wq - 1), kg = warp / wq;
+            const int r0 = qt * 16 + g, r1 = r0 + 8;
+            unsigned qh[DH / 16][4], ql[DH / 16][4];
+#pragma unroll
+            for (int ks = 0; ks < DH / 16; ++ks) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = (q & 1) ? r1 : r0;
+                    const size_t o = (size_t)r * D.d + ks * 16 + 2 * t4 + (q >> 1) * 8;
+                    qh[ks][q] = r < A.t ? ldcg_u32(qhi + o) : 0u;
+                    ql[ks][q] = r < A.t ? ldcg_u32(qlo + o) : 0u;
+                }
+            }
+            RowsState<DH> ws;
+#pragma unroll
+            for (int i = 0; i < DH / 8; ++i) ws.o[i][0] = ws.o[i][1] = ws.o[i][2] = ws.o[i][3] = 0.f;
+            ws.m[0] = ws.m[1] = kNegBig;
+            ws.l[0] = ws.l[1] = 0.f;
+            const int row_lim0 = cross ? D.C - 1 : start + r0, row_lim1 = cross ? D.C - 1 : start + r1;
+            const int last = cross ? D.C - 1 : start + min(qt * 16 + 15, A.t - 1);      // last key of the row tile
+            for (int i = 0; i < p_hi - p_lo; ++i) {
+                const int sl = i % slots;
+                mbar_wait(smem_u32(&full[sl]), (uint32_t)((i / slots) & 1), D.mbar_limit, D.status);
+                const uint32_t kt = ring + (uint32_t)sl * 2u * tile_bytes;
+                for (int uu = 0; uu < upp; ++uu) {
+                    const int base = (p_lo + i) * P + uu * 32;
+                    if (((i * upp + uu) & (kg_n - 1)) != kg || base > last || qt >= qt_n) continue;
+                    rows_unit<DH>(qh, ql, kt, kt + tile_bytes, uu * 32, row_lim0 - base, row_lim1 - base, ws);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
+            }
+            __syncthreads();             // (1)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                ws.l[c] += __shfl_xor_sync(0xffffffffu, ws.l[c], 1);
+                ws.l[c] += __shfl_xor_sync(0xffffffffu, ws.l[c], 2);
+                const int r = c ? r1 : r0;
+                if (r < A.t) {
+                    float *dst = st + (warp * 16 + g + 8 * c) * LD;
+#pragma unroll
+                    for (int dn = 0; dn < DH / 8; ++dn) {
+                        dst[8 * dn + 2 * t4] = ws.o[dn][2 * c];
+                        dst[8 * dn + 2 * t4 + 1] = ws.o[dn][2 * c + 1];
+                    }
+                    if (t4 == 0) { dst[DH] = ws.m[c]; dst[DH + 1] = ws.l[c]; }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    // the warps' states of a row -> the output, or this CTA's partial result.  Two neighbouring columns a thread.
+    bf16 *out = A.out + (size_t)set * 2 * A.Mp * D.d;
+    const int item = blockIdx.z * D.H + h, n_pairs = A.t * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
+    float *mine = A.part + ((size_t)(item * A.S + rank) * A.t) * LD;
+    auto store = [&](int r, int c, float v0, float v1) {
+        bf16 h0, l0, h1, l1;
+        split_bf16(v0, h0, l0);
+        split_bf16(v1, h1, l1);
+        bf16 *p = out + plane_off(A.Mp, b * A.t + r, h * DH + c);
+        *reinterpret_cast<__nv_bfloat162 *>(p) = __nv_bfloat162(h0, h1);
+        *reinterpret_cast<__nv_bfloat162 *>(p + kLo) = __nv_bfloat162(l0, l1);
+    };
+    for (int e = tid; e < n_pairs; e += kAttnThreads) {
+        const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
+        const float *src = st + r * LD;                   // (row r of a row tile: the tiles of the first kg follow each other)
+        float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
+        for (int w = 0; w < kg_n; ++w) m = fmaxf(m, src[w * step + DH]);
+        for (int w = 0; w < kg_n; ++w) {
+            const float f = ex2(src[w * step + DH] - m);
+            const float2 o = *reinterpret_cast<const float2 *>(src + w * step + c);
+            o0 += f * o.x;
+            o1 += f * o.y;
+            l += f * src[w * step + DH + 1];
+        }
+        if (S == 1) {
+            store(r, c, o0 / l, o1 / l);
+        } else {
+            float *dst = mine + (size_t)r * LD;
+            __stcg(reinterpret_cast<float2 *>(dst + c), make_float2(o0, o1));
+            if (c == 0) __stcg(reinterpret_cast<float2 *>(dst + DH), make_float2(m, l));
+        }
+    }
+    if (S > 1) {
+        __shared__ int s_last;
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(A.count + item, 1) == S - 1;
+        __syncthreads();
+        if (s_last) {
+            __threadfence();
+            const float *all = A.part + ((size_t)item * A.S * A.t) * LD;
+            for (int e = tid; e < n_pairs; e += kAttnThreads) {
+                const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
+                float2 ml[8], os[8];
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    const float *src = all + ((size_t)s * A.t + r) * LD;
+                    ml[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + DH)) : make_float2(kNegBig, 0.f);
+                    os[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + c)) : make_float2(0.f, 0.f);
+                }
+                float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
+#pragma unroll
+                for (int s = 0; s < 8; ++s) m = fmaxf(m, ml[s].x);
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    const float f = ex2(ml[s].x - m);
+                    o0 += f * os[s].x;
+                    o1 += f * os[s].y;
+                    l += f * ml[s].y;
+                }
+                store(r, c, o0 / l, o1 / l);
+            }
+            if (tid == 0) A.count[item] = 0;
+        }
+    }
+    trace_mark(D, 2 + 2 * A.stage);
+}
+
+template <int DH, bool FEW>
+static cudaError_t launch_instance(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    void (*fn)(const Dev, const AttnArgs) = attn_kernel<DH, FEW>;
+    const int ring = A.slots * 2 * D.P * DH * 2;
+    const int park = kAttnWarps * (FEW ? A.t : 16) * (DH + 2) * 4;
+    const int smem = ring > park ? ring : park;
+    cudaError_t e = open_kernel((const void *)fn, smem, false);
+    if (e != cudaSuccess) return e;
+    return L.launch(dim3(A.S, D.H, D.B * A.sets), dim3(kAttnThreads), smem, 1, (const void *)fn, D, A);
+}
+
+cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    const bool few = A.t <= 8;
+    if (D.dh == 32) return few ? launch_instance<32, true>(D, A, L) : launch_instance<32, false>(D, A, L);
+    if (D.dh == 64) return few ? launch_instance<64, true>(D, A, L) : launch_instance<64, false>(D, A, L);
+    return few ? launch_instance<128, true>(D, A, L) : launch_instance<128, false>(D, A, L);
+}
+
+}  // namespace xsm

@@ -1,0 +1,402 @@
+// Host side of the launch chain: tensor maps, how each stage is cut over the chip, recording and replay of a step.
+#include "xsm_host.h"
+
+#include <cuda.h>
+#include <string.h>
+
+#include <algorithm>
+#include <mutex>
+#include <unordered_map>
+
+namespace xsm {
+
+static_assert(sizeof(TensorMap) == sizeof(CUtensorMap), "tensor map size");
+
+constexpr int kMaxPlans = 8;                      // batch sizes whose recordings are kept
+constexpr int kProjSmemMax = 224 * 1024;          // dynamic shared memory of a projection (a CTA may have 227 KB in all)
+
+cudaError_t open_kernel(const void *fn, int smem, bool large_cluster) {
+    static std::mutex mu;
+    struct Opened { int smem = 0; bool large = false; };
+    static std::unordered_map<const void *, Opened> opened[kMaxDevices];      // what each kernel has been opened for, by device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    Opened &o = opened[dev][fn];
+    if (large_cluster && !o.large) {
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+        o.large = true;
+    }
+    if (smem > o.smem) {
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+        o.smem = smem;
+    }
+    return cudaSuccess;
+}
+
+StepPlan::~StepPlan() {
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
+}
+
+Chain::~Chain() {
+    forget();
+    if (record_) cudaStreamDestroy(record_);
+}
+
+void Chain::forget() {
+    plan_ = nullptr;
+    plans_.clear();
+}
+
+// ------------------------------------------------------------------------------------- tensor maps
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
+                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+static bool encode(void *fn, TensorMap *out, const void *base, int cols, int rows, int sets, size_t set_bytes, int box_rows) {
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)sets};
+    cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)set_bytes};
+    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1}, estr[3] = {1, 1, 1};
+    return ((EncodeTiledFn)fn)(reinterpret_cast<CUtensorMap *>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides,
+                               box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// `count` matrices [rows][kdim] of bf16, stride_elems apart (the layers' copies, or the decoding heads'): boxes of 64 columns
+bool Chain::weight_map(TensorMap *out, size_t elem_off, int rows, int kdim, int count, size_t stride_elems, int box_rows) {
+    const size_t stride = count > 1 ? stride_elems * 2 : (size_t)rows * kdim * 2;
+    return encode(encode_, out, weights_ + elem_off * 2, kdim, rows, count, stride, box_rows);
+}
+bool Chain::init(const xsm_model_config &c, const WeightOffsets &w, const char *weights, int sm_count) {
+    c_ = c;
+    w_ = w;
+    weights_ = weights;
+    sms_ = sm_count;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &encode_, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    for (int s = 2; s <= 8; ++s) clusters_[s] = resident_clusters(s);
+    const int d = c.d_model, f = c.d_ff, V = c.vocab, L = c.n_layers, K = c.n_draft;
+    const size_t ls = L > 1 ? w.wq[1] - w.wq[0] : 0;
+    bool ok = weight_map(&qkv_, w.wq[0], 3 * d, d, L, ls, 128) && weight_map(&o_, w.wo[0], d, d, L, ls, 128) &&
+              weight_map(&qc_, w.wqc[0], d, d, L, ls, 128) && weight_map(&oc_, w.woc[0], d, d, L, ls, 128) &&
+              weight_map(&gate_, w.wgate[0], f, d, L, ls, 64) && weight_map(&up_, w.wup[0], f, d, L, ls, 64) &&
+              weight_map(&down_, w.wdown[0], d, f, L, ls, 128) && weight_map(&lm_, w.W0, V, d, 1, 0, 128);
+    if (K > 0) {
+        const size_t hs = K > 1 ? w.Wout[1] - w.Wout[0] : 0;
+        ok = ok && weight_map(&head_out_, w.Wout[0], V, d, K, hs, 128);
+        if (c.head_kind == 1)
+            ok = ok && weight_map(&head_in_, w.hq[0], d, d, K, hs, 128) && weight_map(&head_o_, w.ho[0], d, d, K, hs, 128);
+        else
+            ok = ok && weight_map(&head_in_, w.W1[0], d, d, K, hs, 128);
+    }
+    return ok;
+}
+
+// ------------------------------------------------------------------------------------- cuts of a stage
+
+// Cluster size, rings and shared memory of a projection over `rows` token rows.  The row tiles of a stage (8 to 128) leave
+// SMs idle at one CTA each, so the columns are cut as far as all clusters still run at once.
+void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
+    if (plan_few(op, rows, Mp, kdim)) return;
+    ProjArgs &A = op.proj;
+    A.kdim = kdim;
+    A.rows = rows;
+    A.Mp = Mp;
+    const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
+    // (clusters have to fit into a GPC: of six CTAs 22 run at a time, of eight 15; a cluster more than that is a second wave)
+    int S = 1;
+    for (int s = 2; s <= std::min(8, nblk); ++s)
+        if (tiles <= clusters_[s]) S = s;
+    A.S = S;
+    A.tps = ((rows + 3) / 4 + S - 1) / S * 4;
+    const int n = (nblk + S - 1) / S, b_bytes = 2 * Mp * 128, a_bytes = 128 * 128;
+    const int room = kProjSmemMax - 1024 - S * A.tps * 512;
+    A.nb = std::min(n, std::max(2, std::min(kProjRing, (room / 3) / b_bytes)));
+    A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
+    A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
+    A.tmem_cols = 32;
+    while (A.tmem_cols < 2 * Mp) A.tmem_cols *= 2;
+    op.smem = 1024 + A.na * a_bytes + A.nb * b_bytes + S * A.tps * 512;
+}
+
+// The projections over few token rows: how the units are dealt out, passes over the columns, shared memory.  False: the
+// shape does not fit, or there are more token rows than the path serves.
+bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
+    ProjArgs &A = op.proj;
+    if (rows > kFewRows) return false;
+    const bool pairs = A.epi0 == PE_QKV || A.epi0 == PE_GATEUP;
+    const int units = A.epi0 == PE_QKV ? A.g[0].units / 2 : A.g[0].units + (A.epi1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
+    const int share = A.x_jobs ? std::max(1, sms_ / A.g[0].jobs) : sms_;      // CTAs for `units`
+    A.upc = (units + share - 1) / share;
+    A.ctas = (units + A.upc - 1) / A.upc;
+    const FewShape f = few_shape(rows, kdim);
+    const int passes = (kdim + f.pass - 1) / f.pass;
+    A.chunk = (kdim / passes + 63) / 64 * 64;
+    if (A.chunk * passes < kdim) A.chunk += 64;
+    const int n_rows = A.upc * (pairs ? 2 : 1), tiles = (n_rows + 15) / 16, pitch = A.chunk * 2 + 64;
+    const int red = tiles * f.warps * 16 * (f.nt * 8 + 1) * 4, stages = tiles * passes;
+    const int slots = std::min(std::min(stages, kProjRing), (kProjSmemMax - red) / (16 * pitch));
+    if (slots < std::min(stages, 2) || A.upc > 32 && A.epi0 == PE_ADD || A.ctas > 160) return false;
+    A.kdim = kdim;
+    A.rows = rows;
+    A.Mp = Mp;
+    A.S = 1;
+    A.slots = slots;
+    op.kind = ChainOp::FEW;
+    op.smem = slots * 16 * pitch + red;
+    return true;
+}
+
+AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
+    AttnArgs A;
+    memset(&A, 0, sizeof(A));
+    A.cross = cross;
+    A.sets = sets;
+    A.t = t;
+    A.Mp = Mp;
+    const int items = D.B * D.H * sets, upp = D.P / 32, pair = 2 * D.P * D.dh * 2;
+    // about one CTA per SM at most; few rows: one more for every 640 keys (a merge costs as much as four units of 32 keys)
+    A.S = 1;
+    while (A.S < 8 && items * A.S * 2 <= sms_ + sms_ / 8) A.S *= 2;
+    A.split = t <= 8 ? 640 : 128;
+    if (cross) A.S = std::min(A.S, (D.C + A.split - 1) / A.split);
+    A.part = D.apart;
+    A.count = D.acount;
+    const int round = upp == 1 || upp == 2 || upp == 4 ? 8 / upp : 1;
+    const int pages = ((cross ? D.cpages : D.max_blocks) + A.S - 1) / A.S;
+    const int budget = items * A.S > sms_ ? 100 * 1024 : 128 * 1024;
+    int slots = std::min(16, budget / pair) / round * round;
+    slots = std::max(round, std::min(slots, (pages + round - 1) / round * round));
+    A.slots = slots;
+    return A;
+}
+
+bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
+    const xsm_model_config &c = c_;
+    const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers, rows = D.B * t, Mp = (rows + 7) / 8 * 8;
+    const bool ca = c.head_kind == 1;
+    const float qscale = D.scale * 1.4426950408889634f;      // softmax in base 2
+    auto gain = [&](size_t off) { return (const void *)(weights_ + off * 2); };
+    const size_t head_stride = K > 1 ? w_.Wout[1] - w_.Wout[0] : 0;
+    int shares = 1;                       // of the sums of squares of h: one from the embedding, then four per row tile of the writer
+    auto proj = [&](int epi0, int epi1, int layer, const TensorMap &w0, const TensorMap *w1, size_t w_off, size_t w1_off, const void *x) -> ChainOp & {
+        ops.emplace_back();
+        ChainOp &op = ops.back();
+        op.kind = ChainOp::PROJ;
+        memset(&op.proj, 0, sizeof(op.proj));
+        op.maps.w0 = w0;
+        op.maps.w1 = w1 ? *w1 : w0;
+        ProjArgs &A = op.proj;
+        A.x = (const bf16 *)x;
+        A.g[0].w = (const bf16 *)weights_ + w_off;
+        A.g[1].w = (const bf16 *)weights_ + w1_off;
+        A.g[0].w_stride = A.g[1].w_stride = head_stride;
+        A.epi0 = epi0; A.epi1 = epi1; A.layer = layer; A.t = t; A.pos0 = -1; A.scale = qscale;
+        return op;
+    };
+    auto group = [&](ProjGroup &g, int units, int tile_rows, int jobs, int ld, void *out, float *logits) {
+        g.units = units; g.jobs = jobs; g.job_tiles = (units + tile_rows - 1) / tile_rows; g.tiles = g.job_tiles * jobs;
+        g.ld = ld; g.out = (bf16 *)out; g.logits = logits;
+    };
+    auto attn = [&](bool cross, int sets, int layer, const void *pool, const void *q, void *out) {
+        ops.emplace_back();
+        ChainOp &op = ops.back();
+        op.kind = ChainOp::ATTN;
+        op.attn = plan_attn(D, cross, sets, t, Mp);
+        op.attn.layer = layer; op.attn.rows = rows; op.attn.pos0 = -1;
+        op.attn.pool = pool; op.attn.q = (const __half *)q; op.attn.out = (bf16 *)out;
+    };
+    auto residual = [&](int layer, const TensorMap &w, size_t w_off, const void *x, int kdim, size_t next_gain) {
+        ChainOp &op = proj(PE_ADD, -1, layer, w, nullptr, w_off, 0, x);
+        group(op.proj.g[0], d, 128, 1, d, D.xa_, nullptr);
+        op.proj.gain = gain(next_gain);
+        plan_proj(op, rows, Mp, kdim);
+        shares = op.kind == ChainOp::FEW ? op.proj.ctas : d / 128 * 4;
+    };
+    auto normed = [&](ChainOp &op) {
+        op.proj.norm = 1;
+        op.proj.ss_parts = shares;
+        plan_proj(op, rows, Mp, d);
+    };
+    if (prompt) { ops.emplace_back(); ops.back().kind = ChainOp::EMBED; }
+    for (int l = 0; l < L; ++l) {
+        {
+            ChainOp &op = proj(PE_QKV, -1, l, qkv_, nullptr, w_.wq[l], 0, D.xa_);
+            group(op.proj.g[0], 3 * d, 128, 1, 0, nullptr, nullptr);
+            op.proj.q = (__half *)D.qp_;
+            op.proj.late_go = l == 0;
+            normed(op);
+        }
+        if (prompt && l == L - 1) break;      // the last keys and values are in the cache
+        attn(false, 1, l, D.kv_pool, D.qp_, D.aa_);
+        residual(l, o_, w_.wo[l], D.aa_, d, w_.g2[l]);
+        {
+            ChainOp &op = proj(PE_QUERY, -1, l, qc_, nullptr, w_.wqc[l], 0, D.xa_);
+            group(op.proj.g[0], d, 128, 1, 0, nullptr, nullptr);
+            op.proj.q = (__half *)D.qp_;
+            normed(op);
+        }
+        attn(true, 1, l, D.ckv_pool, D.qp_, D.aa_);
+        residual(l, oc_, w_.woc[l], D.aa_, d, w_.g3[l]);
+        {
+            ChainOp &op = proj(PE_GATEUP, -1, l, gate_, &up_, w_.wgate[l], w_.wup[l], D.xa_);
+            group(op.proj.g[0], f, 64, 1, f, D.actp_, nullptr);
+            normed(op);
+        }
+        residual(l, down_, w_.wdown[l], D.actp_, f, l + 1 < L ? w_.g1[l + 1] : w_.gf);
+    }
+    if (prompt) return true;
+    {
+        ChainOp &op = proj(PE_LOGITS, K == 0 ? -1 : ca ? PE_QUERY : PE_HEADY, 0, lm_, K > 0 ? &head_in_ : nullptr, w_.W0,
+                            K == 0 ? 0 : ca ? w_.hq[0] : w_.W1[0], D.xa_);
+        group(op.proj.g[0], V, 128, 1, V, nullptr, D.logits0);
+        if (K > 0) group(op.proj.g[1], d, 128, K, d, D.yp_, nullptr);
+        op.proj.gain = gain(w_.gf);
+        op.proj.q = (__half *)D.hq_;
+        normed(op);
+    }
+    if (K > 0 && ca) {
+        attn(true, K, 0, D.hckv_pool, D.hq_, D.ha_);
+        ChainOp &op = proj(PE_HEADADD, -1, 0, head_o_, nullptr, w_.ho[0], 0, D.ha_);
+        group(op.proj.g[0], d, 128, K, d, D.yp_, nullptr);
+        op.proj.gain = gain(w_.gf);
+        op.proj.z_jobs = op.proj.x_jobs = 1;
+        op.proj.ss_parts = shares;
+        plan_proj(op, rows, Mp, d);
+    }
+    if (K > 0) {
+        ChainOp &op = proj(PE_LOGITS, -1, 0, head_out_, nullptr, w_.Wout[0], 0, D.yp_);
+        group(op.proj.g[0], V, 128, K, V, nullptr, D.hlogits);
+        op.proj.z_jobs = op.proj.x_jobs = 1;
+        plan_proj(op, rows, Mp, d);
+    }
+    ops.emplace_back();
+    ops.back().kind = ChainOp::TAIL;
+    return true;
+}
+
+// The weights of a step in the order of their use are one stream (of bytes, closed to a ring: the first layer follows the
+// last projection).  Every projection fetches as much of it ahead as it reads itself, kAheadBytes further on.
+void Chain::plan_ahead(std::vector<ChainOp> &ops) {
+    constexpr size_t kAheadBytes = 32 << 20;
+    struct Piece { const char *p; size_t n, at; };      // at: offset in the stream
+    std::vector<Piece> pieces;
+    size_t total = 0;
+    auto add = [&](const bf16 *p, size_t elems) { pieces.push_back({(const char *)p, elems * 2, total}); total += elems * 2; };
+    struct Use { ProjArgs *A; size_t begin, end; };
+    std::vector<Use> uses;
+    for (ChainOp &op : ops) {
+        if (op.kind != ChainOp::PROJ && op.kind != ChainOp::FEW) continue;
+        ProjArgs &A = op.proj;
+        const size_t begin = total;
+        for (int q = 0; q < (A.epi1 >= 0 || A.epi0 == PE_GATEUP ? 2 : 1); ++q) {
+            const size_t one = (size_t)(A.epi0 == PE_GATEUP ? A.g[0].units : A.g[q].units) * A.kdim;
+            const int jobs = A.epi0 == PE_GATEUP ? 1 : A.g[q].jobs;
+            for (int j = 0; j < jobs; ++j) add(A.g[q].w + j * A.g[q].w_stride, one);
+        }
+        uses.push_back({&A, begin, total});
+    }
+    if (total <= 2 * kAheadBytes) return;      // the model stays in L2 anyway
+    for (Use &u : uses) {
+        size_t lo = (u.begin + kAheadBytes) % total, left = u.end - u.begin;
+        for (int q = 0; q < 2 && left > 0; ++q) {
+            size_t i = 0;
+            while (pieces[i].at + pieces[i].n <= lo) ++i;
+            const size_t off = lo - pieces[i].at, n = std::min(left, pieces[i].n - off);
+            u.A->ahead[q] = pieces[i].p + off;
+            u.A->ahead_bytes[q] = (unsigned)n;
+            left -= n;
+            lo = (lo + n) % total;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------- running
+
+cudaError_t Chain::run(const Dev &D, const ChainOp &op, int t, const ChainLaunch &L) {
+    switch (op.kind) {
+        case ChainOp::PROJ: return launch_proj_umma(D, op.proj, &op.maps, op.smem, L);
+        case ChainOp::FEW: return launch_proj_few(D, op.proj, op.smem, L);
+        case ChainOp::ATTN: return launch_attn(D, op.attn, L);
+        case ChainOp::TAIL: return launch_tail(D, op.proj.stage, L);
+        case ChainOp::EMBED: return launch_embed_rows(D, t, (D.B * t + 7) / 8 * 8, op.attn.pos0, L);
+    }
+    return cudaErrorInvalidValue;
+}
+
+bool Chain::select(const Dev &D) {
+    auto it = plans_.find(D.B);
+    if (it == plans_.end()) {
+        if ((int)plans_.size() >= kMaxPlans) plans_.clear();
+        std::unique_ptr<StepPlan> p(new StepPlan());
+        if (!build(D, D.K1, false, p->ops)) return false;
+        plan_ahead(p->ops);
+        for (size_t i = 0; i < p->ops.size(); ++i) p->ops[i].proj.stage = p->ops[i].attn.stage = (int)i;
+        it = plans_.emplace(D.B, std::move(p)).first;
+    }
+    plan_ = it->second.get();
+    return true;
+}
+
+cudaError_t Chain::run_op(const Dev &D, int i, cudaStream_t st, unsigned long long *count) {
+    return run(D, plan_->ops[i], D.K1, ChainLaunch{st, false, count});
+}
+
+cudaError_t Chain::step(const Dev &D, cudaStream_t st, bool graph, bool overlap, unsigned long long *count) {
+    cudaError_t e;
+    if (graph) {
+        // a stream that is being captured by the caller takes the kernels themselves
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if ((e = cudaStreamIsCapturing(st, &cs)) != cudaSuccess) return e;
+        if (cs != cudaStreamCaptureStatusNone) graph = false;
+    }
+    if (!graph) {
+        const ChainLaunch L{st, overlap, count};
+        for (const ChainOp &op : plan_->ops)
+            if ((e = run(D, op, D.K1, L)) != cudaSuccess) return e;
+        return cudaSuccess;
+    }
+    StepPlan &p = *plan_;
+    if (!p.exec) {
+        if (!record_ && (e = cudaStreamCreateWithFlags(&record_, cudaStreamNonBlocking)) != cudaSuccess) return e;
+        if ((e = cudaStreamBeginCapture(record_, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
+        unsigned long long n = 0;
+        const ChainLaunch L{record_, true, &n};
+        for (const ChainOp &op : p.ops)
+            if ((e = run(D, op, D.K1, L)) != cudaSuccess) break;
+        const cudaError_t end = cudaStreamEndCapture(record_, &p.graph);
+        if (e != cudaSuccess) return e;
+        if (end != cudaSuccess) return end;
+        if ((e = cudaGraphInstantiate(&p.exec, p.graph, 0)) != cudaSuccess) return e;
+        p.kernels = n;
+    }
+    *count += p.kernels;
+    return cudaGraphLaunch(p.exec, st);
+}
+
+cudaError_t Chain::ingest(const Dev &D, int n, cudaStream_t st, unsigned long long *count) {
+    // chunks of as many positions of every sequence as fit 128 token rows, of equal length
+    const int most = std::max(1, kMaxTokens / D.B), chunks = (n + most - 1) / most, t = (n + chunks - 1) / chunks;
+    std::vector<ChainOp> ops;
+    if (!build(D, t, true, ops)) return cudaErrorInvalidValue;
+    plan_ahead(ops);
+    const ChainLaunch L{st, true, count};
+    cudaError_t e;
+    for (int pos = 0; pos < n; pos += t) {
+        for (ChainOp &op : ops) {
+            op.attn.pos0 = op.proj.pos0 = pos;
+            op.attn.pos_end = op.proj.pos_end = n;
+            if ((e = run(D, op, t, L)) != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+}  // namespace xsm

@@ -1,0 +1,131 @@
+// The launch chain: one decoding step (or one chunk of a prompt) as a sequence of kernels on one stream, each launched
+// with programmatic stream serialization so that it starts, and fetches what does not depend on the step, while its
+// predecessor still runs.
+#pragma once
+#include "xsm_common.cuh"
+
+#include <stddef.h>
+
+namespace xsm {
+
+// what a projection does with its dot products
+enum ProjEpilogue : int {
+    PE_QKV = 0,       // self-attention: rotated, scaled queries as fp16 planes; rotated keys and values into the cache
+    PE_ADD = 1,       // residual stream: h += y, and h * (next RMSNorm gain) as bf16 planes, with its sums of squares
+    PE_QUERY = 2,     // cross-attention queries, scaled, as fp16 planes
+    PE_GATEUP = 3,    // SiLU(gate) * up as bf16 planes
+    PE_LOGITS = 4,    // fp32
+    PE_HEADY = 5,     // g + SiLU(y) as bf16 planes (MLP decoding head)
+    PE_HEADADD = 6    // g + y as bf16 planes (cross-attention decoding head)
+};
+
+constexpr int kProjRing = 16;         // most operand blocks of one kind that a CTA keeps in shared memory
+
+// A group of weight matrices of one shape in a projection stage: one matrix, or one per decoding head.
+struct ProjGroup {
+    int units, jobs, ld;              // output units of one matrix; matrices; row length of the output
+    int job_tiles, tiles;             // row tiles of one matrix, of the group
+    bf16 *out;                        // planes of ld columns (a set per decoding head; layout: xsm_proj.cuh)
+    float *logits;                    // PE_LOGITS: [jobs][M][ld]
+    const bf16 *w;                    // first matrix (few token rows: read without tensor maps)
+    size_t w_stride;                  // elements from one matrix of the group to the next
+};
+
+struct ProjArgs {
+    int epi0, epi1;                   // of the two groups; epi1 < 0: one group
+    int stage;                        // index of the kernel in its chain
+    int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8)
+    int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
+    int S, tps;                       // CTAs per cluster (cuts of the columns), token rows each of them finishes
+    int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns
+    int norm, ss_parts;               // the input is an RMSNorm input; shares of its sums of squares (0: not needed)
+    int z_jobs, x_jobs;               // group 0 has one matrix per decoding head; the activations too
+    const bf16 *x;                    // planes of kdim columns (x_jobs: a set per decoding head)
+    int upc, ctas;                    // few token rows: units (pairs of rows) per CTA, CTAs (per decoding head with x_jobs)
+    int slots, chunk;                 // weight tiles in shared memory, columns of one
+    int late_go;                      // let the next kernel start only after this one's wait
+    float scale;                      // queries
+    const char *ahead[2];             // weights that a later kernel of the step reads: fetched into L2 meanwhile
+    unsigned ahead_bytes[2];
+    const void *gain;                 // PE_ADD: gain of the RMSNorm that reads h next; PE_HEADY / PE_HEADADD: of the final RMSNorm
+    __half *q;                        // PE_QKV, PE_QUERY: planes [2][Mp][d] (a set per decoding head)
+    ProjGroup g[2];
+};
+
+// Attention of a stage: t query rows of every sequence against the cached keys of the sequence (self) or of the condition.
+struct AttnArgs {
+    int stage;
+    int cross, sets, layer;           // sets: decoding heads that attend in this stage (cross-attention heads), else 1
+    int t, rows, Mp, pos0, pos_end;   // as in ProjArgs
+    int S, split, slots;              // most CTAs per (sequence, head), keys for each; page pairs in shared memory
+    float *part;                      // partial results [items][S][t][d_head + 2]
+    int *count;                       // [items] CTAs that have left theirs (zero between kernels)
+    const void *pool;                 // cache tiles
+    const __half *q;                  // planes [2][Mp][d] (a set per decoding head)
+    bf16 *out;                        // planes of d columns (a set per decoding head; layout: xsm_proj.cuh)
+};
+
+// How the kernels of a chain are launched.
+struct ChainLaunch {
+    cudaStream_t stream;
+    bool overlap;                     // programmatic stream serialization
+    unsigned long long *count;        // launches
+
+    template <typename... Args>
+    cudaError_t launch(dim3 grid, dim3 block, int smem, int cluster, const void *fn, const Args &...args) const {
+        cudaLaunchConfig_t c = {};
+        c.gridDim = grid;
+        c.blockDim = block;
+        c.dynamicSmemBytes = (size_t)smem;
+        c.stream = stream;
+        cudaLaunchAttribute at[2];
+        int n = 0;
+        if (overlap) {
+            at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[n++].val.programmaticStreamSerializationAllowed = 1;
+        }
+        if (cluster > 1) {
+            at[n].id = cudaLaunchAttributeClusterDimension;
+            at[n].val.clusterDim.x = (unsigned)cluster;
+            at[n].val.clusterDim.y = 1;
+            at[n++].val.clusterDim.z = 1;
+        }
+        c.attrs = at;
+        c.numAttrs = (unsigned)n;
+        void *p[] = {const_cast<void *>(static_cast<const void *>(&args))...};
+        ++*count;
+        return cudaLaunchKernelExC(&c, fn, p);
+    }
+};
+
+// opens a kernel for `smem` bytes of dynamic shared memory (and for clusters of more than eight CTAs) on the current device
+cudaError_t open_kernel(const void *fn, int smem, bool large_cluster);
+
+// Instance of the projection over few token rows that serves `rows` token rows and rows of kdim weights: warps that
+// multiply, tiles of eight token rows, columns of one pass
+struct FewShape { int warps, nt, blocks, pass; bool pack; };
+constexpr int kFewRows = 16;
+inline FewShape few_shape(int rows, int kdim) {
+    FewShape f;
+    f.pack = rows <= 4;
+    f.nt = rows <= 8 ? 1 : 2;
+    f.warps = kdim > 2048 ? 15 : 8;
+    f.blocks = kdim > 2048 ? (f.nt == 1 ? 9 : 4) : kdim > 1024 ? 8 : 4;
+    f.pass = f.warps * f.blocks * 32;
+    return f;
+}
+cudaError_t launch_proj_few(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L);
+int resident_clusters(int size);      // clusters of the projection below that the device runs at a time, an SM for each CTA
+cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L);
+cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
+cudaError_t launch_tail(const Dev &D, int stage, const ChainLaunch &L);
+// embeds the window of every sequence (pos0 < 0) or t prompt tokens of each from position pos0 on
+cudaError_t launch_embed_rows(const Dev &D, int t, int Mp, int pos0, const ChainLaunch &L);
+// state of a new request: pool, sequences with prompt_len - 1 positions in the cache, first window
+cudaError_t launch_begin(const Dev &D, const RunParams &R, cudaStream_t st);
+// single stages (inspection): waits until the stages before `stage` have run one by one; notes that `done` of them have
+cudaError_t launch_stage_gate(const Dev &D, int stage, cudaStream_t st);
+cudaError_t launch_stage_mark(const Dev &D, int done, cudaStream_t st);
+cudaError_t launch_set_run(const Dev &D, const RunParams &R, cudaStream_t st);
+
+}  // namespace xsm

@@ -98,6 +98,19 @@ constexpr int kUmmaActsBytes = 4 * kUmmaPlaneBytes;        // two buffers of two
 
 constexpr int kSmallRedBytes = 512;   // at most eight token rows: partial products of one warp for one tile, [8 tokens][16 rows] floats
 
+// What a request may change without changing the launch chain (which is recorded once): kept in device memory.
+struct RunParams {
+    int verify_mode, k_accept, sample_mode, k_sample;
+    float delta, temperature;
+    uint32_t key0, key1;
+    int max_new, prompt_len;
+    int request;                   // number of the request: what the host is told when every sequence has ended
+    // scripted drafts (load generator of the benchmark): null, or [B][script_n] tokens by absolute position; the commit
+    // then drafts script tokens, of which the first floor((t+1) a) - floor(t a) are left intact at step t (a = script_acc / 1024)
+    const int *script;
+    int script_n, script_acc;
+};
+
 // Everything a kernel needs; passed by value.
 struct Dev {
     // shape
@@ -148,6 +161,17 @@ struct Dev {
     float *sspub;                  // [grid][M] bf16 models: each CTA's share of the sum of squares of the rows of hpub
     const void *gain_first;        // RMSNorm gain that the first stage of a step applies to the embeddings
     unsigned long long *trace;     // null, or [1 + 2 * n_stages][grid] nanosecond timestamps of the launch's first step
+    // launch chain (bf16 models): activations as hi and lo planes of Mp rows: bf16 (layout: xsm_proj.cuh), queries fp16 [2][Mp][d]
+    RunParams *rp;
+    int *host_done;                // host memory: the last request of which every sequence has ended
+    int *stage_word;               // single stages (inspection): stages of the current step that have run
+    int Mp, tail_row_bytes;        // rows of a plane for a step of the batch; largest logits row that the tail keeps in shared memory
+    void *xa_;                     // the residual stream times the gain of the RMSNorm that reads it next (bf16)
+    void *qp_, *aa_, *actp_, *yp_; // queries, attention rows, gated activations, decoding heads' hidden states (a set per head)
+    void *hq_, *ha_;               // cross-attention heads: queries, attention rows (a set per head)
+    float *apart;                  // attention: partial results of the key splits; acount: splits that have left theirs
+    int *acount;
+    float *ss;                     // [kMaxTokens][kShareLd] shares of the sums of squares of the rows of h
     // untagged
     float *h;                      // master copy of the residual stream (each column range has one owner CTA)
     float2 *rope_cs;               // [max_seq_len + K + 2][dh/2] cos, sin of position * theta^(-2i/dh)

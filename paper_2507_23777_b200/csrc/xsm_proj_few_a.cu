@@ -1,0 +1,9 @@
+// Instances of the projections over few token rows.
+#include "xsm_proj_few.cuh"
+
+namespace xsm {
+
+cudaError_t few_8_1_p_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, true, 4>(D, A, smem, L); }
+cudaError_t few_8_1_n_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, false, 4>(D, A, smem, L); }
+
+}  // namespace xsm

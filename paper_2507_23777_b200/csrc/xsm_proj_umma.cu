@@ -1,0 +1,338 @@
+// Projections of bf16 models on the tensor cores of the 5th generation (tcgen05), as kernels of the launch chain.
+//
+// y[m][u] = W[u] . x[m] for the token rows m of a step (or of a chunk of the prompt).  The weight rows are the M side of the
+// product (128 rows a tile, one accumulator lane each), the token rows the N side, twice: the activations are fp32 values
+// split into bf16 hi + lo, published by their writer as two planes, and the two products are added after the fact, so
+// nothing of the activations is lost and a weight tile serves all token rows in one pass.  A tile's columns are cut over
+// the S CTAs of a cluster (a step has at most 128 token rows, so the row tiles alone would leave most of the chip idle).
+// Each of them hands the partial sums of a share of the token rows to the CTA that finishes those rows, straight from the
+// accumulator (asynchronous 16-byte stores that count on the receiver's barrier), and they are added in rank order:
+// results do not depend on timing.
+//
+// Weights do not depend on the rest of the step: their copies start before the kernel waits for its predecessor.
+#include "xsm_proj.cuh"
+
+#include <cuda.h>
+
+namespace xsm {
+
+constexpr int kProjThreads = 512;
+constexpr int kBlockK = 64;                        // columns of one operand block (128 bytes: one swizzled row)
+constexpr int kABytes = 128 * kBlockK * 2;         // weight block
+
+struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate), group 1 (or up)
+
+template <int EPI0, int EPI1>
+__global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
+    extern __shared__ char smem_raw[];
+    char *const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);      // (swizzled tiles: 1024-byte boundaries)
+    __shared__ __align__(8) uint64_t bars[4 * kProjRing + 1];      // A full, A empty, B full, B empty, done
+    __shared__ __align__(8) uint64_t recv_bar;                      // the peers' shares of this CTA's token rows
+    __shared__ uint32_t tmem_slot;
+    __shared__ float s_inv[kMaxTokens];
+    __shared__ int s_pos[kMaxTokens], s_swz[kMaxTokens];
+    __shared__ long long s_cache[kMaxTokens];
+    constexpr bool TWO = EPI0 == PE_GATEUP;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int S = A.S, rank = S > 1 ? (int)cluster_rank() : 0, Mp = A.Mp;
+    if (A.pos0 < 0 && !A.late_go && __ldcg(D.n_active) == 0) {      // every sequence has ended in an earlier step
+        chain_wait();
+        return;
+    }
+    int tile = blockIdx.x / S, job = 0, z = A.layer, grp = 0;
+    if (EPI1 >= 0 && tile >= A.g[0].tiles) {
+        tile -= A.g[0].tiles;
+        grp = 1;
+    }
+    const ProjGroup &G = A.g[grp];
+    if (EPI1 >= 0 || A.z_jobs) {          // the matrices of a group (one per decoding head) share its map, one behind the other
+        z = job = grp == 1 || A.z_jobs ? tile / G.job_tiles : 0;
+        tile -= job * G.job_tiles;
+    }
+    const int u0 = tile * (TWO ? 64 : 128);
+    const int nblk = A.kdim / kBlockK, k_lo = rank * nblk / S, n = (rank + 1) * nblk / S - k_lo;
+    const int na = A.na, nb = A.nb;
+    const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, A.rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
+    const uint32_t b_bytes = (uint32_t)(2 * Mp) * kBlockK * 2u;
+    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = sb + (uint32_t)nb * b_bytes;
+    float *recv = reinterpret_cast<float *>(smem + (srecv - sa));
+    auto bar = [&](int kind, int i) { return smem_u32(&bars[kind * kProjRing + i]); };
+    const uint32_t done = smem_u32(&bars[4 * kProjRing]);
+    if (tid == 0) {
+        for (int i = 0; i < na; ++i) { mbar_init(bar(0, i), 1u); mbar_init(bar(1, i), 1u); }
+        for (int i = 0; i < nb; ++i) { mbar_init(bar(2, i), 1u); mbar_init(bar(3, i), 1u); }
+        mbar_init(done, 1u);
+        mbar_init(smem_u32(&recv_bar), 1u);
+        mbar_init_fence();
+        if (S > 1 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)((S - 1) * ((nm + 3) >> 2)) * 2048u);
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tcgen05_before_sync();
+    __syncthreads();
+    tcgen05_after_sync();
+    // (the tensor memory is taken before the next kernel may start: kernels further down the chain can then never hold
+    // columns that this one still waits for)
+    if (!A.late_go) chain_go();
+    if (S > 1) cluster_arrive();          // "this CTA runs": peers may write to its shared memory after cluster_wait
+    const void *wmap = grp == 1 ? &T.w1 : &T.w0;
+    auto load_a = [&](int i) {
+        const uint32_t dst = sa + (uint32_t)(i % na) * kABytes, b = bar(0, i % na);
+        const int x = (k_lo + i) * kBlockK;
+        mbar_arrive_expect_tx(b, kABytes);
+        if (TWO) {
+            tma_box(dst, &T.w0, x, u0, z, b);
+            tma_box(dst + kABytes / 2, &T.w1, x, u0, z, b);
+        } else {
+            tma_box(dst, wmap, x, u0, z, b);
+        }
+    };
+    if (tid == 0)
+        for (int i = 0; i < min(n, na); ++i) load_a(i);
+    if (warp == 3) fetch_ahead(A, blockIdx.x, gridDim.x);
+    if (A.stage == 0) trace_mark(D, 0);
+    const bf16 *x = A.x + (A.x_jobs ? (size_t)job * 2 * Mp * A.kdim : 0);
+    chain_wait();
+    if (A.late_go) chain_go();
+    trace_mark(D, 1 + 2 * A.stage);
+    if (tid == 0) {
+        fence_proxy_async();              // the activations were written by ordinary stores
+        for (int i = 0; i < n; ++i) {
+            if (i >= nb) mbar_wait(bar(3, i % nb), (uint32_t)((i / nb - 1) & 1), D.mbar_limit, D.status);
+            const uint32_t b = bar(2, i % nb);
+            mbar_arrive_expect_tx(b, b_bytes);
+            bulk_g2s(sb + (uint32_t)(i % nb) * b_bytes, x + (size_t)(k_lo + i) * (128 * Mp), b_bytes, b);
+            if (i >= na) {
+                mbar_wait(bar(1, i % na), (uint32_t)((i / na - 1) & 1), D.mbar_limit, D.status);
+                load_a(i);
+            }
+        }
+    } else if (tid == 32) {
+        const uint32_t idesc = umma_idesc(128, 2 * Mp), tmem = tmem_slot;
+        for (int i = 0; i < n; ++i) {
+            mbar_wait(bar(0, i % na), (uint32_t)((i / na) & 1), D.mbar_limit, D.status);
+            mbar_wait(bar(2, i % nb), (uint32_t)((i / nb) & 1), D.mbar_limit, D.status);
+            tcgen05_after_sync();
+            const uint64_t da = umma_desc_sw128(sa + (uint32_t)(i % na) * kABytes), db = umma_desc_sw128(sb + (uint32_t)(i % nb) * b_bytes);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, da + 2 * ks, db + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
+            if (i + na < n) umma_commit(bar(1, i % na));
+            if (i + nb < n) umma_commit(bar(3, i % nb));
+        }
+        umma_commit(done);
+    }
+    // meanwhile: what the epilogue needs to know of the token rows that this CTA finishes
+    if (warp >= 2) {
+        for (int i = tid - 64; i < nm; i += kProjThreads - 64) {
+            const int m = m0 + i;
+            float inv = 1.f;
+            if (A.ss_parts > 0) {
+                float ss = 0.f;
+                const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)m * kShareLd);
+                for (int p0 = 0; p0 < A.ss_parts; p0 += 32) {        // 32 shares in flight, added in order
+                    float4 v[8];
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) v[p] = p0 + 4 * p < A.ss_parts ? __ldcg(sh + (p0 >> 2) + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        const int k = A.ss_parts - p0 - 4 * p;       // (the last quad may hold shares that nobody writes)
+                        ss += (v[p].x + (k > 1 ? v[p].y : 0.f)) + ((k > 2 ? v[p].z : 0.f) + (k > 3 ? v[p].w : 0.f));
+                    }
+                }
+                inv = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+            }
+            s_inv[i] = inv;
+            if (EPI0 == PE_QKV) {
+                const int b = m / A.t, j = m - b * A.t;
+                const int pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + j;
+                const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
+                const int page = live ? __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos)) : 0, rp = row_in_page(D, pos);
+                s_pos[i] = live ? pos : 0;
+                s_cache[i] = live ? ((long long)page * D.H * D.P + rp) * D.dh : -1;      // place of head 0 in a page set
+                s_swz[i] = D.dh >= 64 ? rp & 7 : (rp >> 1) & 3;
+            }
+        }
+    }
+    // The epilogue takes four token rows (a quad) of a weight row at a time; what it reads from memory is requested before the
+    // products are waited for, or a round ahead.
+    constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
+    constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
+    const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
+    const bool live_row = u_row < G.units;
+    const float gain = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u_row)) : 0.f;
+    float hn[4];
+    float2 csn[4];
+    auto request = [&](int quad) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = 4 * quad + q;
+            if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(m0 + i) * D.d + u_row);
+            if (EPI0 == PE_QKV && i < nm) csn[q] = __ldg(D.rope_cs + (size_t)s_pos[i] * half + (e < half ? e : e - half));
+        }
+    };
+    __syncwarp();
+    if (EPI0 == PE_QKV) __syncthreads();      // the rows' positions
+    request(side);
+    mbar_wait(done, 0u, D.mbar_limit, D.status);
+    __syncwarp();
+    tcgen05_after_sync();
+    if (S > 1) cluster_wait();                // the peers run: their barriers and shared memory are there
+    {
+        // accumulator -> the CTA that finishes the token rows, hi and lo parts added: [sender][quad][weight row][4]
+        const int lanes = warp & 3, r = lanes * 32 + lane;               // this thread's accumulator lane = weight row
+        const uint32_t tbase = tmem_slot + ((uint32_t)(lanes * 32) << 16);
+        for (int c = warp >> 2; c < (Mp >> 3); c += kProjThreads / 128) {
+            uint32_t v[16];
+            tmem_ld16(v, tbase + (uint32_t)c * 16u);
+            tmem_wait_ld();
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int quad = 2 * c + q;
+                if (quad * 4 < A.rows) {
+                    float f[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
+                    const int owner = S > 1 ? quad / qps : 0, place = rank * qps + quad - owner * qps;
+                    if (owner == rank) {
+                        *reinterpret_cast<float4 *>(recv + (size_t)(place * 128 + r) * 4) = make_float4(f[0], f[1], f[2], f[3]);
+                    } else {
+                        st_async_v4(map_rank(srecv + (uint32_t)(place * 128 + r) * 16u, (uint32_t)owner), f, map_rank(smem_u32(&recv_bar), (uint32_t)owner));
+                    }
+                }
+            }
+        }
+    }
+    tcgen05_before_sync();
+    __syncthreads();
+    if (warp == 2) {
+        tcgen05_after_sync();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
+    }
+    if (S > 1 && nm > 0) mbar_wait(smem_u32(&recv_bar), 0u, D.mbar_limit, D.status);
+    __syncwarp();
+    // sums over the cluster in rank order, epilogue
+    auto total = [&](int quad, int r, float (&o)[4]) {
+        const float4 *p = reinterpret_cast<const float4 *>(recv) + quad * 128 + r;
+        float4 v = p[0];
+        for (int s = 1; s < S; ++s) {
+            const float4 w = p[s * qps * 128];
+            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
+        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+    };
+    // where this thread's weight row goes
+    const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
+    __half *qrow = A.q + (size_t)job * 2 * Mp * D.d + (EPI0 == PE_QKV ? col : u_row);
+    bf16 *xrow = G.out + (size_t)job * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
+    const int xchunk = (u_row >> 3) & 7;
+    float *lrow = G.logits + (size_t)job * D.M * G.ld + u_row;
+    __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
+    auto put_x = [&](int m, float v) {
+        bf16 hi, lo;
+        split_bf16(v, hi, lo);
+        bf16 *p = xrow + (m >> 3) * 1024 + (m & 7) * 64 + ((xchunk ^ (m & 7)) << 3);
+        p[0] = hi;
+        p[512] = lo;
+    };
+    auto put_q = [&](int m, float v) {
+        __half hi, lo;
+        split_f16(v * A.scale, hi, lo);
+        qrow[(size_t)m * D.d] = hi;
+        qrow[(size_t)(Mp + m) * D.d] = lo;
+    };
+    for (int quad = side; 4 * quad < nm; quad += SIDES) {
+        float h[4], v[4], w[4];
+        float2 cs[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
+        request(quad + SIDES);
+        total(quad, row, v);
+        if (EPI0 == PE_QKV) total(quad, e < half ? row + half : row - half, w);
+        if (TWO) total(quad, row + 64, w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = 4 * quad + q, m = m0 + i;
+            if (i >= nm) break;
+            if (EPI0 == PE_ADD) {
+                const float o = live_row ? h[q] + v[q] : 0.f;
+                if (live_row) {
+                    D.h[(size_t)m * D.d + u_row] = o;
+                    put_x(m, o * gain);
+                }
+                const float ssq = warp_sum(o * o);
+                if (lane == 0) D.ss[(size_t)m * kShareLd + tile * 4 + (row >> 5)] = ssq;
+            } else if (live_row) {
+                const float inv = s_inv[i], x1 = v[q] * inv;
+                if (EPI0 == PE_QKV) {
+                    const float x2 = w[q] * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
+                    if (sec == 0) put_q(m, o);
+                    else if (s_cache[i] >= 0) crow[s_cache[i] + (((e >> 3) ^ s_swz[i]) << 3)] = from_f<__half>(o);
+                } else if (TWO) {
+                    put_x(m, silu_f(x1) * (w[q] * inv));
+                } else if (EPI0 == PE_QUERY || (EPI1 == PE_QUERY && grp == 1)) {
+                    put_q(m, x1);
+                } else if (EPI0 == PE_HEADADD) {
+                    put_x(m, h[q] * inv * gain + v[q]);
+                } else if (EPI1 == PE_HEADY && grp == 1) {
+                    put_x(m, h[q] * inv * gain + silu_f(x1));
+                } else {
+                    lrow[(size_t)m * G.ld] = A.norm ? x1 : v[q];
+                }
+            }
+        }
+    }
+    if (S > 1) { cluster_arrive(); cluster_wait(); }      // (what this CTA sent has been received before its peers leave)
+    if (D.trace != nullptr) {
+        __syncthreads();
+        trace_mark(D, 2 + 2 * A.stage);
+    }
+}
+
+template <int EPI0, int EPI1>
+static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
+    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1>;
+    cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
+    if (e != cudaSuccess) return e;
+    const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
+    return L.launch(dim3(tiles * A.S), dim3(kProjThreads), smem, A.S, (const void *)fn, D, A, T);
+}
+
+int resident_clusters(int size) {
+    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1>;
+    constexpr int smem = 200 * 1024;
+    int n = 0;
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)size;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.gridDim = dim3(size);
+    c.blockDim = dim3(kProjThreads);
+    c.dynamicSmemBytes = smem;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    if (open_kernel(fn, smem, false) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, fn, &c) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L) {
+    const ProjMaps &T = *reinterpret_cast<const ProjMaps *>(maps);
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_instance<a, b>(D, A, T, smem, L)
+    XSM_EPI(PE_QKV, -1);
+    XSM_EPI(PE_ADD, -1);
+    XSM_EPI(PE_QUERY, -1);
+    XSM_EPI(PE_GATEUP, -1);
+    XSM_EPI(PE_LOGITS, -1);
+    XSM_EPI(PE_LOGITS, PE_HEADY);
+    XSM_EPI(PE_LOGITS, PE_QUERY);
+    XSM_EPI(PE_HEADADD, -1);
+#undef XSM_EPI
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace xsm

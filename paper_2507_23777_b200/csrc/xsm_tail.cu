@@ -1,0 +1,503 @@
+// The end of a decoding step and the start of a request, as kernels of the launch chain: verification of the drafts,
+// resampling, commit and the embedding of the next window; the state of a new request; the embedding of prompt tokens.
+#include "xsm_proj.cuh"
+
+namespace xsm {
+
+constexpr int kTailThreads = 256, kTailWarps = kTailThreads / 32;
+constexpr int kMaxCand = 64;
+
+__device__ __forceinline__ uint32_t rand24(const RunParams &R, int seq, uint32_t step, uint32_t slot, uint32_t purpose) {
+    return philox_word0(step, slot, purpose, 0u, R.key0 ^ (uint32_t)seq, R.key1) >> 8;
+}
+
+// ---------------------------------------------------------------------------------------- embedding
+
+// Row m of the window <- the embedding of `tok`: master copy, planes (times the gain of the first RMSNorm) and sum of squares.
+// All threads of the block; d / 8 <= kTailThreads.
+static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, float *sh) {
+    const bf16 *E = reinterpret_cast<const bf16 *>(D.E), *gain = reinterpret_cast<const bf16 *>(D.gain_first);
+    const int c = threadIdx.x * 8, d = D.d;
+    float ssq = 0.f;
+    if (c < d) {
+        tok = min(max(tok, 0), D.V - 1);
+        const uint4 ev = __ldg(reinterpret_cast<const uint4 *>(E + (size_t)tok * d + c)), gv = __ldg(reinterpret_cast<const uint4 *>(gain + c));
+        const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
+        float v[8];
+        __align__(16) bf16 hi[8], lo[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            v[q] = __uint_as_float((q & 1) ? ew[q >> 1] & 0xFFFF0000u : ew[q >> 1] << 16);
+            const float g = __uint_as_float((q & 1) ? gw[q >> 1] & 0xFFFF0000u : gw[q >> 1] << 16);
+            split_bf16(v[q] * g, hi[q], lo[q]);
+            ssq += v[q] * v[q];
+        }
+        float4 *h = reinterpret_cast<float4 *>(D.h + (size_t)m * d + c);
+        h[0] = make_float4(v[0], v[1], v[2], v[3]);
+        h[1] = make_float4(v[4], v[5], v[6], v[7]);
+        bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + plane_off(Mp, m, c);
+        *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
+        *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
+    }
+    ssq = warp_sum(ssq);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ssq;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float s = 0.f;
+        for (int w = 0; w < kTailWarps; ++w) s += sh[w];
+        D.ss[(size_t)m * kShareLd] = s;      // the only share
+    }
+}
+
+__global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0) {
+    __shared__ float sh[kTailWarps];
+    chain_wait();
+    chain_go();      // (only now: kernels further down may read what earlier chunks wrote before they wait themselves)
+    const int b = blockIdx.x / t, j = blockIdx.x - b * t;
+    int tok;
+    if (pos0 >= 0) {
+        const int n = D.rp->prompt_len;
+        tok = pos0 + j < n ? D.prompt[(size_t)b * n + pos0 + j] : 0;
+    } else {
+        if (__ldcg(D.finished + b)) return;
+        tok = __ldcg(D.window + b * t + j);
+    }
+    embed_row(D, blockIdx.x, Mp, tok, sh);
+}
+cudaError_t launch_embed_rows(const Dev &D, int t, int Mp, int pos0, const ChainLaunch &L) {
+    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, (const void *)embed_rows_kernel, D, t, Mp, pos0);
+}
+
+// ------------------------------------------------------------------------------------ block reductions
+
+static __device__ float block_sum(float v, float *sh) {
+    v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kTailWarps; ++w) s += sh[w];
+    return s;
+}
+static __device__ float block_max(float v, float *sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    float s = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kTailWarps; ++w) s = fmaxf(s, sh[w]);
+    return s;
+}
+// (logit, token) as one 64-bit key whose unsigned order is the ranking: larger logit first, then smaller token.
+// 0 is below every key ("no candidate").  -0.0 ranks with +0.0.
+__device__ __forceinline__ unsigned long long rank_key(float z, int idx) {
+    uint32_t u = __float_as_uint(z + 0.0f);
+    u ^= (u & 0x80000000u) ? 0xFFFFFFFFu : 0x80000000u;
+    return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)idx);
+}
+__device__ __forceinline__ float key_logit(unsigned long long k) {
+    uint32_t u = (uint32_t)(k >> 32);
+    u ^= (u & 0x80000000u) ? 0x80000000u : 0xFFFFFFFFu;
+    return __uint_as_float(u);
+}
+__device__ __forceinline__ int key_token(unsigned long long k) { return (int)(0xFFFFFFFFu - (uint32_t)k); }
+// largest key over the block; every thread gets it
+static __device__ unsigned long long block_best(unsigned long long k, unsigned long long *sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
+        k = other > k ? other : k;
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
+    __syncthreads();
+    k = sh[0];
+#pragma unroll
+    for (int w = 1; w < kTailWarps; ++w) k = sh[w] > k ? sh[w] : k;
+    return k;
+}
+
+// ------------------------------------------------------------------------------- verify and resample
+
+struct TailShared {
+    float red[kTailWarps];
+    unsigned long long redk[kTailWarps];
+    float cv[kMaxCand];
+    int ci[kMaxCand];
+    int accepted;                       // of the draft behind this CTA's row
+    int tok;                            // this slot's candidate
+    int cand[kMaxDraft], win[kMaxDraft];
+    int old_win[kMaxDraft];
+    int state[8];                       // len, n_gen, step_idx, n_blocks; new len, finished
+    float tree_p[8];                    // probability tree: this head's best tokens
+    int tree_t[8];
+    double m[kMaxDraft * 8];            // the tree's tables (slot 1)
+    int tk[kMaxDraft * 8];
+    int path[kMaxDraft];
+};
+
+// copies a logits row into shared memory
+static __device__ void stage_row(const float *z, float *row, int V) {
+    __syncthreads();
+    if ((V & 3) == 0) {
+        for (int i = threadIdx.x; i < (V >> 2); i += kTailThreads)
+            reinterpret_cast<float4 *>(row)[i] = __ldcg(reinterpret_cast<const float4 *>(z) + i);
+    } else {
+        for (int i = threadIdx.x; i < V; i += kTailThreads) row[i] = __ldcg(z + i);
+    }
+    __syncthreads();
+}
+
+// acceptance of token x under backbone logits z, block-wide; every thread returns the same answer
+static __device__ bool accept_token(const Dev &D, const RunParams &R, const float *z, int x, TailShared &sh) {
+    const int V = D.V;
+    if (x < 0 || x >= V) return false;
+    if (R.verify_mode == 2) {     // p0(x) > delta
+        float m = -INFINITY;
+        for (int v = threadIdx.x; v < V; v += kTailThreads) m = fmaxf(m, z[v]);
+        m = block_max(m, sh.red);
+        float sum = 0.f;
+        for (int v = threadIdx.x; v < V; v += kTailThreads) sum += expf(z[v] - m);
+        sum = block_sum(sum, sh.red);
+        return expf(z[x] - m) / sum > R.delta;
+    }
+    const int ka = R.verify_mode == 0 ? 1 : R.k_accept;
+    const unsigned long long kx = rank_key(z[x], x);
+    int cnt = 0;
+    for (int v = threadIdx.x; v < V; v += kTailThreads) cnt += rank_key(z[v], v) > kx ? 1 : 0;
+    return (int)block_sum((float)cnt, sh.red) < ka;
+}
+
+// the k best (logit, token) pairs of z, ranked, left in sh.cv, sh.ci
+static __device__ void top_candidates(const Dev &D, const float *z, int k, TailShared &sh) {
+    const int V = D.V;
+    // every thread keeps the best of its own elements; after each pick only the thread that owned the winner
+    // looks for its next best (among its elements ranked after the winner)
+    unsigned long long mine = 0ull;
+    for (int v = threadIdx.x; v < V; v += kTailThreads) {
+        const unsigned long long kv = rank_key(z[v], v);
+        mine = kv > mine ? kv : mine;
+    }
+    for (int j = 0; j < k; ++j) {
+        const unsigned long long win = block_best(mine, sh.redk);
+        if (threadIdx.x == 0) { sh.cv[j] = key_logit(win); sh.ci[j] = key_token(win); }
+        if (win == mine && j + 1 < k) {      // mine was picked
+            mine = 0ull;
+            for (int v = threadIdx.x; v < V; v += kTailThreads) {
+                const unsigned long long kv = rank_key(z[v], v);
+                if (kv < win && kv > mine) mine = kv;
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// one candidate by inverse CDF over the ranked best (thread 0's answer counts)
+static __device__ int pick_candidate(const RunParams &R, int k, uint32_t r24, const TailShared &sh) {
+    if (R.sample_mode == 0) return sh.ci[0];
+    float total = 0.f;
+    for (int j = 0; j < k; ++j) total += expf((sh.cv[j] - sh.cv[0]) / R.temperature);
+    const float u = (float)r24 * (1.0f / 16777216.0f);
+    float cum = 0.f;
+    for (int j = 0; j < k; ++j) {
+        cum += expf((sh.cv[j] - sh.cv[0]) / R.temperature);
+        if (cum > u * total) return sh.ci[j];
+    }
+    return sh.ci[k - 1];
+}
+
+// Top-K_s probability tree over the decoding heads (Appendix, Ablation of Sampling Strategies): the leaves are the
+// K_s^K paths in lexicographic order of the heads' ranked candidates, a path weighs the product of its tokens'
+// full-vocabulary probabilities, paths whose product falls below 1e-5 are pruned, and the first leaf whose cumulative
+// weight exceeds u * total is drawn (the last surviving leaf if rounding keeps the sum below; the most probable token of
+// every head if no path survives).  One warp; m: [K][8] in shared memory.  Returns the leaf's index.
+static __device__ int tree_pick(int K, int ks, const double *m, double u) {
+    const int lane = threadIdx.x & 31;
+    int n_leaves = 1;
+    for (int d = 0; d < K; ++d) n_leaves *= ks;
+    auto weight = [&](int idx) -> double {
+        if (idx >= n_leaves) return 0.0;
+        double w = 1.0;
+        int div = n_leaves;
+        for (int d = 0; d < K; ++d) {
+            div /= ks;
+            const int k = idx / div;
+            idx -= k * div;
+            w *= m[d * 8 + k];
+            if (w < 1e-5) return 0.0;
+        }
+        return w;
+    };
+    double total = 0.0;
+    for (int base = 0; base < n_leaves; base += 32) total += weight(base + lane);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    if (!(total > 0.0)) return 0;
+    const double target = u * total;
+    double cum = 0.0;
+    int last = 0;
+    for (int base = 0; base < n_leaves; base += 32) {
+        const double w = weight(base + lane);
+        double c = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double up = __shfl_up_sync(0xffffffffu, c, o);
+            if (lane >= o) c += up;
+        }
+        c += cum;
+        const unsigned alive = __ballot_sync(0xffffffffu, w > 0.0), hit = __ballot_sync(0xffffffffu, w > 0.0 && c > target);
+        if (hit) return base + __ffs(hit) - 1;
+        if (alive) last = base + 31 - __clz(alive);
+        cum = __shfl_sync(0xffffffffu, c, 31);
+    }
+    return last;
+}
+
+static __device__ void draw_initial_drafts(const Dev &D, const RunParams &R, int b, int *win) {
+    for (int i = 1; i <= D.K; ++i) {
+        const unsigned long long m = rand24(R, b, 0u, (uint32_t)i, 1u);
+        win[i] = (int)((m * (unsigned long long)D.V) >> 24);
+    }
+}
+
+// pages for positions < len + K + 1 of sequence b (one thread)
+static __device__ void reserve_pages(const Dev &D, int b, int len, int held) {
+    const int need = page_of(D, len + D.K1 + D.P - 1);
+    int nb = held;
+    while (nb < need) {
+        const int idx = atomicSub(D.n_free, 1) - 1;
+        if (idx < 0 || nb >= D.max_blocks) {
+            atomicAdd(D.n_free, 1);
+            atomicExch(D.status, XSM_STATUS_CAPACITY);
+            break;
+        }
+        __stcg(D.block_table + (size_t)b * D.max_blocks + nb, __ldcg(D.free_stack + idx));
+        ++nb;
+    }
+    if (nb != held) __stcg(D.n_blocks + b, nb);
+}
+
+// Algorithm 1 lines 7-12 for one sequence by a cluster of K + 1 CTAs, one per window row and slot: CTA j < K decides on
+// the draft behind row j; with the accept length a known to all, CTA i draws candidate i from row a of the backbone (i = 0)
+// or of head i; every CTA works out the commit, CTA 0 writes it down, and CTA i embeds row i of the next window.
+__global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int stage) {
+    extern __shared__ __align__(16) float row_buf[];
+    __shared__ TailShared sh;
+    const int K1 = D.K1, K = D.K, V = D.V, tid = threadIdx.x;
+    const int b = blockIdx.x / K1, slot = blockIdx.x - b * K1;
+    const bool staged = (size_t)V * 4 <= (size_t)D.tail_row_bytes;      // else the rows are read where they are
+    chain_go();
+    const RunParams &R = *D.rp;
+    if (__ldcg(D.finished + b)) {
+        chain_wait();
+        if (slot == 0 && tid == 0) __stcg(D.step_n_new + b, 0);
+        return;
+    }
+    if (tid == 32) sh.state[0] = __ldcg(D.len + b);
+    if (tid == 33) sh.state[1] = __ldcg(D.n_gen + b);
+    if (tid == 34) sh.state[2] = (int)__ldcg(D.step_idx + b);
+    if (tid == 35) sh.state[3] = __ldcg(D.n_blocks + b);
+    if (tid >= 64 && tid < 64 + K1) sh.old_win[tid - 64] = __ldcg(D.window + b * K1 + tid - 64);
+    chain_wait();
+    trace_mark(D, 1 + 2 * stage);
+    __syncthreads();
+    const float *z = D.logits0 + (size_t)(b * K1 + slot) * V;
+    int a = 0;
+    if (K > 0) {
+        if (slot < K) {
+            const float *row = z;
+            if (staged) { stage_row(z, row_buf, V); row = row_buf; }
+            const bool ok = accept_token(D, R, row, sh.old_win[slot + 1], sh);
+            if (tid == 0) sh.accepted = ok ? 1 : 0;
+        }
+        __syncthreads();
+        cluster_arrive();
+        cluster_wait();
+        int flag = 1;
+        const int lane = tid & 31;
+        if (lane < K) asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(flag) : "r"(map_rank(smem_u32(&sh.accepted), (uint32_t)lane)) : "memory");
+        const unsigned no = __ballot_sync(0xffffffffu, lane < K && flag == 0);
+        a = no ? __ffs(no) - 1 : K;
+    }
+    // candidate of this slot
+    if (slot == 0) z = D.logits0 + (size_t)(b * K1 + a) * V;
+    else z = D.hlogits + ((size_t)(slot - 1) * D.M + b * K1 + a) * V;
+    if (staged) {
+        if (!(slot == 0 && a == 0 && K > 0)) stage_row(z, row_buf, V);      // (slot 0 has row 0 already)
+        z = row_buf;
+    }
+    const bool tree = R.sample_mode == 2 && slot > 0;
+    const int k = tree ? min(max(R.k_sample, 1), min(V, 8)) : R.sample_mode == 0 ? 1 : min(max(R.k_sample, 1), min(V, kMaxCand));
+    top_candidates(D, z, k, sh);
+    if (!tree) {
+        if (tid == 0) sh.tok = pick_candidate(R, k, rand24(R, b, (uint32_t)sh.state[2], (uint32_t)slot, 0u), sh);
+    } else {
+        // probability tree: this head's K_s best tokens and their probabilities, for slot 1, which draws one path for all heads
+        const float mx = sh.cv[0];
+        float sum = 0.f;
+        for (int v = tid; v < V; v += kTailThreads) sum += expf(z[v] - mx);
+        sum = block_sum(sum, sh.red);
+        if (tid < k) {
+            sh.tree_t[tid] = sh.ci[tid];
+            sh.tree_p[tid] = expf(sh.cv[tid] - mx) / sum;
+        }
+    }
+    if (R.sample_mode == 2 && K > 0) {
+        __syncthreads();
+        cluster_arrive();
+        cluster_wait();
+        if (slot == 1) {
+            const int ks = k;
+            for (int i = tid; i < K * ks; i += kTailThreads) {
+                const int d = i / ks, j = i - d * ks;
+                sh.m[d * 8 + j] = (double)ld_cluster_f32(map_rank(smem_u32(&sh.tree_p[j]), (uint32_t)(d + 1)));
+                asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(sh.tk[d * 8 + j]) : "r"(map_rank(smem_u32(&sh.tree_t[j]), (uint32_t)(d + 1))) : "memory");
+            }
+            __syncthreads();
+            if (tid < 32) {
+                const double u = (double)rand24(R, b, (uint32_t)sh.state[2], 1u, 0u) * (1.0 / 16777216.0);
+                int leaf = tree_pick(K, ks, sh.m, u), div = 1;
+                for (int d = 0; d < K; ++d) div *= ks;
+                for (int d = 0; d < K; ++d) {
+                    div /= ks;
+                    const int kk = leaf / div;
+                    leaf -= kk * div;
+                    if (tid == 0) sh.path[d] = sh.tk[d * 8 + kk];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (K > 0) { cluster_arrive(); cluster_wait(); }
+    if (tid < K1) {
+        int v = sh.tok;
+        if (K > 0) {
+            const bool from_path = R.sample_mode == 2 && tid > 0;
+            const uint32_t src = from_path ? map_rank(smem_u32(&sh.path[tid - 1]), 1u) : map_rank(smem_u32(&sh.tok), (uint32_t)tid);
+            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(src) : "memory");
+        }
+        sh.cand[tid] = v;
+    }
+    __syncthreads();
+    // commit x_{s+1..s*}, s <- s*, next window <- candidates: worked out by every CTA, written by CTA 0
+    if (tid == 0) {
+        const bool w = slot == 0;
+        const int len0 = sh.state[0], len = len0 + a + 1;
+        // scripted drafts: the token at the first rejected position is the script's as well, so that a near-tie
+        // of the backbone's two best logits cannot take the run off the script for good
+        if (R.script != nullptr && len < R.script_n) sh.cand[0] = R.script[(size_t)b * R.script_n + len];
+        int n_gen = sh.state[1], fin = 0, n_out = 0;
+        for (int j = 0; j <= a; ++j) {
+            const int tok = j < a ? sh.old_win[j + 1] : sh.cand[0];
+            if (n_gen >= R.max_new) break;
+            if (w) {
+                __stcg(D.tok_log + (size_t)b * D.tok_ld + n_gen, tok);
+                __stcg(D.step_tokens + b * K1 + n_out, tok);
+            }
+            ++n_gen; ++n_out;
+            if (D.eos >= 0 && tok == D.eos) { fin = 1; break; }
+        }
+        if (n_gen >= R.max_new || len > D.max_seq_len) fin = 1;
+        for (int j = 0; j < K1; ++j) sh.win[j] = sh.cand[j];
+        if (R.script != nullptr) {
+            // scripted drafts: the next window drafts the script's tokens; the first `keep` stay as they
+            // are, the others are made wrong (a forced accept length for a backbone that reproduces the script)
+            const long long t = (long long)sh.state[2] + 1;
+            const int keep = (int)((((t + 1) * R.script_acc) >> 10) - ((t * R.script_acc) >> 10));
+            const int *sc = R.script + (size_t)b * R.script_n;
+            for (int j = 1; j < K1; ++j) {
+                const int pos = len + j;
+                int tok = pos < R.script_n ? sc[pos] : 0;
+                if (j > keep) tok = tok + 1 < D.V ? tok + 1 : 0;
+                sh.win[j] = tok;
+            }
+        }
+        sh.state[5] = fin;
+        if (w) {
+            for (int j = n_out; j < K1; ++j) __stcg(D.step_tokens + b * K1 + j, -1);
+            __stcg(D.step_n_new + b, n_out);
+            __stcg(D.n_gen + b, n_gen);
+            __stcg(D.step_idx + b, (uint32_t)sh.state[2] + 1u);
+            D.hist[(size_t)b * (kMaxDraft + 1) + a] += 1ull;
+            D.steps[b] += 1ull;
+            if (fin) {
+                __stcg(D.finished + b, 1);
+                if (atomicSub(D.n_active, 1) == 1) {      // the last one: tell the host which request is done
+                    __threadfence_system();
+                    *reinterpret_cast<volatile int *>(D.host_done) = R.request;
+                }
+            } else {
+                reserve_pages(D, b, len, sh.state[3]);
+            }
+            __stcg(D.len + b, len);
+            for (int j = 0; j < K1; ++j) __stcg(D.window + b * K1 + j, sh.win[j]);
+        }
+    }
+    __syncthreads();
+    if (!sh.state[5]) embed_row(D, b * K1 + slot, D.Mp, sh.win[slot], sh.red);
+    if (K > 0) { cluster_arrive(); cluster_wait(); }      // peers may still read this CTA's candidate
+    trace_mark(D, 2 + 2 * stage);
+}
+
+cudaError_t launch_tail(const Dev &D, int stage, const ChainLaunch &L) {
+    const int smem = (size_t)D.V * 4 <= (size_t)D.tail_row_bytes ? (D.V * 4 + 15) / 16 * 16 : 16;
+    cudaError_t e = open_kernel((const void *)tail_kernel, smem, D.K1 > 8);
+    if (e != cudaSuccess) return e;
+    return L.launch(dim3(D.B * D.K1), dim3(kTailThreads), smem, D.K1, (const void *)tail_kernel, D, stage);
+}
+
+// --------------------------------------------------------------------------------- start of a request
+
+// Algorithm 1 line 1: the pool, the run's parameters, and per sequence s = prompt_len - 1, its pages, the first window.
+__global__ void set_run_kernel(const Dev D, const RunParams R) { *D.rp = R; }
+__global__ void begin_pool_kernel(const Dev D, const RunParams R) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < D.n_pages) D.free_stack[i] = D.n_pages - 1 - i;
+    if (i < 256) D.acount[i] = 0;
+    if (i == 0) { *D.n_free = D.n_pages; *D.n_active = D.B; *D.status = 0; *D.stage_word = 0; *D.rp = R; }
+}
+__global__ void begin_seq_kernel(const Dev D) {
+    const int b = blockIdx.x;
+    const RunParams &R = *D.rp;
+    const int len = R.prompt_len - 1;
+    if (threadIdx.x <= kMaxDraft) D.hist[(size_t)b * (kMaxDraft + 1) + threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) {
+        int win[kMaxDraft];
+        D.len[b] = len; D.finished[b] = 0; D.n_gen[b] = 0; D.n_blocks[b] = 0; D.step_idx[b] = 0u;
+        D.steps[b] = 0ull; D.step_n_new[b] = 0;
+        win[0] = D.prompt[(size_t)b * R.prompt_len + len];
+        draw_initial_drafts(D, R, b, win);
+        for (int j = 0; j < D.K1; ++j) D.window[b * D.K1 + j] = win[j];
+        reserve_pages(D, b, len, 0);
+    }
+}
+cudaError_t launch_begin(const Dev &D, const RunParams &R, cudaStream_t st) {
+    begin_pool_kernel<<<(D.n_pages + 255) / 256, 256, 0, st>>>(D, R);
+    begin_seq_kernel<<<D.B, 32, 0, st>>>(D);
+    return cudaGetLastError();
+}
+// bounded: after D.spin_limit polls the status word is raised
+__global__ void stage_gate_kernel(const Dev D, int stage) {
+    for (unsigned n = 0; n < D.spin_limit; ++n)
+        if (__ldcg(D.stage_word) == stage) return;
+    atomicExch(D.status, XSM_STATUS_TIMEOUT);
+}
+__global__ void stage_mark_kernel(const Dev D, int done) { *D.stage_word = done; }
+cudaError_t launch_stage_gate(const Dev &D, int stage, cudaStream_t st) {
+    stage_gate_kernel<<<1, 1, 0, st>>>(D, stage);
+    return cudaGetLastError();
+}
+cudaError_t launch_stage_mark(const Dev &D, int done, cudaStream_t st) {
+    stage_mark_kernel<<<1, 1, 0, st>>>(D, done);
+    return cudaGetLastError();
+}
+cudaError_t launch_set_run(const Dev &D, const RunParams &R, cudaStream_t st) {
+    set_run_kernel<<<1, 1, 0, st>>>(D, R);
+    return cudaGetLastError();
+}
+
+}  // namespace xsm
