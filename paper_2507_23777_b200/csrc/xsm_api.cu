@@ -1,9 +1,6 @@
-// Host side of the C ABI declared in include/xsm.h: argument checks, workspace layout, phase tables,
-// launches.  No device memory is allocated here; everything lives in the caller's workspace.
+// Host side of the C ABI declared in include/xsm.h: argument checks, workspace layout, requests.  No device memory is allocated here; everything lives in the caller's workspace.
 #include "../../include/xsm.h"
 #include "xsm_host.h"
-
-#include <cuda.h>
 
 #include <limits.h>
 #include <math.h>
@@ -18,24 +15,19 @@ using namespace xsm;
 
 namespace {
 
-constexpr int kSizingGrid = 256;      // CTA count assumed when sizing split-partial buffers and per-CTA marks
 constexpr int kKvStagePositions = 256;
-constexpr int kMinSlots = 5;          // ring slots the shared-memory plan keeps at least
-constexpr int kChunkSteps = 64;       // decoding steps per persistent-kernel launch in xsm_generate
 
 thread_local std::string g_create_error;
 
 struct Layout {
     size_t total = 0;
-    size_t phases, jobs, wkc_off, wvc_off, hk_off, hv_off, tmaps;
-    size_t len, window, cand, acc_len, finished, n_gen, n_blocks, ingest_left, step_idx, block_table, free_stack,
-        scalars, hist, steps, tok_log, step_tokens, step_n_new, prompt, script;
-    size_t h, rope_cs;
-    size_t xchg_begin, hpub, qkv, attn, qc, cattn, act, y, logits0, hlogits, part, cpart, candx, header, done, sspub, qh, hattn, gpub,
-        hpart, treex, xchg_end;
-    size_t rp, xa, qp, aa, actp, yp, hq, ha, ss, apart, acount;      // launch chain
+    size_t wkc_off, wvc_off, hk_off, hv_off;
+    size_t len, window, finished, n_gen, n_blocks, step_idx, block_table, free_stack, scalars, hist, steps, tok_log, step_tokens,
+        step_n_new, prompt, script;
+    size_t h, rope_cs, logits0, hlogits;
+    size_t rp, xa, qp, aa, actp, yp, hq, ha, ss, apart, acount;
     size_t stage_cond, stage_kv, stage_tok, trace, ckv_pool, hckv_pool, kv_pool;
-    int n_pages = 0, max_blocks = 0, cpages = 0, tok_ld = 0, n_phases = 0, n_jobs = 0;
+    int n_pages = 0, max_blocks = 0, cpages = 0, tok_ld = 0, n_stages = 0;
     size_t page_bytes = 0;
 };
 
@@ -55,27 +47,20 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.cpages = (int)((c.n_cond + P - 1) / P);
     L.tok_ld = c.max_seq_len + (int)K1;
     const bool ca = c.head_kind == 1 && c.n_draft > 0;
-    L.n_phases = c.n_layers * 8 + 3 + (c.n_draft > 0 ? 1 : 0) + (ca ? 2 : 0);
-    L.n_jobs = c.n_layers * 6 + 1 + (ca ? 3 : 2) * c.n_draft;
+    L.n_stages = c.n_layers * 8 + 2 + (c.n_draft > 0 ? 1 : 0) + (ca ? 2 : 0);
     size_t cur = 0;
-    L.phases = take(cur, sizeof(Tables));
-    L.jobs = take(cur, 256);
     L.wkc_off = take(cur, sizeof(size_t) * c.n_layers);
     L.wvc_off = take(cur, sizeof(size_t) * c.n_layers);
-    L.tmaps = take(cur, 128 * 2 * (size_t)(kLayerJobs + kMaxTailJobs));      // two tensor maps per job
     L.hk_off = take(cur, sizeof(size_t) * (c.n_draft + 1));
     L.hv_off = take(cur, sizeof(size_t) * (c.n_draft + 1));
     L.len = take(cur, 4 * B);
     L.window = take(cur, 4 * M);
-    L.cand = take(cur, 4 * M);
-    L.acc_len = take(cur, 4 * B);
     L.finished = take(cur, 4 * B);
     L.n_gen = take(cur, 4 * B);
     L.n_blocks = take(cur, 4 * B);
-    L.ingest_left = take(cur, 4 * B);
     L.step_idx = take(cur, 4 * B);
     L.block_table = take(cur, 4 * B * L.max_blocks);
-    L.scalars = take(cur, 256);   // n_free, n_active, status, bar
+    L.scalars = take(cur, 256);   // n_active, status, n_free, stage_word
     L.hist = take(cur, 8 * B * (kMaxDraft + 1));
     L.steps = take(cur, 8 * B);
     L.tok_log = take(cur, 4 * B * L.tok_ld);
@@ -83,51 +68,27 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.step_n_new = take(cur, 4 * B);
     L.prompt = take(cur, 4 * B * (c.max_seq_len + 1));
     L.script = take(cur, 4 * B * L.tok_ld);
-    L.h = take(cur, 4 * (size_t)kMaxTokens * d);
+    L.rp = take(cur, sizeof(RunParams));
+    // activations of a step or of a chunk of a prompt: four bytes an element (bf16 models: hi and lo parts)
+    const size_t row = 4 * (size_t)kMaxTokens, nh = ca ? (size_t)c.n_draft : 0;
+    L.h = take(cur, row * d);
     L.rope_cs = take(cur, 8 * (size_t)(c.max_seq_len + K1 + 1) * (dh / 2));
-    // tagged exchange buffers, cleared together at every xsm_prefill
-    L.xchg_begin = cur;
-    L.hpub = take(cur, 4 * M * d);
-    L.qkv = take(cur, 4 * M * 3 * d);
-    L.attn = take(cur, 4 * M * d);
-    L.qc = take(cur, 4 * M * d);
-    L.cattn = take(cur, 4 * M * d);
-    L.act = take(cur, 4 * M * f);
-    L.y = take(cur, 4 * M * d * (c.n_draft > 0 ? c.n_draft : 1));
+    L.xa = take(cur, row * d);
+    L.qp = take(cur, row * d);
+    L.aa = take(cur, row * d);
+    L.actp = take(cur, row * f);
+    L.yp = take(cur, row * d * c.n_draft);
+    L.hq = take(cur, row * d * nh);
+    L.ha = take(cur, row * d * nh);
+    L.ss = take(cur, row * kShareLd);
+    L.apart = take(cur, row * kSplitCtas * (dh + 2));
+    L.acount = take(cur, 4 * kSplitCtas);
     L.logits0 = take(cur, 4 * M * V);
     L.hlogits = take(cur, 4 * M * V * (c.n_draft > 0 ? c.n_draft : 1));
-    const size_t part_items = B * H + kSizingGrid;      // >= B * H * S_max for every batch
-    L.part = take(cur, 4 * part_items * K1 * (dh + 2));
-    L.cpart = take(cur, 4 * part_items * K1 * (dh + 2));
-    L.candx = take(cur, 4 * B * (K1 + 1));
-    L.header = take(cur, 4 * B * kHeaderWords);
-    L.done = take(cur, 4 * kSizingGrid);
-    L.sspub = take(cur, 4 * (size_t)kSizingGrid * M);
-    const size_t nh = ca ? (size_t)c.n_draft : 0;       // cross-attention heads: their own exchange buffers
-    L.qh = take(cur, 4 * M * d * nh);
-    L.hattn = take(cur, 4 * M * d * nh);
-    L.gpub = take(cur, 4 * M * d * (ca ? 1 : 0));
-    L.hpart = take(cur, 4 * nh * part_items * K1 * (dh + 2));
-    L.treex = take(cur, 4 * B * (c.n_draft > 0 ? c.n_draft : 1) * 8 * 2);
-    L.xchg_end = cur;
-    if (c.dtype == 1) {      // launch chain: planes of at most kMaxTokens token rows, twice (hi, lo), two bytes an element
-        const size_t row = 4 * (size_t)kMaxTokens;
-        L.rp = take(cur, sizeof(RunParams) + 64);
-        L.xa = take(cur, row * d);
-        L.qp = take(cur, row * d);
-        L.aa = take(cur, row * d);
-        L.actp = take(cur, row * f);
-        L.yp = take(cur, row * d * c.n_draft);
-        L.hq = take(cur, row * d * nh);
-        L.ha = take(cur, row * d * nh);
-        L.ss = take(cur, 4 * (size_t)kMaxTokens * 160);
-        L.apart = take(cur, 4 * (size_t)kSizingGrid * kMaxTokens * (dh + 2));      // (split items: at most 9/8 of the SMs)
-        L.acount = take(cur, 4 * kSizingGrid);
-    }
     L.stage_cond = take(cur, esize(c) * B * c.n_cond * c.d_cond);
     L.stage_kv = take(cur, 4 * 2 * (size_t)kKvStagePositions * d);
     L.stage_tok = take(cur, 4 * B * (c.max_seq_len + 1));
-    L.trace = take(cur, 8 * (size_t)(1 + 2 * L.n_phases) * kSizingGrid);
+    L.trace = take(cur, 8 * (size_t)(1 + 2 * L.n_stages) * kTraceCtas);
     L.ckv_pool = take(cur, esize(c) * (size_t)c.n_layers * 2 * B * L.cpages * H * P * dh);
     L.hckv_pool = take(cur, esize(c) * nh * 2 * B * L.cpages * H * P * dh);
     L.page_bytes = esize(c) * (size_t)c.n_layers * 2 * H * P * dh;
@@ -221,30 +182,20 @@ WeightOffsets weight_offsets(const xsm_model_config &c) {
 
 struct xsm_ctx {
     xsm_model_config cfg;
-    xsm_decode_config dc;
     Layout lay;
     WeightOffsets wo;
     const char *weights;
     char *ws;
-    size_t ws_bytes;
     cudaStream_t stream;
     Dev dev;
-    int grid, sm_count, smem_bytes, phase_launch, prefilled, batch;
-    uint32_t serial;          // decoding steps launched since the last xsm_prefill
-    int static_steps;         // the latest step kept its attention partials in the library's own scratch array
+    int sm_count, phase_launch, prefilled, n_stages;
     unsigned long long launches;
     std::string err;
-    Tables h_tab;
-    std::vector<CUtensorMap> h_tmaps;   // tcgen05 path: host copies of the jobs' tensor maps (uploaded by xsm_prefill)
-    int n_stages;             // stages of one decoding step
-    Chain chain;              // bf16 models: the launch chain
-    bool use_chain;
-    RunParams run;
+    Chain chain;              // the kernels of a decoding step
+    RunParams run;            // as in device memory
     int request;              // number of the latest xsm_prefill
-    void *encode_tiled;       // cuTensorMapEncodeTiled of the driver (null: the tcgen05 path is not used)
-    int *pinned;              // [4] n_active, status
+    int *pinned;              // [16] n_active and status; at 8: the last request of which every sequence has ended
     cudaEvent_t ev0, ev1, step_ev[2];
-    double last_wall_ms;
 };
 
 namespace {
@@ -266,223 +217,6 @@ xsm_status cuda_fail(xsm_ctx *ctx, cudaError_t e, const char *what) {
 template <typename T> T *at(xsm_ctx *ctx, size_t off) { return reinterpret_cast<T *>(ctx->ws + off); }
 const void *wptr(const xsm_ctx *ctx, size_t elem_off) { return ctx->weights + elem_off * esize(ctx->cfg); }
 
-// Shared memory of the step kernel for a batch of `batch` sequences: header, ring slots, activation area
-// (also the scratch of attention, verification and the cross-warp reduction), sums of squares.
-// Returns nullptr or the reason why the shape cannot run.
-// do the projections of this batch run on the tcgen05 path?
-bool umma_shape(const xsm_model_config &c, int batch) {
-    const int M = batch * (c.n_draft + 1);
-    // (measured: below about 27 token rows the mma.sync paths are faster; the tensor-core path pays a fixed cost per
-    // block of 64 columns that only a well-filled tile repays)
-    return c.dtype == 1 && M >= kUmmaMinRows && M <= 128 && c.d_model % kUmmaK == 0 && c.d_ff % kUmmaK == 0;
-}
-
-// jobs in the tail of a step: the LM head, then per decoding head W1 and Wout, or Wq, Wo and Wout
-int tail_jobs(const xsm_model_config &c) { return 1 + (c.head_kind == 1 ? 3 : 2) * c.n_draft; }
-
-// grid: CTAs of the step kernel if known (it sizes the staging of the sums-of-squares shares on the path for at most
-// eight token rows), 0: not known yet, plan for the largest
-const char *plan_smem(const xsm_model_config &c, int batch, Dev &D, int &smem_bytes, int grid = 0) {
-    const int K1 = c.n_draft + 1, M = batch * K1, dh = c.d_head;
-    D.tab_bytes = smem_tab_bytes(tail_jobs(c));
-    D.plan_bytes = smem_plan_bytes(tail_jobs(c));
-    if (D.umma)      // swizzled tensor-core tiles: the ring starts on a 1024-byte boundary
-        D.plan_bytes = (kSmemHeader + D.tab_bytes + D.plan_bytes + 1023) / 1024 * 1024 - kSmemHeader - D.tab_bytes;
-    const int kSmemTables = D.tab_bytes, kSmemPlans = D.plan_bytes;
-    if (D.umma) {
-        // tcgen05 path: the activation area holds two buffers of two planes (hi, lo) of 128 token rows x 64 columns; the
-        // other users of the area (attention, verification, commit) fit inside
-        const int tail = (kMaxTokens + 1536) * 4;
-        const int avail = kSmemMax - kSmemHeader - kSmemTables - kSmemPlans - tail;
-        int need = 2 * 16 * (dh + 8) * 2 + 4 * K1 * dh * 4 + 128 * dh + (kConsumerWarps + 1) * K1 * (dh + 2) * 4;
-        const int samp = (((c.vocab + 3) & ~3) + 1024) * 4;
-        if (samp > need) need = samp;
-        const int emb = 512 + K1 * (c.d_model / 8) * 4;
-        if (emb > need) need = emb;
-        int acts = kUmmaActsBytes > need ? kUmmaActsBytes : (need + 1023) / 1024 * 1024;
-        int slots = (avail - acts) / kSlotBytes;
-        if (slots > kMaxSlots) slots = kMaxSlots;
-        if (slots < kMinSlots) return "the shape needs more shared memory than one CTA has";
-        D.n_slots = slots;
-        D.acts_bytes = acts;
-        D.kca = c.d_model > c.d_ff ? c.d_model : c.d_ff;
-        D.tile_bytes = c.page_size * dh * 2;
-        D.kv_one_item = 2 * D.tile_bytes <= kSlotBytes ? 1 : 0;
-        smem_bytes = kSmemHeader + kSmemTables + kSmemPlans + slots * kSlotBytes + acts + tail;
-        return nullptr;
-    }
-    const int kmax = c.d_model > c.d_ff ? c.d_model : c.d_ff;
-    // sums of squares and their partials; at most eight token rows of a bf16 model: the CTAs' shares [row][CTA]
-    int tail = (kMaxTokens + 1536) * 4;
-    if (grid > 0 && c.dtype == 1 && M <= 8 && grid * M <= 1536) tail = (kMaxTokens + ((grid * M + 31) & ~31)) * 4;
-    const int avail = kSmemMax - kSmemHeader - kSmemTables - kSmemPlans - tail;
-    // what the other users of the activation area need
-    const int np = c.dtype == 1 ? (M <= 8 ? 8 : M <= 16 ? 16 : M <= 32 ? 32 : M <= 80 ? 80 : 128) : 8;
-    int need = kConsumerWarps * np * 16 * 4 + 2 * 16 * M * 4;         // reduction of the projections, new residual values
-    const int attn = 2 * 16 * (dh + 8) * 2 + 4 * K1 * dh * 4 + 128 * dh + (kConsumerWarps + 1) * K1 * (dh + 2) * 4;
-    if (attn > need) need = attn;
-    const int samp = (((c.vocab + 3) & ~3) + 1024) * 4;      // a logits row, reduction scratch, candidates, the probability tree's tables
-    if (samp > need) need = samp;
-    const int emb = 512 + K1 * (c.d_model / (c.dtype == 1 ? 8 : 4)) * 4;   // commit: scalars, partial sums of the new window's rows
-    if (emb > need) need = emb;
-    const int full = M * (kmax * 4 + 16) + (kConsumerWarps * np * 16 + kConsumerWarps * M) * 4;   // all activations of the widest projection, and the partial products behind them
-    int acts = full > need ? full : need;
-    if (acts > avail - kMinSlots * kSlotBytes) acts = avail - kMinSlots * kSlotBytes;
-    if (acts < need) return "the shape needs more shared memory than one CTA has";
-    acts = (acts + 127) / 128 * 128;
-    if (acts > avail - kMinSlots * kSlotBytes) acts -= 128;
-    int kca = ((acts / M - 16) / 4) / 128 * 128;
-    if (kca > kmax) kca = kmax;
-    if (kca < kmax && c.dtype == 1) {
-        // the widest projection is staged in chunks: room for the accumulators and the per-token partial sums behind
-        // a chunk, and chunks of at most 2048 columns (four rows of a chunk fit one ring slot)
-        kca = (((acts - kAccumBytes - kAccumBytes / 16) / M - 16) / 4) / 128 * 128;
-        if (kca > 2048) kca = 2048;
-    }
-    if (kca < 128) return "batch * (n_draft + 1) is too large for the activation staging area";
-    if (c.dtype == 0 && kca < kmax) return "fp32 models need all activations of a projection in shared memory: reduce the batch";
-    if (c.dtype == 0 && M > 24) return "fp32 models support at most 24 token rows per step";
-    int slots = (avail - acts) / kSlotBytes;
-    if (slots > kMaxSlots) slots = kMaxSlots;
-    D.n_slots = slots;
-    D.acts_bytes = acts;
-    D.kca = kca;
-    D.tile_bytes = c.page_size * dh * (c.dtype == 1 ? 2 : 4);
-    D.kv_one_item = 2 * D.tile_bytes <= kSlotBytes ? 1 : 0;
-    smem_bytes = kSmemHeader + kSmemTables + kSmemPlans + slots * kSlotBytes + acts + tail;
-    return nullptr;
-}
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                                  const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Tensor map of a bf16 weight matrix [layers][rows][kdim] (rows of kdim elements, layers layer_bytes apart): boxes of 64
-// columns x 8 rows of one layer, 128-byte swizzle (the layout the tcgen05 matrix descriptors of the step kernel name).
-bool encode_weight_map(xsm_ctx *ctx, CUtensorMap *out, const void *W, int rows, int kdim, int layers, long long layer_bytes) {
-    if (!ctx->encode_tiled || !W) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)kdim, (cuuint64_t)rows, (cuuint64_t)(layers > 0 ? layers : 1)};
-    cuuint64_t strides[2] = {(cuuint64_t)kdim * 2, (cuuint64_t)(layers > 1 ? layer_bytes : (long long)rows * kdim * 2)};
-    cuuint32_t box[3] = {(cuuint32_t)kUmmaK, 8, 1}, estr[3] = {1, 1, 1};
-    return ((EncodeTiledFn)ctx->encode_tiled)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(W), dims, strides, box, estr,
-                                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// stage and job tables for the current batch: the eight stages of layer 0, then the tail of the step
-void build_tables(xsm_ctx *ctx) {
-    const xsm_model_config &c = ctx->cfg;
-    const Dev &D = ctx->dev;
-    const WeightOffsets &w = ctx->wo;
-    const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers;
-    const size_t M = D.M;
-    const int hw = 3 * L + 1;      // writes of the residual stream per step: the embedding and three per layer
-    Tables &T = ctx->h_tab;
-    memset(&T, 0, sizeof(T));
-    T.layer_bytes = L > 1 ? (long long)((w.wq[1] - w.wq[0]) * esize(c)) : 0;
-    T.gain_last = wptr(ctx, w.gf);
-    int n_jobs = 0, n_stages = 0;
-    auto job = [&](const void *W, const void *W2, int rows, int kdim, const float *x, const void *gain, float *out,
-                   int out_ld, int epi, TagRef in, int in_jinc, TagRef outt, int out_jinc, const void *gain_out = nullptr,
-                   int out_plain = 0) -> GemvJob & {
-        GemvJob &j = T.jobs[n_jobs++];
-        j.W = W; j.W2 = W2; j.x = x; j.gain = gain; j.out = out; j.hm = epi == EPI_ADD ? D.h : nullptr;
-        j.rows = rows; j.kdim = kdim; j.out_ld = out_ld; j.epi = epi; j.in = in; j.outt = outt;
-        j.in_jinc = in_jinc; j.out_jinc = out_jinc; j.gain_out = gain_out; j.out_plain = out_plain;
-        return j;
-    };
-    auto gemv1 = [&](int j0, int n) {
-        Stage &s = T.stages[n_stages++];
-        s.kind = ST_GEMV; s.job0 = j0; s.njobs = n;
-    };
-    auto attn = [&](int kind) {
-        Stage &s = T.stages[n_stages++];
-        s.kind = kind;
-        s.in = TagRef{L, 0}; s.outt = TagRef{L, 0}; s.part = TagRef{L, 0}; s.jinc = 1;
-    };
-    // layer 0.  Buffers written once per layer have write index serial * L + l, the residual stream 3 l + which.
-    // A stage that adds to the residual stream publishes it with the gain of the RMSNorm that reads it next.
-    const TagRef per_layer{L, 0};
-    job(wptr(ctx, w.wq[0]), nullptr, 3 * d, d, D.hpub, wptr(ctx, w.g1[0]), D.qkv, 3 * d, EPI_STORE, TagRef{hw, 0}, 3, per_layer, 1);
-    gemv1(0, 1);
-    attn(ST_ATTN_SELF);
-    job(wptr(ctx, w.wo[0]), nullptr, d, d, D.attn, nullptr, D.hpub, d, EPI_ADD, per_layer, 1, TagRef{hw, 1}, 3, wptr(ctx, w.g2[0]));
-    gemv1(1, 1);
-    job(wptr(ctx, w.wqc[0]), nullptr, d, d, D.hpub, wptr(ctx, w.g2[0]), D.qc, d, EPI_STORE, TagRef{hw, 1}, 3, per_layer, 1);
-    gemv1(2, 1);
-    attn(ST_ATTN_CROSS);
-    job(wptr(ctx, w.woc[0]), nullptr, d, d, D.cattn, nullptr, D.hpub, d, EPI_ADD, per_layer, 1, TagRef{hw, 2}, 3, wptr(ctx, w.g3[0]));
-    gemv1(3, 1);
-    job(wptr(ctx, w.wgate[0]), wptr(ctx, w.wup[0]), f, d, D.hpub, wptr(ctx, w.g3[0]), D.act, f, EPI_GATEUP, TagRef{hw, 2}, 3,
-        per_layer, 1);
-    gemv1(4, 1);
-    {   // the down projection's published copy is read through the first RMSNorm of the NEXT layer (or the final one)
-        GemvJob &j = job(wptr(ctx, w.wdown[0]), nullptr, d, f, D.act, nullptr, D.hpub, d, EPI_ADD, per_layer, 1, TagRef{hw, 3}, 3,
-                         wptr(ctx, w.g1[0]));
-        j.gain_out_step = T.layer_bytes != 0 ? T.layer_bytes : 1;
-        gemv1(5, 1);
-    }
-    // tail
-    const TagRef once{1, 0};
-    int j0 = n_jobs;
-    job(wptr(ctx, w.W0), nullptr, V, d, D.hpub, wptr(ctx, w.gf), D.logits0, V, EPI_STORE, TagRef{hw, 3 * L}, 0, once, 0, nullptr, 1);
-    if (c.head_kind == 1 && K > 0) {
-        // cross-attention heads (Eq. 3): q = Wq g beside the LM head (every CTA also publishes its columns of g), the
-        // heads' attention over their own keys and values of the condition, y = g + Wo a
-        for (int i = 0; i < K; ++i)
-            job(wptr(ctx, w.hq[i]), nullptr, d, d, D.hpub, wptr(ctx, w.gf), D.qh + (size_t)i * M * d, d, EPI_STORE, TagRef{hw, 3 * L}, 0, once, 0);
-        gemv1(j0, 1 + K);
-        T.stages[n_stages - 1].norm_out = 1;
-        {
-            Stage &s = T.stages[n_stages++];
-            s.kind = ST_ATTN_HEAD;
-            s.in = once; s.outt = once; s.part = once; s.jinc = 0;
-        }
-        j0 = n_jobs;
-        for (int i = 0; i < K; ++i)
-            job(wptr(ctx, w.ho[i]), nullptr, d, d, D.hattn + (size_t)i * M * d, nullptr, D.y + (size_t)i * M * d, d, EPI_ADDG, once, 0, once, 0)
-                .res = D.gpub;
-        gemv1(j0, K);
-    } else {
-        for (int i = 0; i < K; ++i)
-            job(wptr(ctx, w.W1[i]), nullptr, d, d, D.hpub, wptr(ctx, w.gf), D.y + (size_t)i * M * d, d, EPI_HEADY,
-                TagRef{hw, 3 * L}, 0, once, 0);
-        gemv1(j0, 1 + K);
-    }
-    if (K > 0) {
-        j0 = n_jobs;
-        for (int i = 0; i < K; ++i)
-            job(wptr(ctx, w.Wout[i]), nullptr, V, d, D.y + (size_t)i * M * d, nullptr, D.hlogits + (size_t)i * M * V, V,
-                EPI_STORE, once, 0, once, 0, nullptr, 1);
-        gemv1(j0, K);
-    }
-    T.stages[n_stages++].kind = ST_SAMPLE;
-    T.stages[n_stages++].kind = ST_COMMIT;
-    T.n_tail_stages = n_stages - kLayerStages;
-    T.n_tail_jobs = n_jobs - kLayerJobs;
-    ctx->n_stages = kLayerStages * L + T.n_tail_stages;
-    if (ctx->dev.umma) {
-        // tcgen05 path: the weights come by TMA; one tensor map per matrix (all layers of a layer job in one map)
-        ctx->h_tmaps.assign(2 * (size_t)n_jobs, CUtensorMap{});
-        char *d_maps = ctx->ws + ctx->lay.tmaps;
-        bool ok = true;
-        for (int i = 0; i < n_jobs && ok; ++i) {
-            GemvJob &j = T.jobs[i];
-            const int layers = i < kLayerJobs ? L : 1;
-            ok = encode_weight_map(ctx, &ctx->h_tmaps[2 * i], j.W, j.rows, j.kdim, layers, T.layer_bytes);
-            j.tmap = d_maps + 128 * (2 * (size_t)i);
-            if (ok && j.W2 != nullptr) {
-                ok = encode_weight_map(ctx, &ctx->h_tmaps[2 * i + 1], j.W2, j.rows, j.kdim, layers, T.layer_bytes);
-                j.tmap2 = d_maps + 128 * (2 * (size_t)i + 1);
-            }
-        }
-        if (!ok) {        // no tensor maps: the projections take the mma.sync path
-            ctx->dev.umma = 0;
-            for (int i = 0; i < n_jobs; ++i) T.jobs[i].tmap = T.jobs[i].tmap2 = nullptr;
-        }
-    }
-}
-
 xsm_status check_device_status(xsm_ctx *ctx) {
     XSM_CUDA(ctx, cudaMemcpyAsync(ctx->pinned, ctx->dev.n_active, 8, cudaMemcpyDeviceToHost, ctx->stream));
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -493,39 +227,14 @@ xsm_status check_device_status(xsm_ctx *ctx) {
     return XSM_OK;
 }
 
-// n_steps decoding steps on the stream
-xsm_status run_steps(xsm_ctx *ctx, int n_steps, bool static_scratch = false) {
-    if (ctx->use_chain) {
-        // a recording is replayed unless single launches were asked for, a timeline is taken (the recording has none), or
-        // the call must not make the driver allocate anything
-        const bool graph = !ctx->phase_launch && !static_scratch && ctx->dev.trace == nullptr;
-        for (int t = 0; t < n_steps; ++t)
-            XSM_CUDA(ctx, ctx->chain.step(ctx->dev, ctx->stream, graph, !ctx->phase_launch, &ctx->launches));
-        return XSM_OK;
-    }
-    const int np = ctx->n_stages;
-    if (!static_scratch && ctx->static_steps) {
-        // The steps since the workspace partials were last written went through the library's scratch array, so the
-        // workspace copy still carries the tags of an older step; tags repeat with period three, and a stale word
-        // could pass for a fresh partial.  It restarts from "never written".
-        XSM_CUDA(ctx, cudaMemsetAsync(ctx->ws + ctx->lay.part, 0, ctx->lay.candx - ctx->lay.part, ctx->stream));
-        if (ctx->lay.xchg_end > ctx->lay.hpart)
-            XSM_CUDA(ctx, cudaMemsetAsync(ctx->ws + ctx->lay.hpart, 0, ctx->lay.xchg_end - ctx->lay.hpart, ctx->stream));
-    }
-    ctx->static_steps = static_scratch ? 1 : 0;
-    if (!ctx->phase_launch) {
-        XSM_CUDA(ctx, launch_step(ctx->dev, ctx->cfg.dtype, 0, np, n_steps, ctx->serial, ctx->grid, ctx->smem_bytes, ctx->stream));
-        ctx->launches += 1;
-        ctx->serial += (uint32_t)n_steps;
-    } else {
-        for (int t = 0; t < n_steps; ++t) {
-            for (int p = 0; p < np; ++p) {
-                XSM_CUDA(ctx, launch_step(ctx->dev, ctx->cfg.dtype, p, p + 1, 1, ctx->serial, ctx->grid, ctx->smem_bytes, ctx->stream));
-                ctx->launches += 1;
-            }
-            ctx->serial += 1u;
-        }
-    }
+// one decoding step on the stream; scratch: device memory for the partial results of the key splits (null: the workspace's)
+xsm_status run_step(xsm_ctx *ctx, float *scratch = nullptr) {
+    // a recording is replayed unless single launches were asked for, a timeline is taken (the recording has none), or the
+    // call must not make the driver allocate anything
+    const bool graph = !ctx->phase_launch && scratch == nullptr && ctx->dev.trace == nullptr;
+    Dev D = ctx->dev;
+    if (scratch) D.apart = scratch;
+    XSM_CUDA(ctx, ctx->chain.step(D, ctx->stream, graph, !ctx->phase_launch, &ctx->launches));
     return XSM_OK;
 }
 
@@ -538,41 +247,17 @@ xsm_status set_run(xsm_ctx *ctx, const RunParams &r) {
     return XSM_OK;
 }
 xsm_status set_max_new(xsm_ctx *ctx, int max_new) {
-    ctx->dev.max_new = max_new;
-    if (!ctx->use_chain) return XSM_OK;
     RunParams r = ctx->run;
     r.max_new = max_new;
     return set_run(ctx, r);
 }
-
-// Algorithm 1 line 1 on the launch chain: state, the condition's keys and values, the prompt, the first window
-xsm_status chain_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_t *d_prompt, int prompt_len, const xsm_decode_config *dc) {
-    const xsm_model_config &c = ctx->cfg;
-    Dev &D = ctx->dev;
-    D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8;
-    if (!ctx->chain.select(D)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
-    ctx->n_stages = ctx->chain.n_ops();
-    RunParams &r = ctx->run;
-    memset(&r, 0, sizeof(r));
-    r.verify_mode = dc->verify_mode; r.k_accept = dc->k_accept; r.delta = dc->delta;
-    r.sample_mode = dc->sample_mode; r.k_sample = dc->k_sample; r.temperature = dc->temperature;
-    r.key0 = (uint32_t)dc->seed; r.key1 = (uint32_t)(dc->seed >> 32);
-    r.max_new = INT_MAX; r.prompt_len = prompt_len;
-    r.request = ++ctx->request;
-    if ((const void *)d_prompt != (const void *)D.prompt)
-        XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
-    XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
-    XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off), at<size_t>(ctx, ctx->lay.wvc_off), d_cond,
-                                  D.ckv_pool, D.L, ctx->stream));
-    if (c.head_kind == 1 && D.K > 0) {
-        XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off), at<size_t>(ctx, ctx->lay.hv_off), d_cond,
-                                      D.hckv_pool, D.K, ctx->stream));
-        ctx->launches += 1;
-    }
-    ctx->launches += 3;
-    if (prompt_len > 1) XSM_CUDA(ctx, ctx->chain.ingest(D, prompt_len - 1, ctx->stream, &ctx->launches));
-    XSM_CUDA(ctx, launch_embed_rows(D, D.K1, D.Mp, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
-    ctx->prefilled = 1;
+// the tokens committed by the latest step -> the caller
+xsm_status copy_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
+    const Dev &D = ctx->dev;
+    if (d_new_tokens)
+        XSM_CUDA(ctx, cudaMemcpyAsync(d_new_tokens, D.step_tokens, sizeof(int32_t) * D.M, cudaMemcpyDeviceToDevice, ctx->stream));
+    if (d_n_new)
+        XSM_CUDA(ctx, cudaMemcpyAsync(d_n_new, D.step_n_new, sizeof(int32_t) * D.B, cudaMemcpyDeviceToDevice, ctx->stream));
     return XSM_OK;
 }
 
@@ -601,21 +286,14 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     Layout L;
     if (!make_layout(*cfg, workspace_bytes, L))
         return fail(nullptr, XSM_ERR_CAPACITY, "workspace cannot hold the buffers plus one sequence of cache pages");
-    Dev probe;
-    memset(&probe, 0, sizeof(probe));
-    int smem_one = 0;
-    if (const char *m = plan_smem(*cfg, 1, probe, smem_one)) return fail(nullptr, XSM_ERR_INVALID_ARG, m);
     xsm_ctx *ctx = new xsm_ctx();
     ctx->cfg = *cfg;
     ctx->lay = L;
     ctx->wo = weight_offsets(*cfg);
     ctx->weights = (const char *)d_weights;
     ctx->ws = (char *)d_workspace;
-    ctx->ws_bytes = workspace_bytes;
     ctx->stream = (cudaStream_t)cuda_stream;
-    ctx->phase_launch = 0; ctx->prefilled = 0; ctx->batch = 0; ctx->launches = 0; ctx->last_wall_ms = 0; ctx->serial = 0;
-    ctx->static_steps = 0;
-    ctx->request = 0; ctx->use_chain = false;
+    ctx->phase_launch = 0; ctx->prefilled = 0; ctx->launches = 0; ctx->request = 0; ctx->n_stages = 0;
     memset(&ctx->run, 0, sizeof(ctx->run));
     ctx->pinned = nullptr; ctx->ev0 = ctx->ev1 = ctx->step_ev[0] = ctx->step_ev[1] = nullptr;
     auto bail = [&](cudaError_t e, const char *what) {
@@ -629,30 +307,13 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
         return XSM_ERR_CUDA;
     };
     cudaError_t e;
-    int grid = 0;
     {
         int dev = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return bail(e, "cudaGetDevice");
-        if ((e = cudaDeviceGetAttribute(&grid, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return bail(e, "device query");
+        if ((e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return bail(e, "device query");
     }
-    if (grid < 1) { delete ctx; return fail(nullptr, XSM_ERR_CUDA, "no multiprocessors reported"); }
-    ctx->sm_count = grid;
-    // every CTA must own at least one row of every projection (the exchange protocol relies on it), and the
-    // buffers that are sized per CTA bound the grid from above
-    if (grid > cfg->d_model) grid = cfg->d_model;
-    if (grid > kSizingGrid) grid = kSizingGrid;
-    ctx->grid = grid;
     if ((e = cudaHostAlloc((void **)&ctx->pinned, 64, cudaHostAllocDefault)) != cudaSuccess) return bail(e, "cudaHostAlloc");
-    {   // the driver's tensor-map encoder, for the weights of the tcgen05 projections (absent: those take the mma.sync path)
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        ctx->encode_tiled = nullptr;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            ctx->encode_tiled = fn;
-        else
-            (void)cudaGetLastError();
-    }
+    if (!ctx->chain.init(*cfg, ctx->wo, ctx->weights, ctx->sm_count)) return bail(cudaErrorNotSupported, "tensor maps of the weights");
     if ((e = cudaEventCreate(&ctx->ev0)) != cudaSuccess) return bail(e, "cudaEventCreate");
     if ((e = cudaEventCreate(&ctx->ev1)) != cudaSuccess) return bail(e, "cudaEventCreate");
     for (cudaEvent_t &ev : ctx->step_ev)
@@ -696,42 +357,28 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
         if ((1 << sh) == cfg->page_size) D.p_shift = sh;
     D.max_seq_len = cfg->max_seq_len; D.tok_ld = L.tok_ld;
     D.eps = cfg->rms_eps; D.scale = (float)(1.0 / sqrt((double)cfg->d_head)); D.bos = cfg->bos_id; D.eos = cfg->eos_id;
-    D.max_new = INT_MAX;
     D.spin_limit = kSpinLimit; D.mbar_limit = kMbarSpinLimit;
-    D.tables = at<Tables>(ctx, L.phases);
-    D.E = wptr(ctx, ctx->wo.E);
-    D.len = at<int>(ctx, L.len); D.window = at<int>(ctx, L.window); D.cand = at<int>(ctx, L.cand);
-    D.acc_len = at<int>(ctx, L.acc_len); D.finished = at<int>(ctx, L.finished); D.n_gen = at<int>(ctx, L.n_gen);
+    D.E = wptr(ctx, ctx->wo.E); D.gain_first = wptr(ctx, ctx->wo.g1[0]);
+    D.head_kind = cfg->head_kind;
+    D.len = at<int>(ctx, L.len); D.window = at<int>(ctx, L.window);
+    D.finished = at<int>(ctx, L.finished); D.n_gen = at<int>(ctx, L.n_gen);
     D.n_blocks = at<int>(ctx, L.n_blocks); D.block_table = at<int>(ctx, L.block_table);
-    D.ingest_left = at<int>(ctx, L.ingest_left); D.step_idx = at<uint32_t>(ctx, L.step_idx);
+    D.step_idx = at<uint32_t>(ctx, L.step_idx);
     D.free_stack = at<int>(ctx, L.free_stack);
     int *sc = at<int>(ctx, L.scalars);
-    D.n_active = sc; D.status = sc + 1; D.n_free = sc + 2;
+    D.n_active = sc; D.status = sc + 1; D.n_free = sc + 2; D.stage_word = sc + 3;
     D.hist = at<unsigned long long>(ctx, L.hist); D.steps = at<unsigned long long>(ctx, L.steps);
     D.tok_log = at<int>(ctx, L.tok_log); D.step_tokens = at<int>(ctx, L.step_tokens);
     D.step_n_new = at<int>(ctx, L.step_n_new); D.prompt = at<int>(ctx, L.prompt);
+    D.rp = at<RunParams>(ctx, L.rp);
+    D.host_done = ctx->pinned + 8;
     D.h = at<float>(ctx, L.h); D.rope_cs = at<float2>(ctx, L.rope_cs);
-    D.hpub = at<float>(ctx, L.hpub); D.qkv = at<float>(ctx, L.qkv); D.attn = at<float>(ctx, L.attn);
-    D.qc = at<float>(ctx, L.qc); D.cattn = at<float>(ctx, L.cattn); D.act = at<float>(ctx, L.act);
-    D.y = at<float>(ctx, L.y); D.logits0 = at<float>(ctx, L.logits0); D.hlogits = at<float>(ctx, L.hlogits);
-    D.part = at<float>(ctx, L.part); D.cpart = at<float>(ctx, L.cpart);
-    D.candx = at<uint32_t>(ctx, L.candx); D.header = at<uint32_t>(ctx, L.header); D.done = at<uint32_t>(ctx, L.done);
-    D.sspub = at<float>(ctx, L.sspub); D.gain_first = wptr(ctx, ctx->wo.g1[0]); D.grid = grid;
-    D.kv_pool = ctx->ws + L.kv_pool; D.ckv_pool = ctx->ws + L.ckv_pool;
-    D.head_kind = cfg->head_kind;
-    D.qh = at<float>(ctx, L.qh); D.hattn = at<float>(ctx, L.hattn); D.gpub = at<float>(ctx, L.gpub); D.hpart = at<float>(ctx, L.hpart);
-    D.hckv_pool = ctx->ws + L.hckv_pool;
-    D.treex = at<uint32_t>(ctx, L.treex);
-    if (cfg->dtype == 1) {
-        ctx->use_chain = ctx->chain.init(*cfg, ctx->wo, ctx->weights, ctx->sm_count);
-        D.rp = at<RunParams>(ctx, L.rp);
-        D.stage_word = reinterpret_cast<int *>(ctx->ws + L.rp + sizeof(RunParams) + 32);
-        D.host_done = ctx->pinned + 8;
-        D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
-        D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
-        D.apart = at<float>(ctx, L.apart); D.acount = at<int>(ctx, L.acount);
-        D.tail_row_bytes = 160 * 1024;
-    }
+    D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
+    D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
+    D.apart = at<float>(ctx, L.apart); D.acount = at<int>(ctx, L.acount);
+    D.tail_row_bytes = 160 * 1024;
+    D.logits0 = at<float>(ctx, L.logits0); D.hlogits = at<float>(ctx, L.hlogits);
+    D.kv_pool = ctx->ws + L.kv_pool; D.ckv_pool = ctx->ws + L.ckv_pool; D.hckv_pool = ctx->ws + L.hckv_pool;
     *out = ctx;
     return XSM_OK;
 }
@@ -758,82 +405,31 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     if ((long long)batch * ctx->lay.max_blocks > ctx->lay.n_pages)
         return fail(ctx, XSM_ERR_CAPACITY, "the page pool cannot hold `batch` sequences of max_seq_len positions");
     Dev &D = ctx->dev;
-    ctx->dc = *dc;
-    ctx->batch = batch;
-    {
-        const int bh = batch * D.H, s_max = ctx->grid / bh;
-        D.S_max = s_max < 1 ? 1 : (s_max > 64 ? 64 : s_max);
-    }
-    if (ctx->use_chain) return chain_prefill(ctx, batch, d_cond, d_prompt, prompt_len, dc);
-    int smem_bytes = 0;
-    D.umma = (umma_shape(c, batch) && ctx->encode_tiled != nullptr) ? 1 : 0;
-    if (const char *m = plan_smem(c, batch, D, smem_bytes, ctx->grid)) return fail(ctx, XSM_ERR_CAPACITY, m);
-    {   // at most eight token rows, all activations of the widest projection staged at once with room for the warps'
-        // partial products behind them, the CTAs' shares of a row readable by one warp pass: the compact instance
-        const int M = batch * D.K1, kmax = c.d_model > c.d_ff ? c.d_model : c.d_ff;
-        D.small = (c.dtype == 1 && M <= 8 && D.kca >= kmax && ctx->grid * M <= 1536 && (ctx->grid & 3) == 0 &&
-                   D.acts_bytes - M * (kmax * 4 + 16) >= kConsumerWarps * kSmallRedBytes) ? 1 : 0;
-        // (the other paths stage their partial sums of squares in the full-size area)
-        if (!D.small)
-            if (const char *m = plan_smem(c, batch, D, smem_bytes)) return fail(ctx, XSM_ERR_CAPACITY, m);
-    }
-    ctx->smem_bytes = smem_bytes;
-    {   // the step kernel instance for this batch must fit one CTA per multiprocessor
-        Dev probe = D;
-        probe.M = batch * D.K1;
-        int resident = 0;
-        XSM_CUDA(ctx, step_kernel_setup(probe, c.dtype, smem_bytes, &resident));
-        if (resident < ctx->grid) return fail(ctx, XSM_ERR_CUDA, "the step kernel does not fit on this device");
-    }
-    D.B = batch; D.M = batch * D.K1;
-    D.inv_m = ((1 << 20) + D.M - 1) / D.M;
-    D.verify_mode = dc->verify_mode; D.k_accept = dc->k_accept; D.delta = dc->delta;
-    D.sample_mode = dc->sample_mode; D.k_sample = dc->k_sample; D.temperature = dc->temperature;
-    D.key0 = (uint32_t)dc->seed; D.key1 = (uint32_t)(dc->seed >> 32);
-    D.max_new = INT_MAX; D.prompt_len = prompt_len;
-    // the condition's keys and values of one head: one item while that is at most 96 KB, else split over CTAs
-    int s_cross = 1;
-    if ((long long)D.cpages * 2 * D.tile_bytes > 96 * 1024) {
-        s_cross = D.S_max < D.cpages ? D.S_max : D.cpages;
-        if (s_cross < 1) s_cross = 1;
-    }
-    D.S_cross = s_cross;
-    D.B = batch; D.M = batch * D.K1;
-    build_tables(ctx);
-    if (!D.umma && umma_shape(c, batch)) {      // the tensor maps could not be made: plan the shared memory of the mma.sync path
-        if (const char *m = plan_smem(c, batch, D, smem_bytes)) return fail(ctx, XSM_ERR_CAPACITY, m);
-        ctx->smem_bytes = smem_bytes;
-    }
-    if (D.umma)
-        XSM_CUDA(ctx, cudaMemcpyAsync(ctx->ws + ctx->lay.tmaps, ctx->h_tmaps.data(), sizeof(CUtensorMap) * ctx->h_tmaps.size(),
-                                      cudaMemcpyHostToDevice, ctx->stream));
-    D.n_stages = ctx->n_stages;
-    XSM_CUDA(ctx, cudaMemcpyAsync(ctx->ws + ctx->lay.phases, &ctx->h_tab, sizeof(Tables), cudaMemcpyHostToDevice, ctx->stream));
+    if (c.dtype == 0 && batch * D.K1 > kF32Rows) return fail(ctx, XSM_ERR_CAPACITY, "fp32 models support at most 24 token rows per step");
+    D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8;
+    if (!ctx->chain.select(D)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
+    ctx->n_stages = ctx->chain.n_ops();
+    RunParams &r = ctx->run;
+    memset(&r, 0, sizeof(r));
+    r.verify_mode = dc->verify_mode; r.k_accept = dc->k_accept; r.delta = dc->delta;
+    r.sample_mode = dc->sample_mode; r.k_sample = dc->k_sample; r.temperature = dc->temperature;
+    r.key0 = (uint32_t)dc->seed; r.key1 = (uint32_t)(dc->seed >> 32);
+    r.max_new = INT_MAX; r.prompt_len = prompt_len;
+    r.request = ++ctx->request;
     if ((const void *)d_prompt != (const void *)D.prompt)
-        XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len,
-                                      cudaMemcpyDeviceToDevice, ctx->stream));
-    // no tag of an earlier generation may survive: the exchange buffers restart from "never written"
-    XSM_CUDA(ctx, cudaMemsetAsync(ctx->ws + ctx->lay.xchg_begin, 0, ctx->lay.xchg_end - ctx->lay.xchg_begin, ctx->stream));
-    ctx->serial = 0;
-    ctx->static_steps = 0;
-    D.script = nullptr; D.script_n = 0; D.script_acc = 0;
-    // the table above is read from host memory that the next prefill rewrites
-    XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    XSM_CUDA(ctx, launch_init(D, c.dtype, ctx->serial, ctx->stream));      // also clears the status word
-    XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off),
-                                  at<size_t>(ctx, ctx->lay.wvc_off), d_cond, D.ckv_pool, D.L, ctx->stream));
+        XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
+    XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
+    XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off), at<size_t>(ctx, ctx->lay.wvc_off), d_cond,
+                                  D.ckv_pool, D.L, ctx->stream));
     if (c.head_kind == 1 && D.K > 0) {
-        XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off),
-                                      at<size_t>(ctx, ctx->lay.hv_off), d_cond, D.hckv_pool, D.K, ctx->stream));
+        XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off), at<size_t>(ctx, ctx->lay.hv_off), d_cond,
+                                      D.hckv_pool, D.K, ctx->stream));
         ctx->launches += 1;
     }
     ctx->launches += 3;
+    if (prompt_len > 1) XSM_CUDA(ctx, ctx->chain.ingest(D, prompt_len - 1, ctx->stream, &ctx->launches));
+    XSM_CUDA(ctx, launch_embed_rows(D, c.dtype, D.K1, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
     ctx->prefilled = 1;
-    const int ingest_steps = (prompt_len - 1 + D.K1 - 1) / D.K1;
-    if (ingest_steps > 0) {
-        xsm_status st = run_steps(ctx, ingest_steps);
-        if (st != XSM_OK) return st;
-    }
     return XSM_OK;
 }
 
@@ -841,14 +437,8 @@ xsm_status xsm_spec_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) 
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_spec_step before xsm_prefill");
     xsm_status st = set_max_new(ctx, INT_MAX);
-    if (st == XSM_OK) st = run_steps(ctx, 1);
-    if (st != XSM_OK) return st;
-    const Dev &D = ctx->dev;
-    if (d_new_tokens)
-        XSM_CUDA(ctx, cudaMemcpyAsync(d_new_tokens, D.step_tokens, sizeof(int32_t) * D.M, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (d_n_new)
-        XSM_CUDA(ctx, cudaMemcpyAsync(d_n_new, D.step_n_new, sizeof(int32_t) * D.B, cudaMemcpyDeviceToDevice, ctx->stream));
-    return XSM_OK;
+    if (st == XSM_OK) st = run_step(ctx);
+    return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
 
 // ---- scratch owned by the library, for xsm_spec_step_static
@@ -861,26 +451,17 @@ static std::atomic<void *> g_static_scratch_addr[kMaxDevices];   // by device or
 xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_spec_step_static before xsm_prefill");
-    Dev &D = ctx->dev;
-    // the split partials of self- and cross-attention: [B * H * S_max][K + 1][d_head + 2] floats each; cross-attention
-    // heads have K more such sets
-    const size_t one = (size_t)D.B * D.H * D.S_max * D.K1 * (D.dh + 2) * sizeof(float);
+    const Dev &D = ctx->dev;
+    // the partial results of the key splits of self- and cross-attention: [batch * n_heads * splits][K + 1][d_head + 2] floats
+    // each, with as many splits as leave an SM for each (one stage's at a time are in use); cross-attention heads count K more
+    const int splits = ctx->sm_count / (D.B * D.H);
+    const size_t one = (size_t)D.B * D.H * (splits < 1 ? 1 : splits > 64 ? 64 : splits) * D.K1 * (D.dh + 2) * sizeof(float);
     const size_t half = (one + 255) / 256 * 256;
     const size_t n_sets = 2 + (D.head_kind == 1 ? (size_t)D.K : 0);
     if (n_sets * half > kStaticScratchBytes)
         return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch need " +
                                                std::to_string(n_sets * half) + " bytes, the built-in scratch holds " +
                                                std::to_string(kStaticScratchBytes));
-    if (ctx->use_chain) {      // the key splits meet in distributed shared memory: no scratch, and no recording either
-        xsm_status st = set_max_new(ctx, INT_MAX);
-        if (st == XSM_OK) st = run_steps(ctx, 1, true);
-        if (st != XSM_OK) return st;
-        if (d_new_tokens)
-            XSM_CUDA(ctx, cudaMemcpyAsync(d_new_tokens, D.step_tokens, sizeof(int32_t) * D.M, cudaMemcpyDeviceToDevice, ctx->stream));
-        if (d_n_new)
-            XSM_CUDA(ctx, cudaMemcpyAsync(d_n_new, D.step_n_new, sizeof(int32_t) * D.B, cudaMemcpyDeviceToDevice, ctx->stream));
-        return XSM_OK;
-    }
     int dev = 0;
     XSM_CUDA(ctx, cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return fail(ctx, XSM_ERR_INVALID_ARG, "device ordinal out of range");
@@ -889,24 +470,9 @@ xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_
         XSM_CUDA(ctx, cudaGetSymbolAddress(&p, g_static_scratch));
         g_static_scratch_addr[dev].store(p);
     }
-    char *scratch = static_cast<char *>(g_static_scratch_addr[dev].load());
-    // the array keeps what the last call left; a stale tag would pass for a fresh partial, so it restarts from zero
-    XSM_CUDA(ctx, cudaMemsetAsync(scratch, 0, n_sets * half, ctx->stream));
-    float *const ws_part = D.part, *const ws_cpart = D.cpart, *const ws_hpart = D.hpart;
-    D.part = reinterpret_cast<float *>(scratch);
-    D.cpart = reinterpret_cast<float *>(scratch + half);
-    if (D.head_kind == 1) D.hpart = reinterpret_cast<float *>(scratch + 2 * half);
-    D.max_new = INT_MAX;
-    const xsm_status st = run_steps(ctx, 1, true);     // the kernel arguments are copied at launch
-    D.part = ws_part;
-    D.cpart = ws_cpart;
-    D.hpart = ws_hpart;
-    if (st != XSM_OK) return st;
-    if (d_new_tokens)
-        XSM_CUDA(ctx, cudaMemcpyAsync(d_new_tokens, D.step_tokens, sizeof(int32_t) * D.M, cudaMemcpyDeviceToDevice, ctx->stream));
-    if (d_n_new)
-        XSM_CUDA(ctx, cudaMemcpyAsync(d_n_new, D.step_n_new, sizeof(int32_t) * D.B, cudaMemcpyDeviceToDevice, ctx->stream));
-    return XSM_OK;
+    xsm_status st = set_max_new(ctx, INT_MAX);
+    if (st == XSM_OK) st = run_step(ctx, static_cast<float *>(g_static_scratch_addr[dev].load()));
+    return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
 
 xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int32_t *d_lengths, xsm_stats *host_stats) {
@@ -918,29 +484,14 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     xsm_status set = set_max_new(ctx, max_new_tokens);
     if (set != XSM_OK) return set;
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
-    long long budget = (long long)max_new_tokens + 2;   // every step commits at least one token per live sequence
-    if (ctx->use_chain) {
-        // one step ahead of the device: the next is on its way while one runs, and the one too many at the end finds
-        // every sequence ended and does nothing
-        volatile int *const done = ctx->pinned + 8;
-        for (long long i = 0; i < budget && *done != ctx->request; ++i) {
-            xsm_status st = run_steps(ctx, 1);
-            if (st != XSM_OK) return st;
-            XSM_CUDA(ctx, cudaEventRecord(ctx->step_ev[i & 1], ctx->stream));
-            if (i > 0) XSM_CUDA(ctx, cudaEventSynchronize(ctx->step_ev[(i - 1) & 1]));
-        }
-        budget = 0;
-        xsm_status st = check_device_status(ctx);
+    // One step ahead of the device: the next is on its way while one runs, and the one too many at the end finds every
+    // sequence ended and does nothing.  Every step commits at least one token per live sequence.
+    volatile int *const done = ctx->pinned + 8;
+    for (long long i = 0; i < (long long)max_new_tokens + 2 && *done != ctx->request; ++i) {
+        xsm_status st = run_step(ctx);
         if (st != XSM_OK) return st;
-    }
-    while (budget > 0) {
-        const int n = (int)(budget < kChunkSteps ? budget : kChunkSteps);
-        xsm_status st = run_steps(ctx, n);
-        if (st != XSM_OK) return st;
-        budget -= n;
-        st = check_device_status(ctx);
-        if (st != XSM_OK) return st;
-        if (ctx->pinned[0] <= 0) break;
+        XSM_CUDA(ctx, cudaEventRecord(ctx->step_ev[i & 1], ctx->stream));
+        if (i > 0) XSM_CUDA(ctx, cudaEventSynchronize(ctx->step_ev[(i - 1) & 1]));
     }
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev1, ctx->stream));
     if (d_tokens || d_lengths) {
@@ -950,7 +501,6 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     float ms = 0.f;
     XSM_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-    ctx->last_wall_ms = ms;
     if (host_stats) {
         std::vector<unsigned long long> hist((size_t)D.B * (kMaxDraft + 1)), steps(D.B);
         std::vector<int> ngen(D.B);
@@ -1012,26 +562,16 @@ const char *xsm_last_error(const xsm_ctx *ctx) { return ctx ? ctx->err.c_str() :
 
 uint64_t xsm_kernel_launches(const xsm_ctx *ctx) { return ctx ? ctx->launches : 0; }
 
-// the exchange buffers hold fp32 words whose two lowest mantissa bits are a tag
-static void strip_tags(float *p, size_t n) {
-    uint32_t *u = reinterpret_cast<uint32_t *>(p);
-    for (size_t i = 0; i < n; ++i) u[i] &= ~3u;
-}
-
 xsm_status xsm_debug_get_logits(xsm_ctx *ctx, float *h_logits0, float *h_head_logits) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "no step has run");
     const Dev &D = ctx->dev;
     xsm_status st = check_device_status(ctx);
     if (st != XSM_OK) return st;
-    if (h_logits0) {
+    if (h_logits0)
         XSM_CUDA(ctx, cudaMemcpy(h_logits0, D.logits0, sizeof(float) * (size_t)D.M * D.V, cudaMemcpyDeviceToHost));
-        if (!ctx->use_chain) strip_tags(h_logits0, (size_t)D.M * D.V);
-    }
-    if (h_head_logits && D.K > 0) {
+    if (h_head_logits && D.K > 0)
         XSM_CUDA(ctx, cudaMemcpy(h_head_logits, D.hlogits, sizeof(float) * (size_t)D.K * D.M * D.V, cudaMemcpyDeviceToHost));
-        if (!ctx->use_chain) strip_tags(h_head_logits, (size_t)D.K * D.M * D.V);
-    }
     return XSM_OK;
 }
 
@@ -1068,12 +608,7 @@ xsm_status xsm_debug_set_drafts(xsm_ctx *ctx, const int32_t *h_drafts) {
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy2D(D.window + 1, sizeof(int32_t) * D.K1, h_drafts, sizeof(int32_t) * D.K,
                                sizeof(int32_t) * D.K, D.B, cudaMemcpyHostToDevice));
-    if (ctx->use_chain) {
-        XSM_CUDA(ctx, launch_embed_rows(D, D.K1, D.Mp, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
-        return XSM_OK;
-    }
-    XSM_CUDA(ctx, launch_embed(D, ctx->cfg.dtype, ctx->serial, ctx->stream));
-    ctx->launches += 1;
+    XSM_CUDA(ctx, launch_embed_rows(D, ctx->cfg.dtype, D.K1, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
     return XSM_OK;
 }
 
@@ -1095,24 +630,23 @@ xsm_status xsm_debug_get_state(xsm_ctx *ctx, int32_t *h_len, int32_t *h_window, 
 xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t capacity, int *n_rows, int *n_ctas) {
     if (!ctx || !h_times || !n_rows || !n_ctas) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_trace_step before xsm_prefill");
-    if (ctx->phase_launch) return fail(ctx, XSM_ERR_STATE, "the timeline is taken from the persistent kernel");
+    if (ctx->phase_launch) return fail(ctx, XSM_ERR_STATE, "the timeline is taken from overlapping launches");
     const int rows = 1 + 2 * ctx->n_stages;
-    const int ctas = ctx->use_chain ? kTraceCtas : ctx->grid;
-    const size_t words = (size_t)rows * ctas;
+    const size_t words = (size_t)rows * kTraceCtas;
     if (capacity < words) return fail(ctx, XSM_ERR_CAPACITY, "h_times is too small");
     unsigned long long *d_trace = at<unsigned long long>(ctx, ctx->lay.trace);
     XSM_CUDA(ctx, cudaMemsetAsync(d_trace, 0, 8 * words, ctx->stream));
     xsm_status st = set_max_new(ctx, INT_MAX);
     if (st != XSM_OK) return st;
     ctx->dev.trace = d_trace;
-    st = run_steps(ctx, 1);
+    st = run_step(ctx);
     ctx->dev.trace = nullptr;
     if (st != XSM_OK) return st;
     st = check_device_status(ctx);
     if (st != XSM_OK) return st;
     XSM_CUDA(ctx, cudaMemcpy(h_times, d_trace, 8 * words, cudaMemcpyDeviceToHost));
     *n_rows = rows;
-    *n_ctas = ctas;
+    *n_ctas = kTraceCtas;
     return XSM_OK;
 }
 
@@ -1122,8 +656,8 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     Dev &D = ctx->dev;
     RunParams r = ctx->run;
     if (h_tokens == nullptr || n <= 0) {
-        D.script = r.script = nullptr; D.script_n = r.script_n = 0; D.script_acc = r.script_acc = 0;
-        return ctx->use_chain ? set_run(ctx, r) : XSM_OK;
+        r.script = nullptr; r.script_n = r.script_acc = 0;
+        return set_run(ctx, r);
     }
     if (n > ctx->lay.tok_ld) return fail(ctx, XSM_ERR_INVALID_ARG, "script longer than max_seq_len + n_draft + 1");
     if (!(mean_accept >= 0.f) || mean_accept > (float)D.K) return fail(ctx, XSM_ERR_INVALID_ARG, "mean_accept must be in [0, n_draft]");
@@ -1132,16 +666,15 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     int *d_script = at<int>(ctx, ctx->lay.script);
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy(d_script, h_tokens, sizeof(int32_t) * (size_t)D.B * n, cudaMemcpyHostToDevice));
-    D.script = d_script; D.script_n = n; D.script_acc = (int)lrintf(mean_accept * 1024.f);
-    r.script = d_script; r.script_n = n; r.script_acc = D.script_acc;
-    return ctx->use_chain ? set_run(ctx, r) : XSM_OK;
+    r.script = d_script; r.script_n = n; r.script_acc = (int)lrintf(mean_accept * 1024.f);
+    return set_run(ctx, r);
 }
 
 xsm_status xsm_debug_set_wait_limits(xsm_ctx *ctx, uint32_t polls, uint32_t barrier_tries) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     ctx->dev.spin_limit = polls ? polls : kSpinLimit;
     ctx->dev.mbar_limit = barrier_tries ? barrier_tries : kMbarSpinLimit;
-    if (ctx->use_chain && ctx->prefilled) {      // the limits are part of the recordings
+    if (ctx->prefilled) {      // the limits are part of the recordings
         ctx->chain.forget();
         if (!ctx->chain.select(ctx->dev)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
     }
@@ -1152,15 +685,10 @@ xsm_status xsm_debug_launch_stage(xsm_ctx *ctx, int stage) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_launch_stage before xsm_prefill");
     if (stage < 0 || stage >= ctx->n_stages) return fail(ctx, XSM_ERR_INVALID_ARG, "no such stage");
-    if (ctx->use_chain) {
-        XSM_CUDA(ctx, launch_stage_gate(ctx->dev, stage, ctx->stream));
-        XSM_CUDA(ctx, ctx->chain.run_op(ctx->dev, stage, ctx->stream, &ctx->launches));
-        XSM_CUDA(ctx, launch_stage_mark(ctx->dev, (stage + 1) % ctx->n_stages, ctx->stream));
-        ctx->launches += 2;
-        return XSM_OK;
-    }
-    XSM_CUDA(ctx, launch_step(ctx->dev, ctx->cfg.dtype, stage, stage + 1, 1, ctx->serial, ctx->grid, ctx->smem_bytes, ctx->stream));
-    ctx->launches += 1;
+    XSM_CUDA(ctx, launch_stage_gate(ctx->dev, stage, ctx->stream));
+    XSM_CUDA(ctx, ctx->chain.run_op(ctx->dev, stage, ctx->stream, &ctx->launches));
+    XSM_CUDA(ctx, launch_stage_mark(ctx->dev, (stage + 1) % ctx->n_stages, ctx->stream));
+    ctx->launches += 2;
     return XSM_OK;
 }
 

@@ -347,7 +347,8 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     // the warps' states of a row -> the output, or this CTA's partial result.  Two neighbouring columns a thread.
     bf16 *out = A.out + (size_t)set * 2 * A.Mp * D.d;
     const int item = blockIdx.z * D.H + h, n_pairs = A.t * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
-    float *mine = A.part + ((size_t)(item * A.S + rank) * A.t) * LD;
+    // partial results: [items][S][t][DH + 2]; acount: CTAs of an item that have left theirs (zero between kernels)
+    float *mine = D.apart + ((size_t)(item * A.S + rank) * A.t) * LD;
     auto store = [&](int r, int c, float v0, float v1) {
         bf16 h0, l0, h1, l1;
         split_bf16(v0, h0, l0);
@@ -380,11 +381,11 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         __shared__ int s_last;
         __threadfence();
         __syncthreads();
-        if (tid == 0) s_last = atomicAdd(A.count + item, 1) == S - 1;
+        if (tid == 0) s_last = atomicAdd(D.acount + item, 1) == S - 1;
         __syncthreads();
         if (s_last) {
             __threadfence();
-            const float *all = A.part + ((size_t)item * A.S * A.t) * LD;
+            const float *all = D.apart + ((size_t)item * A.S * A.t) * LD;
             for (int e = tid; e < n_pairs; e += kAttnThreads) {
                 const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
                 float2 ml[8], os[8];
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
                 }
                 store(r, c, o0 / l, o1 / l);
             }
-            if (tid == 0) A.count[item] = 0;
+            if (tid == 0) D.acount[item] = 0;
         }
     }
     trace_mark(D, 2 + 2 * A.stage);

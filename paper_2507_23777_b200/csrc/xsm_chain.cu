@@ -76,6 +76,7 @@ bool Chain::init(const xsm_model_config &c, const WeightOffsets &w, const char *
     w_ = w;
     weights_ = weights;
     sms_ = sm_count;
+    if (c.dtype == 0) return true;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &encode_, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
         (void)cudaGetLastError();
@@ -104,8 +105,19 @@ bool Chain::init(const xsm_model_config &c, const WeightOffsets &w, const char *
 // Cluster size, rings and shared memory of a projection over `rows` token rows.  The row tiles of a stage (8 to 128) leave
 // SMs idle at one CTA each, so the columns are cut as far as all clusters still run at once.
 void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
-    if (plan_few(op, rows, Mp, kdim)) return;
     ProjArgs &A = op.proj;
+    if (c_.dtype == 0) {      // a warp for every unit as long as there are SMs; the activations of a chunk of columns in 96 KB
+        const int units = A.epi0 == PE_QKV ? A.g[0].units / 2 : A.g[0].units + (A.epi1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
+        A.kdim = kdim;
+        A.rows = rows;
+        A.Mp = rows;
+        A.ctas = std::min((units + 7) / 8, std::max(1, A.x_jobs ? sms_ / A.g[0].jobs : sms_));
+        A.chunk = std::min(kdim, 96 * 1024 / (4 * rows) / 128 * 128);
+        op.kind = ChainOp::F32;
+        op.smem = std::max(A.chunk * rows * 4, 8 * kF32Rows * 4);
+        return;
+    }
+    if (plan_few(op, rows, Mp, kdim)) return;
     A.kdim = kdim;
     A.rows = rows;
     A.Mp = Mp;
@@ -167,8 +179,6 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
     while (A.S < 8 && items * A.S * 2 <= sms_ + sms_ / 8) A.S *= 2;
     A.split = t <= 8 ? 640 : 128;
     if (cross) A.S = std::min(A.S, (D.C + A.split - 1) / A.split);
-    A.part = D.apart;
-    A.count = D.acount;
     const int round = upp == 1 || upp == 2 || upp == 4 ? 8 / upp : 1;
     const int pages = ((cross ? D.cpages : D.max_blocks) + A.S - 1) / A.S;
     const int budget = items * A.S > sms_ ? 100 * 1024 : 128 * 1024;
@@ -183,7 +193,8 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers, rows = D.B * t, Mp = (rows + 7) / 8 * 8;
     const bool ca = c.head_kind == 1;
     const float qscale = D.scale * 1.4426950408889634f;      // softmax in base 2
-    auto gain = [&](size_t off) { return (const void *)(weights_ + off * 2); };
+    const size_t es = c.dtype == 1 ? 2 : 4;
+    auto gain = [&](size_t off) { return (const void *)(weights_ + off * es); };
     const size_t head_stride = K > 1 ? w_.Wout[1] - w_.Wout[0] : 0;
     int shares = 1;                       // of the sums of squares of h: one from the embedding, then four per row tile of the writer
     auto proj = [&](int epi0, int epi1, int layer, const TensorMap &w0, const TensorMap *w1, size_t w_off, size_t w1_off, const void *x) -> ChainOp & {
@@ -195,8 +206,8 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
         op.maps.w1 = w1 ? *w1 : w0;
         ProjArgs &A = op.proj;
         A.x = (const bf16 *)x;
-        A.g[0].w = (const bf16 *)weights_ + w_off;
-        A.g[1].w = (const bf16 *)weights_ + w1_off;
+        A.g[0].w = (const bf16 *)(weights_ + w_off * es);
+        A.g[1].w = (const bf16 *)(weights_ + w1_off * es);
         A.g[0].w_stride = A.g[1].w_stride = head_stride;
         A.epi0 = epi0; A.epi1 = epi1; A.layer = layer; A.t = t; A.pos0 = -1; A.scale = qscale;
         return op;
@@ -218,7 +229,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
         group(op.proj.g[0], d, 128, 1, d, D.xa_, nullptr);
         op.proj.gain = gain(next_gain);
         plan_proj(op, rows, Mp, kdim);
-        shares = op.kind == ChainOp::FEW ? op.proj.ctas : d / 128 * 4;
+        shares = op.kind == ChainOp::PROJ ? d / 128 * 4 : op.proj.ctas;
     };
     auto normed = [&](ChainOp &op) {
         op.proj.norm = 1;
@@ -282,51 +293,16 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     return true;
 }
 
-// The weights of a step in the order of their use are one stream (of bytes, closed to a ring: the first layer follows the
-// last projection).  Every projection fetches as much of it ahead as it reads itself, kAheadBytes further on.
-void Chain::plan_ahead(std::vector<ChainOp> &ops) {
-    constexpr size_t kAheadBytes = 32 << 20;
-    struct Piece { const char *p; size_t n, at; };      // at: offset in the stream
-    std::vector<Piece> pieces;
-    size_t total = 0;
-    auto add = [&](const bf16 *p, size_t elems) { pieces.push_back({(const char *)p, elems * 2, total}); total += elems * 2; };
-    struct Use { ProjArgs *A; size_t begin, end; };
-    std::vector<Use> uses;
-    for (ChainOp &op : ops) {
-        if (op.kind != ChainOp::PROJ && op.kind != ChainOp::FEW) continue;
-        ProjArgs &A = op.proj;
-        const size_t begin = total;
-        for (int q = 0; q < (A.epi1 >= 0 || A.epi0 == PE_GATEUP ? 2 : 1); ++q) {
-            const size_t one = (size_t)(A.epi0 == PE_GATEUP ? A.g[0].units : A.g[q].units) * A.kdim;
-            const int jobs = A.epi0 == PE_GATEUP ? 1 : A.g[q].jobs;
-            for (int j = 0; j < jobs; ++j) add(A.g[q].w + j * A.g[q].w_stride, one);
-        }
-        uses.push_back({&A, begin, total});
-    }
-    if (total <= 2 * kAheadBytes) return;      // the model stays in L2 anyway
-    for (Use &u : uses) {
-        size_t lo = (u.begin + kAheadBytes) % total, left = u.end - u.begin;
-        for (int q = 0; q < 2 && left > 0; ++q) {
-            size_t i = 0;
-            while (pieces[i].at + pieces[i].n <= lo) ++i;
-            const size_t off = lo - pieces[i].at, n = std::min(left, pieces[i].n - off);
-            u.A->ahead[q] = pieces[i].p + off;
-            u.A->ahead_bytes[q] = (unsigned)n;
-            left -= n;
-            lo = (lo + n) % total;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------------------- running
 
 cudaError_t Chain::run(const Dev &D, const ChainOp &op, int t, const ChainLaunch &L) {
     switch (op.kind) {
         case ChainOp::PROJ: return launch_proj_umma(D, op.proj, &op.maps, op.smem, L);
         case ChainOp::FEW: return launch_proj_few(D, op.proj, op.smem, L);
-        case ChainOp::ATTN: return launch_attn(D, op.attn, L);
-        case ChainOp::TAIL: return launch_tail(D, op.proj.stage, L);
-        case ChainOp::EMBED: return launch_embed_rows(D, t, (D.B * t + 7) / 8 * 8, op.attn.pos0, L);
+        case ChainOp::F32: return launch_proj_f32(D, op.proj, op.smem, L);
+        case ChainOp::ATTN: return c_.dtype == 1 ? launch_attn(D, op.attn, L) : launch_attn_f32(D, op.attn, L);
+        case ChainOp::TAIL: return launch_tail(D, c_.dtype, op.proj.stage, L);
+        case ChainOp::EMBED: return launch_embed_rows(D, c_.dtype, t, op.attn.pos0, L);
     }
     return cudaErrorInvalidValue;
 }
@@ -337,7 +313,6 @@ bool Chain::select(const Dev &D) {
         if ((int)plans_.size() >= kMaxPlans) plans_.clear();
         std::unique_ptr<StepPlan> p(new StepPlan());
         if (!build(D, D.K1, false, p->ops)) return false;
-        plan_ahead(p->ops);
         for (size_t i = 0; i < p->ops.size(); ++i) p->ops[i].proj.stage = p->ops[i].attn.stage = (int)i;
         it = plans_.emplace(D.B, std::move(p)).first;
     }
@@ -382,11 +357,10 @@ cudaError_t Chain::step(const Dev &D, cudaStream_t st, bool graph, bool overlap,
 }
 
 cudaError_t Chain::ingest(const Dev &D, int n, cudaStream_t st, unsigned long long *count) {
-    // chunks of as many positions of every sequence as fit 128 token rows, of equal length
-    const int most = std::max(1, kMaxTokens / D.B), chunks = (n + most - 1) / most, t = (n + chunks - 1) / chunks;
+    // chunks of as many positions of every sequence as fit the token rows that the kernels take, of equal length
+    const int most = std::max(1, (c_.dtype == 1 ? kMaxTokens : kF32Rows) / D.B), chunks = (n + most - 1) / most, t = (n + chunks - 1) / chunks;
     std::vector<ChainOp> ops;
     if (!build(D, t, true, ops)) return cudaErrorInvalidValue;
-    plan_ahead(ops);
     const ChainLaunch L{st, true, count};
     cudaError_t e;
     for (int pos = 0; pos < n; pos += t) {

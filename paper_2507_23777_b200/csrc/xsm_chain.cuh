@@ -45,8 +45,6 @@ struct ProjArgs {
     int slots, chunk;                 // weight tiles in shared memory, columns of one
     int late_go;                      // let the next kernel start only after this one's wait
     float scale;                      // queries
-    const char *ahead[2];             // weights that a later kernel of the step reads: fetched into L2 meanwhile
-    unsigned ahead_bytes[2];
     const void *gain;                 // PE_ADD: gain of the RMSNorm that reads h next; PE_HEADY / PE_HEADADD: of the final RMSNorm
     __half *q;                        // PE_QKV, PE_QUERY: planes [2][Mp][d] (a set per decoding head)
     ProjGroup g[2];
@@ -58,8 +56,6 @@ struct AttnArgs {
     int cross, sets, layer;           // sets: decoding heads that attend in this stage (cross-attention heads), else 1
     int t, rows, Mp, pos0, pos_end;   // as in ProjArgs
     int S, split, slots;              // most CTAs per (sequence, head), keys for each; page pairs in shared memory
-    float *part;                      // partial results [items][S][t][d_head + 2]
-    int *count;                       // [items] CTAs that have left theirs (zero between kernels)
     const void *pool;                 // cache tiles
     const __half *q;                  // planes [2][Mp][d] (a set per decoding head)
     bf16 *out;                        // planes of d columns (a set per decoding head; layout: xsm_proj.cuh)
@@ -118,9 +114,13 @@ cudaError_t launch_proj_few(const Dev &D, const ProjArgs &A, int smem, const Cha
 int resident_clusters(int size);      // clusters of the projection below that the device runs at a time, an SM for each CTA
 cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L);
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
-cudaError_t launch_tail(const Dev &D, int stage, const ChainLaunch &L);
+// fp32 models: at most this many token rows
+constexpr int kF32Rows = 24;
+cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L);
+cudaError_t launch_attn_f32(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
+cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L);
 // embeds the window of every sequence (pos0 < 0) or t prompt tokens of each from position pos0 on
-cudaError_t launch_embed_rows(const Dev &D, int t, int Mp, int pos0, const ChainLaunch &L);
+cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, const ChainLaunch &L);
 // state of a new request: pool, sequences with prompt_len - 1 positions in the cache, first window
 cudaError_t launch_begin(const Dev &D, const RunParams &R, cudaStream_t st);
 // single stages (inspection): waits until the stages before `stage` have run one by one; notes that `done` of them have

@@ -1,0 +1,348 @@
+// The kernels of the launch chain for fp32 models (the parity configuration: at most kF32Rows token rows, plain FMA).
+// Activations are [token row][column] floats; the cache holds fp32 tiles.
+#include "xsm_proj.cuh"
+
+namespace xsm {
+
+constexpr int kF32Warps = 8, kF32Threads = kF32Warps * 32;
+
+// ------------------------------------------------------------------------------------ projections
+
+// A warp owns units (a row, or a pair of rows: rotation partners, gate and up), its lanes the columns.  The weights of the
+// first unit are in registers before the wait; the activations are staged in shared memory, a chunk of columns at a time.
+// MT: token rows that a warp accumulates (at least A.rows).
+template <int MT, int EPI0, int EPI1>
+__global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, const ProjArgs A) {
+    extern __shared__ __align__(16) float xs[];       // [rows][chunk]
+    __shared__ float s_inv[MT];
+    constexpr bool PAIRS = EPI0 == PE_QKV || EPI0 == PE_GATEUP;
+    constexpr int R = PAIRS ? 2 : 1, AHEAD = 4;       // rows of a unit; quads of columns fetched before the wait
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (A.pos0 < 0 && !A.late_go && __ldcg(D.n_active) == 0) {      // every sequence has ended in an earlier step
+        chain_wait();
+        return;
+    }
+    if (!A.late_go) chain_go();
+    const int job = A.x_jobs ? blockIdx.x / A.ctas : 0, cta = A.x_jobs ? blockIdx.x - job * A.ctas : blockIdx.x;
+    const int units = EPI0 == PE_QKV ? A.g[0].units >> 1 : A.g[0].units + (EPI1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
+    const int K = A.kdim, M = A.rows, half = D.dh >> 1, chunk = A.chunk;
+    // weight row r (0, 1) of a unit; u and j become its place in its group
+    auto weights = [&](int unit, int r, int &u, int &j, bool &second) -> const float * {
+        u = unit; j = job; second = false;
+        if (EPI0 == PE_QKV) {
+            const int hd = D.d >> 1, sec = unit / hd, i = unit - sec * hd, head = i / half;
+            u = sec * D.d + head * D.dh + (i - head * half);
+            return reinterpret_cast<const float *>(A.g[0].w) + (size_t)(u + r * half) * K;
+        }
+        if (EPI0 == PE_GATEUP) return reinterpret_cast<const float *>(A.g[r].w) + (size_t)unit * K;
+        if (EPI1 >= 0 && u >= A.g[0].units) {
+            u -= A.g[0].units;
+            j = u / A.g[1].units;
+            u -= j * A.g[1].units;
+            second = true;
+            return reinterpret_cast<const float *>(A.g[1].w) + (size_t)j * A.g[1].w_stride + (size_t)u * K;
+        }
+        return reinterpret_cast<const float *>(A.g[0].w) + (size_t)job * A.g[0].w_stride + (size_t)u * K;
+    };
+    const int first = cta * kF32Warps + warp, step = A.ctas * kF32Warps;
+    int u, j;
+    bool second;
+    const float *w[R];
+    float4 wa[R][AHEAD];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        w[r] = weights(min(first, units - 1), r, u, j, second);
+#pragma unroll
+        for (int q = 0; q < AHEAD; ++q)
+            if (q * 128 + lane * 4 < min(chunk, K)) wa[r][q] = __ldg(reinterpret_cast<const float4 *>(w[r] + q * 128 + lane * 4));
+    }
+    if (A.stage == 0) trace_mark(D, 0);
+    chain_wait();
+    if (A.late_go) chain_go();
+    trace_mark(D, 1 + 2 * A.stage);
+    if (A.ss_parts > 0)
+        for (int m = warp; m < M; m += kF32Warps) {
+            float ss = 0.f;
+            for (int p = lane; p < A.ss_parts; p += 32) ss += __ldcg(D.ss + (size_t)m * kShareLd + p);
+            ss = warp_sum(ss);
+            if (lane == 0) s_inv[m] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+        }
+    const float *x = reinterpret_cast<const float *>(A.x) + (A.x_jobs ? (size_t)job * M * K : 0);
+    auto stage = [&](int k0) {      // columns [k0, k0 + chunk) of all token rows
+        const int n4 = min(chunk, K - k0) >> 2;
+        __syncthreads();
+        for (int i = tid; i < M * n4; i += kF32Threads) {
+            const int m = i / n4, c = i - m * n4;
+            reinterpret_cast<float4 *>(xs + m * chunk)[c] = __ldcg(reinterpret_cast<const float4 *>(x + (size_t)m * K + k0) + c);
+        }
+        __syncthreads();
+    };
+    if (chunk >= K) stage(0);
+    float ssq_mine = 0.f;      // PE_ADD: lane m sums the squares of its token row over the warp's units
+    for (int base = cta * kF32Warps; base < units; base += step) {      // (all warps of the CTA together: they share the staged columns)
+        const int unit = base + warp;
+        float acc[R][MT];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int m = 0; m < MT; ++m) acc[r][m] = 0.f;
+        const bool mine = unit < units;
+#pragma unroll
+        for (int r = 0; r < R; ++r) w[r] = weights(min(unit, units - 1), r, u, j, second);
+        for (int k0 = 0; k0 < K; k0 += chunk) {
+            if (chunk < K) stage(k0);
+            if (!mine) continue;
+            const int n = min(chunk, K - k0);
+            auto columns = [&](int c, const float4 (&wv)[R]) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    if (m < M) {
+                        const float4 xv = *reinterpret_cast<const float4 *>(xs + m * chunk + c);
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            acc[r][m] = fmaf(wv[r].x, xv.x, fmaf(wv[r].y, xv.y, fmaf(wv[r].z, xv.z, fmaf(wv[r].w, xv.w, acc[r][m]))));
+                    }
+                }
+            };
+            int q0 = 0;
+            if (unit == first && k0 == 0) {
+#pragma unroll
+                for (int q = 0; q < AHEAD; ++q) {
+                    float4 wv[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) wv[r] = wa[r][q];
+                    if (q * 128 + lane * 4 < n) columns(q * 128 + lane * 4, wv);
+                }
+                q0 = AHEAD;
+            }
+            for (int c = q0 * 128 + lane * 4; c < n; c += 128) {
+                float4 wv[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) wv[r] = __ldg(reinterpret_cast<const float4 *>(w[r] + k0 + c));
+                columns(c, wv);
+            }
+        }
+        if (!mine) continue;
+        // sums over the lanes; lane m keeps token row m
+        float v = 0.f, v2 = 0.f;
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            if (m < M) {
+                const float s = warp_sum(acc[0][m]);
+                if (lane == m) v = s;
+                if (PAIRS) {
+                    const float s2 = warp_sum(acc[R - 1][m]);
+                    if (lane == m) v2 = s2;
+                }
+            }
+        }
+        const int m = lane;
+        if (m >= M) continue;
+        const float inv = A.ss_parts > 0 ? s_inv[m] : 1.f;
+        if (EPI0 == PE_ADD) {
+            const float h = __ldcg(D.h + (size_t)m * D.d + u) + v;
+            D.h[(size_t)m * D.d + u] = h;
+            reinterpret_cast<float *>(A.g[0].out)[(size_t)m * A.g[0].ld + u] = h * __ldg(reinterpret_cast<const float *>(A.gain) + u);
+            ssq_mine += h * h;
+        } else if (EPI0 == PE_QKV) {
+            v *= inv;
+            v2 *= inv;
+            const int sec = u >= D.d ? (u >= 2 * D.d ? 2 : 1) : 0, c = u - sec * D.d, head = c / D.dh, e = c - head * D.dh;
+            const int b = m / A.t, jj = m - b * A.t, pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + jj;
+            const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
+            float o1 = v, o2 = v2;
+            if (sec < 2 && live) {
+                const float2 cs = __ldg(D.rope_cs + (size_t)pos * half + e);
+                o1 = v * cs.x - v2 * cs.y;
+                o2 = v2 * cs.x + v * cs.y;
+            }
+            if (sec == 0) {
+                float *q = reinterpret_cast<float *>(A.q) + (size_t)m * D.d + c;
+                q[0] = o1 * A.scale;
+                q[half] = o2 * A.scale;
+            } else if (live) {
+                const int page = __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos));
+                float *tile = kv_tile<float>(D, D.kv_pool, D.n_pages, A.layer, sec - 1, page, head) + tile_off<float>(row_in_page(D, pos), e, D.dh);
+                tile[0] = o1;
+                tile[half] = o2;
+            }
+        } else if (EPI0 == PE_GATEUP) {
+            reinterpret_cast<float *>(A.g[0].out)[(size_t)m * A.g[0].ld + u] = silu_f(v * inv) * (v2 * inv);
+        } else if (EPI0 == PE_QUERY || (EPI1 == PE_QUERY && second)) {
+            reinterpret_cast<float *>(A.q)[((size_t)j * M + m) * D.d + u] = v * inv * A.scale;
+        } else if (EPI0 == PE_HEADADD || (EPI1 == PE_HEADY && second)) {
+            const float g = __ldcg(D.h + (size_t)m * D.d + u) * inv * __ldg(reinterpret_cast<const float *>(A.gain) + u);
+            const ProjGroup &G = A.g[EPI1 >= 0 ? 1 : 0];
+            reinterpret_cast<float *>(G.out)[((size_t)j * M + m) * G.ld + u] = g + (EPI0 == PE_HEADADD ? v : silu_f(v * inv));
+        } else {
+            A.g[0].logits[((size_t)j * D.M + m) * A.g[0].ld + u] = A.norm ? v * inv : v;
+        }
+    }
+    if (EPI0 == PE_ADD) {
+        // the CTA's shares of the sums of squares
+        __syncthreads();
+        if (lane < M) xs[warp * MT + lane] = ssq_mine;
+        __syncthreads();
+        if (tid < M) {
+            float s = 0.f;
+            for (int q = 0; q < kF32Warps; ++q) s += xs[q * MT + tid];
+            D.ss[(size_t)tid * kShareLd + cta] = s;
+        }
+    }
+    trace_mark(D, 2 + 2 * A.stage);
+}
+
+// -------------------------------------------------------------------------------------- attention
+
+// One CTA per (sequence, head): 256 keys at a time, a thread scores one key against all t rows, then the threads sum the
+// values of a column each, a share of the keys each, and the shares are added in order.
+template <int T>
+__global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, const AttnArgs A) {
+    extern __shared__ __align__(16) float sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, dh = D.dh;
+    const int h = blockIdx.y, b = blockIdx.z % D.B, set = blockIdx.z / D.B;
+    const bool cross = A.cross != 0;
+    float *qs = sm, *p = qs + T * dh, *o = p + T * kF32Threads, *red = o + T * dh;      // queries, weights [T][256], output, per-warp values
+    float *m_run = red + kF32Warps * T, *l_run = m_run + T, *f_run = l_run + T;
+    chain_go();
+    const bool dead = A.pos0 < 0 && __ldcg(D.finished + b) != 0;
+    chain_wait();
+    if (dead) return;
+    trace_mark(D, 1 + 2 * A.stage);
+    const int start = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);
+    const int n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + A.t, A.pos_end) : start + A.t;
+    const float *q = reinterpret_cast<const float *>(A.q) + ((size_t)set * A.rows + (size_t)b * A.t) * D.d + h * dh;
+    for (int i = tid; i < T * dh; i += kF32Threads) {
+        const int r = i / dh;
+        qs[i] = r < A.t ? __ldcg(q + (size_t)r * D.d + i - r * dh) : 0.f;
+        o[i] = 0.f;
+    }
+    if (tid < T) { m_run[tid] = kNegBig; l_run[tid] = 0.f; }
+    auto tile = [&](int kv, int key) -> const float * {
+        const int pg = page_of(D, key), page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
+        return kv_tile<float>(D, const_cast<void *>(A.pool), cross ? D.B * D.cpages : D.n_pages, cross && A.sets > 1 ? set : A.layer, kv, page, h) +
+               (size_t)row_in_page(D, key) * dh;
+    };
+    for (int k0 = 0; k0 < n_keys; k0 += kF32Threads) {
+        const int key = k0 + tid;
+        float s[T];
+#pragma unroll
+        for (int r = 0; r < T; ++r) s[r] = 0.f;
+        __syncthreads();
+        if (key < n_keys) {
+            const float4 *kr = reinterpret_cast<const float4 *>(tile(0, key));
+#pragma unroll 4
+            for (int c = 0; c < (dh >> 2); ++c) {
+                const float4 kv = __ldcg(kr + c);
+#pragma unroll
+                for (int r = 0; r < T; ++r) {
+                    const float4 qv = *reinterpret_cast<const float4 *>(qs + r * dh + 4 * c);
+                    s[r] = fmaf(kv.x, qv.x, fmaf(kv.y, qv.y, fmaf(kv.z, qv.z, fmaf(kv.w, qv.w, s[r]))));
+                }
+            }
+        }
+        // running maximum of every row, weights relative to it
+#pragma unroll
+        for (int r = 0; r < T; ++r) {
+            if (key >= n_keys || (!cross && key > start + r)) s[r] = -INFINITY;
+            float m = s[r];
+#pragma unroll
+            for (int k = 16; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
+            if (lane == 0) red[warp * T + r] = m;
+        }
+        __syncthreads();
+        if (tid < T) {
+            float m = m_run[tid];
+            for (int w = 0; w < kF32Warps; ++w) m = fmaxf(m, red[w * T + tid]);
+            f_run[tid] = exp2f(m_run[tid] - m);
+            m_run[tid] = m;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < T; ++r) {
+            const float e = exp2f(s[r] - m_run[r]);
+            p[r * kF32Threads + tid] = e;
+            const float l = warp_sum(e);
+            if (lane == 0) red[warp * T + r] = l;
+        }
+        __syncthreads();
+        if (tid < T) {
+            float l = l_run[tid] * f_run[tid];
+            for (int w = 0; w < kF32Warps; ++w) l += red[w * T + tid];
+            l_run[tid] = l;
+        }
+        // values: column c, keys part, part + parts, ...; every part its own place, added in order
+        const int parts = kF32Threads / dh, c = tid % dh, part = tid / dh, n = min(kF32Threads, n_keys - k0);
+        float acc[T];
+#pragma unroll
+        for (int r = 0; r < T; ++r) acc[r] = 0.f;
+#pragma unroll 4
+        for (int k = part; k < n; k += parts) {
+            const float v = __ldcg(tile(1, k0 + k) + c);
+#pragma unroll
+            for (int r = 0; r < T; ++r) acc[r] = fmaf(p[r * kF32Threads + k], v, acc[r]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < T; ++r) p[r * kF32Threads + tid] = acc[r];
+        __syncthreads();
+        for (int i = tid; i < T * dh; i += kF32Threads) {
+            const int r = i / dh, cc = i - r * dh;
+            float v = o[i] * f_run[r];
+            for (int k = 0; k < parts; ++k) v += p[r * kF32Threads + k * dh + cc];
+            o[i] = v;
+        }
+    }
+    __syncthreads();
+    float *out = reinterpret_cast<float *>(A.out) + ((size_t)set * A.rows + (size_t)b * A.t) * D.d + h * dh;
+    for (int i = tid; i < A.t * dh; i += kF32Threads) {
+        const int r = i / dh;
+        out[(size_t)r * D.d + i - r * dh] = o[i] / l_run[r];
+    }
+    trace_mark(D, 2 + 2 * A.stage);
+}
+
+// ---------------------------------------------------------------------------------------- launches
+
+template <int MT, int EPI0, int EPI1>
+static cudaError_t launch_proj_instance(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
+    void (*fn)(const Dev, const ProjArgs) = proj_f32_kernel<MT, EPI0, EPI1>;
+    cudaError_t e = open_kernel((const void *)fn, smem, false);
+    if (e != cudaSuccess) return e;
+    return L.launch(dim3(A.x_jobs ? A.ctas * A.g[0].jobs : A.ctas), dim3(kF32Threads), smem, 1, (const void *)fn, D, A);
+}
+template <int MT>
+static cudaError_t launch_proj_rows(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_proj_instance<MT, a, b>(D, A, smem, L)
+    XSM_EPI(PE_QKV, -1);
+    XSM_EPI(PE_ADD, -1);
+    XSM_EPI(PE_QUERY, -1);
+    XSM_EPI(PE_GATEUP, -1);
+    XSM_EPI(PE_LOGITS, -1);
+    XSM_EPI(PE_LOGITS, PE_HEADY);
+    XSM_EPI(PE_LOGITS, PE_QUERY);
+    XSM_EPI(PE_HEADADD, -1);
+#undef XSM_EPI
+    return cudaErrorInvalidValue;
+}
+cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
+    if (A.rows <= 4) return launch_proj_rows<4>(D, A, smem, L);
+    if (A.rows <= 8) return launch_proj_rows<8>(D, A, smem, L);
+    return launch_proj_rows<kF32Rows>(D, A, smem, L);
+}
+
+template <int T>
+static cudaError_t launch_attn_rows(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    void (*fn)(const Dev, const AttnArgs) = attn_f32_kernel<T>;
+    const int smem = (2 * T * D.dh + T * kF32Threads + kF32Warps * T + 3 * T) * 4;
+    cudaError_t e = open_kernel((const void *)fn, smem, false);
+    if (e != cudaSuccess) return e;
+    return L.launch(dim3(1, D.H, D.B * A.sets), dim3(kF32Threads), smem, 1, (const void *)fn, D, A);
+}
+cudaError_t launch_attn_f32(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    if (A.t <= 4) return launch_attn_rows<4>(D, A, L);
+    if (A.t <= 8) return launch_attn_rows<8>(D, A, L);
+    return launch_attn_rows<kF32Rows>(D, A, L);
+}
+
+}  // namespace xsm

@@ -21,7 +21,7 @@ struct WeightMaps { TensorMap w0, w1; };
 
 // one kernel of a chain
 struct ChainOp {
-    enum Kind { PROJ, FEW, ATTN, TAIL, EMBED } kind;
+    enum Kind { PROJ, FEW, F32, ATTN, TAIL, EMBED } kind;
     WeightMaps maps;
     ProjArgs proj;
     AttnArgs attn;
@@ -54,7 +54,6 @@ class Chain {
 
   private:
     bool weight_map(TensorMap *out, size_t elem_off, int rows, int kdim, int count, size_t stride_elems, int box_rows);
-    void plan_ahead(std::vector<ChainOp> &ops);
     bool build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops);
     void plan_proj(ChainOp &op, int rows, int Mp, int kdim);
     bool plan_few(ChainOp &op, int rows, int Mp, int kdim);

@@ -1,29 +1,7 @@
-// Host-side launchers and the kernels around the decoding step: prefill (condition keys and values, first
-// window), inspection, export.  The step kernel itself is compiled in xsm_step_dh*.cu from xsm_device.cuh.
-#include "xsm_device.cuh"
+// The kernels around the decoding step: prefill (keys and values of the condition), inspection, export.
+#include "xsm_common.cuh"
 
 namespace xsm {
-
-cudaError_t launch_step_dh32(const Dev &, int, int, int, int, uint32_t, int, int, cudaStream_t, int *);
-cudaError_t launch_step_dh64(const Dev &, int, int, int, int, uint32_t, int, int, cudaStream_t, int *);
-cudaError_t launch_step_dh128(const Dev &, int, int, int, int, uint32_t, int, int, cudaStream_t, int *);
-
-static cudaError_t step_dispatch(const Dev &D, int dtype, int st_lo, int st_hi, int n_steps, uint32_t serial0, int grid,
-                                 int smem_bytes, cudaStream_t st, int *max_grid) {
-    if (D.dh == 32) return launch_step_dh32(D, dtype, st_lo, st_hi, n_steps, serial0, grid, smem_bytes, st, max_grid);
-    if (D.dh == 64) return launch_step_dh64(D, dtype, st_lo, st_hi, n_steps, serial0, grid, smem_bytes, st, max_grid);
-    return launch_step_dh128(D, dtype, st_lo, st_hi, n_steps, serial0, grid, smem_bytes, st, max_grid);
-}
-
-// resident CTAs of the instance that serves D (D.M and D.dh set)
-cudaError_t step_kernel_setup(const Dev &D, int dtype, int smem_bytes, int *max_grid) {
-    return step_dispatch(D, dtype, 0, 0, 0, 0u, 0, smem_bytes, nullptr, max_grid);
-}
-
-cudaError_t launch_step(const Dev &D, int dtype, int st_lo, int st_hi, int n_steps, uint32_t serial0, int grid,
-                        int smem_bytes, cudaStream_t st) {
-    return step_dispatch(D, dtype, st_lo, st_hi, n_steps, serial0, grid, smem_bytes, st, nullptr);
-}
 
 // ------------------------------------------------------------------------------- prefill kernels
 
@@ -196,61 +174,6 @@ cudaError_t launch_cross_kv(const Dev &D, int dtype, const void *W, const size_t
             cross_kv_kernel<bf16><<<grid, 256, 0, st>>>(D, (const bf16 *)W, wkc_off, wvc_off, (const bf16 *)cond, pool);
     } else
         cross_kv_kernel<float><<<grid, 256, 0, st>>>(D, (const float *)W, wkc_off, wvc_off, (const float *)cond, pool);
-    return cudaGetLastError();
-}
-
-// shared memory of prepare_window's partial sums: one float per 16 bytes of the window's embedding rows
-static size_t window_scratch_bytes(const Dev &D, int elem_bytes) { return (size_t)D.K1 * (D.d / (16 / elem_bytes)) * sizeof(float); }
-
-// Algorithm 1 line 1: pool reset, then per-sequence state, first window and its pages.
-__global__ void init_pool_kernel(const Dev D) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < D.n_pages) D.free_stack[i] = D.n_pages - 1 - i;
-    if (i == 0) { *D.n_free = D.n_pages; *D.n_active = D.B; *D.status = 0; }
-}
-
-template <typename WT> __global__ void __launch_bounds__(256) init_seq_kernel(const Dev D, uint32_t serial) {
-    const int b = blockIdx.x, K1 = D.K1;
-    extern __shared__ float s_scratch[];      // K1 * d_model / (elements per 16 bytes) floats
-    __shared__ int s_win[kMaxDraft + 1];
-    if (threadIdx.x == 0) {
-        D.len[b] = 0; D.finished[b] = 0; D.n_gen[b] = 0; D.n_blocks[b] = 0; D.step_idx[b] = 0u;
-        D.acc_len[b] = 0; D.steps[b] = 0ull; D.step_n_new[b] = 0;
-        for (int a = 0; a <= kMaxDraft; ++a) D.hist[(size_t)b * (kMaxDraft + 1) + a] = 0ull;
-        const int *pr = D.prompt + (size_t)b * D.prompt_len;
-        D.ingest_left[b] = D.prompt_len - 1;
-        if (D.prompt_len == 1) {
-            s_win[0] = pr[0];
-            draw_initial_drafts(D, b, s_win);
-        } else {
-            for (int j = 0; j < K1; ++j) s_win[j] = j < D.prompt_len ? pr[j] : 0;
-        }
-        for (int j = 0; j < K1; ++j) D.window[b * K1 + j] = s_win[j];
-    }
-    __syncthreads();
-    prepare_window<WT>(D, b, serial, 0, 0, s_win, 256, s_scratch);
-    __threadfence();
-    __syncthreads();
-    publish_header(D, b, serial, 0, D.prompt_len > 1 ? 2 : 0);
-}
-
-cudaError_t launch_init(const Dev &D, int dtype, uint32_t serial, cudaStream_t st) {
-    const int n = max(D.n_pages, 1);
-    init_pool_kernel<<<(n + 255) / 256, 256, 0, st>>>(D);
-    if (dtype == 1) init_seq_kernel<bf16><<<D.B, 256, window_scratch_bytes(D, 2), st>>>(D, serial);
-    else init_seq_kernel<float><<<D.B, 256, window_scratch_bytes(D, 4), st>>>(D, serial);
-    return cudaGetLastError();
-}
-
-// re-gather the window embeddings after the drafts were replaced from outside
-template <typename WT> __global__ void __launch_bounds__(256) embed_kernel(const Dev D, uint32_t serial) {
-    const int b = blockIdx.x;
-    extern __shared__ float s_scratch[];
-    if (!D.finished[b]) prepare_window<WT>(D, b, serial, D.len[b], D.n_blocks[b], D.window + b * D.K1, 256, s_scratch);
-}
-cudaError_t launch_embed(const Dev &D, int dtype, uint32_t serial, cudaStream_t st) {
-    if (dtype == 1) embed_kernel<bf16><<<D.B, 256, window_scratch_bytes(D, 2), st>>>(D, serial);
-    else embed_kernel<float><<<D.B, 256, window_scratch_bytes(D, 4), st>>>(D, serial);
     return cudaGetLastError();
 }
 

@@ -20,21 +20,5 @@ __device__ __forceinline__ void store_split(bf16 *x, int Mp, int m, int k, float
     p[0] = hi;
     p[kLo] = lo;
 }
-constexpr int kShareLd = 160;      // shares of a row's sum of squares: [row][kShareLd]
-
-// Asks L2 for this CTA's share of the weights that a later kernel reads (one warp).  The kernels of a step are short against
-// the latency of HBM and its weights' transfer; with what is needed 32 MB further on already on its way, memory is read at
-// an even rate and a kernel's own copies come from L2.
-__device__ __forceinline__ void fetch_ahead(const ProjArgs &A, unsigned cta, unsigned n_ctas) {
-    constexpr unsigned kPiece = 4096;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const unsigned pieces = (A.ahead_bytes[q] + kPiece - 1) / kPiece;
-        for (unsigned i = cta + n_ctas * (threadIdx.x & 31); i < pieces; i += n_ctas * 32) {
-            const unsigned off = i * kPiece, n = min(kPiece, A.ahead_bytes[q] - off);
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(A.ahead[q] + off), "r"(n) : "memory");
-        }
-    }
-}
 
 }  // namespace xsm

@@ -76,7 +76,6 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
             }
         }
         __syncwarp();
-        fetch_ahead(A, blockIdx.x, gridDim.x);
     }
     if (A.stage == 0) trace_mark(D, 0);
 

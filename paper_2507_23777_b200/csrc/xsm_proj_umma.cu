@@ -91,7 +91,6 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     };
     if (tid == 0)
         for (int i = 0; i < min(n, na); ++i) load_a(i);
-    if (warp == 3) fetch_ahead(A, blockIdx.x, gridDim.x);
     if (A.stage == 0) trace_mark(D, 0);
     const bf16 *x = A.x + (A.x_jobs ? (size_t)job * 2 * Mp * A.kdim : 0);
     chain_wait();

@@ -13,31 +13,37 @@ __device__ __forceinline__ uint32_t rand24(const RunParams &R, int seq, uint32_t
 
 // ---------------------------------------------------------------------------------------- embedding
 
-// Row m of the window <- the embedding of `tok`: master copy, planes (times the gain of the first RMSNorm) and sum of squares.
-// All threads of the block; d / 8 <= kTailThreads.
-static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, float *sh) {
-    const bf16 *E = reinterpret_cast<const bf16 *>(D.E), *gain = reinterpret_cast<const bf16 *>(D.gain_first);
-    const int c = threadIdx.x * 8, d = D.d;
+// Row m of the window <- the embedding of `tok`: master copy, the copy that the first projection reads (times the gain of the
+// first RMSNorm) and its sum of squares.  All threads of the block, 16 bytes of a row each.
+template <typename WT> static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, float *sh) {
+    constexpr int N = 16 / (int)sizeof(WT);
+    const WT *E = reinterpret_cast<const WT *>(D.E), *gain = reinterpret_cast<const WT *>(D.gain_first);
+    const int d = D.d;
     float ssq = 0.f;
-    if (c < d) {
-        tok = min(max(tok, 0), D.V - 1);
-        const uint4 ev = __ldg(reinterpret_cast<const uint4 *>(E + (size_t)tok * d + c)), gv = __ldg(reinterpret_cast<const uint4 *>(gain + c));
-        const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
-        float v[8];
-        __align__(16) bf16 hi[8], lo[8];
+    tok = min(max(tok, 0), D.V - 1);
+    for (int c = threadIdx.x * N; c < d; c += kTailThreads * N) {
+        __align__(16) WT e[N], g[N];
+        *reinterpret_cast<uint4 *>(e) = __ldg(reinterpret_cast<const uint4 *>(E + (size_t)tok * d + c));
+        *reinterpret_cast<uint4 *>(g) = __ldg(reinterpret_cast<const uint4 *>(gain + c));
+        float v[N];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            v[q] = __uint_as_float((q & 1) ? ew[q >> 1] & 0xFFFF0000u : ew[q >> 1] << 16);
-            const float g = __uint_as_float((q & 1) ? gw[q >> 1] & 0xFFFF0000u : gw[q >> 1] << 16);
-            split_bf16(v[q] * g, hi[q], lo[q]);
+        for (int q = 0; q < N; ++q) {
+            v[q] = to_f(e[q]);
             ssq += v[q] * v[q];
         }
-        float4 *h = reinterpret_cast<float4 *>(D.h + (size_t)m * d + c);
-        h[0] = make_float4(v[0], v[1], v[2], v[3]);
-        h[1] = make_float4(v[4], v[5], v[6], v[7]);
-        bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + plane_off(Mp, m, c);
-        *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
-        *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
+#pragma unroll
+        for (int q = 0; q < N; q += 4) *reinterpret_cast<float4 *>(D.h + (size_t)m * d + c + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+        if constexpr (sizeof(WT) == 2) {
+            __align__(16) bf16 hi[N], lo[N];
+#pragma unroll
+            for (int q = 0; q < N; ++q) split_bf16(v[q] * to_f(g[q]), hi[q], lo[q]);
+            bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + plane_off(Mp, m, c);
+            *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
+            *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
+        } else {
+            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(D.xa_) + (size_t)m * d + c) =
+                make_float4(v[0] * to_f(g[0]), v[1] * to_f(g[1]), v[2] * to_f(g[2]), v[3] * to_f(g[3]));
+        }
     }
     ssq = warp_sum(ssq);
     __syncthreads();
@@ -50,7 +56,7 @@ static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, float *sh
     }
 }
 
-__global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0) {
+template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0) {
     __shared__ float sh[kTailWarps];
     chain_wait();
     chain_go();      // (only now: kernels further down may read what earlier chunks wrote before they wait themselves)
@@ -63,10 +69,12 @@ __global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, i
         if (__ldcg(D.finished + b)) return;
         tok = __ldcg(D.window + b * t + j);
     }
-    embed_row(D, blockIdx.x, Mp, tok, sh);
+    embed_row<WT>(D, blockIdx.x, Mp, tok, sh);
 }
-cudaError_t launch_embed_rows(const Dev &D, int t, int Mp, int pos0, const ChainLaunch &L) {
-    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, (const void *)embed_rows_kernel, D, t, Mp, pos0);
+cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, const ChainLaunch &L) {
+    const void *fn = dtype == 1 ? (const void *)embed_rows_kernel<bf16> : (const void *)embed_rows_kernel<float>;
+    const int Mp = (D.B * t + 7) / 8 * 8;
+    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, fn, D, t, Mp, pos0);
 }
 
 // ------------------------------------------------------------------------------------ block reductions
@@ -284,7 +292,7 @@ static __device__ void reserve_pages(const Dev &D, int b, int len, int held) {
 // Algorithm 1 lines 7-12 for one sequence by a cluster of K + 1 CTAs, one per window row and slot: CTA j < K decides on
 // the draft behind row j; with the accept length a known to all, CTA i draws candidate i from row a of the backbone (i = 0)
 // or of head i; every CTA works out the commit, CTA 0 writes it down, and CTA i embeds row i of the next window.
-__global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int stage) {
+template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int stage) {
     extern __shared__ __align__(16) float row_buf[];
     __shared__ TailShared sh;
     const int K1 = D.K1, K = D.K, V = D.V, tid = threadIdx.x;
@@ -438,16 +446,17 @@ __global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int sta
         }
     }
     __syncthreads();
-    if (!sh.state[5]) embed_row(D, b * K1 + slot, D.Mp, sh.win[slot], sh.red);
+    if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], sh.red);
     if (K > 0) { cluster_arrive(); cluster_wait(); }      // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }
 
-cudaError_t launch_tail(const Dev &D, int stage, const ChainLaunch &L) {
+cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L) {
+    const void *fn = dtype == 1 ? (const void *)tail_kernel<bf16> : (const void *)tail_kernel<float>;
     const int smem = (size_t)D.V * 4 <= (size_t)D.tail_row_bytes ? (D.V * 4 + 15) / 16 * 16 : 16;
-    cudaError_t e = open_kernel((const void *)tail_kernel, smem, D.K1 > 8);
+    cudaError_t e = open_kernel(fn, smem, D.K1 > 8);
     if (e != cudaSuccess) return e;
-    return L.launch(dim3(D.B * D.K1), dim3(kTailThreads), smem, D.K1, (const void *)tail_kernel, D, stage);
+    return L.launch(dim3(D.B * D.K1), dim3(kTailThreads), smem, D.K1, fn, D, stage);
 }
 
 // --------------------------------------------------------------------------------- start of a request
