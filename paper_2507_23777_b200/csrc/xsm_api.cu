@@ -70,18 +70,18 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.script = take(cur, 4 * B * L.tok_ld);
     L.rp = take(cur, sizeof(RunParams));
     // activations of a step or of a chunk of a prompt: four bytes an element (bf16 models: hi and lo parts)
-    const size_t row = 4 * (size_t)kMaxTokens, nh = ca ? (size_t)c.n_draft : 0;
+    const size_t rows = prompt_rows(c), row = 4 * rows, step_row = 4 * (size_t)kMaxTokens, nh = ca ? (size_t)c.n_draft : 0;
     L.h = take(cur, row * d);
     L.rope_cs = take(cur, 8 * (size_t)(c.max_seq_len + K1 + 1) * (dh / 2));
     L.xa = take(cur, row * d);
     L.qp = take(cur, row * d);
     L.aa = take(cur, row * d);
     L.actp = take(cur, row * f);
-    L.yp = take(cur, row * d * c.n_draft);
-    L.hq = take(cur, row * d * nh);
-    L.ha = take(cur, row * d * nh);
+    L.yp = take(cur, step_row * d * c.n_draft);
+    L.hq = take(cur, step_row * d * nh);
+    L.ha = take(cur, step_row * d * nh);
     L.ss = take(cur, row * kShareLd);
-    L.apart = take(cur, row * kSplitCtas * (dh + 2));
+    L.apart = take(cur, step_row * kSplitCtas * (dh + 2));
     L.acount = take(cur, 4 * kSplitCtas);
     L.logits0 = take(cur, 4 * M * V);
     L.hlogits = take(cur, 4 * M * V * (c.n_draft > 0 ? c.n_draft : 1));

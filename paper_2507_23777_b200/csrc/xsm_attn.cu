@@ -180,11 +180,13 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     extern __shared__ __align__(128) char smem[];
     __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z % D.B, set = blockIdx.z / D.B;
+    // (tiles of a sequence's rows: those that see the most keys first)
+    const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z % D.B, zz = blockIdx.z / D.B, set = zz % A.sets;
+    const int q0 = (A.qt - 1 - zz / A.sets) * kTokenTile, t_rows = min(A.t - q0, kTokenTile), t_cap = min(A.t, kTokenTile);
     const int P = D.P, upp = P >> 5, slots = A.slots;
     const bool cross = A.cross != 0;
-    const int start = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);      // (the state was written by an earlier step)
-    const int n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + A.t, A.pos_end) : start + A.t;
+    const int first = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);      // (the state was written by an earlier step)
+    const int start = first + q0, n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + t_rows, A.pos_end) : start + t_rows;
     const int S = min(A.S, (n_keys + A.split - 1) / A.split);                    // CTAs that take part
     if (rank >= S) return;
     // few rows: a warp looks only at the pages whose units it owns when the units of 1, 2 or 4 pages fill a round of the
@@ -206,19 +208,19 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     }
     const int np = page_of(D, n_keys + P - 1), p_lo = rank * np / S, p_hi = (rank + 1) * np / S;
     const uint32_t tile_bytes = (uint32_t)P * DH * 2u, ring = smem_u32(smem);
-    const int qt_n = FEW ? 1 : (A.t + 15) >> 4;                       // row tiles
+    const int qt_n = FEW ? 1 : (t_rows + 15) >> 4;                       // row tiles
     int wq = 1;                                                       // warps that share the keys between them: kAttnWarps / wq
     if (!FEW)
         while (wq < qt_n) wq <<= 1;
     const int kg_n = kAttnWarps / wq;
     // parked states of the warps [kAttnWarps][rows][DH + 2]; they reuse the ring
     constexpr int LD = DH + 2;
-    const int srows = FEW ? A.t : 16;
+    const int srows = FEW ? t_rows : 16;
     float *st = reinterpret_cast<float *>(smem);
 
     if (warp == kAttnWarps) {
         if (lane == 0) {
-            const int n_old = cross ? np : page_of(D, start);         // pages that nobody writes in this step
+            const int n_old = cross ? np : page_of(D, first);         // pages that nobody writes in this step
             bool waited = false;
             for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
                 if (!waited && pg >= n_old) {
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         __syncthreads();                 // (1) every page has been consumed
     } else {
         const int g = lane >> 2, t4 = lane & 3;
-        const __half *qhi = A.q + (size_t)set * 2 * A.Mp * D.d + (size_t)(b * A.t) * D.d + h * DH, *qlo = qhi + (size_t)A.Mp * D.d;
+        const __half *qhi = A.q + (size_t)set * 2 * A.qp * D.d + (size_t)(b * A.t + q0) * D.d + h * DH, *qlo = qhi + (size_t)A.qp * D.d;
         chain_wait();
         trace_mark(D, 1 + 2 * A.stage);
         if (FEW) {
@@ -251,8 +253,8 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
 #pragma unroll
             for (int c = 0; c < DH / 8; ++c) {
                 const size_t o = (size_t)g * D.d + 8 * c + 2 * t4;
-                qh[c] = g < A.t ? ldcg_u32(qhi + o) : 0u;
-                ql[c] = g < A.t ? ldcg_u32(qlo + o) : 0u;
+                qh[c] = g < t_rows ? ldcg_u32(qhi + o) : 0u;
+                ql[c] = g < t_rows ? ldcg_u32(qlo + o) : 0u;
             }
             FewState<DH> ws;
 #pragma unroll
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int r = 2 * t4 + c;
-                if (r < A.t) {
+                if (r < t_rows) {
                     float *dst = st + (warp * srows + r) * LD;
 #pragma unroll
                     for (int dp = 0; dp < DH / 16; ++dp) {
@@ -302,8 +304,8 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
                 for (int q = 0; q < 4; ++q) {
                     const int r = (q & 1) ? r1 : r0;
                     const size_t o = (size_t)r * D.d + ks * 16 + 2 * t4 + (q >> 1) * 8;
-                    qh[ks][q] = r < A.t ? ldcg_u32(qhi + o) : 0u;
-                    ql[ks][q] = r < A.t ? ldcg_u32(qlo + o) : 0u;
+                    qh[ks][q] = r < t_rows ? ldcg_u32(qhi + o) : 0u;
+                    ql[ks][q] = r < t_rows ? ldcg_u32(qlo + o) : 0u;
                 }
             }
             RowsState<DH> ws;
@@ -312,7 +314,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
             ws.m[0] = ws.m[1] = kNegBig;
             ws.l[0] = ws.l[1] = 0.f;
             const int row_lim0 = cross ? D.C - 1 : start + r0, row_lim1 = cross ? D.C - 1 : start + r1;
-            const int last = cross ? D.C - 1 : start + min(qt * 16 + 15, A.t - 1);      // last key of the row tile
+            const int last = cross ? D.C - 1 : start + min(qt * 16 + 15, t_rows - 1);      // last key of the row tile
             for (int i = 0; i < p_hi - p_lo; ++i) {
                 const int sl = i % slots;
                 mbar_wait(smem_u32(&full[sl]), (uint32_t)((i / slots) & 1), D.mbar_limit, D.status);
@@ -331,7 +333,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
                 ws.l[c] += __shfl_xor_sync(0xffffffffu, ws.l[c], 1);
                 ws.l[c] += __shfl_xor_sync(0xffffffffu, ws.l[c], 2);
                 const int r = c ? r1 : r0;
-                if (r < A.t) {
+                if (r < t_rows) {
                     float *dst = st + (warp * 16 + g + 8 * c) * LD;
 #pragma unroll
                     for (int dn = 0; dn < DH / 8; ++dn) {
@@ -346,14 +348,15 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     __syncthreads();
     // the warps' states of a row -> the output, or this CTA's partial result.  Two neighbouring columns a thread.
     bf16 *out = A.out + (size_t)set * 2 * A.Mp * D.d;
-    const int item = blockIdx.z * D.H + h, n_pairs = A.t * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
+    const int item = blockIdx.z * D.H + h, n_pairs = t_rows * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
     // partial results: [items][S][t][DH + 2]; acount: CTAs of an item that have left theirs (zero between kernels)
-    float *mine = D.apart + ((size_t)(item * A.S + rank) * A.t) * LD;
+    float *mine = D.apart + ((size_t)(item * A.S + rank) * t_cap) * LD;
     auto store = [&](int r, int c, float v0, float v1) {
         bf16 h0, l0, h1, l1;
         split_bf16(v0, h0, l0);
         split_bf16(v1, h1, l1);
-        bf16 *p = out + plane_off(A.Mp, b * A.t + r, h * DH + c);
+        const int row = b * A.t + q0 + r;
+        bf16 *p = out + (size_t)(row / kTokenTile) * 2 * A.Mp * D.d + plane_off(A.Mp, row % kTokenTile, h * DH + c);
         *reinterpret_cast<__nv_bfloat162 *>(p) = __nv_bfloat162(h0, h1);
         *reinterpret_cast<__nv_bfloat162 *>(p + kLo) = __nv_bfloat162(l0, l1);
     };
@@ -385,13 +388,13 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         __syncthreads();
         if (s_last) {
             __threadfence();
-            const float *all = D.apart + ((size_t)item * A.S * A.t) * LD;
+            const float *all = D.apart + ((size_t)item * A.S * t_cap) * LD;
             for (int e = tid; e < n_pairs; e += kAttnThreads) {
                 const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
                 float2 ml[8], os[8];
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
-                    const float *src = all + ((size_t)s * A.t + r) * LD;
+                    const float *src = all + ((size_t)s * t_cap + r) * LD;
                     ml[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + DH)) : make_float2(kNegBig, 0.f);
                     os[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + c)) : make_float2(0.f, 0.f);
                 }
@@ -421,7 +424,7 @@ static cudaError_t launch_instance(const Dev &D, const AttnArgs &A, const ChainL
     const int smem = ring > park ? ring : park;
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
-    return L.launch(dim3(A.S, D.H, D.B * A.sets), dim3(kAttnThreads), smem, 1, (const void *)fn, D, A);
+    return L.launch(dim3(A.S, D.H, D.B * A.sets * A.qt), dim3(kAttnThreads), smem, 1, (const void *)fn, D, A);
 }
 
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {

@@ -124,18 +124,21 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
     // (clusters have to fit into a GPC: of six CTAs 22 run at a time, of eight 15; a cluster more than that is a second wave)
     int S = 1;
+    const int tile_rows = std::min(rows, kTokenTile);
     for (int s = 2; s <= std::min(8, nblk); ++s)
-        if (tiles <= clusters_[s]) S = s;
+        if (tiles * A.tt <= clusters_[s]) S = s;
     A.S = S;
-    A.tps = ((rows + 3) / 4 + S - 1) / S * 4;
-    const int n = (nblk + S - 1) / S, b_bytes = 2 * Mp * 128, a_bytes = 128 * 128;
-    const int room = kProjSmemMax - 1024 - S * A.tps * 512;
+    A.tps = ((tile_rows + 3) / 4 + S - 1) / S * 4;
+    const int n = (nblk + S - 1) / S, b_bytes = 2 * Mp * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
+    // more tiles than SMs: two CTAs to an SM
+    const int room = (tiles * A.tt * S > sms_ ? kProjSmemMax / 2 : kProjSmemMax) - 1024 - (S > 1 ? sums : 0);
     A.nb = std::min(n, std::max(2, std::min(kProjRing, (room / 3) / b_bytes)));
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
     A.tmem_cols = 32;
     while (A.tmem_cols < 2 * Mp) A.tmem_cols *= 2;
-    op.smem = 1024 + A.na * a_bytes + A.nb * b_bytes + S * A.tps * 512;
+    const int rings = A.na * a_bytes + A.nb * b_bytes;
+    op.smem = 1024 + (S > 1 ? rings + sums : std::max(rings, sums));
 }
 
 // The projections over few token rows: how the units are dealt out, passes over the columns, shared memory.  False: the
@@ -173,7 +176,8 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
     A.sets = sets;
     A.t = t;
     A.Mp = Mp;
-    const int items = D.B * D.H * sets, upp = D.P / 32, pair = 2 * D.P * D.dh * 2;
+    A.qt = (t + kTokenTile - 1) / kTokenTile;
+    const int items = D.B * D.H * sets * A.qt, upp = D.P / 32, pair = 2 * D.P * D.dh * 2;
     // about one CTA per SM at most; few rows: one more for every 640 keys (a merge costs as much as four units of 32 keys)
     A.S = 1;
     while (A.S < 8 && items * A.S * 2 <= sms_ + sms_ / 8) A.S *= 2;
@@ -190,7 +194,8 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
 
 bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     const xsm_model_config &c = c_;
-    const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers, rows = D.B * t, Mp = (rows + 7) / 8 * 8;
+    const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers, rows = D.B * t;
+    const int Mp = rows > kTokenTile ? kTokenTile : (rows + 7) / 8 * 8, tt = (rows + kTokenTile - 1) / kTokenTile, qp = tt * Mp;
     const bool ca = c.head_kind == 1;
     const float qscale = D.scale * 1.4426950408889634f;      // softmax in base 2
     const size_t es = c.dtype == 1 ? 2 : 4;
@@ -209,7 +214,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
         A.g[0].w = (const bf16 *)(weights_ + w_off * es);
         A.g[1].w = (const bf16 *)(weights_ + w1_off * es);
         A.g[0].w_stride = A.g[1].w_stride = head_stride;
-        A.epi0 = epi0; A.epi1 = epi1; A.layer = layer; A.t = t; A.pos0 = -1; A.scale = qscale;
+        A.epi0 = epi0; A.epi1 = epi1; A.layer = layer; A.t = t; A.pos0 = -1; A.scale = qscale; A.tt = tt; A.qp = qp;
         return op;
     };
     auto group = [&](ProjGroup &g, int units, int tile_rows, int jobs, int ld, void *out, float *logits) {
@@ -221,7 +226,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
         ChainOp &op = ops.back();
         op.kind = ChainOp::ATTN;
         op.attn = plan_attn(D, cross, sets, t, Mp);
-        op.attn.layer = layer; op.attn.rows = rows; op.attn.pos0 = -1;
+        op.attn.layer = layer; op.attn.rows = rows; op.attn.pos0 = -1; op.attn.qp = qp;
         op.attn.pool = pool; op.attn.q = (const __half *)q; op.attn.out = (bf16 *)out;
     };
     auto residual = [&](int layer, const TensorMap &w, size_t w_off, const void *x, int kdim, size_t next_gain) {
@@ -295,6 +300,14 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
 
 // ---------------------------------------------------------------------------------------- running
 
+// Token rows of a chunk of a prompt.  bf16: 2048, where the narrowest projections (d_model 1024) have a tile for nearly
+// every SM; no more than the prompts of a batch can have.
+int prompt_rows(const xsm_model_config &c) {
+    if (c.dtype == 0) return kF32Rows;
+    const long long all = ((long long)c.max_batch * c.max_seq_len + kTokenTile - 1) / kTokenTile * kTokenTile;
+    return (int)std::max<long long>(kTokenTile, std::min<long long>(2048, all));
+}
+
 cudaError_t Chain::run(const Dev &D, const ChainOp &op, int t, const ChainLaunch &L) {
     switch (op.kind) {
         case ChainOp::PROJ: return launch_proj_umma(D, op.proj, &op.maps, op.smem, L);
@@ -358,7 +371,7 @@ cudaError_t Chain::step(const Dev &D, cudaStream_t st, bool graph, bool overlap,
 
 cudaError_t Chain::ingest(const Dev &D, int n, cudaStream_t st, unsigned long long *count) {
     // chunks of as many positions of every sequence as fit the token rows that the kernels take, of equal length
-    const int most = std::max(1, (c_.dtype == 1 ? kMaxTokens : kF32Rows) / D.B), chunks = (n + most - 1) / most, t = (n + chunks - 1) / chunks;
+    const int most = std::max(1, prompt_rows(c_) / D.B), chunks = (n + most - 1) / most, t = (n + chunks - 1) / chunks;
     std::vector<ChainOp> ops;
     if (!build(D, t, true, ops)) return cudaErrorInvalidValue;
     const ChainLaunch L{st, true, count};

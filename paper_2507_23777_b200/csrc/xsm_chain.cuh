@@ -19,6 +19,7 @@ enum ProjEpilogue : int {
     PE_HEADADD = 6    // g + y as bf16 planes (cross-attention decoding head)
 };
 
+constexpr int kTokenTile = 128;       // token rows that share a plane
 constexpr int kProjRing = 16;         // most operand blocks of one kind that a CTA keeps in shared memory
 
 // A group of weight matrices of one shape in a projection stage: one matrix, or one per decoding head.
@@ -34,7 +35,8 @@ struct ProjGroup {
 struct ProjArgs {
     int epi0, epi1;                   // of the two groups; epi1 < 0: one group
     int stage;                        // index of the kernel in its chain
-    int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8)
+    int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8, at most kTokenTile)
+    int tt, qp;                       // tiles of token rows (a plane set for each); rows of the planes of queries
     int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
     int S, tps;                       // CTAs per cluster (cuts of the columns), token rows each of them finishes
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns
@@ -46,7 +48,7 @@ struct ProjArgs {
     int late_go;                      // let the next kernel start only after this one's wait
     float scale;                      // queries
     const void *gain;                 // PE_ADD: gain of the RMSNorm that reads h next; PE_HEADY / PE_HEADADD: of the final RMSNorm
-    __half *q;                        // PE_QKV, PE_QUERY: planes [2][Mp][d] (a set per decoding head)
+    __half *q;                        // PE_QKV, PE_QUERY: planes [2][qp][d] (a set per decoding head)
     ProjGroup g[2];
 };
 
@@ -54,10 +56,11 @@ struct ProjArgs {
 struct AttnArgs {
     int stage;
     int cross, sets, layer;           // sets: decoding heads that attend in this stage (cross-attention heads), else 1
-    int t, rows, Mp, pos0, pos_end;   // as in ProjArgs
+    int t, rows, Mp, qp, pos0, pos_end;      // as in ProjArgs
+    int qt;                           // tiles of kTokenTile rows of a sequence
     int S, split, slots;              // most CTAs per (sequence, head), keys for each; page pairs in shared memory
     const void *pool;                 // cache tiles
-    const __half *q;                  // planes [2][Mp][d] (a set per decoding head)
+    const __half *q;                  // planes [2][qp][d] (a set per decoding head)
     bf16 *out;                        // planes of d columns (a set per decoding head; layout: xsm_proj.cuh)
 };
 

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
     extern __shared__ __align__(16) float xs[];       // [rows][chunk]
     __shared__ float s_inv[MT];
     constexpr bool PAIRS = EPI0 == PE_QKV || EPI0 == PE_GATEUP;
-    constexpr int R = PAIRS ? 2 : 1, AHEAD = 4;       // rows of a unit; quads of columns fetched before the wait
+    constexpr int R = PAIRS ? 2 : 1, AHEAD = PAIRS ? 4 : 8;       // rows of a unit; quads of columns fetched before the wait
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (A.pos0 < 0 && !A.late_go && __ldcg(D.n_active) == 0) {      // every sequence has ended in an earlier step
         chain_wait();
@@ -194,23 +194,40 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
 
 // -------------------------------------------------------------------------------------- attention
 
-// One CTA per (sequence, head): 256 keys at a time, a thread scores one key against all t rows, then the threads sum the
-// values of a column each, a share of the keys each, and the shares are added in order.
+// One CTA per (sequence, head): 128 keys and values at a time in shared memory (those that the step does not write are
+// fetched before the wait), two threads score a key against all t rows, then the threads sum the values of a column each,
+// a share of the keys each, and the shares are added in order.
+constexpr int kF32Keys = kF32Threads / 2;
 template <int T>
 __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, const AttnArgs A) {
     extern __shared__ __align__(16) float sm[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, dh = D.dh;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, dh = D.dh, ld = dh + 4;
     const int h = blockIdx.y, b = blockIdx.z % D.B, set = blockIdx.z / D.B;
     const bool cross = A.cross != 0;
-    float *qs = sm, *p = qs + T * dh, *o = p + T * kF32Threads, *red = o + T * dh;      // queries, weights [T][256], output, per-warp values
+    float *ks = sm, *vs = ks + kF32Keys * ld, *qs = vs + kF32Keys * ld;
+    float *p = qs + T * dh, *o = p + T * kF32Threads, *red = o + T * dh;      // weights [T][keys] (then shares), output, per-warp values
     float *m_run = red + kF32Warps * T, *l_run = m_run + T, *f_run = l_run + T;
     chain_go();
     const bool dead = A.pos0 < 0 && __ldcg(D.finished + b) != 0;
+    const int start = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);      // (the state was written by an earlier step)
+    const int n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + A.t, A.pos_end) : start + A.t, n_old = cross ? D.C : start;
+    auto fetch = [&](int k0, int lo, int hi) {      // keys and values [lo, hi) into the places of the chunk at k0
+        const int c4 = dh >> 2, n = (hi - lo) * c4;
+        for (int i = tid; i < n; i += kF32Threads) {
+            const int kk = i / c4, c = i - kk * c4, key = lo + kk, pg = page_of(D, key);
+            const int page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
+            const int pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
+            const size_t off = (size_t)row_in_page(D, key) * dh + 4 * c;
+            const float4 kv = __ldcg(reinterpret_cast<const float4 *>(kv_tile<float>(D, const_cast<void *>(A.pool), pages, lay, 0, page, h) + off));
+            const float4 vv = __ldcg(reinterpret_cast<const float4 *>(kv_tile<float>(D, const_cast<void *>(A.pool), pages, lay, 1, page, h) + off));
+            *reinterpret_cast<float4 *>(ks + (key - k0) * ld + 4 * c) = kv;
+            *reinterpret_cast<float4 *>(vs + (key - k0) * ld + 4 * c) = vv;
+        }
+    };
+    if (!dead) fetch(0, 0, min(kF32Keys, n_old));
     chain_wait();
     if (dead) return;
     trace_mark(D, 1 + 2 * A.stage);
-    const int start = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);
-    const int n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + A.t, A.pos_end) : start + A.t;
     const float *q = reinterpret_cast<const float *>(A.q) + ((size_t)set * A.rows + (size_t)b * A.t) * D.d + h * dh;
     for (int i = tid; i < T * dh; i += kF32Threads) {
         const int r = i / dh;
@@ -218,25 +235,21 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
         o[i] = 0.f;
     }
     if (tid < T) { m_run[tid] = kNegBig; l_run[tid] = 0.f; }
-    auto tile = [&](int kv, int key) -> const float * {
-        const int pg = page_of(D, key), page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
-        return kv_tile<float>(D, const_cast<void *>(A.pool), cross ? D.B * D.cpages : D.n_pages, cross && A.sets > 1 ? set : A.layer, kv, page, h) +
-               (size_t)row_in_page(D, key) * dh;
-    };
-    for (int k0 = 0; k0 < n_keys; k0 += kF32Threads) {
-        const int key = k0 + tid;
+    for (int k0 = 0; k0 < n_keys; k0 += kF32Keys) {
+        const int n = min(kF32Keys, n_keys - k0), key = k0 + (tid >> 1), part = tid & 1;
+        fetch(k0, k0 == 0 ? min(kF32Keys, n_old) : k0, k0 + n);
+        __syncthreads();
         float s[T];
 #pragma unroll
         for (int r = 0; r < T; ++r) s[r] = 0.f;
-        __syncthreads();
         if (key < n_keys) {
-            const float4 *kr = reinterpret_cast<const float4 *>(tile(0, key));
+            const float *kr = ks + (tid >> 1) * ld + part * (dh >> 1), *qr = qs + part * (dh >> 1);
 #pragma unroll 4
-            for (int c = 0; c < (dh >> 2); ++c) {
-                const float4 kv = __ldcg(kr + c);
+            for (int c = 0; c < (dh >> 1); c += 4) {
+                const float4 kv = *reinterpret_cast<const float4 *>(kr + c);
 #pragma unroll
                 for (int r = 0; r < T; ++r) {
-                    const float4 qv = *reinterpret_cast<const float4 *>(qs + r * dh + 4 * c);
+                    const float4 qv = *reinterpret_cast<const float4 *>(qr + r * dh + c);
                     s[r] = fmaf(kv.x, qv.x, fmaf(kv.y, qv.y, fmaf(kv.z, qv.z, fmaf(kv.w, qv.w, s[r]))));
                 }
             }
@@ -244,10 +257,11 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
         // running maximum of every row, weights relative to it
 #pragma unroll
         for (int r = 0; r < T; ++r) {
+            s[r] += __shfl_xor_sync(0xffffffffu, s[r], 1);
             if (key >= n_keys || (!cross && key > start + r)) s[r] = -INFINITY;
             float m = s[r];
 #pragma unroll
-            for (int k = 16; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
+            for (int k = 16; k > 1; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
             if (lane == 0) red[warp * T + r] = m;
         }
         __syncthreads();
@@ -261,8 +275,8 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
 #pragma unroll
         for (int r = 0; r < T; ++r) {
             const float e = exp2f(s[r] - m_run[r]);
-            p[r * kF32Threads + tid] = e;
-            const float l = warp_sum(e);
+            if (part == 0) p[r * kF32Keys + (tid >> 1)] = e;
+            const float l = warp_sum(part == 0 ? e : 0.f);
             if (lane == 0) red[warp * T + r] = l;
         }
         __syncthreads();
@@ -271,16 +285,16 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
             for (int w = 0; w < kF32Warps; ++w) l += red[w * T + tid];
             l_run[tid] = l;
         }
-        // values: column c, keys part, part + parts, ...; every part its own place, added in order
-        const int parts = kF32Threads / dh, c = tid % dh, part = tid / dh, n = min(kF32Threads, n_keys - k0);
+        // values: column c, keys share, share + shares, ...; every share its own place, added in order
+        const int shares = kF32Threads / dh, c = tid % dh, share = tid / dh;
         float acc[T];
 #pragma unroll
         for (int r = 0; r < T; ++r) acc[r] = 0.f;
 #pragma unroll 4
-        for (int k = part; k < n; k += parts) {
-            const float v = __ldcg(tile(1, k0 + k) + c);
+        for (int k = share; k < n; k += shares) {
+            const float v = vs[k * ld + c];
 #pragma unroll
-            for (int r = 0; r < T; ++r) acc[r] = fmaf(p[r * kF32Threads + k], v, acc[r]);
+            for (int r = 0; r < T; ++r) acc[r] = fmaf(p[r * kF32Keys + k], v, acc[r]);
         }
         __syncthreads();
 #pragma unroll
@@ -289,7 +303,7 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
         for (int i = tid; i < T * dh; i += kF32Threads) {
             const int r = i / dh, cc = i - r * dh;
             float v = o[i] * f_run[r];
-            for (int k = 0; k < parts; ++k) v += p[r * kF32Threads + k * dh + cc];
+            for (int k = 0; k < shares; ++k) v += p[r * kF32Threads + k * dh + cc];
             o[i] = v;
         }
     }
@@ -334,7 +348,7 @@ cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const Cha
 template <int T>
 static cudaError_t launch_attn_rows(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
     void (*fn)(const Dev, const AttnArgs) = attn_f32_kernel<T>;
-    const int smem = (2 * T * D.dh + T * kF32Threads + kF32Warps * T + 3 * T) * 4;
+    const int smem = (2 * kF32Keys * (D.dh + 4) + 2 * T * D.dh + T * kF32Threads + kF32Warps * T + 3 * T) * 4;
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     return L.launch(dim3(1, D.H, D.B * A.sets), dim3(kF32Threads), smem, 1, (const void *)fn, D, A);

@@ -37,6 +37,8 @@ struct StepPlan {
     ~StepPlan();
 };
 
+int prompt_rows(const xsm_model_config &c);      // most token rows of a chunk of a prompt (buffers are sized for them)
+
 class Chain {
   public:
     ~Chain();

@@ -9,6 +9,9 @@
 // accumulator (asynchronous 16-byte stores that count on the receiver's barrier), and they are added in rank order:
 // results do not depend on timing.
 //
+// A chunk of a prompt has more token rows: tiles of 128 of them, two CTAs to an SM, so that one's products run under the
+// other's epilogue.
+//
 // Weights do not depend on the rest of the step: their copies start before the kernel waits for its predecessor.
 #include "xsm_proj.cuh"
 
@@ -29,9 +32,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     __shared__ __align__(8) uint64_t bars[4 * kProjRing + 1];      // A full, A empty, B full, B empty, done
     __shared__ __align__(8) uint64_t recv_bar;                      // the peers' shares of this CTA's token rows
     __shared__ uint32_t tmem_slot;
-    __shared__ float s_inv[kMaxTokens];
-    __shared__ int s_pos[kMaxTokens], s_swz[kMaxTokens];
-    __shared__ long long s_cache[kMaxTokens];
+    __shared__ float s_inv[kTokenTile];
+    __shared__ int s_pos[kTokenTile], s_swz[kTokenTile];
+    __shared__ long long s_cache[kTokenTile];
     constexpr bool TWO = EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = A.S, rank = S > 1 ? (int)cluster_rank() : 0, Mp = A.Mp;
@@ -39,7 +42,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         chain_wait();
         return;
     }
-    int tile = blockIdx.x / S, job = 0, z = A.layer, grp = 0;
+    // a tile of weight rows and a tile of token rows: neighbours share the weights
+    const int token_tile = A.tt > 1 ? (int)(blockIdx.x / S) % A.tt : 0, mb = token_tile * kTokenTile, rows = min(kTokenTile, A.rows - mb);
+    int tile = blockIdx.x / S / A.tt, job = 0, z = A.layer, grp = 0;
     if (EPI1 >= 0 && tile >= A.g[0].tiles) {
         tile -= A.g[0].tiles;
         grp = 1;
@@ -52,9 +57,10 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const int u0 = tile * (TWO ? 64 : 128);
     const int nblk = A.kdim / kBlockK, k_lo = rank * nblk / S, n = (rank + 1) * nblk / S - k_lo;
     const int na = A.na, nb = A.nb;
-    const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, A.rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
+    const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
     const uint32_t b_bytes = (uint32_t)(2 * Mp) * kBlockK * 2u;
-    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = sb + (uint32_t)nb * b_bytes;
+    // operand rings; behind them (one CTA to a tile: in their place, when the products are done) the partial sums
+    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = S > 1 ? sb + (uint32_t)nb * b_bytes : sa;
     float *recv = reinterpret_cast<float *>(smem + (srecv - sa));
     auto bar = [&](int kind, int i) { return smem_u32(&bars[kind * kProjRing + i]); };
     const uint32_t done = smem_u32(&bars[4 * kProjRing]);
@@ -92,7 +98,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     if (tid == 0)
         for (int i = 0; i < min(n, na); ++i) load_a(i);
     if (A.stage == 0) trace_mark(D, 0);
-    const bf16 *x = A.x + (A.x_jobs ? (size_t)job * 2 * Mp * A.kdim : 0);
+    const bf16 *x = A.x + (size_t)(A.x_jobs ? job : token_tile) * 2 * Mp * A.kdim;
     chain_wait();
     if (A.late_go) chain_go();
     trace_mark(D, 1 + 2 * A.stage);
@@ -129,7 +135,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             float inv = 1.f;
             if (A.ss_parts > 0) {
                 float ss = 0.f;
-                const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)m * kShareLd);
+                const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)(mb + m) * kShareLd);
                 for (int p0 = 0; p0 < A.ss_parts; p0 += 32) {        // 32 shares in flight, added in order
                     float4 v[8];
 #pragma unroll
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             }
             s_inv[i] = inv;
             if (EPI0 == PE_QKV) {
-                const int b = m / A.t, j = m - b * A.t;
+                const int b = (mb + m) / A.t, j = mb + m - b * A.t;
                 const int pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + j;
                 const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
                 const int page = live ? __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos)) : 0, rp = row_in_page(D, pos);
@@ -167,7 +173,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = 4 * quad + q;
-            if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(m0 + i) * D.d + u_row);
+            if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(mb + m0 + i) * D.d + u_row);
             if (EPI0 == PE_QKV && i < nm) csn[q] = __ldg(D.rope_cs + (size_t)s_pos[i] * half + (e < half ? e : e - half));
         }
     };
@@ -189,7 +195,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int quad = 2 * c + q;
-                if (quad * 4 < A.rows) {
+                if (quad * 4 < rows) {
                     float f[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
@@ -223,8 +229,8 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     };
     // where this thread's weight row goes
     const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
-    __half *qrow = A.q + (size_t)job * 2 * Mp * D.d + (EPI0 == PE_QKV ? col : u_row);
-    bf16 *xrow = G.out + (size_t)job * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
+    __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
+    bf16 *xrow = G.out + (size_t)(A.tt > 1 ? token_tile : job) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
     const int xchunk = (u_row >> 3) & 7;
     float *lrow = G.logits + (size_t)job * D.M * G.ld + u_row;
     __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
@@ -239,7 +245,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         __half hi, lo;
         split_f16(v * A.scale, hi, lo);
         qrow[(size_t)m * D.d] = hi;
-        qrow[(size_t)(Mp + m) * D.d] = lo;
+        qrow[(size_t)(A.qp + m) * D.d] = lo;
     };
     for (int quad = side; 4 * quad < nm; quad += SIDES) {
         float h[4], v[4], w[4];
@@ -257,11 +263,11 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             if (EPI0 == PE_ADD) {
                 const float o = live_row ? h[q] + v[q] : 0.f;
                 if (live_row) {
-                    D.h[(size_t)m * D.d + u_row] = o;
+                    D.h[(size_t)(mb + m) * D.d + u_row] = o;
                     put_x(m, o * gain);
                 }
                 const float ssq = warp_sum(o * o);
-                if (lane == 0) D.ss[(size_t)m * kShareLd + tile * 4 + (row >> 5)] = ssq;
+                if (lane == 0) D.ss[(size_t)(mb + m) * kShareLd + tile * 4 + (row >> 5)] = ssq;
             } else if (live_row) {
                 const float inv = s_inv[i], x1 = v[q] * inv;
                 if (EPI0 == PE_QKV) {
@@ -295,7 +301,7 @@ static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMa
     cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
-    return L.launch(dim3(tiles * A.S), dim3(kProjThreads), smem, A.S, (const void *)fn, D, A, T);
+    return L.launch(dim3(tiles * A.tt * A.S), dim3(kProjThreads), smem, A.S, (const void *)fn, D, A, T);
 }
 
 int resident_clusters(int size) {

@@ -37,7 +37,7 @@ template <typename WT> static __device__ void embed_row(const Dev &D, int m, int
             __align__(16) bf16 hi[N], lo[N];
 #pragma unroll
             for (int q = 0; q < N; ++q) split_bf16(v[q] * to_f(g[q]), hi[q], lo[q]);
-            bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + plane_off(Mp, m, c);
+            bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + (size_t)(m / kTokenTile) * 2 * Mp * d + plane_off(Mp, m % kTokenTile, c);
             *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
             *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
         } else {
@@ -73,7 +73,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_row
 }
 cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, const ChainLaunch &L) {
     const void *fn = dtype == 1 ? (const void *)embed_rows_kernel<bf16> : (const void *)embed_rows_kernel<float>;
-    const int Mp = (D.B * t + 7) / 8 * 8;
+    const int Mp = D.B * t > kTokenTile ? kTokenTile : (D.B * t + 7) / 8 * 8;
     return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, fn, D, t, Mp, pos0);
 }
 
