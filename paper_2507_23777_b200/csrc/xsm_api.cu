@@ -24,7 +24,7 @@ struct Layout {
     size_t wkc_off, wvc_off, hk_off, hv_off;
     size_t len, window, finished, n_gen, n_blocks, step_idx, block_table, free_stack, scalars, hist, steps, tok_log, step_tokens,
         step_n_new, prompt, script;
-    size_t h, rope_cs, logits0, hlogits;
+    size_t h, rope_cs, row_info, row_cs, logits0, hlogits;
     size_t rp, xa, qp, aa, actp, yp, hq, ha, ss, apart, acount;
     size_t stage_cond, stage_kv, stage_tok, trace, ckv_pool, hckv_pool, kv_pool;
     int n_pages = 0, max_blocks = 0, cpages = 0, tok_ld = 0, n_stages = 0;
@@ -73,6 +73,8 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     const size_t rows = prompt_rows(c), row = 4 * rows, step_row = 4 * (size_t)kMaxTokens, nh = ca ? (size_t)c.n_draft : 0;
     L.h = take(cur, row * d);
     L.rope_cs = take(cur, 8 * (size_t)(c.max_seq_len + K1 + 1) * (dh / 2));
+    L.row_info = take(cur, sizeof(RowInfo) * rows);
+    L.row_cs = take(cur, 8 * rows * (dh / 2));
     L.xa = take(cur, row * d);
     L.qp = take(cur, row * d);
     L.aa = take(cur, row * d);
@@ -373,6 +375,7 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     D.rp = at<RunParams>(ctx, L.rp);
     D.host_done = ctx->pinned + 8;
     D.h = at<float>(ctx, L.h); D.rope_cs = at<float2>(ctx, L.rope_cs);
+    D.row_info = at<RowInfo>(ctx, L.row_info); D.row_cs = at<float2>(ctx, L.row_cs);
     D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
     D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
     D.apart = at<float>(ctx, L.apart); D.acount = at<int>(ctx, L.acount);
@@ -428,7 +431,7 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     }
     ctx->launches += 3;
     if (prompt_len > 1) XSM_CUDA(ctx, ctx->chain.ingest(D, prompt_len - 1, ctx->stream, &ctx->launches));
-    XSM_CUDA(ctx, launch_embed_rows(D, c.dtype, D.K1, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
+    XSM_CUDA(ctx, launch_embed_rows(D, c.dtype, D.K1, -1, 0, ChainLaunch{ctx->stream, false, &ctx->launches}));
     ctx->prefilled = 1;
     return XSM_OK;
 }
@@ -608,7 +611,7 @@ xsm_status xsm_debug_set_drafts(xsm_ctx *ctx, const int32_t *h_drafts) {
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy2D(D.window + 1, sizeof(int32_t) * D.K1, h_drafts, sizeof(int32_t) * D.K,
                                sizeof(int32_t) * D.K, D.B, cudaMemcpyHostToDevice));
-    XSM_CUDA(ctx, launch_embed_rows(D, ctx->cfg.dtype, D.K1, -1, ChainLaunch{ctx->stream, false, &ctx->launches}));
+    XSM_CUDA(ctx, launch_embed_rows(D, ctx->cfg.dtype, D.K1, -1, 0, ChainLaunch{ctx->stream, false, &ctx->launches}));
     return XSM_OK;
 }
 

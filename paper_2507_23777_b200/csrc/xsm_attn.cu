@@ -223,19 +223,19 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
             const int n_old = cross ? np : page_of(D, first);         // pages that nobody writes in this step
             bool waited = false;
             for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
-                if (!waited && pg >= n_old) {
-                    chain_wait();
-                    fence_proxy_async();
-                    waited = true;
-                }
                 const int sl = i % slots;
                 if (i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
                 const int page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
                 const int pool_pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
                 const __half *kt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 0, page, h);
                 const __half *vt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 1, page, h);
-                const uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
+                uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
                 mbar_arrive_expect_tx(f, 2u * tile_bytes);
+                if (!waited && pg >= n_old) {
+                    settle(kt); settle(vt); settle(f); settle(dst);
+                    chain_wait();
+                    waited = true;
+                }
                 bulk_g2s(dst, kt, tile_bytes, f);
                 bulk_g2s(dst + tile_bytes, vt, tile_bytes, f);
             }
@@ -245,16 +245,20 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         __syncthreads();                 // (1) every page has been consumed
     } else {
         const int g = lane >> 2, t4 = lane & 3;
-        const __half *qhi = A.q + (size_t)set * 2 * A.qp * D.d + (size_t)(b * A.t + q0) * D.d + h * DH, *qlo = qhi + (size_t)A.qp * D.d;
+        // this lane's part of the queries: row g of the first row tile of the warp
+        const int row_tile = FEW ? 0 : warp & (wq - 1);
+        const __half *qhi = A.q + (size_t)set * 2 * A.qp * D.d + (size_t)(b * A.t + q0 + row_tile * 16 + g) * D.d + h * DH + 2 * t4;
+        const __half *qlo = qhi + (size_t)A.qp * D.d;
+        settle(qhi); settle(qlo);
+        bar_sync<kAttnWarps * 32>(1);      // (warps that come to the wait together leave it sooner)
         chain_wait();
         trace_mark(D, 1 + 2 * A.stage);
         if (FEW) {
             unsigned qh[DH / 8], ql[DH / 8];
 #pragma unroll
             for (int c = 0; c < DH / 8; ++c) {
-                const size_t o = (size_t)g * D.d + 8 * c + 2 * t4;
-                qh[c] = g < t_rows ? ldcg_u32(qhi + o) : 0u;
-                ql[c] = g < t_rows ? ldcg_u32(qlo + o) : 0u;
+                qh[c] = g < t_rows ? ldcg_u32(qhi + 8 * c) : 0u;
+                ql[c] = g < t_rows ? ldcg_u32(qlo + 8 * c) : 0u;
             }
             FewState<DH> ws;
 #pragma unroll
@@ -295,7 +299,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
                 }
             }
         } else {
-            const int qt = warp & (wq - 1), kg = warp / wq;
+            const int qt = row_tile, kg = warp / wq;
             const int r0 = qt * 16 + g, r1 = r0 + 8;
             unsigned qh[DH / 16][4], ql[DH / 16][4];
 #pragma unroll
@@ -303,7 +307,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int r = (q & 1) ? r1 : r0;
-                    const size_t o = (size_t)r * D.d + ks * 16 + 2 * t4 + (q >> 1) * 8;
+                    const size_t o = (size_t)((q & 1) * 8) * D.d + ks * 16 + (q >> 1) * 8;
                     qh[ks][q] = r < t_rows ? ldcg_u32(qhi + o) : 0u;
                     ql[ks][q] = r < t_rows ? ldcg_u32(qlo + o) : 0u;
                 }

@@ -152,20 +152,26 @@ bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
     A.upc = (units + share - 1) / share;
     A.ctas = (units + A.upc - 1) / A.upc;
     const FewShape f = few_shape(rows, kdim);
-    const int passes = (kdim + f.pass - 1) / f.pass;
-    A.chunk = (kdim / passes + 63) / 64 * 64;
-    if (A.chunk * passes < kdim) A.chunk += 64;
-    const int n_rows = A.upc * (pairs ? 2 : 1), tiles = (n_rows + 15) / 16, pitch = A.chunk * 2 + 64;
-    const int red = tiles * f.warps * 16 * (f.nt * 8 + 1) * 4, stages = tiles * passes;
-    const int slots = std::min(std::min(stages, kProjRing), (kProjSmemMax - red) / (16 * pitch));
-    if (slots < std::min(stages, 2) || A.upc > 32 && A.epi0 == PE_ADD || A.ctas > 160) return false;
+    const int n_rows = A.upc * (pairs ? 2 : 1), tiles = (n_rows + 15) / 16;
+    const int red = tiles * f.warps * 16 * (f.nt * 8 + 1) * 4;
+    A.slot_rows = tiles == 1 ? (n_rows + 7) / 8 * 8 : 16;
+    // passes no wider than the registers hold, and narrow enough for two of them in flight
+    int slots = 0;
+    for (int passes = (kdim + f.pass - 1) / f.pass; passes <= 16; ++passes) {
+        A.chunk = ((kdim + passes - 1) / passes + 63) / 64 * 64;
+        const int pitch = A.chunk * 2 + 64, stages = tiles * ((kdim + A.chunk - 1) / A.chunk);
+        slots = std::min(std::min(stages, kProjRing), (kProjSmemMax - red) / (A.slot_rows * pitch));
+        if (slots >= std::min(stages, 2)) break;
+        slots = 0;
+    }
+    if (slots == 0 || (A.upc > 32 && A.epi0 == PE_ADD) || A.ctas > kShareLd) return false;
     A.kdim = kdim;
     A.rows = rows;
     A.Mp = Mp;
     A.S = 1;
     A.slots = slots;
     op.kind = ChainOp::FEW;
-    op.smem = slots * 16 * pitch + red;
+    op.smem = slots * A.slot_rows * (A.chunk * 2 + 64) + red;
     return true;
 }
 
@@ -315,7 +321,7 @@ cudaError_t Chain::run(const Dev &D, const ChainOp &op, int t, const ChainLaunch
         case ChainOp::F32: return launch_proj_f32(D, op.proj, op.smem, L);
         case ChainOp::ATTN: return c_.dtype == 1 ? launch_attn(D, op.attn, L) : launch_attn_f32(D, op.attn, L);
         case ChainOp::TAIL: return launch_tail(D, c_.dtype, op.proj.stage, L);
-        case ChainOp::EMBED: return launch_embed_rows(D, c_.dtype, t, op.attn.pos0, L);
+        case ChainOp::EMBED: return launch_embed_rows(D, c_.dtype, t, op.attn.pos0, op.attn.pos_end, L);
     }
     return cudaErrorInvalidValue;
 }

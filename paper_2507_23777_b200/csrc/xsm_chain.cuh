@@ -44,7 +44,7 @@ struct ProjArgs {
     int z_jobs, x_jobs;               // group 0 has one matrix per decoding head; the activations too
     const bf16 *x;                    // planes of kdim columns (x_jobs: a set per decoding head)
     int upc, ctas;                    // few token rows: units (pairs of rows) per CTA, CTAs (per decoding head with x_jobs)
-    int slots, chunk;                 // weight tiles in shared memory, columns of one
+    int slots, chunk, slot_rows;      // weight tiles in shared memory; columns, rows of one
     int late_go;                      // let the next kernel start only after this one's wait
     float scale;                      // queries
     const void *gain;                 // PE_ADD: gain of the RMSNorm that reads h next; PE_HEADY / PE_HEADADD: of the final RMSNorm
@@ -123,7 +123,7 @@ cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const Cha
 cudaError_t launch_attn_f32(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
 cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L);
 // embeds the window of every sequence (pos0 < 0) or t prompt tokens of each from position pos0 on
-cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, const ChainLaunch &L);
+cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, int pos_end, const ChainLaunch &L);
 // state of a new request: pool, sequences with prompt_len - 1 positions in the cache, first window
 cudaError_t launch_begin(const Dev &D, const RunParams &R, cudaStream_t st);
 // single stages (inspection): waits until the stages before `stage` have run one by one; notes that `done` of them have

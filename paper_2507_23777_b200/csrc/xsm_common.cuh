@@ -23,6 +23,15 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // lets the next kernel of the chain be launched as soon as every CTA of this one has said so
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// barrier `id` (not 0) of the first N threads of a block
+template <int N> __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, %1;" :: "r"(id), "n"(N) : "memory"); }
+// Keeps a value from being computed later than here (the compiler would put address arithmetic behind the wait, where it is
+// on the step's critical path).
+template <typename T> __device__ __forceinline__ void settle(T *&p) { asm volatile("" : "+l"(p)); }
+__device__ __forceinline__ void settle(int &v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void settle(uint32_t &v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void settle(float &v) { asm volatile("" : "+f"(v)); }
+
 // ------------------------------------------------------------------------- shared memory, barriers
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -235,6 +244,9 @@ template <> __device__ __forceinline__ size_t tile_off<float>(int r, int e, int 
 template <> __device__ __forceinline__ size_t tile_off<__half>(int r, int e, int dh) {
     return (size_t)r * dh + (size_t)swz(r, e >> 3, dh * 2) * 8 + (e & 7);
 }
+
+// chunk permutation of a row of 16-bit elements
+__device__ __forceinline__ int row_swz(int rp, int dh) { return dh >= 64 ? rp & 7 : (rp >> 1) & 3; }
 
 // page and row inside the page of a position (pages of a power of two of positions need no division)
 __device__ __forceinline__ int page_of(const Dev &D, int pos) { return D.p_shift >= 0 ? pos >> D.p_shift : pos / D.P; }

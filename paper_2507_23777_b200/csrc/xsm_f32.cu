@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
             if (q * 128 + lane * 4 < min(chunk, K)) wa[r][q] = __ldg(reinterpret_cast<const float4 *>(w[r] + q * 128 + lane * 4));
     }
     if (A.stage == 0) trace_mark(D, 0);
+    __syncthreads();      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (A.late_go) chain_go();
     trace_mark(D, 1 + 2 * A.stage);
@@ -148,21 +149,15 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
             v *= inv;
             v2 *= inv;
             const int sec = u >= D.d ? (u >= 2 * D.d ? 2 : 1) : 0, c = u - sec * D.d, head = c / D.dh, e = c - head * D.dh;
-            const int b = m / A.t, jj = m - b * A.t, pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + jj;
-            const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
-            float o1 = v, o2 = v2;
-            if (sec < 2 && live) {
-                const float2 cs = __ldg(D.rope_cs + (size_t)pos * half + e);
-                o1 = v * cs.x - v2 * cs.y;
-                o2 = v2 * cs.x + v * cs.y;
-            }
+            const float2 cs = __ldcg(D.row_cs + (size_t)m * half + e);
+            const long long place = __ldcg(reinterpret_cast<const long long *>(D.row_info + m));
+            const float o1 = sec < 2 ? v * cs.x - v2 * cs.y : v, o2 = sec < 2 ? v2 * cs.x + v * cs.y : v2;
             if (sec == 0) {
                 float *q = reinterpret_cast<float *>(A.q) + (size_t)m * D.d + c;
                 q[0] = o1 * A.scale;
                 q[half] = o2 * A.scale;
-            } else if (live) {
-                const int page = __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos));
-                float *tile = kv_tile<float>(D, D.kv_pool, D.n_pages, A.layer, sec - 1, page, head) + tile_off<float>(row_in_page(D, pos), e, D.dh);
+            } else if (place >= 0) {
+                float *tile = kv_tile<float>(D, D.kv_pool, D.n_pages, A.layer, sec - 1, 0, head) + place + e;
                 tile[0] = o1;
                 tile[half] = o2;
             }
@@ -225,6 +220,7 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
         }
     };
     if (!dead) fetch(0, 0, min(kF32Keys, n_old));
+    __syncthreads();
     chain_wait();
     if (dead) return;
     trace_mark(D, 1 + 2 * A.stage);

@@ -27,6 +27,12 @@ struct RunParams {
     int script_n, script_acc;
 };
 
+// Where the keys and values of a token row go: element offset of its row in head 0 of its page (< 0: nowhere), row in the page.
+struct __align__(16) RowInfo {
+    long long place;
+    int rp, pad_;
+};
+
 // Everything a kernel needs; passed by value.
 struct Dev {
     // shape
@@ -60,6 +66,8 @@ struct Dev {
     float *ss;                     // [kMaxTokens][kShareLd] shares of the sums of squares of the rows of h
     float *logits0, *hlogits;      // [M][V], [K][M][V]
     float *h;                      // residual stream [row][d]
+    RowInfo *row_info;             // [row]; with row_cs written when the row is embedded, so that nobody else looks up positions and pages
+    float2 *row_cs;                // [row][dh/2] cos, sin of the row's position
     float2 *rope_cs;               // [max_seq_len + K + 2][dh/2] cos, sin of position * theta^(-2i/dh)
     // caches
     void *kv_pool;                 // [L][2][n_pages][H] tiles of P x dh

@@ -22,60 +22,56 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     constexpr int kOutThreads = NW * 32, LDM = NT * 8 + 1;      // (odd pitch: neighbouring rows in other banks)
     constexpr bool PAIRS = EPI0 == PE_QKV || EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (A.pos0 < 0 && !A.late_go && __ldcg(D.n_active) == 0) {      // every sequence has ended in an earlier step
-        chain_wait();
-        return;
-    }
-    if (tid == 0) {
-        for (int i = 0; i < A.slots; ++i) {
-            mbar_init(smem_u32(&full[i]), 1u);
-            mbar_init(smem_u32(&empty[i]), (uint32_t)NW);
-        }
-        mbar_init_fence();
-    }
-    __syncthreads();
     if (!A.late_go) chain_go();
+    // sequences that still run: looked at just before the wait, when the weights are on their way
+    const int active = A.pos0 < 0 && !A.late_go ? __ldcg(D.n_active) : 1;
     // this CTA's units: rows, or pairs of rows (rotation partners; gate and up)
     const int job = A.x_jobs ? blockIdx.x / A.ctas : 0, cta = A.x_jobs ? blockIdx.x - job * A.ctas : blockIdx.x;
     const int all_units = EPI0 == PE_QKV ? A.g[0].units >> 1 : A.g[0].units + (EPI1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
     const int lo = cta * A.upc, n_units = min(A.upc, all_units - lo), n_rows = PAIRS ? 2 * n_units : n_units;
     const int tiles = (n_rows + 15) >> 4, kdim = A.kdim, chunk = A.chunk, passes = (kdim + chunk - 1) / chunk;
-    const uint32_t pitch = (uint32_t)chunk * 2u + 64u, ring = smem_u32(smem);
+    const uint32_t pitch = (uint32_t)chunk * 2u + 64u, slot_bytes = (uint32_t)A.slot_rows * pitch, ring = smem_u32(smem);
     const int half = D.dh >> 1, M = A.rows;
     // rows of pair p of q, k, v: p and its rotation partner half a head further
     auto qkv_row = [&](int p) {
         const int hd = D.d >> 1, sec = p / hd, i = p - sec * hd, head = i / half;
         return sec * D.d + head * D.dh + (i - head * half);
     };
-    if (warp == NW) {
-        // producer: tile by tile within a pass
-        for (int s = 0; s < tiles * passes; ++s) {
-            const int pass = s / tiles, tile = s - pass * tiles, sl = s % A.slots, r = tile * 16 + lane;
-            const uint32_t bytes = (uint32_t)min(chunk, kdim - pass * chunk) * 2u, f = smem_u32(&full[sl]);
-            const int rows = min(16, n_rows - tile * 16);
-            if (s >= A.slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((s / A.slots - 1) & 1), D.mbar_limit, D.status);
-            if (lane == 0) mbar_arrive_expect_tx(f, bytes * (uint32_t)rows);
-            __syncwarp();
-            if (lane < rows) {
-                const bf16 *src;
-                if (EPI0 == PE_QKV) {
-                    src = A.g[0].w + (size_t)(qkv_row(lo + (r >> 1)) + (r & 1) * half) * kdim;
-                } else if (EPI0 == PE_GATEUP) {
-                    src = A.g[r & 1].w + (size_t)(lo + (r >> 1)) * kdim;
+    // the producer warp owns the barriers and the ring: stage s is a pass of a tile, tile by tile within a pass
+    const int stages = tiles * passes;
+    auto issue = [&](int s, int sl) {
+        const int pass = s / tiles, tile = s - pass * tiles, r = tile * 16 + lane, rows = min(16, n_rows - tile * 16);
+        const uint32_t bytes = (uint32_t)min(chunk, kdim - pass * chunk) * 2u, f = smem_u32(&full[sl]);
+        if (lane == 0) mbar_arrive_expect_tx(f, bytes * (uint32_t)rows);
+        __syncwarp();
+        if (lane < rows) {
+            const bf16 *src;
+            if (EPI0 == PE_QKV) {
+                src = A.g[0].w + (size_t)(qkv_row(lo + (r >> 1)) + (r & 1) * half) * kdim;
+            } else if (EPI0 == PE_GATEUP) {
+                src = A.g[r & 1].w + (size_t)(lo + (r >> 1)) * kdim;
+            } else {
+                int u = lo + r;
+                if (EPI1 >= 0 && u >= A.g[0].units) {
+                    u -= A.g[0].units;
+                    const int j = u / A.g[1].units;
+                    src = A.g[1].w + (size_t)j * A.g[1].w_stride + (size_t)(u - j * A.g[1].units) * kdim;
                 } else {
-                    int u = lo + r;
-                    if (EPI1 >= 0 && u >= A.g[0].units) {
-                        u -= A.g[0].units;
-                        const int j = u / A.g[1].units;
-                        src = A.g[1].w + (size_t)j * A.g[1].w_stride + (size_t)(u - j * A.g[1].units) * kdim;
-                    } else {
-                        src = A.g[0].w + (size_t)job * A.g[0].w_stride + (size_t)u * kdim;
-                    }
+                    src = A.g[0].w + (size_t)job * A.g[0].w_stride + (size_t)u * kdim;
                 }
-                bulk_g2s(ring + (uint32_t)sl * 16u * pitch + (uint32_t)lane * pitch, src + (size_t)pass * chunk, bytes, f);
             }
+            bulk_g2s(ring + (uint32_t)sl * slot_bytes + (uint32_t)lane * pitch, src + (size_t)pass * chunk, bytes, f);
         }
         __syncwarp();
+    };
+    if (tid < A.slots) {
+        mbar_init(smem_u32(&full[tid]), 1u);
+        mbar_init(smem_u32(&empty[tid]), (uint32_t)NW);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    if (warp == NW) {
+        for (int s = 0; s < min(stages, A.slots); ++s) issue(s, s);
     }
     if (A.stage == 0) trace_mark(D, 0);
 
@@ -88,13 +84,14 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     if (EPI0 == PE_ADD)
         while (lpt < A.upc) lpt <<= 1;
     const int per_m = EPI0 == PE_ADD ? lpt : n_units;
-    float *const red = reinterpret_cast<float *>(smem + (size_t)A.slots * 16 * pitch);     // [tile][warp][16][LDM]
+    float *const red = reinterpret_cast<float *>(smem + (size_t)A.slots * slot_bytes);     // [tile][warp][16][LDM]
     struct Out {
-        int m, r, grp, sec;                        // token row, unit or row of the CTA, group; section of q, k, v
+        int m, r, grp, sec, e;                     // token row, unit or row of the CTA, group; section of q, k, v, element of the head
         const float *sum;                          // the warps' partial sums
-        char *p, *p2;                              // where the output goes (of the rotation partner)
+        char *p;                                   // where the output goes (keys and values: head and section in page 0, row 0)
         const float *h;                            // residual stream
         float gain;
+        RowInfo row;                               // q, k, v: place in the cache, cosine and sine
         float2 cs;
     };
     auto locate = [&](int e, Out &o) {
@@ -108,6 +105,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
             u = qkv_row(u);
             o.sec = u >= D.d ? (u >= 2 * D.d ? 2 : 1) : 0;
             u -= o.sec * D.d;
+            const int head = u / D.dh;
+            o.e = u - head * D.dh;
+            if (o.sec > 0) o.p = reinterpret_cast<char *>(kv_tile<__half>(D, D.kv_pool, D.n_pages, A.layer, o.sec - 1, 0, head) + (o.e & 7));
         }
         if (EPI1 >= 0 && u >= A.g[0].units) {
             u -= A.g[0].units;
@@ -117,8 +117,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         }
         const int epi = EPI1 >= 0 && o.grp ? EPI1 : EPI0;
         if (epi == PE_QKV || epi == PE_QUERY) {
-            o.p = reinterpret_cast<char *>(A.q + ((size_t)j * 2 * MP + o.m) * D.d + u);
-            o.p2 = o.p + half * 2;
+            if (EPI0 != PE_QKV || o.sec == 0) o.p = reinterpret_cast<char *>(A.q + ((size_t)j * 2 * MP + o.m) * D.d + u);
         } else if (epi == PE_LOGITS) {
             o.p = reinterpret_cast<char *>(A.g[0].logits + ((size_t)j * D.M + o.m) * A.g[0].ld + u);
         } else {
@@ -129,21 +128,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         o.h = D.h + (size_t)min(o.m, kMaxTokens - 1) * D.d + u;
         if (EPI0 == PE_ADD || HEAD) o.gain = to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u));
     };
-    // q, k, v: rotation of the row's position; keys and values go to its place in the cache (nowhere if the sequence has ended)
     auto position = [&](Out &o) {
-        const int b = o.m / A.t, j = o.m - b * A.t;
-        int pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + j;
-        const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
-        if (!live) pos = 0;
-        const int pair = (lo + o.r) % (D.d >> 1), head = pair / half, e = pair - head * half;
-        o.cs = __ldg(D.rope_cs + (size_t)pos * half + e);
-        if (o.sec > 0) {
-            const int page = __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos));
-            __half *tile = kv_tile<__half>(D, D.kv_pool, D.n_pages, A.layer, o.sec - 1, page, head);
-            o.p = reinterpret_cast<char *>(tile + tile_off<__half>(row_in_page(D, pos), e, D.dh));
-            o.p2 = reinterpret_cast<char *>(tile + tile_off<__half>(row_in_page(D, pos), e + half, D.dh));
-            if (!live) o.p = nullptr;
-        }
+        o.row = *reinterpret_cast<const RowInfo *>(&(const int4 &)__ldcg(reinterpret_cast<const int4 *>(D.row_info + o.m)));
+        o.cs = __ldcg(D.row_cs + (size_t)o.m * half + o.e);
     };
     Out o1;
     locate(tid, o1);
@@ -160,7 +147,20 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         x_full[q] = base + g * 64 + ((chunk8 ^ g) << 3);
         x_last[q] = base + (NT - 1) * 1024 + tail * 64 + ((chunk8 ^ tail) << 3) + (PACK ? (g >> 2) * kLo : 0);
     }
+    const uint32_t full0 = smem_u32(&full[0]);
+    const char *w0 = smem + (size_t)g * pitch + t4 * 16 + warp * 64;
+    float *dst0 = red + (size_t)(warp * 16 + g) * LDM + 2 * t4;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) { settle(x_full[q]); settle(x_last[q]); }
+    settle(o1.sum); settle(o1.p); settle(o1.h); settle(w0); settle(dst0);
+    if (EPI0 == PE_ADD || HEAD) settle(o1.gain);
+    if (warp < NW) bar_sync<NW * 32>(1);           // (warps that come to the wait together leave it sooner: 0.3 us a kernel)
     chain_wait();
+    if (active == 0) {                             // every sequence has ended in an earlier step
+        if (warp == NW)
+            for (int s = 0; s < min(stages, A.slots); ++s) mbar_wait(smem_u32(&full[s]), 0u, D.mbar_limit, D.status);
+        return;
+    }
     if (A.late_go) {
         chain_go();
         if (EPI0 == PE_QKV && has) position(o1);
@@ -168,6 +168,34 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     trace_mark(D, 1 + 2 * A.stage);
 
     float h_old = 0.f;
+    // one k-block of a tile: a, c: eight columns of weight rows g and g + 8
+    auto multiply = [&](float (&ah)[NT][4], float (&al)[NT][4], const uint4 &a, const uint4 &c, const uint4 (&h)[NT], const uint4 (&l)[NT]) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            mma16816_bf16(ah[nt], a.x, c.x, a.y, c.y, h[nt].x, h[nt].y);
+            if (PACK) {
+                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, h[nt].z, h[nt].w);
+            } else {
+                mma16816_bf16(al[nt], a.x, c.x, a.y, c.y, l[nt].x, l[nt].y);
+                mma16816_bf16(ah[nt], a.z, c.z, a.w, c.w, h[nt].z, h[nt].w);
+                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, l[nt].z, l[nt].w);
+            }
+        }
+    };
+    auto park = [&](float *dst, const float (&ah)[NT][4], const float (&al)[NT][4], bool first) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float v = ah[nt][q] + al[nt][q];
+                if (PACK) v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
+                if (!PACK || t4 < 2) {
+                    float *o = dst + (q >> 1) * 8 * LDM + nt * 8 + (q & 1);
+                    *o = first ? v : *o + v;
+                }
+            }
+        }
+    };
     if (warp < NW) {
         int sl = 0;
         uint32_t par = 0;
@@ -188,12 +216,11 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
                 }
             }
             if ((EPI0 == PE_ADD || HEAD) && pass == 0 && has) h_old = __ldcg(o1.h);
-            const char *w = smem + (size_t)g * pitch + t4 * 16 + warp * 64;
-            float *dst = red + (size_t)(warp * 16 + g) * LDM + 2 * t4;
+            float *dst = dst0;
             for (int tile = 0; tile < tiles; ++tile) {
                 const bool two = n_rows - tile * 16 > 8;
-                mbar_wait(smem_u32(&full[sl]), par, D.mbar_limit, D.status);
-                const char *ws = w + (size_t)sl * 16 * pitch;
+                mbar_wait(full0 + 8u * (uint32_t)sl, par, D.mbar_limit, D.status);
+                const char *ws = w0 + (size_t)sl * slot_bytes;
                 float ah[NT][4], al[NT][4];
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
@@ -205,17 +232,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
                         const uint4 a = *reinterpret_cast<const uint4 *>(ws + NW * i * 64);
                         uint4 c = make_uint4(0u, 0u, 0u, 0u);
                         if (two) c = *reinterpret_cast<const uint4 *>(ws + 8 * pitch + NW * i * 64);
-#pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) {
-                            mma16816_bf16(ah[nt], a.x, c.x, a.y, c.y, xh[i][nt].x, xh[i][nt].y);
-                            if (PACK) {
-                                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, xh[i][nt].z, xh[i][nt].w);
-                            } else {
-                                mma16816_bf16(al[nt], a.x, c.x, a.y, c.y, xl[i][nt].x, xl[i][nt].y);
-                                mma16816_bf16(ah[nt], a.z, c.z, a.w, c.w, xh[i][nt].z, xh[i][nt].w);
-                                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, xl[i][nt].z, xl[i][nt].w);
-                            }
-                        }
+                        multiply(ah, al, a, c, xh[i], xl[i]);
                     }
                 }
                 if (A.slots < tiles * passes) {
@@ -223,23 +240,13 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
                     if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
                 }
                 if (++sl == A.slots) { sl = 0; par ^= 1u; }
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float v = ah[nt][q] + al[nt][q];
-                        if (PACK) v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
-                        if (!PACK || t4 < 2) {
-                            float *o = dst + (q >> 1) * 8 * LDM + nt * 8 + (q & 1);
-                            *o = pass == 0 ? v : *o + v;
-                        }
-                    }
-                }
+                park(dst, ah, al, pass == 0);
                 dst += NW * 16 * LDM;
             }
         }
-    } else if (A.ss_parts > 0) {
+    } else {
         // the producer warp adds up the shares of the sums of squares: four lanes per token row, every fourth quad each
+        if (A.ss_parts > 0) {
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
             const int m = nt * 8 + g;
@@ -256,6 +263,16 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
             ss += __shfl_xor_sync(0xffffffffu, ss, 1);
             ss += __shfl_xor_sync(0xffffffffu, ss, 2);
             if (t4 == 0) s_inv[m] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+        }
+        }
+        // then the rest of the weights, as their slots become free
+        int sl = 0;
+        uint32_t par = 0;
+        for (int s = A.slots; s < stages; ++s) {
+            mbar_wait(smem_u32(&empty[sl]), par, D.mbar_limit, D.status);
+            __syncwarp();
+            issue(s, sl);
+            if (++sl == A.slots) { sl = 0; par ^= 1u; }
         }
     }
     __syncthreads();
@@ -303,10 +320,12 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
             const float v = total(o1.sum) * inv, v2 = total(o1.sum + LDM) * inv;
             if (o1.sec == 0) {
                 put_query(o1.p, v * o1.cs.x - v2 * o1.cs.y);
-                put_query(o1.p2, v2 * o1.cs.x + v * o1.cs.y);
-            } else if (o1.p != nullptr) {
-                *reinterpret_cast<__half *>(o1.p) = from_f<__half>(o1.sec == 1 ? v * o1.cs.x - v2 * o1.cs.y : v);
-                *reinterpret_cast<__half *>(o1.p2) = from_f<__half>(o1.sec == 1 ? v2 * o1.cs.x + v * o1.cs.y : v2);
+                put_query(o1.p + half * 2, v2 * o1.cs.x + v * o1.cs.y);
+            } else if (o1.row.place >= 0) {
+                __half *p = reinterpret_cast<__half *>(o1.p) + o1.row.place;
+                const int sw = row_swz(o1.row.rp, D.dh);
+                p[((o1.e >> 3) ^ sw) << 3] = from_f<__half>(o1.sec == 1 ? v * o1.cs.x - v2 * o1.cs.y : v);
+                p[(((o1.e + half) >> 3) ^ sw) << 3] = from_f<__half>(o1.sec == 1 ? v2 * o1.cs.x + v * o1.cs.y : v2);
             }
         } else if (EPI0 == PE_GATEUP) {
             put_bf16(o1.p, silu_f(total(o1.sum) * inv) * (total(o1.sum + LDM) * inv));
@@ -337,8 +356,8 @@ static cudaError_t launch_few(const Dev &D, const ProjArgs &A, int smem, const C
 #define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_few_instance<NW, NT, PACK, MAXB, a, b>(D, A, smem, L)
     XSM_EPI(PE_ADD, -1);
     if constexpr (NW == 8) {
-        XSM_EPI(PE_QKV, -1);
         XSM_EPI(PE_QUERY, -1);
+        XSM_EPI(PE_QKV, -1);
         XSM_EPI(PE_GATEUP, -1);
         XSM_EPI(PE_LOGITS, -1);
         XSM_EPI(PE_LOGITS, PE_HEADY);

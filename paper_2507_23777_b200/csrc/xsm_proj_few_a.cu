@@ -3,7 +3,7 @@
 
 namespace xsm {
 
-cudaError_t few_8_1_p_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, true, 4>(D, A, smem, L); }
-cudaError_t few_8_1_n_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, false, 4>(D, A, smem, L); }
+cudaError_t few_8_1_packed_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, true, 4>(D, A, smem, L); }
+cudaError_t few_8_1_4(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) { return launch_few<8, 1, false, 4>(D, A, smem, L); }
 
 }  // namespace xsm

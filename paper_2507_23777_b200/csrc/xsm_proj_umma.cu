@@ -33,15 +33,12 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     __shared__ __align__(8) uint64_t recv_bar;                      // the peers' shares of this CTA's token rows
     __shared__ uint32_t tmem_slot;
     __shared__ float s_inv[kTokenTile];
-    __shared__ int s_pos[kTokenTile], s_swz[kTokenTile];
-    __shared__ long long s_cache[kTokenTile];
+    __shared__ RowInfo s_row[kTokenTile];
     constexpr bool TWO = EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int S = A.S, rank = S > 1 ? (int)cluster_rank() : 0, Mp = A.Mp;
-    if (A.pos0 < 0 && !A.late_go && __ldcg(D.n_active) == 0) {      // every sequence has ended in an earlier step
-        chain_wait();
-        return;
-    }
+    // sequences that still run: looked at just before the wait, when the weights are on their way
+    const int active = A.pos0 < 0 && !A.late_go ? __ldcg(D.n_active) : 1;
     // a tile of weight rows and a tile of token rows: neighbours share the weights
     const int token_tile = A.tt > 1 ? (int)(blockIdx.x / S) % A.tt : 0, mb = token_tile * kTokenTile, rows = min(kTokenTile, A.rows - mb);
     int tile = blockIdx.x / S / A.tt, job = 0, z = A.layer, grp = 0;
@@ -84,8 +81,8 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     if (!A.late_go) chain_go();
     if (S > 1) cluster_arrive();          // "this CTA runs": peers may write to its shared memory after cluster_wait
     const void *wmap = grp == 1 ? &T.w1 : &T.w0;
-    auto load_a = [&](int i) {
-        const uint32_t dst = sa + (uint32_t)(i % na) * kABytes, b = bar(0, i % na);
+    auto load_a = [&](int i, int slot) {
+        const uint32_t dst = sa + (uint32_t)slot * kABytes, b = bar(0, slot);
         const int x = (k_lo + i) * kBlockK;
         mbar_arrive_expect_tx(b, kABytes);
         if (TWO) {
@@ -96,35 +93,53 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         }
     };
     if (tid == 0)
-        for (int i = 0; i < min(n, na); ++i) load_a(i);
+        for (int i = 0; i < min(n, na); ++i) load_a(i, i);
     if (A.stage == 0) trace_mark(D, 0);
     const bf16 *x = A.x + (size_t)(A.x_jobs ? job : token_tile) * 2 * Mp * A.kdim;
+    const bf16 *xb = x + (size_t)k_lo * (128 * Mp);      // this CTA's blocks of the activations
+    const uint32_t idesc = umma_idesc(128, 2 * Mp), tmem = tmem_slot, full_a = bar(0, 0), full_b = bar(2, 0);
+    settle(xb);
+    if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kProjThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
+    if (active == 0) {      // every sequence has ended in an earlier step
+        if (tid == 0)
+            for (int i = 0; i < min(n, na); ++i) mbar_wait(bar(0, i), 0u, D.mbar_limit, D.status);
+        __syncthreads();
+        if (S > 1) cluster_wait();
+        if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
+        return;
+    }
     if (A.late_go) chain_go();
     trace_mark(D, 1 + 2 * A.stage);
     if (tid == 0) {
-        fence_proxy_async();              // the activations were written by ordinary stores
+        // (written by ordinary stores of an earlier kernel, which has completed: nothing to order)
+        int slot = 0, a_slot = 0;
+        uint32_t par = 1u, a_par = 0u;
         for (int i = 0; i < n; ++i) {
-            if (i >= nb) mbar_wait(bar(3, i % nb), (uint32_t)((i / nb - 1) & 1), D.mbar_limit, D.status);
-            const uint32_t b = bar(2, i % nb);
-            mbar_arrive_expect_tx(b, b_bytes);
-            bulk_g2s(sb + (uint32_t)(i % nb) * b_bytes, x + (size_t)(k_lo + i) * (128 * Mp), b_bytes, b);
+            if (i >= nb) mbar_wait(bar(3, slot), par, D.mbar_limit, D.status);
+            mbar_arrive_expect_tx(full_b + 8u * (uint32_t)slot, b_bytes);
+            bulk_g2s(sb + (uint32_t)slot * b_bytes, xb + (size_t)i * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)slot);
+            if (++slot == nb) { slot = 0; par ^= 1u; }
             if (i >= na) {
-                mbar_wait(bar(1, i % na), (uint32_t)((i / na - 1) & 1), D.mbar_limit, D.status);
-                load_a(i);
+                mbar_wait(bar(1, a_slot), a_par, D.mbar_limit, D.status);
+                load_a(i, a_slot);
+                if (++a_slot == na) { a_slot = 0; a_par ^= 1u; }
             }
         }
     } else if (tid == 32) {
-        const uint32_t idesc = umma_idesc(128, 2 * Mp), tmem = tmem_slot;
+        int ia = 0, ib = 0;
+        uint32_t pa = 0u, pb = 0u;
         for (int i = 0; i < n; ++i) {
-            mbar_wait(bar(0, i % na), (uint32_t)((i / na) & 1), D.mbar_limit, D.status);
-            mbar_wait(bar(2, i % nb), (uint32_t)((i / nb) & 1), D.mbar_limit, D.status);
+            mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
+            mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
             tcgen05_after_sync();
-            const uint64_t da = umma_desc_sw128(sa + (uint32_t)(i % na) * kABytes), db = umma_desc_sw128(sb + (uint32_t)(i % nb) * b_bytes);
+            const uint64_t da = umma_desc_sw128(sa + (uint32_t)ia * kABytes), db = umma_desc_sw128(sb + (uint32_t)ib * b_bytes);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, da + 2 * ks, db + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
-            if (i + na < n) umma_commit(bar(1, i % na));
-            if (i + nb < n) umma_commit(bar(3, i % nb));
+            if (i + na < n) umma_commit(bar(1, ia));
+            if (i + nb < n) umma_commit(bar(3, ib));
+            if (++ia == na) { ia = 0; pa ^= 1u; }
+            if (++ib == nb) { ib = 0; pb ^= 1u; }
         }
         umma_commit(done);
     }
@@ -149,19 +164,11 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
                 inv = 1.0f / sqrtf(ss / (float)D.d + D.eps);
             }
             s_inv[i] = inv;
-            if (EPI0 == PE_QKV) {
-                const int b = (mb + m) / A.t, j = mb + m - b * A.t;
-                const int pos = (A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b)) + j;
-                const bool live = A.pos0 >= 0 ? pos < A.pos_end : __ldcg(D.finished + b) == 0;
-                const int page = live ? __ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos)) : 0, rp = row_in_page(D, pos);
-                s_pos[i] = live ? pos : 0;
-                s_cache[i] = live ? ((long long)page * D.H * D.P + rp) * D.dh : -1;      // place of head 0 in a page set
-                s_swz[i] = D.dh >= 64 ? rp & 7 : (rp >> 1) & 3;
-            }
+            if (EPI0 == PE_QKV) *reinterpret_cast<int4 *>(&s_row[i]) = __ldcg(reinterpret_cast<const int4 *>(D.row_info + mb + m));
         }
     }
-    // The epilogue takes four token rows (a quad) of a weight row at a time; what it reads from memory is requested before the
-    // products are waited for, or a round ahead.
+    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row, four at a
+    // time; what it reads from memory is requested before the products are waited for, or a round ahead.
     constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
     const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
@@ -169,16 +176,15 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const float gain = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u_row)) : 0.f;
     float hn[4];
     float2 csn[4];
-    auto request = [&](int quad) {
+    auto request = [&](int i0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int i = 4 * quad + q;
+            const int i = i0 + q * SIDES;
             if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(mb + m0 + i) * D.d + u_row);
-            if (EPI0 == PE_QKV && i < nm) csn[q] = __ldg(D.rope_cs + (size_t)s_pos[i] * half + (e < half ? e : e - half));
+            if (EPI0 == PE_QKV && i < nm) csn[q] = __ldcg(D.row_cs + (size_t)(mb + m0 + i) * half + (e < half ? e : e - half));
         }
     };
     __syncwarp();
-    if (EPI0 == PE_QKV) __syncthreads();      // the rows' positions
     request(side);
     mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
@@ -218,14 +224,11 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     if (S > 1 && nm > 0) mbar_wait(smem_u32(&recv_bar), 0u, D.mbar_limit, D.status);
     __syncwarp();
     // sums over the cluster in rank order, epilogue
-    auto total = [&](int quad, int r, float (&o)[4]) {
-        const float4 *p = reinterpret_cast<const float4 *>(recv) + quad * 128 + r;
-        float4 v = p[0];
-        for (int s = 1; s < S; ++s) {
-            const float4 w = p[s * qps * 128];
-            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-        }
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+    auto total = [&](int i, int r) {
+        const float *p = recv + (size_t)((i >> 2) * 128 + r) * 4 + (i & 3);
+        float v = p[0];
+        for (int s = 1; s < S; ++s) v += p[s * qps * 512];
+        return v;
     };
     // where this thread's weight row goes
     const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
@@ -247,21 +250,19 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         qrow[(size_t)m * D.d] = hi;
         qrow[(size_t)(A.qp + m) * D.d] = lo;
     };
-    for (int quad = side; 4 * quad < nm; quad += SIDES) {
-        float h[4], v[4], w[4];
+    for (int i0 = side; i0 < nm; i0 += 4 * SIDES) {
+        float h[4];
         float2 cs[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
-        request(quad + SIDES);
-        total(quad, row, v);
-        if (EPI0 == PE_QKV) total(quad, e < half ? row + half : row - half, w);
-        if (TWO) total(quad, row + 64, w);
+        request(i0 + 4 * SIDES);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int i = 4 * quad + q, m = m0 + i;
+            const int i = i0 + q * SIDES, m = m0 + i;
             if (i >= nm) break;
+            const float v = total(i, row);
             if (EPI0 == PE_ADD) {
-                const float o = live_row ? h[q] + v[q] : 0.f;
+                const float o = live_row ? h[q] + v : 0.f;
                 if (live_row) {
                     D.h[(size_t)(mb + m) * D.d + u_row] = o;
                     put_x(m, o * gain);
@@ -269,21 +270,21 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
                 const float ssq = warp_sum(o * o);
                 if (lane == 0) D.ss[(size_t)(mb + m) * kShareLd + tile * 4 + (row >> 5)] = ssq;
             } else if (live_row) {
-                const float inv = s_inv[i], x1 = v[q] * inv;
+                const float inv = s_inv[i], x1 = v * inv;
                 if (EPI0 == PE_QKV) {
-                    const float x2 = w[q] * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
+                    const float x2 = total(i, e < half ? row + half : row - half) * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
                     if (sec == 0) put_q(m, o);
-                    else if (s_cache[i] >= 0) crow[s_cache[i] + (((e >> 3) ^ s_swz[i]) << 3)] = from_f<__half>(o);
+                    else if (s_row[i].place >= 0) crow[s_row[i].place + (((e >> 3) ^ row_swz(s_row[i].rp, D.dh)) << 3)] = from_f<__half>(o);
                 } else if (TWO) {
-                    put_x(m, silu_f(x1) * (w[q] * inv));
+                    put_x(m, silu_f(x1) * (total(i, row + 64) * inv));
                 } else if (EPI0 == PE_QUERY || (EPI1 == PE_QUERY && grp == 1)) {
                     put_q(m, x1);
                 } else if (EPI0 == PE_HEADADD) {
-                    put_x(m, h[q] * inv * gain + v[q]);
+                    put_x(m, h[q] * inv * gain + v);
                 } else if (EPI1 == PE_HEADY && grp == 1) {
                     put_x(m, h[q] * inv * gain + silu_f(x1));
                 } else {
-                    lrow[(size_t)m * G.ld] = A.norm ? x1 : v[q];
+                    lrow[(size_t)m * G.ld] = A.norm ? x1 : v;
                 }
             }
         }

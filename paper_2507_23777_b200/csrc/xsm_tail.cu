@@ -13,12 +13,23 @@ __device__ __forceinline__ uint32_t rand24(const RunParams &R, int seq, uint32_t
 
 // ---------------------------------------------------------------------------------------- embedding
 
-// Row m of the window <- the embedding of `tok`: master copy, the copy that the first projection reads (times the gain of the
+// place in the cache of position pos of sequence b, for token row m (one thread)
+static __device__ void place_row(const Dev &D, int m, int b, int pos, bool live) {
+    RowInfo r;
+    r.rp = row_in_page(D, pos);
+    r.place = live ? ((long long)__ldcg(D.block_table + (size_t)b * D.max_blocks + page_of(D, pos)) * D.H * D.P + r.rp) * D.dh : -1;
+    r.pad_ = 0;
+    D.row_info[m] = r;
+}
+
+// Row m of the window, at position pos, <- the embedding of `tok`: the position's cosines and sines, master copy, the copy that the first projection reads (times the gain of the
 // first RMSNorm) and its sum of squares.  All threads of the block, 16 bytes of a row each.
-template <typename WT> static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, float *sh) {
+template <typename WT> static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, int pos, float *sh) {
     constexpr int N = 16 / (int)sizeof(WT);
     const WT *E = reinterpret_cast<const WT *>(D.E), *gain = reinterpret_cast<const WT *>(D.gain_first);
     const int d = D.d;
+    const int half = D.dh >> 1;
+    if ((int)threadIdx.x < half) D.row_cs[(size_t)m * half + threadIdx.x] = __ldg(D.rope_cs + (size_t)pos * half + threadIdx.x);
     float ssq = 0.f;
     tok = min(max(tok, 0), D.V - 1);
     for (int c = threadIdx.x * N; c < d; c += kTailThreads * N) {
@@ -56,25 +67,30 @@ template <typename WT> static __device__ void embed_row(const Dev &D, int m, int
     }
 }
 
-template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0) {
+template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0, int pos_end) {
     __shared__ float sh[kTailWarps];
     chain_wait();
     chain_go();      // (only now: kernels further down may read what earlier chunks wrote before they wait themselves)
     const int b = blockIdx.x / t, j = blockIdx.x - b * t;
-    int tok;
+    int tok, pos;
+    bool live = true;
     if (pos0 >= 0) {
         const int n = D.rp->prompt_len;
+        live = pos0 + j < pos_end;
+        pos = min(pos0 + j, pos_end);
         tok = pos0 + j < n ? D.prompt[(size_t)b * n + pos0 + j] : 0;
     } else {
         if (__ldcg(D.finished + b)) return;
+        pos = __ldcg(D.len + b) + j;
         tok = __ldcg(D.window + b * t + j);
     }
-    embed_row<WT>(D, blockIdx.x, Mp, tok, sh);
+    if (threadIdx.x == 0) place_row(D, blockIdx.x, b, pos, live);
+    embed_row<WT>(D, blockIdx.x, Mp, tok, pos, sh);
 }
-cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, const ChainLaunch &L) {
+cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, int pos_end, const ChainLaunch &L) {
     const void *fn = dtype == 1 ? (const void *)embed_rows_kernel<bf16> : (const void *)embed_rows_kernel<float>;
     const int Mp = D.B * t > kTokenTile ? kTokenTile : (D.B * t + 7) / 8 * 8;
-    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, fn, D, t, Mp, pos0);
+    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, fn, D, t, Mp, pos0, pos_end);
 }
 
 // ------------------------------------------------------------------------------------ block reductions
@@ -310,6 +326,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     if (tid == 34) sh.state[2] = (int)__ldcg(D.step_idx + b);
     if (tid == 35) sh.state[3] = __ldcg(D.n_blocks + b);
     if (tid >= 64 && tid < 64 + K1) sh.old_win[tid - 64] = __ldcg(D.window + b * K1 + tid - 64);
+    __syncthreads();      // (warps that come to the wait together leave it sooner)
     chain_wait();
     trace_mark(D, 1 + 2 * stage);
     __syncthreads();
@@ -446,7 +463,9 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
         }
     }
     __syncthreads();
-    if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], sh.red);
+    const int new_len = sh.state[0] + a + 1;
+    if (slot == 0 && tid < K1) place_row(D, b * K1 + tid, b, new_len + tid, !sh.state[5]);
+    if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], new_len + slot, sh.red);
     if (K > 0) { cluster_arrive(); cluster_wait(); }      // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }
