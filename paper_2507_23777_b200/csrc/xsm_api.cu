@@ -422,14 +422,19 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     if ((const void *)d_prompt != (const void *)D.prompt)
         XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
     XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
-    XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off), at<size_t>(ctx, ctx->lay.wvc_off), d_cond,
-                                  D.ckv_pool, D.L, ctx->stream));
-    if (c.head_kind == 1 && D.K > 0) {
-        XSM_CUDA(ctx, launch_cross_kv(D, c.dtype, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off), at<size_t>(ctx, ctx->lay.hv_off), d_cond,
-                                      D.hckv_pool, D.K, ctx->stream));
+    ctx->launches += 2;
+    if (c.dtype == 1) {
+        XSM_CUDA(ctx, ctx->chain.condition(D, d_cond, ctx->stream, &ctx->launches));
+    } else {
+        XSM_CUDA(ctx, launch_cross_kv(D, ctx->weights, at<size_t>(ctx, ctx->lay.wkc_off), at<size_t>(ctx, ctx->lay.wvc_off), d_cond,
+                                      D.ckv_pool, D.L, ctx->stream));
         ctx->launches += 1;
+        if (c.head_kind == 1 && D.K > 0) {
+            XSM_CUDA(ctx, launch_cross_kv(D, ctx->weights, at<size_t>(ctx, ctx->lay.hk_off), at<size_t>(ctx, ctx->lay.hv_off), d_cond,
+                                          D.hckv_pool, D.K, ctx->stream));
+            ctx->launches += 1;
+        }
     }
-    ctx->launches += 3;
     if (prompt_len > 1) XSM_CUDA(ctx, ctx->chain.ingest(D, prompt_len - 1, ctx->stream, &ctx->launches));
     XSM_CUDA(ctx, launch_embed_rows(D, c.dtype, D.K1, -1, 0, ChainLaunch{ctx->stream, false, &ctx->launches}));
     ctx->prefilled = 1;

@@ -88,12 +88,14 @@ bool Chain::init(const xsm_model_config &c, const WeightOffsets &w, const char *
     bool ok = weight_map(&qkv_, w.wq[0], 3 * d, d, L, ls, 128) && weight_map(&o_, w.wo[0], d, d, L, ls, 128) &&
               weight_map(&qc_, w.wqc[0], d, d, L, ls, 128) && weight_map(&oc_, w.woc[0], d, d, L, ls, 128) &&
               weight_map(&gate_, w.wgate[0], f, d, L, ls, 64) && weight_map(&up_, w.wup[0], f, d, L, ls, 64) &&
-              weight_map(&down_, w.wdown[0], d, f, L, ls, 128) && weight_map(&lm_, w.W0, V, d, 1, 0, 128);
+              weight_map(&down_, w.wdown[0], d, f, L, ls, 128) && weight_map(&kc_, w.wkc[0], d, c.d_cond, L, ls, 128) &&
+              weight_map(&vc_, w.wvc[0], d, c.d_cond, L, ls, 128) && weight_map(&lm_, w.W0, V, d, 1, 0, 128);
     if (K > 0) {
         const size_t hs = K > 1 ? w.Wout[1] - w.Wout[0] : 0;
         ok = ok && weight_map(&head_out_, w.Wout[0], V, d, K, hs, 128);
         if (c.head_kind == 1)
-            ok = ok && weight_map(&head_in_, w.hq[0], d, d, K, hs, 128) && weight_map(&head_o_, w.ho[0], d, d, K, hs, 128);
+            ok = ok && weight_map(&head_in_, w.hq[0], d, d, K, hs, 128) && weight_map(&head_o_, w.ho[0], d, d, K, hs, 128) &&
+                 weight_map(&head_kc_, w.hk[0], d, c.d_cond, K, hs, 128) && weight_map(&head_vc_, w.hv[0], d, c.d_cond, K, hs, 128);
         else
             ok = ok && weight_map(&head_in_, w.W1[0], d, d, K, hs, 128);
     }
@@ -373,6 +375,20 @@ cudaError_t Chain::step(const Dev &D, cudaStream_t st, bool graph, bool overlap,
     }
     *count += p.kernels;
     return cudaGraphLaunch(p.exec, st);
+}
+
+cudaError_t Chain::condition(const Dev &D, const void *d_cond, cudaStream_t st, unsigned long long *count) {
+    struct { TensorMap wk, wv, cond; } m;
+    if (!encode(encode_, &m.cond, d_cond, D.dc, D.C, D.B, (size_t)D.C * D.dc * 2, cond_tile(D.C))) return cudaErrorInvalidValue;
+    m.wk = kc_;
+    m.wv = vc_;
+    cudaError_t e = launch_cond_kv(D, &m, D.ckv_pool, D.L, st);
+    *count += 1;
+    if (e != cudaSuccess || c_.head_kind != 1 || D.K == 0) return e;
+    m.wk = head_kc_;
+    m.wv = head_vc_;
+    *count += 1;
+    return launch_cond_kv(D, &m, D.hckv_pool, D.K, st);
 }
 
 cudaError_t Chain::ingest(const Dev &D, int n, cudaStream_t st, unsigned long long *count) {

@@ -121,6 +121,8 @@ cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
 constexpr int kF32Rows = 24;
 cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L);
 cudaError_t launch_attn_f32(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
+int cond_tile(int n_cond);
+cudaError_t launch_cond_kv(const Dev &D, const void *maps, void *pool, int n_sets, cudaStream_t st);
 cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L);
 // embeds the window of every sequence (pos0 < 0) or t prompt tokens of each from position pos0 on
 cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, int pos_end, const ChainLaunch &L);

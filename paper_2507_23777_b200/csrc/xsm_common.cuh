@@ -115,12 +115,9 @@ template <> __device__ __forceinline__ float from_f<float>(float v) { return v; 
 template <> __device__ __forceinline__ bf16 from_f<bf16>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ __half from_f<__half>(float v) { return __float2half_rn(fminf(fmaxf(v, -65504.f), 65504.f)); }
 
-// Element type of the key/value caches.  bf16 models keep them in fp16: the same two bytes, eleven bits of
-// mantissa instead of eight (cached keys and values are normalised activations times small weights, far
-// inside the fp16 range; stores saturate).  Rounding of the cache is the largest error of the whole path.
-template <typename WT> struct CacheT { typedef WT type; };
-template <> struct CacheT<bf16> { typedef __half type; };
-
+// (bf16 models keep cached keys and values in fp16: the same two bytes, eleven bits of mantissa instead of eight; they are
+// normalised activations times small weights, far inside the fp16 range; stores saturate.  Rounding of the cache is the
+// largest error of the whole path.)
 __device__ __forceinline__ float silu_f(float v) { return v / (1.0f + expf(-v)); }
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll

@@ -51,6 +51,8 @@ class Chain {
     // one decoding step; graph: replay the recording (made at the first call)
     cudaError_t step(const Dev &D, cudaStream_t st, bool graph, bool overlap, unsigned long long *count);
     cudaError_t run_op(const Dev &D, int i, cudaStream_t st, unsigned long long *count);
+    // keys and values of the condition: of the layers, and of cross-attention decoding heads
+    cudaError_t condition(const Dev &D, const void *d_cond, cudaStream_t st, unsigned long long *count);
     // runs prompt tokens 0..n-1 of every sequence through the layers: their keys and values enter the cache
     cudaError_t ingest(const Dev &D, int n, cudaStream_t st, unsigned long long *count);
 
@@ -67,7 +69,7 @@ class Chain {
     const char *weights_ = nullptr;
     int sms_ = 0, clusters_[9] = {};      // clusters of s CTAs (with an SM each) that run at a time
     void *encode_ = nullptr;
-    TensorMap qkv_, o_, qc_, oc_, gate_, up_, down_, lm_, head_in_, head_o_, head_out_;
+    TensorMap qkv_, o_, qc_, oc_, gate_, up_, down_, lm_, head_in_, head_o_, head_out_, kc_, vc_, head_kc_, head_vc_;
     std::map<int, std::unique_ptr<StepPlan>> plans_;
     StepPlan *plan_ = nullptr;
     cudaStream_t record_ = nullptr;

@@ -77,8 +77,9 @@ struct Dev {
 };
 
 // Prefill and inspection kernels (xsm_kernels.cu).  All return the CUDA error of the launch.
-cudaError_t launch_cross_kv(const Dev &D, int dtype, const void *W /*flat weights*/, const size_t *wkc_off,
-                            const size_t *wvc_off, const void *cond, void *pool, int n_sets, cudaStream_t st);
+// fp32 models: keys and values of the condition under n_sets projections (offsets into the flat weights W)
+cudaError_t launch_cross_kv(const Dev &D, const void *W, const size_t *wkc_off, const size_t *wvc_off,
+                            const void *cond, void *pool, int n_sets, cudaStream_t st);
 cudaError_t launch_gather_kv(const Dev &D, int dtype, int layer, int seq, int pos0, int n, float *out_k,
                              float *out_v, cudaStream_t st);
 cudaError_t launch_export(const Dev &D, int max_new, int *d_tokens, int *d_lengths, cudaStream_t st);
