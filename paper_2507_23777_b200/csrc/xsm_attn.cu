@@ -17,7 +17,6 @@
 
 namespace xsm {
 
-constexpr int kAttnWarps = 8, kAttnThreads = kAttnWarps * 32 + 32;
 constexpr int kAttnSlots = 16;
 
 // ------------------------------------------------------------------- 32 keys against at most eight rows
@@ -33,9 +32,12 @@ __device__ __forceinline__ void few_unit(const unsigned (&qh)[DH / 8], const uns
                                          int lim0, int lim1, FewState<DH> &ws) {
     constexpr int RB = DH * 2;
     const int lane = threadIdx.x & 31, g = lane >> 2;
-    float s[2][4];
+    float s[2][4], sl[2][4];       // products with the hi and lo parts of the queries
 #pragma unroll
-    for (int kt = 0; kt < 2; ++kt) s[kt][0] = s[kt][1] = s[kt][2] = s[kt][3] = 0.f;
+    for (int kt = 0; kt < 2; ++kt) {
+        s[kt][0] = s[kt][1] = s[kt][2] = s[kt][3] = 0.f;
+        sl[kt][0] = sl[kt][1] = sl[kt][2] = sl[kt][3] = 0.f;
+    }
 #pragma unroll
     for (int ks = 0; ks < DH / 16; ++ks) {
 #pragma unroll
@@ -45,9 +47,13 @@ __device__ __forceinline__ void few_unit(const unsigned (&qh)[DH / 8], const uns
             unsigned ka[4];
             ldmatrix_x4(ka, k_tile + (uint32_t)row * RB + (uint32_t)swz(row, chunk, RB) * 16u);
             mma16816_f16(s[kt], ka[0], ka[1], ka[2], ka[3], qh[2 * ks], qh[2 * ks + 1]);
-            mma16816_f16(s[kt], ka[0], ka[1], ka[2], ka[3], ql[2 * ks], ql[2 * ks + 1]);
+            mma16816_f16(sl[kt], ka[0], ka[1], ka[2], ka[3], ql[2 * ks], ql[2 * ks + 1]);
         }
     }
+#pragma unroll
+    for (int kt = 0; kt < 2; ++kt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[kt][q] += sl[kt][q];
     float mx0 = kNegBig, mx1 = kNegBig;
 #pragma unroll
     for (int kt = 0; kt < 2; ++kt) {
@@ -175,10 +181,21 @@ __device__ __forceinline__ void rows_unit(const unsigned (&qh)[DH / 16][4], cons
 
 __device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(reinterpret_cast<const unsigned *>(p)); }
 
-template <int DH, bool FEW>
-__global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_kernel(const Dev D, const AttnArgs A) {
+// QP (cross-attention of a step, few rows): the kernel projects the queries of its head itself, from the normalised residual
+// stream.  The head's rows of the projection lie in shared memory before the wait, so the stage costs what the products
+// cost (every warp multiplies all rows over its share of the columns, as in the projections over few token rows) instead of
+// a kernel of its own: 7.5 -> 5 us for both at width 1024.
+constexpr int kQueryBlocks = 4;      // blocks of 32 columns per warp: d_model up to 1024
+//
+// NW: warps that attend, beside the producer.  A unit of 32 keys is some 300 dependent instructions, 1 us for a warp on its
+// own, so sixteen warps where a CTA has many units (and where the queries are projected); eight otherwise, of which two
+// CTAs share an SM when a batch has more (sequence, head) pairs than there are SMs.
+template <int DH, bool FEW, bool QP, int NW>
+__global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 : 1) attn_kernel(const Dev D, const AttnArgs A) {
+    constexpr int kThreads = NW * 32 + 32, RB = DH * 2;
     extern __shared__ __align__(128) char smem[];
-    __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots];
+    __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots], w_full;
+    __shared__ float s_inv[8];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // (tiles of a sequence's rows: those that see the most keys first)
     const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z % D.B, zz = blockIdx.z / D.B, set = zz % A.sets;
@@ -191,12 +208,13 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     if (rank >= S) return;
     // few rows: a warp looks only at the pages whose units it owns when the units of 1, 2 or 4 pages fill a round of the
     // warps (the ring is a whole number of rounds, so a warp meets every fill of its slots)
-    const bool owned = FEW && (upp == 1 || upp == 2 || upp == 4);
+    const bool owned = FEW && NW == 8 && (upp == 1 || upp == 2 || upp == 4);
     if (tid == 0) {
-        for (int i = 0; i < slots; ++i) {
+        for (int i = 0; i < kAttnSlots; ++i) {
             mbar_init(smem_u32(&full[i]), 1u);
-            mbar_init(smem_u32(&empty[i]), owned ? (uint32_t)upp : (uint32_t)kAttnWarps);
+            mbar_init(smem_u32(&empty[i]), owned ? (uint32_t)upp : (uint32_t)NW);
         }
+        if (QP) mbar_init(smem_u32(&w_full), 1u);
         mbar_init_fence();
     }
     __syncthreads();
@@ -208,39 +226,84 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     }
     const int np = page_of(D, n_keys + P - 1), p_lo = rank * np / S, p_hi = (rank + 1) * np / S;
     const uint32_t tile_bytes = (uint32_t)P * DH * 2u, ring = smem_u32(smem);
+    // Few rows: where all pages fit the ring (of the last one only the units that hold keys), nothing is waited for but the page
+    // of a unit, and nothing is given back.
+    const int pages = p_hi - p_lo, last_rows = min(P, (n_keys - (p_hi - 1) * P + 31) & ~31);
+    const bool all_in = FEW && pages > 0 && pages <= kAttnSlots && (uint32_t)(pages - 1) * 2u * tile_bytes + (uint32_t)last_rows * 2u * RB <= (uint32_t)A.ring;
+    const int n_units = pages > 0 ? (pages - 1) * upp + (last_rows >> 5) : 0;
     const int qt_n = FEW ? 1 : (t_rows + 15) >> 4;                       // row tiles
-    int wq = 1;                                                       // warps that share the keys between them: kAttnWarps / wq
+    int wq = 1;                                                       // warps that share the keys between them: NW / wq
     if (!FEW)
         while (wq < qt_n) wq <<= 1;
-    const int kg_n = kAttnWarps / wq;
-    // parked states of the warps [kAttnWarps][rows][DH + 2]; they reuse the ring
+    const int kg_n = NW / wq;            // (few rows: warps, at most; those without a unit leave nothing)
+    // parked states of the warps [NW][rows][DH + 2]; they reuse the ring
     constexpr int LD = DH + 2;
     const int srows = FEW ? t_rows : 16;
     float *st = reinterpret_cast<float *>(smem);
+    // QP, behind the ring: the head's weight rows; in their place later partial sums [row tile][8][16][9], queries hi, lo [8][DH + 8]
+    constexpr int LDQ = DH + 8;
+    const uint32_t w_pitch = (uint32_t)D.d * 2u + 64u;
+    char *const w_rows = smem + A.ring;
+    float *const q_sum = reinterpret_cast<float *>(w_rows);
+    __half *const q_hi = reinterpret_cast<__half *>(q_sum + (DH / 16) * 8 * 16 * 9), *const q_lo = q_hi + 8 * LDQ;
 
-    if (warp == kAttnWarps) {
-        if (lane == 0) {
+    if (warp == NW) {
+        if (QP) {
+            const uint32_t bytes = (uint32_t)D.d * 2u, f = smem_u32(&w_full);
+            if (lane == 0) mbar_arrive_expect_tx(f, bytes * DH);
+            __syncwarp();
+            for (int r = lane; r < DH; r += 32) bulk_g2s(smem_u32(w_rows) + (uint32_t)r * w_pitch, A.wq + (size_t)(h * DH + r) * D.d, bytes, f);
+            __syncwarp();
+        }
+        // (QP: 1/rms of the rows, once the predecessor is done)
+        auto scales = [&]() {
+            const int m = lane >> 2, t4 = lane & 3;
+            const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)(b * A.t + min(m, t_rows - 1)) * kShareLd) + t4;
+            chain_wait();
+            float4 v[kShareLd / 16];
+#pragma unroll
+            for (int q = 0; q < kShareLd / 16; ++q) v[q] = 16 * q + 4 * t4 < A.ss_parts ? __ldcg(sh + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float ss = 0.f;
+#pragma unroll
+            for (int q = 0; q < kShareLd / 16; ++q) {
+                const int n = A.ss_parts - 16 * q - 4 * t4;      // (the last quad may hold shares that nobody writes)
+                ss += (v[q].x + (n > 1 ? v[q].y : 0.f)) + ((n > 2 ? v[q].z : 0.f) + (n > 3 ? v[q].w : 0.f));
+            }
+            ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+            ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+            if (t4 == 0) s_inv[m] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+            asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
+        };
+        bool scaled = !QP;
+        if (lane == 0 || QP) {
             const int n_old = cross ? np : page_of(D, first);         // pages that nobody writes in this step
             bool waited = false;
             for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
-                const int sl = i % slots;
-                if (i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
+                const int sl = all_in ? i : i % slots, rows = all_in && pg == p_hi - 1 ? last_rows : P;
+                const uint32_t part = (uint32_t)rows * RB;
+                if (QP && !all_in && i == slots) {      // (due before a slot is free again)
+                    scales();
+                    scaled = true;
+                }
+                if (QP && lane != 0) continue;
+                if (!all_in && i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
                 const int page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
                 const int pool_pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
                 const __half *kt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 0, page, h);
                 const __half *vt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 1, page, h);
                 uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
-                mbar_arrive_expect_tx(f, 2u * tile_bytes);
+                mbar_arrive_expect_tx(f, 2u * part);
                 if (!waited && pg >= n_old) {
                     settle(kt); settle(vt); settle(f); settle(dst);
                     chain_wait();
                     waited = true;
                 }
-                bulk_g2s(dst, kt, tile_bytes, f);
-                bulk_g2s(dst + tile_bytes, vt, tile_bytes, f);
+                bulk_g2s(dst, kt, part, f);
+                bulk_g2s(dst + part, vt, part, f);
             }
         }
         __syncwarp();
+        if (!scaled) scales();
         chain_wait();
         __syncthreads();                 // (1) every page has been consumed
     } else {
@@ -249,12 +312,69 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         const int row_tile = FEW ? 0 : warp & (wq - 1);
         const __half *qhi = A.q + (size_t)set * 2 * A.qp * D.d + (size_t)(b * A.t + q0 + row_tile * 16 + g) * D.d + h * DH + 2 * t4;
         const __half *qlo = qhi + (size_t)A.qp * D.d;
-        settle(qhi); settle(qlo);
-        bar_sync<kAttnWarps * 32>(1);      // (warps that come to the wait together leave it sooner)
+        // QP: of the residual stream, columns 8 t4 .. of the warp's first block of 32 for token row g (the last rows: the first one again)
+        const int xm = b * A.t + (g < t_rows ? g : 0);
+        const bf16 *xp = nullptr;
+        if (QP) xp = A.x + (size_t)((warp & 7) >> 1) * (128 * A.Mp) + (xm >> 3) * 1024 + (xm & 7) * 64 + ((((warp & 1) * 4 + t4) ^ (xm & 7)) << 3);
+        settle(qhi); settle(qlo); settle(xp);
+        bar_sync<NW * 32>(1);      // (warps that come to the wait together leave it sooner)
         chain_wait();
         trace_mark(D, 1 + 2 * A.stage);
         if (FEW) {
             unsigned qh[DH / 8], ql[DH / 8];
+            if constexpr (QP) {
+                constexpr int TILES = DH / 32;       // row tiles of a warp: eight warps share the columns, two such groups the rows
+                const int nb = D.d >> 5, kg = warp & 7, t0 = (warp >> 3) * TILES;
+                uint4 xh[kQueryBlocks], xl[kQueryBlocks];
+#pragma unroll
+                for (int i = 0; i < kQueryBlocks; ++i)
+                    if (kg + 8 * i < nb) {
+                        const bf16 *p = xp + (size_t)i * 4 * (128 * A.Mp);
+                        xh[i] = __ldcg(reinterpret_cast<const uint4 *>(p));
+                        xl[i] = __ldcg(reinterpret_cast<const uint4 *>(p + kLo));
+                    }
+                mbar_wait(smem_u32(&w_full), 0u, D.mbar_limit, D.status);
+                float ah[TILES][4], al[TILES][4];
+#pragma unroll
+                for (int tile = 0; tile < TILES; ++tile) {
+                    const char *w = w_rows + (size_t)((t0 + tile) * 16 + g) * w_pitch + t4 * 16 + kg * 64;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) ah[tile][q] = al[tile][q] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < kQueryBlocks; ++i)
+                        if (kg + 8 * i < nb) {
+                            const uint4 a = *reinterpret_cast<const uint4 *>(w + i * 512);
+                            const uint4 c = *reinterpret_cast<const uint4 *>(w + 8 * w_pitch + i * 512);
+                            mma16816_bf16(ah[tile], a.x, c.x, a.y, c.y, xh[i].x, xh[i].y);
+                            mma16816_bf16(al[tile], a.x, c.x, a.y, c.y, xl[i].x, xl[i].y);
+                            mma16816_bf16(ah[tile], a.z, c.z, a.w, c.w, xh[i].z, xh[i].w);
+                            mma16816_bf16(al[tile], a.z, c.z, a.w, c.w, xl[i].z, xl[i].w);
+                        }
+                }
+                bar_sync<NW * 32>(1);                // the weights' place is free
+#pragma unroll
+                for (int tile = 0; tile < TILES; ++tile) {
+                    float *o = q_sum + (size_t)(((t0 + tile) * 8 + kg) * 16 + g) * 9 + 2 * t4;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) o[(q >> 1) * 8 * 9 + (q & 1)] = ah[tile][q] + al[tile][q];
+                }
+                bar_sync<kThreads>(2);               // (and the producer's scales)
+                for (int i = tid; i < DH * 8; i += NW * 32) {
+                    const int m = i / DH, e = i - m * DH;
+                    const float *p = q_sum + (size_t)((e >> 4) * 8 * 16 + (e & 15)) * 9 + m;
+                    float v = 0.f;
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) v += p[w * 16 * 9];
+                    v = m < t_rows ? v * s_inv[m] * A.scale : 0.f;
+                    split_f16(v, q_hi[m * LDQ + e], q_lo[m * LDQ + e]);
+                }
+                bar_sync<NW * 32>(1);
+#pragma unroll
+                for (int c = 0; c < DH / 8; ++c) {
+                    qh[c] = *reinterpret_cast<const unsigned *>(q_hi + g * LDQ + 8 * c + 2 * t4);
+                    ql[c] = *reinterpret_cast<const unsigned *>(q_lo + g * LDQ + 8 * c + 2 * t4);
+                }
+            } else
 #pragma unroll
             for (int c = 0; c < DH / 8; ++c) {
                 qh[c] = g < t_rows ? ldcg_u32(qhi + 8 * c) : 0u;
@@ -266,18 +386,27 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
             ws.m[0] = ws.m[1] = kNegBig;
             ws.l[0] = ws.l[1] = 0.f;
             const int row_lim0 = cross ? D.C - 1 : start + 2 * t4, row_lim1 = cross ? D.C - 1 : row_lim0 + 1;
-            const int stride = owned ? kAttnWarps / upp : 1;
-            for (int i = owned ? warp / upp : 0; i < p_hi - p_lo; i += stride) {
-                const int sl = i % slots;
-                mbar_wait(smem_u32(&full[sl]), (uint32_t)((i / slots) & 1), D.mbar_limit, D.status);
-                const uint32_t kt = ring + (uint32_t)sl * 2u * tile_bytes;
-                for (int uu = owned ? warp % upp : 0; uu < upp; uu += owned ? upp : 1) {
-                    if (!owned && ((i * upp + uu) & (kAttnWarps - 1)) != warp) continue;
-                    const int base = (p_lo + i) * P + uu * 32;
-                    if (base < n_keys) few_unit<DH>(qh, ql, kt, kt + tile_bytes, uu * 32, row_lim0 - base, row_lim1 - base, ws);
+            if (all_in) {
+                for (int u = warp; u < n_units; u += NW) {
+                    const int i = u / upp, uu = u - i * upp, base = (p_lo + i) * P + uu * 32;
+                    mbar_wait(smem_u32(&full[i]), 0u, D.mbar_limit, D.status);
+                    const uint32_t kt = ring + (uint32_t)i * 2u * tile_bytes, vt = kt + (uint32_t)(i == pages - 1 ? last_rows : P) * RB;
+                    few_unit<DH>(qh, ql, kt, vt, uu * 32, row_lim0 - base, row_lim1 - base, ws);
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
+            } else {
+                const int stride = owned ? NW / upp : 1;
+                for (int i = owned ? warp / upp : 0; i < p_hi - p_lo; i += stride) {
+                    const int sl = i % slots;
+                    mbar_wait(smem_u32(&full[sl]), (uint32_t)((i / slots) & 1), D.mbar_limit, D.status);
+                    const uint32_t kt = ring + (uint32_t)sl * 2u * tile_bytes;
+                    for (int uu = owned ? warp % upp : 0; uu < upp; uu += owned ? upp : 1) {
+                        if (!owned && ((i * upp + uu) & (NW - 1)) != warp) continue;
+                        const int base = (p_lo + i) * P + uu * 32;
+                        if (base < n_keys) few_unit<DH>(qh, ql, kt, kt + tile_bytes, uu * 32, row_lim0 - base, row_lim1 - base, ws);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
+                }
             }
             __syncthreads();             // (1)
 #pragma unroll
@@ -352,6 +481,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     __syncthreads();
     // the warps' states of a row -> the output, or this CTA's partial result.  Two neighbouring columns a thread.
     bf16 *out = A.out + (size_t)set * 2 * A.Mp * D.d;
+    const int states = FEW && all_in ? min(NW, n_units) : kg_n;
     const int item = blockIdx.z * D.H + h, n_pairs = t_rows * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
     // partial results: [items][S][t][DH + 2]; acount: CTAs of an item that have left theirs (zero between kernels)
     float *mine = D.apart + ((size_t)(item * A.S + rank) * t_cap) * LD;
@@ -364,12 +494,12 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         *reinterpret_cast<__nv_bfloat162 *>(p) = __nv_bfloat162(h0, h1);
         *reinterpret_cast<__nv_bfloat162 *>(p + kLo) = __nv_bfloat162(l0, l1);
     };
-    for (int e = tid; e < n_pairs; e += kAttnThreads) {
+    for (int e = tid; e < n_pairs; e += kThreads) {
         const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
         const float *src = st + r * LD;                   // (row r of a row tile: the tiles of the first kg follow each other)
         float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
-        for (int w = 0; w < kg_n; ++w) m = fmaxf(m, src[w * step + DH]);
-        for (int w = 0; w < kg_n; ++w) {
+        for (int w = 0; w < states; ++w) m = fmaxf(m, src[w * step + DH]);
+        for (int w = 0; w < states; ++w) {
             const float f = ex2(src[w * step + DH] - m);
             const float2 o = *reinterpret_cast<const float2 *>(src + w * step + c);
             o0 += f * o.x;
@@ -393,7 +523,7 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
         if (s_last) {
             __threadfence();
             const float *all = D.apart + ((size_t)item * A.S * t_cap) * LD;
-            for (int e = tid; e < n_pairs; e += kAttnThreads) {
+            for (int e = tid; e < n_pairs; e += kThreads) {
                 const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
                 float2 ml[8], os[8];
 #pragma unroll
@@ -420,22 +550,35 @@ __global__ void __launch_bounds__(kAttnThreads, FEW && DH <= 64 ? 2 : 1) attn_ke
     trace_mark(D, 2 + 2 * A.stage);
 }
 
-template <int DH, bool FEW>
-static cudaError_t launch_instance(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
-    void (*fn)(const Dev, const AttnArgs) = attn_kernel<DH, FEW>;
-    const int ring = A.slots * 2 * D.P * DH * 2;
-    const int park = kAttnWarps * (FEW ? A.t : 16) * (DH + 2) * 4;
-    const int smem = ring > park ? ring : park;
-    cudaError_t e = open_kernel((const void *)fn, smem, false);
-    if (e != cudaSuccess) return e;
-    return L.launch(dim3(A.S, D.H, D.B * A.sets * A.qt), dim3(kAttnThreads), smem, 1, (const void *)fn, D, A);
+// shared memory that the states of the warps take when the pages are done with
+int attn_park(const Dev &D, int t, int warps) { return warps * (t <= 8 ? t : 16) * (D.dh + 2) * 4; }
+// shared memory beside the ring of a stage whose queries the kernel projects itself; 0: not possible
+int attn_query_smem(const Dev &D, int t) {
+    if (t > 8 || D.d > kQueryBlocks * 8 * 32 || D.dh > 64) return 0;
+    const int weights = D.dh * (D.d * 2 + 64), later = (D.dh / 16) * 8 * 16 * 9 * 4 + 2 * 8 * (D.dh + 8) * 2;
+    return weights > later ? weights : later;
 }
 
+template <int DH, bool FEW, bool QP, int NW>
+static cudaError_t launch_instance(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    void (*fn)(const Dev, const AttnArgs) = attn_kernel<DH, FEW, QP, NW>;
+    const int smem = A.ring + (QP ? attn_query_smem(D, A.t) : 0);
+    cudaError_t e = open_kernel((const void *)fn, smem, false);
+    if (e != cudaSuccess) return e;
+    return L.launch(dim3(A.S, D.H, D.B * A.sets * A.qt), dim3(NW * 32 + 32), smem, 1, (const void *)fn, D, A);
+}
+
+template <int DH>
+static cudaError_t launch_heads(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
+    if (A.t > 8) return launch_instance<DH, false, false, 8>(D, A, L);
+    if constexpr (DH <= 64) {
+        if (A.wq != nullptr) return launch_instance<DH, true, true, 16>(D, A, L);
+        if (A.warps == 16) return launch_instance<DH, true, false, 16>(D, A, L);
+    }
+    return launch_instance<DH, true, false, 8>(D, A, L);
+}
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
-    const bool few = A.t <= 8;
-    if (D.dh == 32) return few ? launch_instance<32, true>(D, A, L) : launch_instance<32, false>(D, A, L);
-    if (D.dh == 64) return few ? launch_instance<64, true>(D, A, L) : launch_instance<64, false>(D, A, L);
-    return few ? launch_instance<128, true>(D, A, L) : launch_instance<128, false>(D, A, L);
+    return D.dh == 32 ? launch_heads<32>(D, A, L) : D.dh == 64 ? launch_heads<64>(D, A, L) : launch_heads<128>(D, A, L);
 }
 
 }  // namespace xsm

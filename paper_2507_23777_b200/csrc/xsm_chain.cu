@@ -186,18 +186,34 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
     A.Mp = Mp;
     A.qt = (t + kTokenTile - 1) / kTokenTile;
     const int items = D.B * D.H * sets * A.qt, upp = D.P / 32, pair = 2 * D.P * D.dh * 2;
-    // about one CTA per SM at most; few rows: one more for every 640 keys (a merge costs as much as four units of 32 keys)
+    // About one CTA per SM at most; few rows: one more for every 512 keys (two units of 32 for each of eight warps; a merge costs
+    // as much as two), sixteen warps where a CTA can have more than that.
     A.S = 1;
     while (A.S < 8 && items * A.S * 2 <= sms_ + sms_ / 8) A.S *= 2;
-    A.split = t <= 8 ? 640 : 128;
-    if (cross) A.S = std::min(A.S, (D.C + A.split - 1) / A.split);
+    A.split = t <= 8 ? (D.dh <= 64 ? 512 : 640) : 128;
+    const int keys = cross ? D.C : D.max_blocks * D.P;
+    A.S = std::min(A.S, (keys + A.split - 1) / A.split);
+    A.warps = t <= 8 && D.dh <= 64 && items * A.S <= sms_ && keys > 512 * A.S ? 16 : 8;
     const int round = upp == 1 || upp == 2 || upp == 4 ? 8 / upp : 1;
     const int pages = ((cross ? D.cpages : D.max_blocks) + A.S - 1) / A.S;
     const int budget = items * A.S > sms_ ? 100 * 1024 : 128 * 1024;
     int slots = std::min(16, budget / pair) / round * round;
     slots = std::max(round, std::min(slots, (pages + round - 1) / round * round));
     A.slots = slots;
+    A.ring = std::max(slots * pair, attn_park(D, t, A.warps));
     return A;
+}
+
+// Does a cross-attention stage project its own queries?  The head's weights have to fit beside the pages (all of them, else at
+// least two at a time), and every CTA needs an SM to itself.
+bool Chain::own_queries(const Dev &D, AttnArgs &A) const {
+    const int weights = attn_query_smem(D, A.t), pair = 2 * D.P * D.dh * 2;
+    if (c_.dtype != 1 || weights == 0 || A.S * D.H * D.B > sms_) return false;
+    const int room = kProjSmemMax - weights, pages = (D.cpages + A.S - 1) / A.S;
+    const int all = A.S > 1 ? pages * pair : (pages - 1) * pair + ((D.C - (pages - 1) * D.P + 31) / 32 * 32) * D.dh * 4;
+    A.ring = std::max(all <= room ? all : room / pair * pair, attn_park(D, A.t, 16));
+    A.slots = std::min(16, A.ring / pair);
+    return A.ring <= room && (all <= room || A.slots >= 2);
 }
 
 bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
@@ -261,13 +277,22 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
         if (prompt && l == L - 1) break;      // the last keys and values are in the cache
         attn(false, 1, l, D.kv_pool, D.qp_, D.aa_);
         residual(l, o_, w_.wo[l], D.aa_, d, w_.g2[l]);
-        {
+        const size_t at = ops.size();
+        attn(true, 1, l, D.ckv_pool, D.qp_, D.aa_);
+        if (!prompt && own_queries(D, ops[at].attn)) {
+            AttnArgs &A = ops[at].attn;
+            A.wq = (const bf16 *)weights_ + w_.wqc[l];
+            A.x = (const bf16 *)D.xa_;
+            A.ss_parts = shares;
+            A.scale = qscale;
+        } else {
+            ops.pop_back();
             ChainOp &op = proj(PE_QUERY, -1, l, qc_, nullptr, w_.wqc[l], 0, D.xa_);
             group(op.proj.g[0], d, 128, 1, 0, nullptr, nullptr);
             op.proj.q = (__half *)D.qp_;
             normed(op);
+            attn(true, 1, l, D.ckv_pool, D.qp_, D.aa_);
         }
-        attn(true, 1, l, D.ckv_pool, D.qp_, D.aa_);
         residual(l, oc_, w_.woc[l], D.aa_, d, w_.g3[l]);
         {
             ChainOp &op = proj(PE_GATEUP, -1, l, gate_, &up_, w_.wgate[l], w_.wup[l], D.xa_);

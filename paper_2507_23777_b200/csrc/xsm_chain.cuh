@@ -58,10 +58,14 @@ struct AttnArgs {
     int cross, sets, layer;           // sets: decoding heads that attend in this stage (cross-attention heads), else 1
     int t, rows, Mp, qp, pos0, pos_end;      // as in ProjArgs
     int qt;                           // tiles of kTokenTile rows of a sequence
-    int S, split, slots;              // most CTAs per (sequence, head), keys for each; page pairs in shared memory
+    int warps;                        // that attend (few rows: 8 or 16)
+    int S, split, slots, ring;        // most CTAs per (sequence, head), keys for each; page pairs in shared memory, its bytes
     const void *pool;                 // cache tiles
     const __half *q;                  // planes [2][qp][d] (a set per decoding head)
     bf16 *out;                        // planes of d columns (a set per decoding head; layout: xsm_proj.cuh)
+    const bf16 *wq, *x;               // wq not null: the queries are projected here, wq x (x: planes of d columns)
+    int ss_parts;                     // shares of the sums of squares of x
+    float scale;                      // of the queries
 };
 
 // How the kernels of a chain are launched.
@@ -117,6 +121,8 @@ cudaError_t launch_proj_few(const Dev &D, const ProjArgs &A, int smem, const Cha
 int resident_clusters(int size);      // clusters of the projection below that the device runs at a time, an SM for each CTA
 cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L);
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
+int attn_query_smem(const Dev &D, int t);
+int attn_park(const Dev &D, int t, int warps);
 // fp32 models: at most this many token rows
 constexpr int kF32Rows = 24;
 cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L);

@@ -62,6 +62,7 @@ class Chain {
     void plan_proj(ChainOp &op, int rows, int Mp, int kdim);
     bool plan_few(ChainOp &op, int rows, int Mp, int kdim);
     AttnArgs plan_attn(const Dev &D, bool cross, int sets, int t, int Mp);
+    bool own_queries(const Dev &D, AttnArgs &A) const;
     cudaError_t run(const Dev &D, const ChainOp &op, int t, const ChainLaunch &L);
 
     xsm_model_config c_;

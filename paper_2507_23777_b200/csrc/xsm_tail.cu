@@ -129,28 +129,19 @@ __device__ __forceinline__ float key_logit(unsigned long long k) {
     return __uint_as_float(u);
 }
 __device__ __forceinline__ int key_token(unsigned long long k) { return (int)(0xFFFFFFFFu - (uint32_t)k); }
-// largest key over the block; every thread gets it
-static __device__ unsigned long long block_best(unsigned long long k, unsigned long long *sh) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, k, o);
-        k = other > k ? other : k;
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
-    __syncthreads();
-    k = sh[0];
-#pragma unroll
-    for (int w = 1; w < kTailWarps; ++w) k = sh[w] > k ? sh[w] : k;
-    return k;
+// largest key over the warp; every lane gets it
+__device__ __forceinline__ unsigned long long warp_best(unsigned long long k) {
+    const unsigned hi = (unsigned)(k >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned l = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)k : 0u);
+    return ((unsigned long long)m << 32) | l;
 }
 
 // ------------------------------------------------------------------------------- verify and resample
 
 struct TailShared {
     float red[kTailWarps];
-    unsigned long long redk[kTailWarps];
-    float cv[kMaxCand];
+    unsigned long long best[kTailWarps * kMaxCand];      // the warps' ranked candidates
+    float cv[kMaxCand], cw[kMaxCand];   // candidates, ranked: logits, sampling weights
     int ci[kMaxCand];
     int accepted;                       // of the draft behind this CTA's row
     int tok;                            // this slot's candidate
@@ -164,14 +155,30 @@ struct TailShared {
     int path[kMaxDraft];
 };
 
-// copies a logits row into shared memory
+// copies a logits row into shared memory, eight loads of a thread in flight
 static __device__ void stage_row(const float *z, float *row, int V) {
+    constexpr int N = 8;
     __syncthreads();
     if ((V & 3) == 0) {
-        for (int i = threadIdx.x; i < (V >> 2); i += kTailThreads)
-            reinterpret_cast<float4 *>(row)[i] = __ldcg(reinterpret_cast<const float4 *>(z) + i);
+        for (int i0 = threadIdx.x; i0 < (V >> 2); i0 += N * kTailThreads) {
+            float4 v[N];
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                if (i0 + q * kTailThreads < (V >> 2)) v[q] = __ldcg(reinterpret_cast<const float4 *>(z) + i0 + q * kTailThreads);
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                if (i0 + q * kTailThreads < (V >> 2)) reinterpret_cast<float4 *>(row)[i0 + q * kTailThreads] = v[q];
+        }
     } else {
-        for (int i = threadIdx.x; i < V; i += kTailThreads) row[i] = __ldcg(z + i);
+        for (int i0 = threadIdx.x; i0 < V; i0 += 2 * N * kTailThreads) {
+            float v[2 * N];
+#pragma unroll
+            for (int q = 0; q < 2 * N; ++q)
+                if (i0 + q * kTailThreads < V) v[q] = __ldcg(z + i0 + q * kTailThreads);
+#pragma unroll
+            for (int q = 0; q < 2 * N; ++q)
+                if (i0 + q * kTailThreads < V) row[i0 + q * kTailThreads] = v[q];
+        }
     }
     __syncthreads();
 }
@@ -196,24 +203,44 @@ static __device__ bool accept_token(const Dev &D, const RunParams &R, const floa
     return (int)block_sum((float)cnt, sh.red) < ka;
 }
 
-// the k best (logit, token) pairs of z, ranked, left in sh.cv, sh.ci
+// the k best (logit, token) pairs of z, ranked, left in sh.cv, sh.ci: every warp ranks the k best of its share, the first warp
+// merges the lists (a pick is two warp reductions; block-wide picks with two barriers each took a microsecond for two)
 static __device__ void top_candidates(const Dev &D, const float *z, int k, TailShared &sh) {
-    const int V = D.V;
-    // every thread keeps the best of its own elements; after each pick only the thread that owned the winner
-    // looks for its next best (among its elements ranked after the winner)
-    unsigned long long mine = 0ull;
-    for (int v = threadIdx.x; v < V; v += kTailThreads) {
-        const unsigned long long kv = rank_key(z[v], v);
-        mine = kv > mine ? kv : mine;
-    }
+    const int V = D.V, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the two best of this thread's elements below `limit`
+    auto scan = [&](unsigned long long limit, unsigned long long &first, unsigned long long &second) {
+        first = second = 0ull;
+        for (int v = threadIdx.x; v < V; v += kTailThreads) {
+            const unsigned long long kv = rank_key(z[v], v);
+            if (kv < limit) {
+                if (kv > first) { second = first; first = kv; }
+                else if (kv > second) second = kv;
+            }
+        }
+    };
+    unsigned long long mine, next;
+    scan(~0ull, mine, next);
+    bool known = true;                   // next is what follows mine
     for (int j = 0; j < k; ++j) {
-        const unsigned long long win = block_best(mine, sh.redk);
-        if (threadIdx.x == 0) { sh.cv[j] = key_logit(win); sh.ci[j] = key_token(win); }
-        if (win == mine && j + 1 < k) {      // mine was picked
-            mine = 0ull;
-            for (int v = threadIdx.x; v < V; v += kTailThreads) {
-                const unsigned long long kv = rank_key(z[v], v);
-                if (kv < win && kv > mine) mine = kv;
+        const unsigned long long win = warp_best(mine);
+        if (lane == 0) sh.best[warp * kMaxCand + j] = win;
+        if (win == mine && win != 0ull && j + 1 < k) {      // mine was picked
+            if (known) { mine = next; known = false; }
+            else { scan(win, mine, next); known = true; }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        // lane l reads list l / 4, every fourth entry from l % 4 on
+        const unsigned long long *list = sh.best + (lane >> 2) * kMaxCand;
+        int at = lane & 3;
+        unsigned long long head = at < k ? list[at] : 0ull;
+        for (int j = 0; j < k; ++j) {
+            const unsigned long long win = warp_best(head);
+            if (lane == 0) { sh.cv[j] = key_logit(win); sh.ci[j] = key_token(win); }
+            if (win == head) {
+                at += 4;
+                head = at < k ? list[at] : 0ull;
             }
         }
     }
@@ -224,11 +251,11 @@ static __device__ void top_candidates(const Dev &D, const float *z, int k, TailS
 static __device__ int pick_candidate(const RunParams &R, int k, uint32_t r24, const TailShared &sh) {
     if (R.sample_mode == 0) return sh.ci[0];
     float total = 0.f;
-    for (int j = 0; j < k; ++j) total += expf((sh.cv[j] - sh.cv[0]) / R.temperature);
+    for (int j = 0; j < k; ++j) total += sh.cw[j];
     const float u = (float)r24 * (1.0f / 16777216.0f);
     float cum = 0.f;
     for (int j = 0; j < k; ++j) {
-        cum += expf((sh.cv[j] - sh.cv[0]) / R.temperature);
+        cum += sh.cw[j];
         if (cum > u * total) return sh.ci[j];
     }
     return sh.ci[k - 1];
@@ -359,6 +386,10 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     const int k = tree ? min(max(R.k_sample, 1), min(V, 8)) : R.sample_mode == 0 ? 1 : min(max(R.k_sample, 1), min(V, kMaxCand));
     top_candidates(D, z, k, sh);
     if (!tree) {
+        if (R.sample_mode != 0) {
+            if (tid < k) sh.cw[tid] = expf((sh.cv[tid] - sh.cv[0]) / R.temperature);
+            __syncthreads();
+        }
         if (tid == 0) sh.tok = pick_candidate(R, k, rand24(R, b, (uint32_t)sh.state[2], (uint32_t)slot, 0u), sh);
     } else {
         // probability tree: this head's K_s best tokens and their probabilities, for slot 1, which draws one path for all heads
@@ -408,6 +439,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
         sh.cand[tid] = v;
     }
     __syncthreads();
+    if (K > 0) cluster_arrive();         // (this CTA has read its peers' candidates)
     // commit x_{s+1..s*}, s <- s*, next window <- candidates: worked out by every CTA, written by CTA 0
     if (tid == 0) {
         const bool w = slot == 0;
@@ -464,9 +496,10 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     }
     __syncthreads();
     const int new_len = sh.state[0] + a + 1;
-    if (slot == 0 && tid < K1) place_row(D, b * K1 + tid, b, new_len + tid, !sh.state[5]);
+    if (slot == 0 && tid >= kTailThreads - 32 && tid - (kTailThreads - 32) < K1)      // (the last warp: the embedding needs the first ones)
+        place_row(D, b * K1 + tid - (kTailThreads - 32), b, new_len + tid - (kTailThreads - 32), !sh.state[5]);
     if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], new_len + slot, sh.red);
-    if (K > 0) { cluster_arrive(); cluster_wait(); }      // peers may still read this CTA's candidate
+    if (K > 0) cluster_wait();           // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }
 
