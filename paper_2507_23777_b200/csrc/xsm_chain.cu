@@ -194,6 +194,7 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
     const int keys = cross ? D.C : D.max_blocks * D.P;
     A.S = std::min(A.S, (keys + A.split - 1) / A.split);
     A.warps = t <= 8 && D.dh <= 64 && items * A.S <= sms_ && keys > 512 * A.S ? 16 : 8;
+    A.warm = items * A.S <= sms_;
     const int round = upp == 1 || upp == 2 || upp == 4 ? 8 / upp : 1;
     const int pages = ((cross ? D.cpages : D.max_blocks) + A.S - 1) / A.S;
     const int budget = items * A.S > sms_ ? 100 * 1024 : 128 * 1024;

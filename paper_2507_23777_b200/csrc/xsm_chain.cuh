@@ -58,7 +58,7 @@ struct AttnArgs {
     int cross, sets, layer;           // sets: decoding heads that attend in this stage (cross-attention heads), else 1
     int t, rows, Mp, qp, pos0, pos_end;      // as in ProjArgs
     int qt;                           // tiles of kTokenTile rows of a sequence
-    int warps;                        // that attend (few rows: 8 or 16)
+    int warps, warm;                  // that attend (few rows: 8 or 16); run the code once before the wait
     int S, split, slots, ring;        // most CTAs per (sequence, head), keys for each; page pairs in shared memory, its bytes
     const void *pool;                 // cache tiles
     const __half *q;                  // planes [2][qp][d] (a set per decoding head)
