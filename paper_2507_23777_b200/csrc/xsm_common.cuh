@@ -53,11 +53,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 // Waits for the phase of the given parity, bounded: when `limit` tries run out the status word is raised and the caller goes
 // on (its results are then void; the host reports the timeout).
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, unsigned limit, int *status) {
-    if (mbar_try_wait(bar, parity)) return;
+// (false: the limit ran out)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned limit, int *status) {
+    if (mbar_try_wait(bar, parity)) return true;
     for (unsigned n = 0; n < limit; ++n)
-        if (mbar_try_wait(bar, parity)) return;
+        if (mbar_try_wait(bar, parity)) return true;
     atomicExch(status, XSM_STATUS_TIMEOUT);
+    return false;
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         mbar_init(done, 1u);
         mbar_init(smem_u32(&recv_bar), 1u);
         mbar_init_fence();
-        if (S > 1 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)((S - 1) * ((nm + 3) >> 2)) * 2048u);
+        if (S > 1 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
     }
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
@@ -99,13 +99,41 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const bf16 *xb = x + (size_t)k_lo * (128 * Mp);      // this CTA's blocks of the activations
     const uint32_t idesc = umma_idesc(128, 2 * Mp), tmem = tmem_slot, full_a = bar(0, 0), full_b = bar(2, 0);
     settle(xb);
+    constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
+    constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
+    const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
+    const bool live_row = u_row < G.units;
+    float gain = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u_row)) : 0.f;
+    // where this thread's weight row goes
+    const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
+    __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
+    bf16 *xrow = G.out + (size_t)(A.tt > 1 ? token_tile : job) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
+    const int xchunk = (u_row >> 3) & 7;
+    float *lrow = G.logits + (size_t)job * D.M * G.ld + u_row;
+    __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
+    settle(gain); settle(qrow); settle(xrow); settle(lrow); settle(crow);
+    // Accumulator -> the CTA that finishes the token rows: [sender][quad][weight row][4].  This thread's lane of the accumulator
+    // is its weight row; eight token rows at a time, from c0 on.
+    const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = warp >> 2, qinv = 65536 / qps + 1;
+    const uint32_t recv_b = smem_u32(&recv_bar);
+    uint32_t dst[2], dst_bar[2];
+    auto where = [&](int c) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int quad = 2 * c + q, owner = (quad * qinv) >> 16, place = rank * qps + quad - owner * qps;      // (quad / qps: both are below 33)
+            dst[q] = S > 1 ? map_rank(srecv + (uint32_t)(place * 128 + arow) * 16u, (uint32_t)min(owner, S - 1)) : (uint32_t)(quad * 128 + arow) * 16u;
+            dst_bar[q] = S > 1 ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;
+        }
+    };
+    where(c0);
+    settle(dst[0]); settle(dst[1]); settle(dst_bar[0]); settle(dst_bar[1]);
+    if (S > 1) cluster_wait();            // the peers run: their barriers and shared memory are there
     if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kProjThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (active == 0) {      // every sequence has ended in an earlier step
         if (tid == 0)
             for (int i = 0; i < min(n, na); ++i) mbar_wait(bar(0, i), 0u, D.mbar_limit, D.status);
         __syncthreads();
-        if (S > 1) cluster_wait();
         if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
         return;
     }
@@ -169,11 +197,6 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     }
     // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row, four at a
     // time; what it reads from memory is requested before the products are waited for, or a round ahead.
-    constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
-    constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
-    const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
-    const bool live_row = u_row < G.units;
-    const float gain = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u_row)) : 0.f;
     float hn[4];
     float2 csn[4];
     auto request = [&](int i0) {
@@ -186,42 +209,31 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     };
     __syncwarp();
     request(side);
-    mbar_wait(done, 0u, D.mbar_limit, D.status);
+    __syncthreads();      // (what the epilogue needs is in shared memory; the last products are under way)
+    const bool done_ok = mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
     tcgen05_after_sync();
-    if (S > 1) cluster_wait();                // the peers run: their barriers and shared memory are there
-    {
-        // accumulator -> the CTA that finishes the token rows, hi and lo parts added: [sender][quad][weight row][4]
-        const int lanes = warp & 3, r = lanes * 32 + lane;               // this thread's accumulator lane = weight row
-        const uint32_t tbase = tmem_slot + ((uint32_t)(lanes * 32) << 16);
-        for (int c = warp >> 2; c < (Mp >> 3); c += kProjThreads / 128) {
-            uint32_t v[16];
-            tmem_ld16(v, tbase + (uint32_t)c * 16u);
-            tmem_wait_ld();
+    for (int c = c0; c < (Mp >> 3); c += kProjThreads / 128) {      // hi and lo parts added
+        uint32_t v[16];
+        tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
+        if (c != c0) where(c);
+        tmem_wait_ld();
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int quad = 2 * c + q;
-                if (quad * 4 < rows) {
-                    float f[4];
+        for (int q = 0; q < 2; ++q) {
+            if ((2 * c + q) * 4 < rows) {
+                float f[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
-                    const int owner = S > 1 ? quad / qps : 0, place = rank * qps + quad - owner * qps;
-                    if (owner == rank) {
-                        *reinterpret_cast<float4 *>(recv + (size_t)(place * 128 + r) * 4) = make_float4(f[0], f[1], f[2], f[3]);
-                    } else {
-                        st_async_v4(map_rank(srecv + (uint32_t)(place * 128 + r) * 16u, (uint32_t)owner), f, map_rank(smem_u32(&recv_bar), (uint32_t)owner));
-                    }
-                }
+                for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
+                if (S == 1) *reinterpret_cast<float4 *>(smem + (srecv - sa) + dst[q]) = make_float4(f[0], f[1], f[2], f[3]);
+                else if (done_ok) st_async_v4(dst[q], f, dst_bar[q]);      // (a peer that gave up waiting may have left)
             }
         }
     }
     tcgen05_before_sync();
-    __syncthreads();
-    if (warp == 2) {
-        tcgen05_after_sync();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
-    }
-    if (S > 1 && nm > 0) mbar_wait(smem_u32(&recv_bar), 0u, D.mbar_limit, D.status);
+    // One CTA to a tile: a barrier.  In a cluster every CTA waits for all shares of its rows, its own among them, so none leaves
+    // before what is sent to it has come: no barrier at the end, whose wait for all stores took 1600 to 2400 cycles.
+    if (S == 1) __syncthreads();
+    else if (nm > 0 && !mbar_wait(recv_b, 0u, D.mbar_limit, D.status)) mbar_wait(recv_b, 0u, D.mbar_limit, D.status);
     __syncwarp();
     // sums over the cluster in rank order, epilogue
     auto total = [&](int i, int r) {
@@ -230,13 +242,6 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         for (int s = 1; s < S; ++s) v += p[s * qps * 512];
         return v;
     };
-    // where this thread's weight row goes
-    const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
-    __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
-    bf16 *xrow = G.out + (size_t)(A.tt > 1 ? token_tile : job) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
-    const int xchunk = (u_row >> 3) & 7;
-    float *lrow = G.logits + (size_t)job * D.M * G.ld + u_row;
-    __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
     auto put_x = [&](int m, float v) {
         bf16 hi, lo;
         split_bf16(v, hi, lo);
@@ -289,10 +294,17 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             }
         }
     }
-    if (S > 1) { cluster_arrive(); cluster_wait(); }      // (what this CTA sent has been received before its peers leave)
     if (D.trace != nullptr) {
         __syncthreads();
         trace_mark(D, 2 + 2 * A.stage);
+    }
+    // (every warp has read its part of the accumulator)
+    if (warp != 2) {
+        asm volatile("bar.arrive 2, %0;" :: "n"(kProjThreads) : "memory");
+    } else {
+        asm volatile("bar.sync 2, %0;" :: "n"(kProjThreads) : "memory");
+        tcgen05_after_sync();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
     }
 }
 
