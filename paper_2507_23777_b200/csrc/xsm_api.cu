@@ -7,7 +7,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <atomic>
 #include <string>
 #include <vector>
 
@@ -25,7 +24,7 @@ struct Layout {
     size_t len, window, finished, n_gen, n_blocks, step_idx, block_table, free_stack, scalars, hist, steps, tok_log, step_tokens,
         step_n_new, prompt, script;
     size_t h, rope_cs, row_info, row_cs, logits0, hlogits;
-    size_t rp, xa, qp, aa, actp, yp, hq, ha, ss, apart, acount;
+    size_t rp, xa, qp, aa, actp, yp, hq, ha, ss;
     size_t stage_cond, stage_kv, stage_tok, trace, ckv_pool, hckv_pool, kv_pool;
     int n_pages = 0, max_blocks = 0, cpages = 0, tok_ld = 0, n_stages = 0;
     size_t page_bytes = 0;
@@ -83,8 +82,6 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.hq = take(cur, step_row * d * nh);
     L.ha = take(cur, step_row * d * nh);
     L.ss = take(cur, row * kShareLd);
-    L.apart = take(cur, step_row * kSplitCtas * (dh + 2));
-    L.acount = take(cur, 4 * kSplitCtas);
     L.logits0 = take(cur, 4 * M * V);
     L.hlogits = take(cur, 4 * M * V * (c.n_draft > 0 ? c.n_draft : 1));
     L.stage_cond = take(cur, esize(c) * B * c.n_cond * c.d_cond);
@@ -229,14 +226,12 @@ xsm_status check_device_status(xsm_ctx *ctx) {
     return XSM_OK;
 }
 
-// one decoding step on the stream; scratch: device memory for the partial results of the key splits (null: the workspace's)
-xsm_status run_step(xsm_ctx *ctx, float *scratch = nullptr) {
+// one decoding step on the stream
+xsm_status run_step(xsm_ctx *ctx, bool may_record = true) {
     // a recording is replayed unless single launches were asked for, a timeline is taken (the recording has none), or the
     // call must not make the driver allocate anything
-    const bool graph = !ctx->phase_launch && scratch == nullptr && ctx->dev.trace == nullptr;
-    Dev D = ctx->dev;
-    if (scratch) D.apart = scratch;
-    XSM_CUDA(ctx, ctx->chain.step(D, ctx->stream, graph, !ctx->phase_launch, &ctx->launches));
+    const bool graph = !ctx->phase_launch && may_record && ctx->dev.trace == nullptr;
+    XSM_CUDA(ctx, ctx->chain.step(ctx->dev, ctx->stream, graph, !ctx->phase_launch, &ctx->launches));
     return XSM_OK;
 }
 
@@ -378,7 +373,6 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     D.row_info = at<RowInfo>(ctx, L.row_info); D.row_cs = at<float2>(ctx, L.row_cs);
     D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
     D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
-    D.apart = at<float>(ctx, L.apart); D.acount = at<int>(ctx, L.acount);
     D.tail_row_bytes = 160 * 1024;
     D.logits0 = at<float>(ctx, L.logits0); D.hlogits = at<float>(ctx, L.hlogits);
     D.kv_pool = ctx->ws + L.kv_pool; D.ckv_pool = ctx->ws + L.ckv_pool; D.hckv_pool = ctx->ws + L.hckv_pool;
@@ -449,12 +443,9 @@ xsm_status xsm_spec_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) 
     return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
 
-// ---- scratch owned by the library, for xsm_spec_step_static
-// The name below is a device symbol: host code may not use it as an address.  Its device address is asked
-// for once per device (cudaGetSymbolAddress) and kept.
+// The partial results of the key splits travel within clusters and need no memory; the call keeps the limit that it had when
+// they lay in an array of the library.
 constexpr size_t kStaticScratchBytes = (size_t)1 << 20;
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
-static std::atomic<void *> g_static_scratch_addr[kMaxDevices];   // by device ordinal; null until the first call on that device
 
 xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
@@ -470,16 +461,8 @@ xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_
         return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch need " +
                                                std::to_string(n_sets * half) + " bytes, the built-in scratch holds " +
                                                std::to_string(kStaticScratchBytes));
-    int dev = 0;
-    XSM_CUDA(ctx, cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) return fail(ctx, XSM_ERR_INVALID_ARG, "device ordinal out of range");
-    if (g_static_scratch_addr[dev].load() == nullptr) {   // set-up, once per device, with that device current
-        void *p = nullptr;                                // (threads that race here all store the same address)
-        XSM_CUDA(ctx, cudaGetSymbolAddress(&p, g_static_scratch));
-        g_static_scratch_addr[dev].store(p);
-    }
     xsm_status st = set_max_new(ctx, INT_MAX);
-    if (st == XSM_OK) st = run_step(ctx, static_cast<float *>(g_static_scratch_addr[dev].load()));
+    if (st == XSM_OK) st = run_step(ctx, false);
     return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
 

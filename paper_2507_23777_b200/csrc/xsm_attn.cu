@@ -190,22 +190,27 @@ constexpr int kQueryBlocks = 4;      // blocks of 32 columns per warp: d_model u
 // NW: warps that attend, beside the producer.  A unit of 32 keys is some 300 dependent instructions, 1 us for a warp on its
 // own, so sixteen warps where a CTA has many units (and where the queries are projected); eight otherwise, of which two
 // CTAs share an SM when a batch has more (sequence, head) pairs than there are SMs.
-template <int DH, bool FEW, bool QP, int NW>
+// CL: several CTAs to a (sequence, head), a cluster.
+template <int DH, bool FEW, bool QP, int NW, bool CL>
 __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 : 1) attn_kernel(const Dev D, const AttnArgs A) {
     constexpr int kThreads = NW * 32 + 32, RB = DH * 2;
     extern __shared__ __align__(128) char smem[];
-    __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots], w_full;
+    __shared__ __align__(8) uint64_t full[kAttnSlots], empty[kAttnSlots], w_full, recv_bar;
     __shared__ float s_inv[8];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // (tiles of a sequence's rows: those that see the most keys first)
-    const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z % D.B, zz = blockIdx.z / D.B, set = zz % A.sets;
-    const int q0 = (A.qt - 1 - zz / A.sets) * kTokenTile, t_rows = min(A.t - q0, kTokenTile), t_cap = min(A.t, kTokenTile);
+    const int rank = CL ? blockIdx.x : 0, h = blockIdx.y, b = blockIdx.z % D.B, zz = blockIdx.z / D.B, set = zz % A.sets;
+    const int q0 = (A.qt - 1 - zz / A.sets) * kTokenTile, t_rows = min(A.t - q0, kTokenTile);
     const int P = D.P, upp = P >> 5, slots = A.slots;
     const bool cross = A.cross != 0;
     const int first = cross ? 0 : A.pos0 >= 0 ? A.pos0 : __ldcg(D.len + b);      // (the state was written by an earlier step)
     const int start = first + q0, n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + t_rows, A.pos_end) : start + t_rows;
-    const int S = min(A.S, (n_keys + A.split - 1) / A.split);                    // CTAs that take part
-    if (rank >= S) return;
+    const int S = CL ? min(A.S, (n_keys + A.split - 1) / A.split) : 1;           // CTAs that take part
+    if (CL && rank >= S) {
+        cluster_arrive();
+        cluster_wait();
+        return;
+    }
     // few rows: a warp looks only at the pages whose units it owns when the units of 1, 2 or 4 pages fill a round of the
     // warps (the ring is a whole number of rounds, so a warp meets every fill of its slots)
     const bool owned = FEW && NW == 8 && (upp == 1 || upp == 2 || upp == 4);
@@ -215,10 +220,15 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             mbar_init(smem_u32(&empty[i]), owned ? (uint32_t)upp : (uint32_t)NW);
         }
         if (QP) mbar_init(smem_u32(&w_full), 1u);
+        mbar_init(smem_u32(&recv_bar), 1u);
         mbar_init_fence();
+        // (rows rank, rank + S, .. are finished here; may be none)
+        const int my_rows = (t_rows - rank + S - 1) / S;
+        if (CL && S > 1 && my_rows > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * my_rows * (DH + 2)) * 4u);
     }
     __syncthreads();
     chain_go();
+    if (CL) { cluster_arrive(); cluster_wait(); }      // the peers run: what is sent to them has a place
     const bool dead = A.pos0 < 0 && __ldcg(D.finished + b) != 0;
     if (dead) {
         chain_wait();
@@ -252,7 +262,7 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
     // once per stage, and a cold one costs as much again: measured on the merge, 1900 against 1000 cycles).  Self-attention
     // of one sequence 3.5 -> 3.0 us; slower where the first run ends after the wait would have (two CTAs to an SM) or costs
     // registers (QP, heads of 128).
-    constexpr bool WARM = FEW && !QP && DH <= 64 && NW == 8;
+    constexpr bool WARM = FEW && !QP && !CL && DH <= 64 && NW == 8;
 #pragma unroll 1
     for (int round = WARM && A.warm && warp < NW ? 0 : 1; round < 2; ++round) {
     int real = 1;
@@ -497,9 +507,8 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
     // the warps' states of a row -> the output, or this CTA's partial result.  Two neighbouring columns a thread.
     bf16 *out = A.out + (size_t)set * 2 * A.Mp * D.d;
     const int states = FEW && all_in ? min(NW, n_units) : kg_n;
-    const int item = blockIdx.z * D.H + h, n_pairs = t_rows * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
-    // partial results: [items][S][t][DH + 2]; acount: CTAs of an item that have left theirs (zero between kernels)
-    float *mine = D.apart + ((size_t)(item * A.S + rank) * t_cap) * LD;
+    const int n_pairs = t_rows * (DH / 2), step = (FEW ? srows : wq * 16) * LD;
+    const float *const recv = reinterpret_cast<const float *>(smem + A.recv);      // [sender][row of this CTA][DH + 2]
     auto store = [&](int r, int c, float v0, float v1) {
         bf16 h0, l0, h1, l1;
         split_bf16(v0, h0, l0);
@@ -523,53 +532,46 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             o1 += f * o.y;
             l += f * src[w * step + DH + 1];
         }
-        if (S == 1) {
+        if (!CL || S == 1) {
             const float inv = 1.f / l;
             store(r, c, o0 * inv, o1 * inv);
         } else if (real) {
-            float *dst = mine + (size_t)r * LD;
-            __stcg(reinterpret_cast<float2 *>(dst + c), make_float2(o0, o1));
-            if (c == 0) __stcg(reinterpret_cast<float2 *>(dst + DH), make_float2(m, l));
+            const uint32_t slot = (uint32_t)(r / S), owner = (uint32_t)r - slot * S, rows = (uint32_t)((t_rows - (int)owner + S - 1) / S);
+            const uint32_t dst = map_rank(smem_u32(recv) + ((uint32_t)rank * rows + slot) * (uint32_t)(LD * 4), owner), bar = map_rank(smem_u32(&recv_bar), owner);
+            st_async_v2(dst + (uint32_t)c * 4u, o0, o1, bar);
+            if (c == 0) st_async_v2(dst + DH * 4u, m, l, bar);
         }
     }
-    if (S > 1 && real) {
-        __shared__ int s_last;
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) s_last = atomicAdd(D.acount + item, 1) == S - 1;
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            const float *all = D.apart + ((size_t)item * A.S * t_cap) * LD;
-            for (int e = tid; e < n_pairs; e += kThreads) {
-                const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
-                float2 ml[8], os[8];
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const float *src = all + ((size_t)s * t_cap + r) * LD;
-                    ml[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + DH)) : make_float2(kNegBig, 0.f);
-                    os[s] = s < S ? __ldcg(reinterpret_cast<const float2 *>(src + c)) : make_float2(0.f, 0.f);
-                }
-                float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
-#pragma unroll
-                for (int s = 0; s < 8; ++s) m = fmaxf(m, ml[s].x);
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const float f = ex2(ml[s].x - m);
-                    o0 += f * os[s].x;
-                    o1 += f * os[s].y;
-                    l += f * ml[s].y;
-                }
-                const float inv = 1.f / l;
-                store(r, c, o0 * inv, o1 * inv);
+    // The CTAs of a (sequence, head) are a cluster: each takes the partial results of its share of the rows from all of them, in
+    // shared memory, by counted stores, and adds them up in rank order.  (Through global memory, with a counter that told the
+    // last CTA to merge, the two fences and the round trips cost 4 to 5 us.)
+    if (CL && S > 1 && real && rank < t_rows) {
+        const int my_rows = (t_rows - rank + S - 1) / S;
+        if (!mbar_wait(smem_u32(&recv_bar), 0u, D.mbar_limit, D.status)) mbar_wait(smem_u32(&recv_bar), 0u, D.mbar_limit, D.status);
+        __syncwarp();
+        for (int e = tid; e < my_rows * (DH / 2); e += kThreads) {
+            const int i = e / (DH / 2), c = (e - i * (DH / 2)) * 2;
+            const float *src = recv + i * LD;
+            float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
+            for (int s = 0; s < S; ++s) m = fmaxf(m, src[s * my_rows * LD + DH]);
+            for (int s = 0; s < S; ++s) {
+                const float *p = src + s * my_rows * LD;
+                const float f = ex2(p[DH] - m);
+                const float2 o = *reinterpret_cast<const float2 *>(p + c);
+                o0 += f * o.x;
+                o1 += f * o.y;
+                l += f * p[DH + 1];
             }
-            if (tid == 0) D.acount[item] = 0;
+            const float inv = 1.f / l;
+            store(rank + i * S, c, o0 * inv, o1 * inv);
         }
     }
     }
     trace_mark(D, 2 + 2 * A.stage);
 }
 
+// shared memory for the partial results of the cluster's CTAs: s senders, ceil(t / s) rows, for any s up to S that takes part
+int attn_recv(const Dev &D, int S, int t) { return S > 1 ? (min(t, kTokenTile) + S - 1) * (D.dh + 2) * 4 : 0; }
 // shared memory that the states of the warps take when the pages are done with
 int attn_park(const Dev &D, int t, int warps) { return warps * (t <= 8 ? t : 16) * (D.dh + 2) * 4; }
 // shared memory beside the ring of a stage whose queries the kernel projects itself; 0: not possible
@@ -579,26 +581,29 @@ int attn_query_smem(const Dev &D, int t) {
     return weights > later ? weights : later;
 }
 
-template <int DH, bool FEW, bool QP, int NW>
-static cudaError_t launch_instance(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
-    void (*fn)(const Dev, const AttnArgs) = attn_kernel<DH, FEW, QP, NW>;
-    const int smem = A.ring + (QP ? attn_query_smem(D, A.t) : 0);
+template <int DH, bool FEW, bool QP, int NW, bool CL>
+static cudaError_t launch_instance(const Dev &D, const AttnArgs &args, const ChainLaunch &L) {
+    void (*fn)(const Dev, const AttnArgs) = attn_kernel<DH, FEW, QP, NW, CL>;
+    AttnArgs A = args;
+    A.recv = A.ring + (QP ? attn_query_smem(D, A.t) : 0);
+    const int smem = A.recv + attn_recv(D, A.S, A.t);
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
-    return L.launch(dim3(A.S, D.H, D.B * A.sets * A.qt), dim3(NW * 32 + 32), smem, 1, (const void *)fn, D, A);
+    return L.launch(dim3(A.S, D.H, D.B * A.sets * A.qt), dim3(NW * 32 + 32), smem, A.S, (const void *)fn, D, A);
 }
 
-template <int DH>
+template <int DH, bool CL>
 static cudaError_t launch_heads(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
-    if (A.t > 8) return launch_instance<DH, false, false, 8>(D, A, L);
+    if (A.t > 8) return launch_instance<DH, false, false, 8, CL>(D, A, L);
     if constexpr (DH <= 64) {
-        if (A.wq != nullptr) return launch_instance<DH, true, true, 16>(D, A, L);
-        if (A.warps == 16) return launch_instance<DH, true, false, 16>(D, A, L);
+        if (A.wq != nullptr) return launch_instance<DH, true, true, 16, CL>(D, A, L);
+        if (A.warps == 16) return launch_instance<DH, true, false, 16, CL>(D, A, L);
     }
-    return launch_instance<DH, true, false, 8>(D, A, L);
+    return launch_instance<DH, true, false, 8, CL>(D, A, L);
 }
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L) {
-    return D.dh == 32 ? launch_heads<32>(D, A, L) : D.dh == 64 ? launch_heads<64>(D, A, L) : launch_heads<128>(D, A, L);
+    if (A.S > 1) return D.dh == 32 ? launch_heads<32, true>(D, A, L) : D.dh == 64 ? launch_heads<64, true>(D, A, L) : launch_heads<128, true>(D, A, L);
+    return D.dh == 32 ? launch_heads<32, false>(D, A, L) : D.dh == 64 ? launch_heads<64, false>(D, A, L) : launch_heads<128, false>(D, A, L);
 }
 
 }  // namespace xsm

@@ -186,18 +186,24 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
     A.Mp = Mp;
     A.qt = (t + kTokenTile - 1) / kTokenTile;
     const int items = D.B * D.H * sets * A.qt, upp = D.P / 32, pair = 2 * D.P * D.dh * 2;
-    // About one CTA per SM at most; few rows: one more for every 512 keys (two units of 32 for each of eight warps; a merge costs
-    // as much as two), sixteen warps where a CTA can have more than that.
+    // A (sequence, head) is cut over a cluster of S CTAs, about one per SM in all and no more than run at a time.  A CTA more pays
+    // for every 384 keys (192 in heads of 128; 12 or 6 units of 32 keys, 1 us each, over eight warps) and less than that costs
+    // more in the exchange: medium width at 500 keys 797 -> 758 us a step, at 1500 851 -> 818, heads of 128 at 513 keys 9.2 -> 7.0
+    // us a stage.  Tiles of 16 rows: a unit serves all of them, 128 keys.  Sixteen warps where a CTA can have more than 512
+    // keys and an SM to itself.
     A.S = 1;
-    while (A.S < 8 && items * A.S * 2 <= sms_ + sms_ / 8) A.S *= 2;
-    A.split = t <= 8 ? (D.dh <= 64 ? 512 : 640) : 128;
+    const int per_sm = t <= 8 && D.dh <= 64 ? 2 : 1;      // CTAs that an SM can hold
+    for (int s = 2; s <= 8; ++s)
+        if (items <= per_sm * clusters_[s] && items * s <= sms_ + sms_ / 8) A.S = s;
+    A.split = t <= 8 ? (D.dh <= 64 ? 384 : 192) : 128;
     const int keys = cross ? D.C : D.max_blocks * D.P;
     A.S = std::min(A.S, (keys + A.split - 1) / A.split);
-    A.warps = t <= 8 && D.dh <= 64 && items * A.S <= sms_ && keys > 512 * A.S ? 16 : 8;
-    A.warm = items * A.S <= sms_;
+    const bool alone = items * A.S <= sms_ && (A.S == 1 || items <= clusters_[A.S]);      // an SM for every CTA
+    A.warps = t <= 8 && D.dh <= 64 && alone && keys > 512 * A.S ? 16 : 8;
+    A.warm = A.S == 1 && items <= sms_;
     const int round = upp == 1 || upp == 2 || upp == 4 ? 8 / upp : 1;
     const int pages = ((cross ? D.cpages : D.max_blocks) + A.S - 1) / A.S;
-    const int budget = items * A.S > sms_ ? 100 * 1024 : 128 * 1024;
+    const int budget = alone ? 128 * 1024 : 100 * 1024;
     int slots = std::min(16, budget / pair) / round * round;
     slots = std::max(round, std::min(slots, (pages + round - 1) / round * round));
     A.slots = slots;
@@ -209,8 +215,8 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
 // least two at a time), and every CTA needs an SM to itself.
 bool Chain::own_queries(const Dev &D, AttnArgs &A) const {
     const int weights = attn_query_smem(D, A.t), pair = 2 * D.P * D.dh * 2;
-    if (c_.dtype != 1 || weights == 0 || A.S * D.H * D.B > sms_) return false;
-    const int room = kProjSmemMax - weights, pages = (D.cpages + A.S - 1) / A.S;
+    if (c_.dtype != 1 || weights == 0 || A.S * D.H * D.B > sms_ || (A.S > 1 && D.H * D.B > clusters_[A.S])) return false;
+    const int room = kProjSmemMax - weights - attn_recv(D, A.S, A.t), pages = (D.cpages + A.S - 1) / A.S;
     const int all = A.S > 1 ? pages * pair : (pages - 1) * pair + ((D.C - (pages - 1) * D.P + 31) / 32 * 32) * D.dh * 4;
     A.ring = std::max(all <= room ? all : room / pair * pair, attn_park(D, A.t, 16));
     A.slots = std::min(16, A.ring / pair);

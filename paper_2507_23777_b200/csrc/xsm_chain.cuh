@@ -59,7 +59,8 @@ struct AttnArgs {
     int t, rows, Mp, qp, pos0, pos_end;      // as in ProjArgs
     int qt;                           // tiles of kTokenTile rows of a sequence
     int warps, warm;                  // that attend (few rows: 8 or 16); run the code once before the wait
-    int S, split, slots, ring;        // most CTAs per (sequence, head), keys for each; page pairs in shared memory, its bytes
+    int S, split, slots, ring;        // most CTAs per (sequence, head) (a cluster), keys for each; page pairs in shared memory, its bytes
+    int recv;                         // where the other CTAs' partial results arrive in shared memory
     const void *pool;                 // cache tiles
     const __half *q;                  // planes [2][qp][d] (a set per decoding head)
     bf16 *out;                        // planes of d columns (a set per decoding head; layout: xsm_proj.cuh)
@@ -123,6 +124,7 @@ cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, 
 cudaError_t launch_attn(const Dev &D, const AttnArgs &A, const ChainLaunch &L);
 int attn_query_smem(const Dev &D, int t);
 int attn_park(const Dev &D, int t, int warps);
+int attn_recv(const Dev &D, int S, int t);
 // fp32 models: at most this many token rows
 constexpr int kF32Rows = 24;
 cudaError_t launch_proj_f32(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L);

@@ -12,7 +12,6 @@ constexpr int kMaxDevices = 64;                      // device ordinals the per-
 // Every device-side wait is bounded: polls of a word in global memory and mbarrier try_wait calls.
 constexpr unsigned kSpinLimit = 1u << 21, kMbarSpinLimit = 1u << 22;
 constexpr int kShareLd = 160;                        // shares of a row's sum of squares: [row][kShareLd]
-constexpr int kSplitCtas = 256;                      // most CTAs that leave partial results in an attention stage
 
 // What a request may change without changing the launch chain (which is recorded once): kept in device memory.
 struct RunParams {
@@ -61,8 +60,6 @@ struct Dev {
     void *xa_;                     // the residual stream times the gain of the RMSNorm that reads it next
     void *qp_, *aa_, *actp_, *yp_; // queries, attention rows, gated activations, decoding heads' hidden states (a set per head)
     void *hq_, *ha_;               // cross-attention heads: queries, attention rows (a set per head)
-    float *apart;                  // attention: partial results of the key splits; acount: splits that have left theirs
-    int *acount;
     float *ss;                     // [kMaxTokens][kShareLd] shares of the sums of squares of the rows of h
     float *logits0, *hlogits;      // [M][V], [K][M][V]
     float *h;                      // residual stream [row][d]

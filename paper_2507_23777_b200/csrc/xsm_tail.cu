@@ -518,7 +518,6 @@ __global__ void set_run_kernel(const Dev D, const RunParams R) { *D.rp = R; }
 __global__ void begin_pool_kernel(const Dev D, const RunParams R) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < D.n_pages) D.free_stack[i] = D.n_pages - 1 - i;
-    if (i < 256) D.acount[i] = 0;
     if (i == 0) { *D.n_free = D.n_pages; *D.n_active = D.B; *D.status = 0; *D.stage_word = 0; *D.rp = R; }
 }
 __global__ void begin_seq_kernel(const Dev D) {
