@@ -124,21 +124,41 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.rows = rows;
     A.Mp = Mp;
     const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
-    // (clusters have to fit into a GPC: of six CTAs 22 run at a time, of eight 15; a cluster more than that is a second wave)
-    int S = 1;
-    const int tile_rows = std::min(rows, kTokenTile);
-    for (int s = 2; s <= std::min(8, nblk); ++s)
-        if (tiles * A.tt <= clusters_[s]) S = s;
+    // How a tile of weight rows is cut: its columns over a cluster of S CTAs, as many as fit into the GPCs at a time (of six CTAs
+    // 22 clusters, of eight 15; a cluster more is a second wave).  More than 96 token rows in one plane: these into T parts too,
+    // each with the weights for itself, which leaves less to exchange and to finish in a CTA.  The stage's time after the wait
+    // in cycles, as measured, chooses among S and T: a product 47, or N / 2 where the token rows (hi and lo) bound it;
+    // activations, and weights that do not fit the ring, 59 bytes a cycle; 45 for every token row that is sent, 250 for every
+    // one that is finished.  125 rows of width 1024: 2079 -> 1834 us a step.  Below, the CTAs of more parts keep the next stage's
+    // weights out of shared memory for longer than they save: 90 rows of width 768 703 -> 716, 80 rows 1494 -> 1498, 40 rows 1221 -> 1273.
+    int S = 1, T = 1;
+    const bool parts = A.tt == 1 && rows > 96;
+    double best = 1e30;
+    for (int t = 1; t <= (parts ? Mp / 8 : 1); ++t) {
+        const int nt = parts ? (Mp / 8 + t - 1) / t * 8 : std::min(Mp, kTokenTile);
+        if ((Mp + nt - 1) / nt != t) continue;
+        for (int s = 1; s <= std::min(8, nblk); ++s) {
+            const int n = (nblk + s - 1) / s;
+            if (s > 1 ? tiles * A.tt * t > clusters_[s] : t > 1 && tiles * t > sms_) continue;
+            const double late = std::max(0.0, n * 16384.0 - 160 * 1024), sent = s > 1 ? 600 + 45.0 * nt : 0;
+            const double cost = n * 4 * std::max(47.0, nt * 1.0) + (n * 256.0 * nt + late) / 59 + sent + 250.0 * ((nt + 4 * s - 1) / (4 * s) * 4);
+            if (!parts || cost < best) { best = cost; S = s; T = t; }
+        }
+    }
     A.S = S;
+    const int planes = A.tt;
+    A.tok = planes > 1 ? Mp : (Mp / 8 + T - 1) / T * 8;
+    A.tt = planes * T;
+    const int tile_rows = std::min(rows, A.tok);
     A.tps = ((tile_rows + 3) / 4 + S - 1) / S * 4;
-    const int n = (nblk + S - 1) / S, b_bytes = 2 * Mp * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
+    const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
     // more tiles than SMs: two CTAs to an SM
     const int room = (tiles * A.tt * S > sms_ ? kProjSmemMax / 2 : kProjSmemMax) - 1024 - (S > 1 ? sums : 0);
     A.nb = std::min(n, std::max(2, std::min(kProjRing, (room / 3) / b_bytes)));
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
     A.tmem_cols = 32;
-    while (A.tmem_cols < 2 * Mp) A.tmem_cols *= 2;
+    while (A.tmem_cols < 2 * A.tok) A.tmem_cols *= 2;
     const int rings = A.na * a_bytes + A.nb * b_bytes;
     op.smem = 1024 + (S > 1 ? rings + sums : std::max(rings, sums));
 }

@@ -36,7 +36,7 @@ struct ProjArgs {
     int epi0, epi1;                   // of the two groups; epi1 < 0: one group
     int stage;                        // index of the kernel in its chain
     int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8, at most kTokenTile)
-    int tt, qp;                       // tiles of token rows (a plane set for each); rows of the planes of queries
+    int tt, tok, qp;                  // tiles of tok token rows (parts of one plane set, or one for each); rows of the planes of queries
     int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
     int S, tps;                       // CTAs per cluster (cuts of the columns), token rows each of them finishes
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns

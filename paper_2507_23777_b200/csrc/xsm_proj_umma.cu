@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     // sequences that still run: looked at just before the wait, when the weights are on their way
     const int active = A.pos0 < 0 && !A.late_go ? __ldcg(D.n_active) : 1;
     // a tile of weight rows and a tile of token rows: neighbours share the weights
-    const int token_tile = A.tt > 1 ? (int)(blockIdx.x / S) % A.tt : 0, mb = token_tile * kTokenTile, rows = min(kTokenTile, A.rows - mb);
+    const int token_tile = A.tt > 1 ? (int)(blockIdx.x / S) % A.tt : 0, mb = token_tile * A.tok, rows = min(A.tok, A.rows - mb);
+    const int plane = mb / Mp, pm = mb - plane * Mp, Nt = min(A.tok, Mp - pm);      // where they are: plane set, first row; rows with padding
     int tile = blockIdx.x / S / A.tt, job = 0, z = A.layer, grp = 0;
     if (EPI1 >= 0 && tile >= A.g[0].tiles) {
         tile -= A.g[0].tiles;
@@ -55,9 +56,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const int nblk = A.kdim / kBlockK, k_lo = rank * nblk / S, n = (rank + 1) * nblk / S - k_lo;
     const int na = A.na, nb = A.nb;
     const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
-    const uint32_t b_bytes = (uint32_t)(2 * Mp) * kBlockK * 2u;
+    const uint32_t b_bytes = (uint32_t)(2 * Nt) * kBlockK * 2u, b_pitch = (uint32_t)(2 * A.tok) * kBlockK * 2u;
     // operand rings; behind them (one CTA to a tile: in their place, when the products are done) the partial sums
-    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = S > 1 ? sb + (uint32_t)nb * b_bytes : sa;
+    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = S > 1 ? sb + (uint32_t)nb * b_pitch : sa;
     float *recv = reinterpret_cast<float *>(smem + (srecv - sa));
     auto bar = [&](int kind, int i) { return smem_u32(&bars[kind * kProjRing + i]); };
     const uint32_t done = smem_u32(&bars[4 * kProjRing]);
@@ -95,9 +96,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     if (tid == 0)
         for (int i = 0; i < min(n, na); ++i) load_a(i, i);
     if (A.stage == 0) trace_mark(D, 0);
-    const bf16 *x = A.x + (size_t)(A.x_jobs ? job : token_tile) * 2 * Mp * A.kdim;
-    const bf16 *xb = x + (size_t)k_lo * (128 * Mp);      // this CTA's blocks of the activations
-    const uint32_t idesc = umma_idesc(128, 2 * Mp), tmem = tmem_slot, full_a = bar(0, 0), full_b = bar(2, 0);
+    const bf16 *x = A.x + (size_t)(A.x_jobs ? job : plane) * 2 * Mp * A.kdim;
+    const bf16 *xb = x + (size_t)k_lo * (128 * Mp) + (size_t)pm * 128;      // this CTA's blocks of the activations
+    const uint32_t idesc = umma_idesc(128, 2 * Nt), tmem = tmem_slot, full_a = bar(0, 0), full_b = bar(2, 0);
     settle(xb);
     constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
@@ -107,9 +108,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     // where this thread's weight row goes
     const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
     __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
-    bf16 *xrow = G.out + (size_t)(A.tt > 1 ? token_tile : job) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (u_row & 7);
+    bf16 *xrow = G.out + (size_t)(job + plane) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (size_t)pm * 128 + (u_row & 7);
     const int xchunk = (u_row >> 3) & 7;
-    float *lrow = G.logits + (size_t)job * D.M * G.ld + u_row;
+    float *lrow = G.logits + ((size_t)job * D.M + mb) * G.ld + u_row;
     __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
     settle(gain); settle(qrow); settle(xrow); settle(lrow); settle(crow);
     // Accumulator -> the CTA that finishes the token rows: [sender][quad][weight row][4].  This thread's lane of the accumulator
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         for (int i = 0; i < n; ++i) {
             if (i >= nb) mbar_wait(bar(3, slot), par, D.mbar_limit, D.status);
             mbar_arrive_expect_tx(full_b + 8u * (uint32_t)slot, b_bytes);
-            bulk_g2s(sb + (uint32_t)slot * b_bytes, xb + (size_t)i * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)slot);
+            bulk_g2s(sb + (uint32_t)slot * b_pitch, xb + (size_t)i * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)slot);
             if (++slot == nb) { slot = 0; par ^= 1u; }
             if (i >= na) {
                 mbar_wait(bar(1, a_slot), a_par, D.mbar_limit, D.status);
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
             mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
             tcgen05_after_sync();
-            const uint64_t da = umma_desc_sw128(sa + (uint32_t)ia * kABytes), db = umma_desc_sw128(sb + (uint32_t)ib * b_bytes);
+            const uint64_t da = umma_desc_sw128(sa + (uint32_t)ia * kABytes), db = umma_desc_sw128(sb + (uint32_t)ib * b_pitch);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, da + 2 * ks, db + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
             if (i + na < n) umma_commit(bar(1, ia));
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const bool done_ok = mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
     tcgen05_after_sync();
-    for (int c = c0; c < (Mp >> 3); c += kProjThreads / 128) {      // hi and lo parts added
+    for (int c = c0; c < (Nt >> 3); c += kProjThreads / 128) {      // hi and lo parts added
         uint32_t v[16];
         tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
         if (c != c0) where(c);
