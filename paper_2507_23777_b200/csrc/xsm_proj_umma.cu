@@ -17,6 +17,8 @@
 
 #include <cuda.h>
 
+#include <atomic>
+
 namespace xsm {
 
 constexpr int kProjThreads = 512;
@@ -318,7 +320,12 @@ static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMa
     return L.launch(dim3(tiles * A.tt * A.S), dim3(kProjThreads), smem, A.S, (const void *)fn, D, A, T);
 }
 
+// (asked for once per device: the answer does not change, and asking takes longer than the rest of a context's creation)
 int resident_clusters(int size) {
+    static std::atomic<int> known[kMaxDevices][9];      // the answer + 1
+    int dev = 0;
+    if (size < 2 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    if (const int k = known[dev][size].load()) return k - 1;
     const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1>;
     constexpr int smem = 200 * 1024;
     int n = 0;
@@ -336,6 +343,7 @@ int resident_clusters(int size) {
         (void)cudaGetLastError();
         return 0;
     }
+    known[dev][size].store(n + 1);
     return n;
 }
 

@@ -25,12 +25,9 @@ def speedup(scr: float, latency_base: float, latency_spec: float) -> float:
     return scr * latency_base / latency_spec
 
 
-# DRAM traffic of the step kernel measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum of one launch of 64
-# decoding steps at contexts 0..63, see profiles/), as a ratio to the algorithmic bytes of the same launch.  Traffic
-# grows in proportion to the units processed (weights once per step plus the cache), so a launch of the benchmark is
-# its algorithmic bytes times this ratio.  None: no capture of the current kernel for that configuration.
-_TRAFFIC_RATIO = {1: (19.537792e9 + 47.306752e6) / 19304546304.0,
-                  2: (63.641296e9 + 80.708864e6) / 63021514752.0}
+# DRAM traffic of a decoding step measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum over its launches), as a
+# ratio to the algorithmic bytes of the same step.  Empty: there is no capture of the present kernels.
+_TRAFFIC_RATIO: dict[int, float] = {}
 
 
 def measured_traffic(config_index: int, algorithmic_bytes_per_launch: float, head_kind: int = 0):

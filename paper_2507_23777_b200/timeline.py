@@ -4,8 +4,8 @@
 
 Runs `warm` decoding steps of the chosen configuration (batch 1 unless --batch), then one traced step, and prints
 for every kind of stage: how long the step spends in it (last CTA of the previous stage done -> last CTA of this
-stage done), how long a CTA waits for its inputs after finishing the previous stage, and how long it takes from
-"inputs are in shared memory" to "outputs are published".  Every mark is a read of the GPU's global timer plus a
+stage done), how long after the previous stage's end a CTA is past the wait for it, and how long it takes from there
+to its end.  Every mark is a read of the GPU's global timer plus a
 store (a few hundred nanoseconds), so a traced step is slower than an untraced one; compare shares, not totals.
 """
 from __future__ import annotations
@@ -16,32 +16,39 @@ import numpy as np
 
 from . import binding, build, inputs
 
-LAYER_STAGES = ["RMSNorm + QKV", "self-attention", "out-projection + residual", "RMSNorm + cross q", "cross-attention",
-                "cross out-projection + residual", "RMSNorm + gate/up + SiLU*mul", "down projection + residual"]
-
-
-def stage_names(cfg):
-    tail = ["LM head + head blocks"] + (["head output projections"] if cfg["n_draft"] else []) + ["verify / resample", "commit"]
-    return LAYER_STAGES, tail
+def stage_names(cfg, n_stages: int):
+    """Names of a layer's stages and of the tail's.  A layer has seven stages where the cross-attention projects its own
+    queries, else eight."""
+    tail = ["LM head" + (" + head blocks" if cfg["n_draft"] else "")]
+    if cfg["n_draft"] and cfg.get("head_kind", 0) == 1:
+        tail += ["heads' cross-attention", "heads' out-projection"]
+    if cfg["n_draft"]:
+        tail.append("head output projections")
+    tail.append("verify / resample / commit / embed")
+    cross = ["RMSNorm + cross q + cross-attention"]
+    if n_stages - len(tail) == 8 * cfg["n_layers"]:
+        cross = ["RMSNorm + cross q", "cross-attention"]
+    return (["RMSNorm + QKV", "self-attention", "out-projection + residual"] + cross +
+            ["cross out-projection + residual", "RMSNorm + gate/up + SiLU*mul", "down projection + residual"], tail)
 
 
 def table(cfg, t: np.ndarray) -> str:
     t = t.astype(np.int64)
     rows, G = t.shape
     L = cfg["n_layers"]
-    layer, tail = stage_names(cfg)
-    end_prev = t[0].copy()
+    layer, tail = stage_names(cfg, (rows - 1) // 2)
+    end_prev = t[0][t[0] > 0].max()
     acc: dict[str, list] = {}
     for p in range((rows - 1) // 2):
         a, e = t[1 + 2 * p], t[2 + 2 * p]
-        name = layer[p % 8] if p < 8 * L else tail[p - 8 * L]
-        has = a > 0
-        wait = (a[has] - end_prev[has]) if has.any() else np.zeros(1)
-        comp = (e[has] - a[has]) if has.any() else np.zeros(1)
-        acc.setdefault(name, []).append((e.max() - end_prev.max(), wait.mean(), comp.mean(), int(has.sum())))
-        end_prev = e
-    total = t[-1].max() - t[0].min()
-    out = [f"traced step: {total / 1e3:.1f} us, {G} CTAs", f"{'stage':34s} {'n':>3s} {'us each':>8s} {'share':>7s} {'wait in':>8s} {'compute':>8s} {'CTAs':>5s}"]
+        name = layer[p % len(layer)] if p < len(layer) * L else tail[p - len(layer) * L]
+        has = (a > 0) & (e > 0)
+        if not has.any():
+            continue
+        acc.setdefault(name, []).append((e.max() - end_prev, (a[has] - end_prev).mean(), (e[has] - a[has]).mean(), int(has.sum())))
+        end_prev = e.max()
+    total = end_prev - t[0][t[0] > 0].min()
+    out = [f"traced step: {total / 1e3:.1f} us (at most {G} CTAs of a stage are recorded)", f"{'stage':34s} {'n':>3s} {'us each':>8s} {'share':>7s} {'wait in':>8s} {'compute':>8s} {'CTAs':>5s}"]
     for k, v in acc.items():
         v = np.array(v, dtype=float)
         out.append(f"{k:34s} {len(v):3d} {v[:, 0].mean() / 1e3:8.2f} {100 * v[:, 0].sum() / total:6.1f}% {v[:, 1].mean() / 1e3:8.2f} {v[:, 2].mean() / 1e3:8.2f} {v[:, 3].mean():5.0f}")
