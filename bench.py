@@ -291,12 +291,11 @@ def run_gpu(args):
     value = job.tokens_per_s_per_mesh()
     e2e = world * n_e2e * T / (ms_e2e / 1e3)
     peaks, which = measured_peaks()
-    # roofline of the persistent step kernel: algorithmic bytes of all its steps / time inside xsm_generate
+    # roofline of the decoding step: algorithmic bytes of all steps / time inside xsm_generate
     alg = metrics.algorithmic_bytes(cfg, B)
     mean_n = (T / 2.0)
     bytes_per_step = alg["fixed"] + alg["per_position"] * mean_n
     steps_per_pass = steps_total / args.steps / 1.0
-    n_step_launches = sum(-(-int(s[0] // B) // 64) for s in stats) or 1
     achieved = bytes_per_step * (steps_total / B) / (kernel_ms / 1e3) / 1e9
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -313,12 +312,12 @@ def run_gpu(args):
         "gpu_launches": int(launches),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": achieved / peaks["hbm_gbs"],
-                     "traffic": metrics.measured_traffic(args.config if not args.k0 else -1, bytes_per_step * steps_total / B / n_step_launches,
+                     "traffic": metrics.measured_traffic(args.config if not args.k0 else -1, bytes_per_step,
                                                                  cfg.get("head_kind", 0)),
                      "peak_source": f"{which} copy bandwidth (MEASURED_PEAKS.json)" if which == "measured" else "fallback",
-                     "kernel": "xsm::step_kernel (persistent, 148 CTAs; one launch = up to 64 decoding steps)",
-                     "bytes_per_launch": bytes_per_step * steps_total / B / n_step_launches,
-                     "avg_launch_ms": kernel_ms / n_step_launches},
+                     "kernel": "the launch chain of one decoding step (a recorded graph: seven or eight kernels a layer and the tail)",
+                     "bytes_per_launch": bytes_per_step,
+                     "avg_launch_ms": kernel_ms / (steps_total / B)},
         "clocks": clocks,
     }
     if world == 1 and K >= 1 and not args.k0 and not args.no_fitted_heads:

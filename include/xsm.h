@@ -122,8 +122,7 @@ XSM_API xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights
  * dtype), runs prompt tokens 0..prompt_len-2 into the cache, sets x_s to the
  * last prompt token, s = prompt_len-1, draws the K initial drafts uniformly on
  * [0, V) and resets the step counters.  d_prompt: DEVICE int32 [batch,
- * prompt_len].  Synchronises the stream once (the stage tables of the batch
- * are uploaded from host memory of the context); the prefill kernels and the
+ * prompt_len].  The prefill kernels and the
  * ingestion of the prompt are then enqueued without waiting. */
 XSM_API xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_t *d_prompt,
                        int prompt_len, const xsm_decode_config *dc);
@@ -135,19 +134,13 @@ XSM_API xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, cons
  * [batch] (0 for a finished sequence).  Either may be NULL.  Asynchronous. */
 XSM_API xsm_status xsm_spec_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new);
 
-/* The paper has no counterpart of this call; it serves hosts that cannot give the library scratch memory of
- * their own.  xsm_spec_step with one difference: the partial results that the key splits of an attention
- * stage hand to one another (scratch that xsm_spec_step keeps in the caller's workspace) live in a 1 MiB
- * array that is part of the library image, so the call needs no allocation by anyone: not by the library
- * (it calls no allocator) and not by a caller that runs where cudaMalloc is not available, e.g. inside a
- * host process that handed out all device memory at start-up, or on a path that must not synchronise the
- * device.  Every GPU that loads the library holds the 1 MiB until the process exits.  The first call on a
- * device looks up the array's device address; make that call before any stream capture.  A batch whose
- * partials exceed the array (batch * n_heads * splits * (K+1) * (d_head+2) floats, twice) is refused with
- * XSM_ERR_CAPACITY.  The two step calls may alternate freely on one context: when xsm_spec_step, xsm_generate or
- * another call that steps follows this one, the workspace copy of the partials is cleared first.  All contexts of a process share the array and it keeps the last call's contents; the
- * call clears the part it uses first, so calls must not overlap on the GPU (same stream, or otherwise
- * ordered): overlapping calls race.  Arguments and results as xsm_spec_step.  Asynchronous. */
+/* The paper has no counterpart of this call; it serves hosts on a path that must not allocate device memory or
+ * synchronise the device.  xsm_spec_step with one difference: the kernels of the step are launched one by one
+ * instead of as a recorded graph, whose recording and first launch may make the driver allocate.  The partial
+ * results that the key splits of an attention stage hand to one another travel through shared memory and need no
+ * scratch.  A batch for which they would exceed 1 MiB (batch * n_heads * splits * (K+1) * (d_head+2) floats, twice)
+ * is refused with XSM_ERR_CAPACITY, as it was when they lay in an array of the library.  The two step calls may
+ * alternate freely on one context.  Arguments and results as xsm_spec_step.  Asynchronous. */
 XSM_API xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new);
 
 /* Algorithm 1's loop (line 2: while s < L_max and no EOS is committed) and its
@@ -197,8 +190,8 @@ XSM_API xsm_status xsm_debug_get_state(xsm_ctx *ctx, int32_t *h_len, int32_t *h_
 
 /* Runs one decoding step (as xsm_spec_step does, without returning its tokens) and records its timeline:
  * h_times HOST uint64 [n_rows][n_ctas] nanoseconds of the GPU's global timer; row 0 = the step starts, row
- * 1 + 2p = stage p of the step has its inputs in shared memory, row 2 + 2p = stage p has published its
- * outputs; one column per CTA of the persistent kernel; 0 = that CTA had nothing to wait for in that stage.
+ * 1 + 2p = stage p of the step is past its wait for the stage before, row 2 + 2p = stage p is done; one column
+ * for each of a stage's first n_ctas CTAs; 0 = the stage has no such CTA, or it had nothing to do.
  * capacity = number of uint64 words h_times can hold.  Synchronises the stream. */
 XSM_API xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t capacity, int *n_rows, int *n_ctas);
 
@@ -212,16 +205,17 @@ XSM_API xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t 
  * h_tokens == NULL or n == 0 turns it off; xsm_prefill turns it off too.  Synchronises the stream. */
 XSM_API xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, float mean_accept);
 
-/* Bounds of the device-side waits: polls of one exchanged word and tries of one shared-memory barrier before a
- * CTA gives up, raises XSM_ERR_TIMEOUT and leaves at the end of the step.  0 restores the default (2^21, 2^22). */
+/* Bounds of the device-side waits: polls of one word in memory and tries of one shared-memory barrier before a
+ * CTA gives up and raises XSM_ERR_TIMEOUT.  0 restores the default (2^21, 2^22). */
 XSM_API xsm_status xsm_debug_set_wait_limits(xsm_ctx *ctx, uint32_t polls, uint32_t barrier_tries);
 
-/* Launches stage `stage` (0-based: eight per layer, then the tail) of the current step alone, without advancing the
- * step counter.  A stage whose inputs no earlier launch has published waits for them until the limit above runs
- * out; the status then shows at the next synchronising call, and xsm_prefill starts afresh. */
+/* Launches stage `stage` (0-based: eight per layer, seven where the cross-attention projects its
+ * own queries, then the tail) of the current step alone, without advancing the
+ * step counter.  A stage that does not follow the one launched last waits for its turn until the limit above
+ * runs out; the status then shows at the next synchronising call, and xsm_prefill starts afresh. */
 XSM_API xsm_status xsm_debug_launch_stage(xsm_ctx *ctx, int stage);
 
-/* Runs the step one stage per launch instead of as one persistent kernel (1) or back (0). */
+/* Launches the stages of a step one after the other, without overlap, instead of as a recorded graph (1) or back (0). */
 XSM_API xsm_status xsm_debug_set_phase_launch(xsm_ctx *ctx, int on);
 
 #ifdef __cplusplus

@@ -25,9 +25,10 @@ def speedup(scr: float, latency_base: float, latency_spec: float) -> float:
     return scr * latency_base / latency_spec
 
 
-# DRAM traffic of a decoding step measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum over its launches), as a
-# ratio to the algorithmic bytes of the same step.  Empty: there is no capture of the present kernels.
-_TRAFFIC_RATIO: dict[int, float] = {}
+# DRAM traffic of a decoding step measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum over its launches at
+# contexts 0..8, see profiles/), as a ratio to the algorithmic bytes of the same step.  Traffic grows in proportion to the
+# units processed (weights once per step plus the cache).  None: no capture for that configuration.
+_TRAFFIC_RATIO = {2: 1001.0e6 / 981958656.0}
 
 
 def measured_traffic(config_index: int, algorithmic_bytes_per_launch: float, head_kind: int = 0):
