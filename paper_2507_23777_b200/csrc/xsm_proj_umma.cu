@@ -27,8 +27,10 @@ constexpr int kABytes = 128 * kBlockK * 2;         // weight block
 
 struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate), group 1 (or up)
 
-template <int EPI0, int EPI1>
-__global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
+// CL: a tile's columns are cut over a cluster.  Without it 64 registers a thread, so that two CTAs share an SM; with it 64 cost
+// 1 to 2 % of a step.
+template <int EPI0, int EPI1, bool CL>
+__global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
     extern __shared__ char smem_raw[];
     char *const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);      // (swizzled tiles: 1024-byte boundaries)
     __shared__ __align__(8) uint64_t bars[4 * kProjRing + 1];      // A full, A empty, B full, B empty, done
@@ -38,7 +40,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     __shared__ RowInfo s_row[kTokenTile];
     constexpr bool TWO = EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int S = A.S, rank = S > 1 ? (int)cluster_rank() : 0, Mp = A.Mp;
+    const int S = CL ? A.S : 1, rank = CL ? (int)cluster_rank() : 0, Mp = A.Mp;
     // sequences that still run: looked at just before the wait, when the weights are on their way
     const int active = A.pos0 < 0 && !A.late_go ? __ldcg(D.n_active) : 1;
     // a tile of weight rows and a tile of token rows: neighbours share the weights
@@ -60,7 +62,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
     const uint32_t b_bytes = (uint32_t)(2 * Nt) * kBlockK * 2u, b_pitch = (uint32_t)(2 * A.tok) * kBlockK * 2u;
     // operand rings; behind them (one CTA to a tile: in their place, when the products are done) the partial sums
-    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = S > 1 ? sb + (uint32_t)nb * b_pitch : sa;
+    const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = CL ? sb + (uint32_t)nb * b_pitch : sa;
     float *recv = reinterpret_cast<float *>(smem + (srecv - sa));
     auto bar = [&](int kind, int i) { return smem_u32(&bars[kind * kProjRing + i]); };
     const uint32_t done = smem_u32(&bars[4 * kProjRing]);
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         mbar_init(done, 1u);
         mbar_init(smem_u32(&recv_bar), 1u);
         mbar_init_fence();
-        if (S > 1 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
+        if (CL && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
     }
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
@@ -82,7 +84,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     // (the tensor memory is taken before the next kernel may start: kernels further down the chain can then never hold
     // columns that this one still waits for)
     if (!A.late_go) chain_go();
-    if (S > 1) cluster_arrive();          // "this CTA runs": peers may write to its shared memory after cluster_wait
+    if (CL) cluster_arrive();          // "this CTA runs": peers may write to its shared memory after cluster_wait
     const void *wmap = grp == 1 ? &T.w1 : &T.w0;
     auto load_a = [&](int i, int slot) {
         const uint32_t dst = sa + (uint32_t)slot * kABytes, b = bar(0, slot);
@@ -124,13 +126,13 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int quad = 2 * c + q, owner = (quad * qinv) >> 16, place = rank * qps + quad - owner * qps;      // (quad / qps: both are below 33)
-            dst[q] = S > 1 ? map_rank(srecv + (uint32_t)(place * 128 + arow) * 16u, (uint32_t)min(owner, S - 1)) : (uint32_t)(quad * 128 + arow) * 16u;
-            dst_bar[q] = S > 1 ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;
+            dst[q] = CL ? map_rank(srecv + (uint32_t)(place * 128 + arow) * 16u, (uint32_t)min(owner, S - 1)) : (uint32_t)(quad * 128 + arow) * 16u;
+            dst_bar[q] = CL ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;
         }
     };
     where(c0);
     settle(dst[0]); settle(dst[1]); settle(dst_bar[0]); settle(dst_bar[1]);
-    if (S > 1) cluster_wait();            // the peers run: their barriers and shared memory are there
+    if (CL) cluster_wait();            // the peers run: their barriers and shared memory are there
     if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kProjThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (active == 0) {      // every sequence has ended in an earlier step
@@ -198,14 +200,16 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             if (EPI0 == PE_QKV) *reinterpret_cast<int4 *>(&s_row[i]) = __ldcg(reinterpret_cast<const int4 *>(D.row_info + mb + m));
         }
     }
-    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row, four at a
-    // time; what it reads from memory is requested before the products are waited for, or a round ahead.
+    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row in groups
+    // of four, which lie side by side in shared memory (one 16-byte load for each sender; four single ones met four-way bank
+    // conflicts, half of an epilogue's time at 80 token rows); what it reads from memory is requested before the products
+    // are waited for, or a round ahead.
     float hn[4];
     float2 csn[4];
-    auto request = [&](int i0) {
+    auto request = [&](int quad) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int i = i0 + q * SIDES;
+            const int i = 4 * quad + q;
             if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(mb + m0 + i) * D.d + u_row);
             if (EPI0 == PE_QKV && i < nm) csn[q] = __ldcg(D.row_cs + (size_t)(mb + m0 + i) * half + (e < half ? e : e - half));
         }
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
                 float f[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
-                if (S == 1) *reinterpret_cast<float4 *>(smem + (srecv - sa) + dst[q]) = make_float4(f[0], f[1], f[2], f[3]);
+                if (!CL) *reinterpret_cast<float4 *>(smem + (srecv - sa) + dst[q]) = make_float4(f[0], f[1], f[2], f[3]);
                 else if (done_ok) st_async_v4(dst[q], f, dst_bar[q]);      // (a peer that gave up waiting may have left)
             }
         }
@@ -235,15 +239,19 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     tcgen05_before_sync();
     // One CTA to a tile: a barrier.  In a cluster every CTA waits for all shares of its rows, its own among them, so none leaves
     // before what is sent to it has come: no barrier at the end, whose wait for all stores took 1600 to 2400 cycles.
-    if (S == 1) __syncthreads();
+    if (!CL) __syncthreads();
     else if (nm > 0 && !mbar_wait(recv_b, 0u, D.mbar_limit, D.status)) mbar_wait(recv_b, 0u, D.mbar_limit, D.status);
     __syncwarp();
     // sums over the cluster in rank order, epilogue
-    auto total = [&](int i, int r) {
-        const float *p = recv + (size_t)((i >> 2) * 128 + r) * 4 + (i & 3);
-        float v = p[0];
-        for (int s = 1; s < S; ++s) v += p[s * qps * 512];
-        return v;
+    auto total = [&](int quad, int r, float (&v)[4]) {
+        const float4 *p = reinterpret_cast<const float4 *>(recv) + quad * 128 + r;
+        constexpr int kMost = CL ? 8 : 1;
+        float4 part[kMost];
+#pragma unroll
+        for (int s = 0; s < kMost; ++s) part[s] = s < S ? p[s * qps * 128] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 1; s < kMost; ++s) { part[0].x += part[s].x; part[0].y += part[s].y; part[0].z += part[s].z; part[0].w += part[s].w; }
+        v[0] = part[0].x; v[1] = part[0].y; v[2] = part[0].z; v[3] = part[0].w;
     };
     auto put_x = [&](int m, float v) {
         bf16 hi, lo;
@@ -258,17 +266,21 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
         qrow[(size_t)m * D.d] = hi;
         qrow[(size_t)(A.qp + m) * D.d] = lo;
     };
-    for (int i0 = side; i0 < nm; i0 += 4 * SIDES) {
+    for (int quad = side; 4 * quad < nm; quad += SIDES) {
         float h[4];
         float2 cs[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
-        request(i0 + 4 * SIDES);
+        request(quad + SIDES);
+        float sum[4], other[4];      // other: the rotation partner's, or up's
+        total(quad, row, sum);
+        if (TWO) total(quad, row + 64, other);
+        if (EPI0 == PE_QKV) total(quad, e < half ? row + half : row - half, other);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int i = i0 + q * SIDES, m = m0 + i;
+            const int i = 4 * quad + q, m = m0 + i;
             if (i >= nm) break;
-            const float v = total(i, row);
+            const float v = sum[q];
             if (EPI0 == PE_ADD) {
                 const float o = live_row ? h[q] + v : 0.f;
                 if (live_row) {
@@ -280,11 +292,11 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
             } else if (live_row) {
                 const float inv = s_inv[i], x1 = v * inv;
                 if (EPI0 == PE_QKV) {
-                    const float x2 = total(i, e < half ? row + half : row - half) * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
+                    const float x2 = other[q] * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
                     if (sec == 0) put_q(m, o);
                     else if (s_row[i].place >= 0) crow[s_row[i].place + (((e >> 3) ^ row_swz(s_row[i].rp, D.dh)) << 3)] = from_f<__half>(o);
                 } else if (TWO) {
-                    put_x(m, silu_f(x1) * (total(i, row + 64) * inv));
+                    put_x(m, silu_f(x1) * (other[q] * inv));
                 } else if (EPI0 == PE_QUERY || (EPI1 == PE_QUERY && grp == 1)) {
                     put_q(m, x1);
                 } else if (EPI0 == PE_HEADADD) {
@@ -311,9 +323,9 @@ __global__ void __launch_bounds__(kProjThreads) proj_umma_kernel(const Dev D, co
     }
 }
 
-template <int EPI0, int EPI1>
+template <int EPI0, int EPI1, bool CL>
 static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
-    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1>;
+    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL>;
     cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
@@ -326,7 +338,7 @@ int resident_clusters(int size) {
     int dev = 0;
     if (size < 2 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
     if (const int k = known[dev][size].load()) return k - 1;
-    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1>;
+    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1, true>;
     constexpr int smem = 200 * 1024;
     int n = 0;
     cudaLaunchConfig_t c = {};
@@ -349,7 +361,7 @@ int resident_clusters(int size) {
 
 cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L) {
     const ProjMaps &T = *reinterpret_cast<const ProjMaps *>(maps);
-#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_instance<a, b>(D, A, T, smem, L)
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return A.S > 1 ? launch_instance<a, b, true>(D, A, T, smem, L) : launch_instance<a, b, false>(D, A, T, smem, L)
     XSM_EPI(PE_QKV, -1);
     XSM_EPI(PE_ADD, -1);
     XSM_EPI(PE_QUERY, -1);
