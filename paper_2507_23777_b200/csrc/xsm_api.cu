@@ -193,7 +193,7 @@ struct xsm_ctx {
     Chain chain;              // the kernels of a decoding step
     RunParams run;            // as in device memory
     int request;              // number of the latest xsm_prefill
-    int *pinned;              // [16] n_active and status; at 8: the last request of which every sequence has ended
+    int *pinned;              // [16] n_active and status; at 8: the last request that needs no more steps
     cudaEvent_t ev0, ev1, step_ev[2];
 };
 
@@ -476,7 +476,8 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     if (set != XSM_OK) return set;
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     // One step ahead of the device: the next is on its way while one runs, and the one too many at the end finds every
-    // sequence ended and does nothing.  Every step commits at least one token per live sequence.
+    // sequence ended and does nothing.  Every step commits at least one token per live sequence.  A step that finds the status
+    // word raised ends the loop too: the rest would be void, and each might wait out its limits again.
     volatile int *const done = ctx->pinned + 8;
     for (long long i = 0; i < (long long)max_new_tokens + 2 && *done != ctx->request; ++i) {
         xsm_status st = run_step(ctx);
@@ -489,7 +490,8 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
         XSM_CUDA(ctx, launch_export(D, max_new_tokens, d_tokens, d_lengths, ctx->stream));
         ctx->launches += 1;
     }
-    XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const xsm_status end = check_device_status(ctx);      // waits for the stream
+    if (end != XSM_OK) return end;
     float ms = 0.f;
     XSM_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
     if (host_stats) {

@@ -357,6 +357,8 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     chain_wait();
     trace_mark(D, 1 + 2 * stage);
     __syncthreads();
+    // (requested here and looked at in the end: nothing waits for it)
+    const int raised = slot == 0 && tid == kTailThreads - 1 ? __ldcg(D.status) : 0;
     const float *z = D.logits0 + (size_t)(b * K1 + slot) * V;
     int a = 0;
     if (K > 0) {
@@ -499,6 +501,8 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     if (slot == 0 && tid >= kTailThreads - 32 && tid - (kTailThreads - 32) < K1)      // (the last warp: the embedding needs the first ones)
         place_row(D, b * K1 + tid - (kTailThreads - 32), b, new_len + tid - (kTailThreads - 32), !sh.state[5]);
     if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], new_len + slot, sh.red);
+    // a wait of this request ran out, or its pages: more steps are of no use (the host reads the status word itself)
+    if (raised != 0) *reinterpret_cast<volatile int *>(D.host_done) = R.request;
     if (K > 0) cluster_wait();           // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }

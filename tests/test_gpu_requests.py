@@ -1,0 +1,50 @@
+"""How a request ends and what its caller is told, on the hand-sized model."""
+import numpy as np
+import pytest
+
+from conftest import gpu_cfg
+from paper_2507_23777_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    import torch
+    assert torch.cuda.is_available(), "these tests need a B200"
+    from paper_2507_23777_b200 import binding, build
+    build.build()
+    return binding
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_generate_reports_a_wait_that_ran_out_and_launches_no_more_steps(binding, dtype):
+    """A single stage launched out of turn gives up after a shortened limit and raises the status word.  xsm_generate then
+    says XSM_ERR_TIMEOUT, after the two steps that it has on their way at a time and not after all of the sixty that the
+    request could take; so does every further call until the next prefill, which starts clean."""
+    cfg = gpu_cfg(dtype=dtype, n_draft=2, sigma=0.05, max_seq_len=128)
+    w = inputs.make_weights(cfg, random_gains=True)
+    cond = inputs.make_cond(cfg, 1)
+    dc = binding.decode_config(cfg)
+    ctx = binding.Context(cfg, w)
+    ctx.prefill(cond, [0], dc)
+    want, _, _ = ctx.generate(60)
+    ctx.prefill(cond, [0], dc)
+    before = ctx.xsm_kernel_launches()
+    ctx.xsm_spec_step()
+    step = ctx.xsm_kernel_launches() - before
+    ctx.xsm_debug_set_wait_limits(3000, 0)
+    ctx.xsm_debug_launch_stage(2)
+    ctx.xsm_debug_set_wait_limits(0, 0)
+    before = ctx.xsm_kernel_launches()
+    with pytest.raises(binding.XsmError) as e:
+        ctx.generate(60)
+    assert e.value.status == binding.XSM_ERR_TIMEOUT
+    assert ctx.xsm_kernel_launches() - before <= 3 * step
+    with pytest.raises(binding.XsmError) as e:
+        ctx.generate(60)
+    assert e.value.status == binding.XSM_ERR_TIMEOUT
+    toks, lens = np.zeros((1, 60), dtype=np.int32), np.zeros(1, dtype=np.int32)
+    ctx.xsm_generate_host(ctx.cond_to_host(cond), np.zeros((1, 1), dtype=np.int32), dc, 60, toks, lens)
+    assert lens[0] == 60 and np.array_equal(toks, want)
+    ctx.xsm_destroy()
