@@ -192,8 +192,8 @@ struct xsm_ctx {
     std::string err;
     Chain chain;              // the kernels of a decoding step
     RunParams run;            // as in device memory
-    int request;              // number of the latest xsm_prefill
-    int *pinned;              // [16] n_active and status; at 8: the last request that needs no more steps
+    int generate_call;        // number of the latest xsm_generate
+    int *pinned;              // [16] n_active and status; at 8: the last xsm_generate that needs no more steps
     cudaEvent_t ev0, ev1, step_ev[2];
 };
 
@@ -290,7 +290,7 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     ctx->weights = (const char *)d_weights;
     ctx->ws = (char *)d_workspace;
     ctx->stream = (cudaStream_t)cuda_stream;
-    ctx->phase_launch = 0; ctx->prefilled = 0; ctx->launches = 0; ctx->request = 0; ctx->n_stages = 0;
+    ctx->phase_launch = 0; ctx->prefilled = 0; ctx->launches = 0; ctx->generate_call = 0; ctx->n_stages = 0;
     memset(&ctx->run, 0, sizeof(ctx->run));
     ctx->pinned = nullptr; ctx->ev0 = ctx->ev1 = ctx->step_ev[0] = ctx->step_ev[1] = nullptr;
     auto bail = [&](cudaError_t e, const char *what) {
@@ -412,7 +412,6 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     r.sample_mode = dc->sample_mode; r.k_sample = dc->k_sample; r.temperature = dc->temperature;
     r.key0 = (uint32_t)dc->seed; r.key1 = (uint32_t)(dc->seed >> 32);
     r.max_new = INT_MAX; r.prompt_len = prompt_len;
-    r.request = ++ctx->request;
     if ((const void *)d_prompt != (const void *)D.prompt)
         XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
     XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
@@ -472,14 +471,18 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     if (max_new_tokens < 1 || max_new_tokens > ctx->cfg.max_seq_len)
         return fail(ctx, XSM_ERR_INVALID_ARG, "max_new_tokens must be in [1, max_seq_len]");
     Dev &D = ctx->dev;
-    xsm_status set = set_max_new(ctx, max_new_tokens);
-    if (set != XSM_OK) return set;
+    // Stored anew by every call, under a number of its own: a prefill that the caller has captured begins the same request
+    // whenever it is replayed, without this code's knowledge.
+    const int call = ++ctx->generate_call;
+    XSM_CUDA(ctx, launch_set_limit(D, max_new_tokens, call, ctx->stream));
+    ctx->launches += 1;
+    ctx->run.max_new = max_new_tokens;
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     // One step ahead of the device: the next is on its way while one runs, and the one too many at the end finds every
     // sequence ended and does nothing.  Every step commits at least one token per live sequence.  A step that finds the status
     // word raised ends the loop too: the rest would be void, and each might wait out its limits again.
     volatile int *const done = ctx->pinned + 8;
-    for (long long i = 0; i < (long long)max_new_tokens + 2 && *done != ctx->request; ++i) {
+    for (long long i = 0; i < (long long)max_new_tokens + 2 && *done != call; ++i) {
         xsm_status st = run_step(ctx);
         if (st != XSM_OK) return st;
         XSM_CUDA(ctx, cudaEventRecord(ctx->step_ev[i & 1], ctx->stream));

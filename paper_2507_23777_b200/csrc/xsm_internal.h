@@ -19,7 +19,7 @@ struct RunParams {
     float delta, temperature;
     uint32_t key0, key1;
     int max_new, prompt_len;
-    int request;                   // number of the request: what the host is told when it needs no more steps
+    int call;                      // number of the xsm_generate that runs: what the host is told when it needs no more steps
     // scripted drafts (load generator of the benchmark): null, or [B][script_n] tokens by absolute position; the commit
     // then drafts script tokens, of which the first floor((t+1) a) - floor(t a) are left intact at step t (a = script_acc / 1024)
     const int *script;
@@ -52,7 +52,7 @@ struct Dev {
     int *tok_log, *step_tokens, *step_n_new;
     const int *prompt;
     RunParams *rp;
-    int *host_done;                // host memory: the last request that needs no more steps (every sequence has ended, or the status word is raised)
+    int *host_done;                // host memory: the last xsm_generate that needs no more steps (every sequence has ended, or the status word is raised)
     int *stage_word;               // single stages (inspection): stages of the current step that have run
     // activations: bf16 models as hi and lo planes of Mp rows (layout: xsm_proj.cuh), queries fp16 [2][Mp][d]; fp32 models
     // [row][column]

@@ -485,9 +485,9 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
             D.steps[b] += 1ull;
             if (fin) {
                 __stcg(D.finished + b, 1);
-                if (atomicSub(D.n_active, 1) == 1) {      // the last one: tell the host which request is done
+                if (atomicSub(D.n_active, 1) == 1) {      // the last one: tell the host that its call is done
                     __threadfence_system();
-                    *reinterpret_cast<volatile int *>(D.host_done) = R.request;
+                    *reinterpret_cast<volatile int *>(D.host_done) = R.call;
                 }
             } else {
                 reserve_pages(D, b, len, sh.state[3]);
@@ -502,7 +502,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
         place_row(D, b * K1 + tid - (kTailThreads - 32), b, new_len + tid - (kTailThreads - 32), !sh.state[5]);
     if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], new_len + slot, sh.red);
     // a wait of this request ran out, or its pages: more steps are of no use (the host reads the status word itself)
-    if (raised != 0) *reinterpret_cast<volatile int *>(D.host_done) = R.request;
+    if (raised != 0) *reinterpret_cast<volatile int *>(D.host_done) = R.call;
     if (K > 0) cluster_wait();           // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }
@@ -557,6 +557,16 @@ cudaError_t launch_stage_gate(const Dev &D, int stage, cudaStream_t st) {
 }
 cudaError_t launch_stage_mark(const Dev &D, int done, cudaStream_t st) {
     stage_mark_kernel<<<1, 1, 0, st>>>(D, done);
+    return cudaGetLastError();
+}
+// The token limit of the steps that follow and the call that they are for, which is told at once if it needs none.
+__global__ void set_limit_kernel(const Dev D, int max_new, int call) {
+    D.rp->max_new = max_new;
+    D.rp->call = call;
+    if (*D.n_active == 0 || *D.status != 0) *reinterpret_cast<volatile int *>(D.host_done) = call;
+}
+cudaError_t launch_set_limit(const Dev &D, int max_new, int call, cudaStream_t st) {
+    set_limit_kernel<<<1, 1, 0, st>>>(D, max_new, call);
     return cudaGetLastError();
 }
 cudaError_t launch_set_run(const Dev &D, const RunParams &R, cudaStream_t st) {

@@ -48,3 +48,47 @@ def test_generate_reports_a_wait_that_ran_out_and_launches_no_more_steps(binding
     ctx.xsm_generate_host(ctx.cond_to_host(cond), np.zeros((1, 1), dtype=np.int32), dc, 60, toks, lens)
     assert lens[0] == 60 and np.array_equal(toks, want)
     ctx.xsm_destroy()
+
+
+def capture(ctx, stream, calls):
+    """The kernels that `calls` enqueues on the context's stream, as a graph; they do not run."""
+    import torch
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        calls()
+    return g
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_a_captured_prefill_begins_a_request_at_every_replay(binding, dtype):
+    """A caller captures its prefill and the first steps and replays the graph for one request after another, each of which
+    xsm_generate finishes: the same tokens, lengths and counts every time.  A prefill and a request in between that are not
+    captured change nothing."""
+    import torch
+    cfg = gpu_cfg(dtype=dtype, n_draft=2, sigma=0.05)
+    w = inputs.make_weights(cfg, random_gains=True)
+    cond = inputs.make_cond(cfg, 2)
+    dc = binding.decode_config(cfg)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = binding.Context(cfg, w, max_batch=2)
+        d_cond = ctx.cond_to_device(cond)
+        d_prompt = torch.tensor([[0, 7, 9], [0, 3, 4]], dtype=torch.int32, device="cuda")
+
+        def begin():
+            ctx.xsm_prefill(d_cond, d_prompt, 3, dc)
+            ctx.xsm_spec_step()
+            ctx.xsm_spec_step()
+
+        begin()
+        want, _, want_st = ctx.generate(24)
+        g = capture(ctx, stream, begin)
+        for i in range(4):
+            if i == 2:
+                begin()
+                ctx.generate(12)
+            g.replay()
+            toks, lens, st = ctx.generate(24)
+            assert (lens == 24).all() and np.array_equal(toks, want), f"replay {i}"
+            assert st.tokens == 48 and st.steps == want_st.steps, f"replay {i}"
+        ctx.xsm_destroy()
