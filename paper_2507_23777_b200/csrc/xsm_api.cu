@@ -191,7 +191,7 @@ struct xsm_ctx {
     unsigned long long launches;
     std::string err;
     Chain chain;              // the kernels of a decoding step
-    RunParams run;            // as in device memory
+    bool limited;             // the token limit of an xsm_generate may be in device memory
     int generate_call;        // number of the latest xsm_generate
     int *pinned;              // [16] n_active and status; at 8: the last xsm_generate that needs no more steps
     cudaEvent_t ev0, ev1, step_ev[2];
@@ -235,18 +235,23 @@ xsm_status run_step(xsm_ctx *ctx, bool may_record = true) {
     return XSM_OK;
 }
 
-// the request's parameters in device memory, if they are not there already
-xsm_status set_run(xsm_ctx *ctx, const RunParams &r) {
-    if (memcmp(&r, &ctx->run, sizeof(r)) == 0) return XSM_OK;
-    ctx->run = r;
-    XSM_CUDA(ctx, launch_set_run(ctx->dev, r, ctx->stream));
-    ctx->launches += 1;
+// does the stream record into a graph of the caller's, so that what is launched does not run now, but at every replay?
+xsm_status is_captured(xsm_ctx *ctx, bool *yes) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    XSM_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &cs));
+    *yes = cs != cudaStreamCaptureStatusNone;
     return XSM_OK;
 }
-xsm_status set_max_new(xsm_ctx *ctx, int max_new) {
-    RunParams r = ctx->run;
-    r.max_new = max_new;
-    return set_run(ctx, r);
+// A step on its own has no token limit: one that xsm_generate has stored is taken back, unless xsm_prefill has done so.  A
+// captured step takes it back at every replay, since nothing is known of what will have run before.
+xsm_status lift_limit(xsm_ctx *ctx) {
+    bool captured = false;
+    const xsm_status st = is_captured(ctx, &captured);
+    if (st != XSM_OK || (!captured && !ctx->limited)) return st;
+    XSM_CUDA(ctx, launch_set_limit(ctx->dev, INT_MAX, 0, ctx->stream));
+    ctx->launches += 1;
+    if (!captured) ctx->limited = false;
+    return XSM_OK;
 }
 // the tokens committed by the latest step -> the caller
 xsm_status copy_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
@@ -291,7 +296,7 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     ctx->ws = (char *)d_workspace;
     ctx->stream = (cudaStream_t)cuda_stream;
     ctx->phase_launch = 0; ctx->prefilled = 0; ctx->launches = 0; ctx->generate_call = 0; ctx->n_stages = 0;
-    memset(&ctx->run, 0, sizeof(ctx->run));
+    ctx->limited = true;
     ctx->pinned = nullptr; ctx->ev0 = ctx->ev1 = ctx->step_ev[0] = ctx->step_ev[1] = nullptr;
     auto bail = [&](cudaError_t e, const char *what) {
         g_create_error = std::string(what) + ": " + cudaGetErrorString(e);
@@ -401,12 +406,15 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     }
     if ((long long)batch * ctx->lay.max_blocks > ctx->lay.n_pages)
         return fail(ctx, XSM_ERR_CAPACITY, "the page pool cannot hold `batch` sequences of max_seq_len positions");
+    bool captured = false;
+    const xsm_status capture = is_captured(ctx, &captured);
+    if (capture != XSM_OK) return capture;
     Dev &D = ctx->dev;
     if (c.dtype == 0 && batch * D.K1 > kF32Rows) return fail(ctx, XSM_ERR_CAPACITY, "fp32 models support at most 24 token rows per step");
     D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8;
     if (!ctx->chain.select(D)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
     ctx->n_stages = ctx->chain.n_ops();
-    RunParams &r = ctx->run;
+    RunParams r;
     memset(&r, 0, sizeof(r));
     r.verify_mode = dc->verify_mode; r.k_accept = dc->k_accept; r.delta = dc->delta;
     r.sample_mode = dc->sample_mode; r.k_sample = dc->k_sample; r.temperature = dc->temperature;
@@ -416,6 +424,7 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
         XSM_CUDA(ctx, cudaMemcpyAsync((void *)D.prompt, d_prompt, sizeof(int32_t) * batch * prompt_len, cudaMemcpyDeviceToDevice, ctx->stream));
     XSM_CUDA(ctx, launch_begin(D, r, ctx->stream));
     ctx->launches += 2;
+    if (!captured) ctx->limited = false;
     if (c.dtype == 1) {
         XSM_CUDA(ctx, ctx->chain.condition(D, d_cond, ctx->stream, &ctx->launches));
     } else {
@@ -437,7 +446,7 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
 xsm_status xsm_spec_step(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_n_new) {
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_spec_step before xsm_prefill");
-    xsm_status st = set_max_new(ctx, INT_MAX);
+    xsm_status st = lift_limit(ctx);
     if (st == XSM_OK) st = run_step(ctx);
     return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
@@ -460,7 +469,7 @@ xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_
         return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch need " +
                                                std::to_string(n_sets * half) + " bytes, the built-in scratch holds " +
                                                std::to_string(kStaticScratchBytes));
-    xsm_status st = set_max_new(ctx, INT_MAX);
+    xsm_status st = lift_limit(ctx);
     if (st == XSM_OK) st = run_step(ctx, false);
     return st == XSM_OK ? copy_step(ctx, d_new_tokens, d_n_new) : st;
 }
@@ -474,9 +483,9 @@ xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int
     // Stored anew by every call, under a number of its own: a prefill that the caller has captured begins the same request
     // whenever it is replayed, without this code's knowledge.
     const int call = ++ctx->generate_call;
+    ctx->limited = true;
     XSM_CUDA(ctx, launch_set_limit(D, max_new_tokens, call, ctx->stream));
     ctx->launches += 1;
-    ctx->run.max_new = max_new_tokens;
     XSM_CUDA(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
     // One step ahead of the device: the next is on its way while one runs, and the one too many at the end finds every
     // sequence ended and does nothing.  Every step commits at least one token per live sequence.  A step that finds the status
@@ -632,7 +641,7 @@ xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t capacity
     if (capacity < words) return fail(ctx, XSM_ERR_CAPACITY, "h_times is too small");
     unsigned long long *d_trace = at<unsigned long long>(ctx, ctx->lay.trace);
     XSM_CUDA(ctx, cudaMemsetAsync(d_trace, 0, 8 * words, ctx->stream));
-    xsm_status st = set_max_new(ctx, INT_MAX);
+    xsm_status st = lift_limit(ctx);
     if (st != XSM_OK) return st;
     ctx->dev.trace = d_trace;
     st = run_step(ctx);
@@ -650,10 +659,10 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     if (!ctx) return XSM_ERR_INVALID_ARG;
     if (!ctx->prefilled) return fail(ctx, XSM_ERR_STATE, "xsm_debug_set_script before xsm_prefill");
     Dev &D = ctx->dev;
-    RunParams r = ctx->run;
     if (h_tokens == nullptr || n <= 0) {
-        r.script = nullptr; r.script_n = r.script_acc = 0;
-        return set_run(ctx, r);
+        XSM_CUDA(ctx, launch_set_script(D, nullptr, 0, 0, ctx->stream));
+        ctx->launches += 1;
+        return XSM_OK;
     }
     if (n > ctx->lay.tok_ld) return fail(ctx, XSM_ERR_INVALID_ARG, "script longer than max_seq_len + n_draft + 1");
     if (!(mean_accept >= 0.f) || mean_accept > (float)D.K) return fail(ctx, XSM_ERR_INVALID_ARG, "mean_accept must be in [0, n_draft]");
@@ -662,8 +671,9 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     int *d_script = at<int>(ctx, ctx->lay.script);
     XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     XSM_CUDA(ctx, cudaMemcpy(d_script, h_tokens, sizeof(int32_t) * (size_t)D.B * n, cudaMemcpyHostToDevice));
-    r.script = d_script; r.script_n = n; r.script_acc = (int)lrintf(mean_accept * 1024.f);
-    return set_run(ctx, r);
+    XSM_CUDA(ctx, launch_set_script(D, d_script, n, (int)lrintf(mean_accept * 1024.f), ctx->stream));
+    ctx->launches += 1;
+    return XSM_OK;
 }
 
 xsm_status xsm_debug_set_wait_limits(xsm_ctx *ctx, uint32_t polls, uint32_t barrier_tries) {

@@ -139,7 +139,8 @@ cudaError_t launch_begin(const Dev &D, const RunParams &R, cudaStream_t st);
 // single stages (inspection): waits until the stages before `stage` have run one by one; notes that `done` of them have
 cudaError_t launch_stage_gate(const Dev &D, int stage, cudaStream_t st);
 cudaError_t launch_stage_mark(const Dev &D, int done, cudaStream_t st);
+// request parameters that change between prefills: the token limit and the xsm_generate it is for, scripted drafts
 cudaError_t launch_set_limit(const Dev &D, int max_new, int call, cudaStream_t st);
-cudaError_t launch_set_run(const Dev &D, const RunParams &R, cudaStream_t st);
+cudaError_t launch_set_script(const Dev &D, const int *script, int n, int acc, cudaStream_t st);
 
 }  // namespace xsm

@@ -518,7 +518,6 @@ cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L
 // --------------------------------------------------------------------------------- start of a request
 
 // Algorithm 1 line 1: the pool, the run's parameters, and per sequence s = prompt_len - 1, its pages, the first window.
-__global__ void set_run_kernel(const Dev D, const RunParams R) { *D.rp = R; }
 __global__ void begin_pool_kernel(const Dev D, const RunParams R) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < D.n_pages) D.free_stack[i] = D.n_pages - 1 - i;
@@ -569,8 +568,13 @@ cudaError_t launch_set_limit(const Dev &D, int max_new, int call, cudaStream_t s
     set_limit_kernel<<<1, 1, 0, st>>>(D, max_new, call);
     return cudaGetLastError();
 }
-cudaError_t launch_set_run(const Dev &D, const RunParams &R, cudaStream_t st) {
-    set_run_kernel<<<1, 1, 0, st>>>(D, R);
+__global__ void set_script_kernel(const Dev D, const int *script, int n, int acc) {
+    D.rp->script = script;
+    D.rp->script_n = n;
+    D.rp->script_acc = acc;
+}
+cudaError_t launch_set_script(const Dev &D, const int *script, int n, int acc, cudaStream_t st) {
+    set_script_kernel<<<1, 1, 0, st>>>(D, script, n, acc);
     return cudaGetLastError();
 }
 

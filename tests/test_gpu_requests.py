@@ -92,3 +92,46 @@ def test_a_captured_prefill_begins_a_request_at_every_replay(binding, dtype):
             assert (lens == 24).all() and np.array_equal(toks, want), f"replay {i}"
             assert st.tokens == 48 and st.steps == want_st.steps, f"replay {i}"
         ctx.xsm_destroy()
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_parameters_that_were_only_captured_count_as_not_stored(binding, dtype):
+    """Scripted drafts are switched off in a graph that has not run yet: the next direct call still has to switch them off.
+    The graph, replayed in a request with another seed, switches the script off and leaves the rest of the request's
+    parameters alone.  A captured step brings the store of its own limit, a direct one behind a prefill needs none."""
+    import torch
+    K, T = 3, 60
+    cfg = gpu_cfg(dtype=dtype, n_draft=K, sigma=0.3, max_seq_len=128, verify_mode=1, k_accept=2, sample_mode=1, k_sample=3, temperature=0.8)
+    w = inputs.make_weights(cfg, random_gains=True)
+    cond = inputs.make_cond(cfg, 1)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = binding.Context(cfg, w)
+        script = np.tile(np.arange(T + K + 2, dtype=np.int32) % cfg["vocab"], (1, 1))
+
+        def scripted(seed):
+            ctx.prefill(cond, [0], binding.decode_config(dict(cfg, seed=seed)))
+            ctx.xsm_debug_set_script(script, 1.0)
+
+        def run(seed):
+            ctx.prefill(cond, [0], binding.decode_config(dict(cfg, seed=seed)))
+            return ctx.generate(T)[0]
+
+        one, two = run(1), run(2)
+        assert not np.array_equal(one, two)
+        scripted(1)
+        assert not np.array_equal(ctx.generate(T)[0], one)      # (the token after a rejection is the script's)
+        scripted(1)
+        g = capture(ctx, stream, lambda: ctx.xsm_debug_set_script(None, 0.0))
+        ctx.xsm_debug_set_script(None, 0.0)
+        assert np.array_equal(ctx.generate(T)[0], one)
+        scripted(2)
+        g.replay()
+        assert np.array_equal(ctx.generate(T)[0], two)
+        ctx.prefill(cond, [0], binding.decode_config(cfg))
+        before = ctx.xsm_kernel_launches()
+        ctx.xsm_spec_step()
+        direct = ctx.xsm_kernel_launches() - before
+        capture(ctx, stream, ctx.xsm_spec_step)
+        assert ctx.xsm_kernel_launches() - before == 2 * direct + 1
+        ctx.xsm_destroy()
