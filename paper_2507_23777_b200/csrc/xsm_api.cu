@@ -610,7 +610,8 @@ xsm_status xsm_debug_set_drafts(xsm_ctx *ctx, const int32_t *h_drafts) {
     if (D.K == 0) return XSM_OK;
     for (int i = 0; i < D.B * D.K; ++i)
         if (h_drafts[i] < 0 || h_drafts[i] >= D.V) return fail(ctx, XSM_ERR_INVALID_ARG, "draft token out of range");
-    XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const xsm_status st = check_device_status(ctx);
+    if (st != XSM_OK) return st;
     XSM_CUDA(ctx, cudaMemcpy2D(D.window + 1, sizeof(int32_t) * D.K1, h_drafts, sizeof(int32_t) * D.K,
                                sizeof(int32_t) * D.K, D.B, cudaMemcpyHostToDevice));
     XSM_CUDA(ctx, launch_embed_rows(D, ctx->cfg.dtype, D.K1, -1, 0, ChainLaunch{ctx->stream, false, &ctx->launches}));
@@ -669,7 +670,8 @@ xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, fl
     for (long long i = 0; i < (long long)D.B * n; ++i)
         if (h_tokens[i] < 0 || h_tokens[i] >= D.V) return fail(ctx, XSM_ERR_INVALID_ARG, "script token out of range");
     int *d_script = at<int>(ctx, ctx->lay.script);
-    XSM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    const xsm_status st = check_device_status(ctx);
+    if (st != XSM_OK) return st;
     XSM_CUDA(ctx, cudaMemcpy(d_script, h_tokens, sizeof(int32_t) * (size_t)D.B * n, cudaMemcpyHostToDevice));
     XSM_CUDA(ctx, launch_set_script(D, d_script, n, (int)lrintf(mean_accept * 1024.f), ctx->stream));
     ctx->launches += 1;

@@ -21,7 +21,7 @@ def binding():
 def test_generate_reports_a_wait_that_ran_out_and_launches_no_more_steps(binding, dtype):
     """A single stage launched out of turn gives up after a shortened limit and raises the status word.  xsm_generate then
     says XSM_ERR_TIMEOUT, after the two steps that it has on their way at a time and not after all of the sixty that the
-    request could take; so does every further call until the next prefill, which starts clean."""
+    request could take; so does every further call that synchronises, until the next prefill, which starts clean."""
     cfg = gpu_cfg(dtype=dtype, n_draft=2, sigma=0.05, max_seq_len=128)
     w = inputs.make_weights(cfg, random_gains=True)
     cond = inputs.make_cond(cfg, 1)
@@ -41,9 +41,10 @@ def test_generate_reports_a_wait_that_ran_out_and_launches_no_more_steps(binding
         ctx.generate(60)
     assert e.value.status == binding.XSM_ERR_TIMEOUT
     assert ctx.xsm_kernel_launches() - before <= 3 * step
-    with pytest.raises(binding.XsmError) as e:
-        ctx.generate(60)
-    assert e.value.status == binding.XSM_ERR_TIMEOUT
+    for call in (lambda: ctx.generate(60), lambda: ctx.xsm_debug_set_drafts([[1, 2]]), lambda: ctx.xsm_debug_set_script([[1] * 8], 1.0)):
+        with pytest.raises(binding.XsmError) as e:
+            call()
+        assert e.value.status == binding.XSM_ERR_TIMEOUT
     toks, lens = np.zeros((1, 60), dtype=np.int32), np.zeros(1, dtype=np.int32)
     ctx.xsm_generate_host(ctx.cond_to_host(cond), np.zeros((1, 1), dtype=np.int32), dc, 60, toks, lens)
     assert lens[0] == 60 and np.array_equal(toks, want)
