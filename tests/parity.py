@@ -90,6 +90,14 @@ def assert_logits(gpu, ref, atol, rtol, what):
     assert ok.all(), f"{what} off by {float(np.abs(gpu - ref).max())} ({int((~ok).sum())} of {ok.size} beyond the bound)"
 
 
+def self_attention_ctas(ctx, heads):
+    """How many CTAs share the keys of one (sequence, head) in the first layer's self-attention: one more step is run and
+    its timeline counted (CTAs without keys leave no mark)."""
+    marks = int((ctx.xsm_debug_trace_step()[1 + 2 * 1] > 0).sum())
+    assert marks and marks % (ctx.batch * heads) == 0, (marks, ctx.batch, heads)
+    return marks // (ctx.batch * heads)
+
+
 class LockStep:
     def __init__(self, cfg, batch=1, random_gains=False, weights=None, phase_launch=False, workspace_bytes=None):
         self.cfg = dict(cfg)

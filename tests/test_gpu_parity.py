@@ -168,20 +168,23 @@ def test_config4_large_bf16_prefix(P):
 
 @pytest.mark.parametrize("shape", ["heads of 64", "heads of 128, batch 2"])
 def test_long_context_split_attention(P, shape):
-    """Contexts of many pages: self-attention is split over several CTAs per head and merged (6 and 4 splits
-    here), on two-layer models with the widths of configurations 2 and 4.  The oracle is teacher-forced through
+    """Contexts of many pages: the keys of a head are cut over the CTAs of a cluster and the partial results merged, a CTA
+    more for every 384 keys (192 in heads of 128), on two-layer models with the widths of configurations 2 and 4.  The
+    prompt ends where three CTAs share a head; a fourth joins while the steps run.  The oracle is teacher-forced through
     the whole run; logits and the cache are compared at the end, decisions at every step."""
+    steps = 60
     if shape == "heads of 64":
-        cfg, batch, steps = inputs.config(2, n_layers=2, max_seq_len=2048), 1, 300
+        cfg, batch, prompt = inputs.config(2, n_layers=2, max_seq_len=2048), 1, 1120
     else:
-        cfg, batch, steps = inputs.config(4, n_layers=2, d_ff=2048, max_seq_len=2048, n_draft=3, n_cond=70), 2, 260
+        cfg, batch, prompt = inputs.config(4, n_layers=2, d_ff=2048, max_seq_len=2048, n_draft=3, n_cond=70), 2, 545
     ls = P.LockStep(cfg, batch=batch)
-    ls.begin()
+    ls.begin([0] + [int(t) for t in np.random.default_rng(6).integers(1, cfg["vocab"], prompt)])
     for it in range(steps):
         ls.step(check_logits=it >= steps - 3, **BF16_TOL)
     st = ls.ctx.xsm_debug_get_state()
-    assert st["len"].min() >= steps and ls.excused <= max(3, batch * steps // 20)
+    assert st["len"].min() >= prompt + steps and ls.excused <= max(3, batch * steps // 20)
     ls.compare_cache(layers=[1], **BF16_TOL)
+    assert P.self_attention_ctas(ls.ctx, cfg["n_heads"]) == 4
     ls.close()
 
 
@@ -200,9 +203,9 @@ SHAPES = {
     "rows of 3 KB and 12 KB": (_shape(1536, 12, 128, 6144, 2), 2),
     "rows of 1280 and 3840 bytes": (_shape(640, 10, 64, 1920, 3), 1),
     "no heads, five sequences": (_shape(768, 12, 64, 3072, 0), 5),
-    "several tile groups per projection": (_shape(2048, 16, 128, 2048, 3, V=3000), 2),
-    "two attention items per CTA, pages owned by warps": (_shape(1024, 16, 64, 4096, 0), 16),
-    "two attention items per CTA, three token rows each": (_shape(512, 8, 64, 2048, 2, V=900), 24),
+    "eight token rows of two sequences, width 2048": (_shape(2048, 16, 128, 2048, 3, V=3000), 2),
+    "two attention CTAs to an SM, one token row each": (_shape(1024, 16, 64, 4096, 0), 16),
+    "two attention CTAs to an SM, three token rows each": (_shape(512, 8, 64, 2048, 2, V=900), 24),
     "eight token rows of one sequence (all eight query columns of the transposed attention unit)": (_shape(1024, 16, 64, 4096, 7), 1),
     "six token rows of one sequence, heads of 128": (_shape(1024, 8, 128, 2048, 5, V=1200), 1),
 }
@@ -210,8 +213,8 @@ SHAPES = {
 
 @pytest.mark.parametrize("shape", list(SHAPES))
 def test_shape_sweep_bf16(P, shape):
-    """Shapes between the five configurations: each makes the projections pick another tiling (rows per ring
-    item, tiles per group, token tiles, activation chunks).  Three steps, logits and cache against the oracle."""
+    """Shapes between the five configurations: each makes the projections pick another cut (rows and tiles of a CTA, passes
+    over the columns, mma.sync or tcgen05, CTAs of a cluster).  Three steps, logits and cache against the oracle."""
     ov, batch = SHAPES[shape]
     ls = P.LockStep(inputs.config(2, **ov), batch=batch)
     ls.begin()
@@ -222,9 +225,8 @@ def test_shape_sweep_bf16(P, shape):
 
 
 def test_long_prompt_many_pages_per_attention_split(P):
-    """64 heads leave two key splits per head, so at a context of 1100 tokens a split walks nine cache pages and a warp
-    owns more than one of them.  The prompt is ingested through the same step kernel; then logits, decisions and the
-    whole cache of the last layer are compared with the oracle."""
+    """64 heads leave two CTAs for each, so at a context of 1100 tokens a CTA has nine cache pages of two units each, more
+    units than its sixteen warps.  Logits, decisions and the whole cache of the last layer are compared with the oracle."""
     cfg = inputs.config(2, **_shape(2048, 64, 32, 2048, 4, max_seq_len=1400))
     cfg["max_seq_len"] = 1400
     ls = P.LockStep(cfg, batch=1)
@@ -234,6 +236,7 @@ def test_long_prompt_many_pages_per_attention_split(P):
     for _ in range(8):
         ls.step(**BF16_TOL)
     ls.compare_cache(layers=[1], **BF16_TOL)
+    assert P.self_attention_ctas(ls.ctx, cfg["n_heads"]) == 2
     ls.close()
 
 
@@ -360,24 +363,25 @@ def planted_chain(ls, b, n_good, rank=1):
     return win[1:]
 
 
-def test_twelve_key_splits_merge_in_two_batches(P):
-    """Twelve heads of 64 leave twelve key splits per head; at a context of about 3000 tokens the last split folds in
-    eleven partials, in two batches of up to eight.  The prompt is ingested by the step kernel."""
+def test_eight_key_splits(P):
+    """Twelve heads of 64 at a context of about 3000 tokens: the keys of a head are cut over a cluster of eight CTAs, the
+    most there are."""
     cfg = inputs.config(1, n_layers=2, vocab=1500, n_cond=40, max_seq_len=3200)
     ls = P.LockStep(cfg, batch=1)
     prompt = [0] + [int(t) for t in np.random.default_rng(11).integers(1, cfg["vocab"], 3010)]
     st = ls.begin(prompt)
-    assert st["len"][0] == len(prompt) - 1 and (-(-int(st["len"][0]) // 64) + 3) // 4 >= 12
+    assert st["len"][0] == len(prompt) - 1
     for _ in range(6):
         ls.step(**BF16_TOL)
     assert ls.excused <= 2
     ls.compare_cache(layers=[1], **BF16_TOL)
+    assert P.self_attention_ctas(ls.ctx, cfg["n_heads"]) == 8
     ls.close()
 
 
-def test_block_table_reload_after_32_pages_of_one_split(P):
-    """Sixteen heads and four sequences leave two key splits per item; with 32-token pages a context of about 2400
-    tokens gives each split 38 pages, so the producer fetches a second batch of block-table entries."""
+def test_pages_of_a_split_pass_through_the_ring_several_times(P):
+    """Sixteen heads and four sequences leave two CTAs for each; with 32-token pages a context of about 2400 tokens gives
+    each of them 38 pages, more than twice as many as its ring has places."""
     cfg = inputs.config(2, **_shape(512, 16, 32, 1024, 2, V=900, C=33, page_size=32, max_seq_len=2600))
     ls = P.LockStep(cfg, batch=4)
     prompt = [0] + [int(t) for t in np.random.default_rng(12).integers(1, cfg["vocab"], 2420)]
@@ -387,12 +391,13 @@ def test_block_table_reload_after_32_pages_of_one_split(P):
         ls.step(**BF16_TOL)
     assert ls.excused <= 4
     ls.compare_cache(layers=[1], **BF16_TOL)
+    assert P.self_attention_ctas(ls.ctx, cfg["n_heads"]) == 2
     ls.close()
 
 
 def test_context_of_twelve_thousand_tokens_at_the_width_of_configuration_2(P):
-    """The regime the benchmark ends in: 16 heads of 64, nine key splits per head, 21 pages per split (a warp owns
-    three of them).  One layer and a narrow feed-forward block keep the oracle's ingestion affordable."""
+    """The regime the benchmark ends in: 16 heads of 64, the keys of each cut over eight CTAs of 24 pages.  One layer and a
+    narrow feed-forward block keep the oracle's ingestion affordable."""
     cfg = inputs.config(2, n_layers=1, d_ff=1024, vocab=1500, n_cond=40, max_seq_len=12288)
     ls = P.LockStep(cfg, batch=1)
     prompt = [0] + [int(t) for t in np.random.default_rng(13).integers(1, cfg["vocab"], 12050)]
@@ -407,6 +412,7 @@ def test_context_of_twelve_thousand_tokens_at_the_width_of_configuration_2(P):
     ok = np.stack([ls.seqs[0].kv(0, 0, p) for p in range(n - 200, n)])
     ov = np.stack([ls.seqs[0].kv(0, 1, p) for p in range(n - 200, n)])
     assert P.logits_close(k, ok, **BF16_TOL).all() and P.logits_close(v, ov, **BF16_TOL).all()
+    assert P.self_attention_ctas(ls.ctx, cfg["n_heads"]) == 8
     ls.close()
 
 
@@ -463,9 +469,9 @@ def test_multi_token_commits_on_a_bf16_model(P, mode):
 
 
 def test_a_wait_that_runs_out_ends_the_kernel_cleanly_and_prefill_recovers(P):
-    """A stage is launched alone whose inputs no launch has published (the out-projection of layer 0, which reads the
-    attention rows), with the poll limit cut to a few thousand: every CTA gives up, finishes its ring protocol and
-    leaves; the host reports XSM_ERR_TIMEOUT at the next synchronising call; the context works again after xsm_prefill.
+    """A stage is launched alone although the stages before it have not run (the out-projection of layer 0), with the poll
+    limit cut to a few thousand: the kernel that waits for its turn gives up and raises the status word; the host reports
+    XSM_ERR_TIMEOUT at the next synchronising call; the context works again after xsm_prefill.
     Nothing here faults or hangs: the wait is a bounded loop of loads that ends by counting."""
     from paper_2507_23777_b200 import binding
     cfg = gpu_cfg(dtype=1, n_draft=2, sigma=0.05)
@@ -530,7 +536,7 @@ def test_cross_attention_heads_at_the_width_of_configuration_2(P):
 
 def test_cross_attention_heads_with_split_condition_keys(P):
     """Heads of 128 and 513 condition latents (configuration 4's width at reduced depth): the condition's keys of one
-    head exceed a CTA's ring, so the heads' attention is split over CTAs and merged, as the layers' is."""
+    head are cut over the CTAs of a cluster and merged, in the heads' attention as in the layers'."""
     cfg = inputs.config(4, n_layers=1, d_ff=2048, n_draft=2, head_kind=1, max_seq_len=256)
     ls = P.LockStep(cfg, batch=1)
     ls.begin()
