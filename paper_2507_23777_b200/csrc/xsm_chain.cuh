@@ -19,6 +19,7 @@ enum ProjEpilogue : int {
     PE_HEADADD = 6    // g + y as bf16 planes (cross-attention decoding head)
 };
 
+constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kTokenTile = 128;       // token rows that share a plane
 constexpr int kProjRing = 16;         // most operand blocks of one kind that a CTA keeps in shared memory
 

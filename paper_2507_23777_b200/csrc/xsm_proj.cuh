@@ -13,13 +13,5 @@ __device__ __forceinline__ size_t plane_off(int Mp, int m, int k) {
     return (size_t)(k >> 6) * (size_t)(128 * Mp) + (size_t)((m >> 3) * 1024 + (m & 7) * 64 + ((((k >> 3) & 7) ^ (m & 7)) << 3) + (k & 7));
 }
 constexpr int kLo = 512;           // elements from a hi part to its lo part
-// hi and lo of one value
-__device__ __forceinline__ void store_split(bf16 *x, int Mp, int m, int k, float v) {
-    bf16 hi, lo;
-    split_bf16(v, hi, lo);
-    bf16 *p = x + plane_off(Mp, m, k);
-    p[0] = hi;
-    p[kLo] = lo;
-}
 
 }  // namespace xsm
