@@ -149,7 +149,8 @@ XSM_API xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int
  * xsm_prefill, met EOS, or reached max_seq_len.  d_tokens: DEVICE int32
  * [batch, max_new_tokens] (x_1, x_2, ...; unused tail -1); d_lengths: DEVICE
  * int32 [batch].  host_stats (HOST, may be NULL) is filled before returning.
- * Synchronises the stream. */
+ * Synchronises the stream.  XSM_ERR_TIMEOUT where a device-side wait of the
+ * request ran out: the tokens are void, and xsm_prefill starts afresh. */
 XSM_API xsm_status xsm_generate(xsm_ctx *ctx, int max_new_tokens, int32_t *d_tokens, int32_t *d_lengths,
                         xsm_stats *host_stats);
 
@@ -170,7 +171,7 @@ XSM_API const char *xsm_last_error(const xsm_ctx *ctx);
 /* Number of kernels this context has launched so far. */
 XSM_API uint64_t xsm_kernel_launches(const xsm_ctx *ctx);
 
-/* ---- inspection, for tests and parity checks; all synchronise the stream ---- */
+/* ---- inspection, for tests and parity checks; what reads or replaces state synchronises the stream ---- */
 
 /* Logits of the last step: h_logits0 HOST float [batch, K+1, V] (Eq. 2 before the
  * softmax), h_head_logits HOST float [K, batch, K+1, V].  Either may be NULL. */
@@ -202,7 +203,7 @@ XSM_API xsm_status xsm_debug_trace_step(xsm_ctx *ctx, uint64_t *h_times, size_t 
  * script's too.  With a script that the backbone reproduces (its own greedy continuation under strict-greedy
  * verification) the accept length of every step is forced, and SCR = 1 + a; where the backbone's two best logits
  * nearly tie and it disagrees with the script, that one step accepts less and the run stays on the script.
- * h_tokens == NULL or n == 0 turns it off; xsm_prefill turns it off too.  Synchronises the stream. */
+ * h_tokens == NULL or n == 0 turns it off (without waiting); xsm_prefill turns it off too. */
 XSM_API xsm_status xsm_debug_set_script(xsm_ctx *ctx, const int32_t *h_tokens, int n, float mean_accept);
 
 /* Bounds of the device-side waits: polls of one word in memory and tries of one shared-memory barrier before a

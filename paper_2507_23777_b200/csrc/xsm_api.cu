@@ -466,8 +466,8 @@ xsm_status xsm_spec_step_static(xsm_ctx *ctx, int32_t *d_new_tokens, int32_t *d_
     const size_t half = (one + 255) / 256 * 256;
     const size_t n_sets = 2 + (D.head_kind == 1 ? (size_t)D.K : 0);
     if (n_sets * half > kStaticScratchBytes)
-        return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch need " +
-                                               std::to_string(n_sets * half) + " bytes, the built-in scratch holds " +
+        return fail(ctx, XSM_ERR_CAPACITY, "xsm_spec_step_static: the attention partials of this batch would need " +
+                                               std::to_string(n_sets * half) + " bytes of scratch, more than " +
                                                std::to_string(kStaticScratchBytes));
     xsm_status st = lift_limit(ctx);
     if (st == XSM_OK) st = run_step(ctx, false);

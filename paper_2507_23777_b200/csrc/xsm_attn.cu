@@ -1,17 +1,17 @@
 // Attention of bf16 models over the paged fp16 caches, as a kernel of the launch chain.
 //
-// Up to S CTAs serve one (sequence, head): they cut the keys by pages, a producer warp streams (page, head) tiles of
-// keys and values through a ring in shared memory, eight warps attend with mma.sync over 32 keys at a time (a unit).  How
-// many of the S take part depends on the context of the step (one up to 640 keys: a merge costs as much as four units);
-// they leave partial results in global memory and the last one to finish merges them, in the order of the keys.  (A
-// cluster that merges through distributed shared memory took 3 us longer: two cluster barriers with eight CTAs.)
+// A cluster of up to S CTAs serves one (sequence, head): they cut the keys by pages, a producer warp streams (page, head)
+// tiles of keys and values through a ring in shared memory, eight or sixteen warps attend with mma.sync over 32 keys at a
+// time (a unit).  How many of the S take part depends on the keys of the step (one CTA for every 384, 192 in heads of 128,
+// 128 where the rows form tiles: the rule and its figures stand at plan_attn).  Each of them finishes a share of the rows:
+// the others send it their partial results by counted stores into its shared memory, and it adds them up in rank order.
 // The keys and values of the rows themselves have been written to the cache by the projection before, so self-attention
 // is the same walk with a causal limit per row.  Pages that the step does not write (and the condition's) are fetched
 // before the kernel waits for its predecessor.
 //
 // Few rows (at most eight, every step of a batch of any size with up to seven heads): the product is transposed,
 // S^T = K Q^T and O^T = V^T P^T, so that the 16 keys of a product sit on its M side and the rows on its 8-wide N side;
-// all eight warps take different keys.  More rows (chunks of a prompt, many heads): tiles of 16 rows on the M side; the
+// all warps take different keys.  More rows (chunks of a prompt, many heads): tiles of 16 rows on the M side; the
 // warps are divided over the row tiles first and over the keys with what is left.
 #include "xsm_proj.cuh"
 
@@ -182,9 +182,11 @@ __device__ __forceinline__ void rows_unit(const unsigned (&qh)[DH / 16][4], cons
 __device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(reinterpret_cast<const unsigned *>(p)); }
 
 // QP (cross-attention of a step, few rows): the kernel projects the queries of its head itself, from the normalised residual
-// stream.  The head's rows of the projection lie in shared memory before the wait, so the stage costs what the products
-// cost (every warp multiplies all rows over its share of the columns, as in the projections over few token rows) instead of
-// a kernel of its own: 7.5 -> 5 us for both at width 1024.
+// stream (every warp multiplies all rows over its share of the columns, as in the projections over few token rows), instead
+// of a kernel of its own: 7.5 -> 5 us for both at width 1024.  The head's rows of the projection and the pages are requested
+// before the wait, but a CTA (544 threads of 96 registers) shares an SM with none of the out-projection before it (288 of 94
+// or 96).  Where that leaves SMs free, they have arrived when the wait is over; at width 1024 it holds 147 of 148, so all but
+// one of the sixteen CTAs of a sequence start when it ends, and fetch about 200 KB in full view: 4.4 to 4.9 us after the wait.
 constexpr int kQueryBlocks = 4;      // blocks of 32 columns per warp: d_model up to 1024
 //
 // NW: warps that attend, beside the producer.  A unit of 32 keys is some 300 dependent instructions, 1 us for a warp on its

@@ -126,11 +126,12 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
     // How a tile of weight rows is cut: its columns over a cluster of S CTAs, as many as fit into the GPCs at a time (of six CTAs
     // 22 clusters, of eight 15; a cluster more is a second wave).  More than 96 token rows in one plane: these into T parts too,
-    // each with the weights for itself, which leaves less to exchange and to finish in a CTA.  The stage's time after the wait
-    // in cycles, as measured, chooses among S and T: a product 47, or N / 2 where the token rows (hi and lo) bound it;
+    // each with the weights for itself, which leaves less to exchange and to finish in a CTA.  There the stage's time after the
+    // wait in cycles, as measured, chooses among S and T: a product 47, or N / 2 where the token rows (hi and lo) bound it;
     // activations, and weights that do not fit the ring, 59 bytes a cycle; 45 for every token row that is sent, 250 for every
-    // one that is finished.  125 rows of width 1024: 2079 -> 1834 us a step.  Below, the CTAs of more parts keep the next stage's
-    // weights out of shared memory for longer than they save: 90 rows of width 768 703 -> 716, 80 rows 1494 -> 1498, 40 rows 1221 -> 1273.
+    // one that is finished.  125 rows of width 1024: 2079 -> 1834 us a step.  Up to 96 rows T is 1 and the largest S that fits is
+    // taken, without weighing: the CTAs of more parts keep the next stage's weights out of shared memory for longer than they
+    // save (90 rows of width 768 703 -> 716, 80 rows 1494 -> 1498, 40 rows 1221 -> 1273).
     int S = 1, T = 1;
     const bool parts = A.tt == 1 && rows > 96;
     double best = 1e30;
@@ -248,7 +249,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     const int d = c.d_model, f = c.d_ff, V = c.vocab, K = c.n_draft, L = c.n_layers, rows = D.B * t;
     const int Mp = rows > kTokenTile ? kTokenTile : (rows + 7) / 8 * 8, tt = (rows + kTokenTile - 1) / kTokenTile, qp = tt * Mp;
     const bool ca = c.head_kind == 1;
-    const float qscale = D.scale * 1.4426950408889634f;      // softmax in base 2
+    const float qscale = D.scale * kLog2e;      // softmax in base 2
     const size_t es = c.dtype == 1 ? 2 : 4;
     auto gain = [&](size_t off) { return (const void *)(weights_ + off * es); };
     const size_t head_stride = K > 1 ? w_.Wout[1] - w_.Wout[0] : 0;

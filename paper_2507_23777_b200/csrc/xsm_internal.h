@@ -6,7 +6,7 @@
 namespace xsm {
 
 constexpr int kMaxDraft = 16;                        // size of the histogram rows (n_draft itself is <= 15)
-constexpr int kMaxTokens = 128;                      // largest M = batch * (K + 1), and token rows of a chunk of a prompt
+constexpr int kMaxTokens = 128;                      // largest M = batch * (K + 1)
 constexpr int kMaxBatch = 128;
 constexpr int kMaxDevices = 64;                      // device ordinals the per-device host tables cover
 // Every device-side wait is bounded: polls of a word in global memory and mbarrier try_wait calls.
@@ -60,7 +60,7 @@ struct Dev {
     void *xa_;                     // the residual stream times the gain of the RMSNorm that reads it next
     void *qp_, *aa_, *actp_, *yp_; // queries, attention rows, gated activations, decoding heads' hidden states (a set per head)
     void *hq_, *ha_;               // cross-attention heads: queries, attention rows (a set per head)
-    float *ss;                     // [kMaxTokens][kShareLd] shares of the sums of squares of the rows of h
+    float *ss;                     // [row][kShareLd] shares of the sums of squares of the rows of h
     float *logits0, *hlogits;      // [M][V], [K][M][V]
     float *h;                      // residual stream [row][d]
     RowInfo *row_info;             // [row]; with row_cs written when the row is embedded, so that nobody else looks up positions and pages

@@ -1,12 +1,13 @@
 """Per-stage timeline of one decoding step (xsm_debug_trace_step), as a table.
 
-    python -m paper_2507_23777_b200.timeline --config 2 --warm 64
+    python -m paper_2507_23777_b200.timeline --config 2 --warm 64 [--batch B] [--prompt TOKENS] [--room TOKENS]
 
-Runs `warm` decoding steps of the chosen configuration (batch 1 unless --batch), then one traced step, and prints
-for every kind of stage: how long the step spends in it (last CTA of the previous stage done -> last CTA of this
-stage done), how long after the previous stage's end a CTA is past the wait for it, and how long it takes from there
-to its end.  Every mark is a read of the GPU's global timer plus a
-store (a few hundred nanoseconds), so a traced step is slower than an untraced one; compare shares, not totals.
+Runs `warm` decoding steps of the chosen configuration (batch 1, a prompt of one token and the configured room unless
+told otherwise), then eleven traced steps, and prints for the one in the middle by duration and every kind of stage: how
+long the step spends in it (last CTA of the previous stage done -> last CTA of this stage done), how long after the
+previous stage's end a CTA is past the wait for it, and how long it takes from there to its end.  Every mark is a read of
+the GPU's global timer plus a store (a few hundred nanoseconds), so a traced step is slower than an untraced one; compare
+shares, not totals.
 """
 from __future__ import annotations
 
@@ -60,16 +61,22 @@ def main():
     ap.add_argument("--config", type=int, default=2)
     ap.add_argument("--warm", type=int, default=64)
     ap.add_argument("--batch", type=int, default=1)
+    ap.add_argument("--prompt", type=int, default=1, help="tokens of the prompt (random behind the first)")
+    ap.add_argument("--room", type=int, default=0, help="max_seq_len in place of the configured one")
     args = ap.parse_args()
     build.build()
     cfg = inputs.config(args.config)
+    if args.room:
+        cfg["max_seq_len"] = args.room
     w = inputs.make_weights(cfg)
     ctx = binding.Context(cfg, w, max_batch=args.batch)
-    ctx.prefill(inputs.make_cond(cfg, args.batch), [cfg["bos_id"]], binding.decode_config(cfg))
+    prompt = [cfg["bos_id"]] + [int(t) for t in np.random.default_rng(1).integers(1, cfg["vocab"], args.prompt - 1)]
+    ctx.prefill(inputs.make_cond(cfg, args.batch), prompt, binding.decode_config(cfg))
     for _ in range(args.warm):
         ctx.xsm_spec_step()
     print(f"config {args.config} ({cfg['name']}), batch {args.batch}, context {int(ctx.xsm_debug_get_state()['len'][0])}")
-    print(table(cfg, ctx.xsm_debug_trace_step()))
+    steps = sorted((ctx.xsm_debug_trace_step() for _ in range(11)), key=lambda t: int(t[-1].max()) - int(t[0][t[0] > 0].min()))
+    print(table(cfg, steps[5]))
     ctx.xsm_destroy()
 
 
