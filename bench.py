@@ -178,7 +178,7 @@ def fitted_heads_arm(args, cfg, w, cond, T):
     from paper_2507_23777_b200 import binding, fit_heads
     gdc = binding.decode_config(cfg)
 
-    def timed(c, ww):
+    def timed(c, ww, T=T):
         ctx = binding.Context(c, ww, max_batch=1)
         ctx.prefill(cond[:1], [c["bos_id"]], gdc)
         ctx.generate(min(T, 256))                           # warm-up
@@ -190,7 +190,8 @@ def fitted_heads_arm(args, cfg, w, cond, T):
                 "accept_hist": [int(x) for x in list(st.accept_hist)[:c["n_draft"] + 1]]}
 
     cfg0 = dict(cfg, n_draft=0)
-    k0 = timed(cfg0, np.ascontiguousarray(w[:inputs.n_weight_elements(cfg0)]))
+    w0 = np.ascontiguousarray(w[:inputs.n_weight_elements(cfg0)])
+    k0 = timed(cfg0, w0)
     seqs, conds = fit_heads.corpus(cfg, w, args.fit_meshes, 512)
     fitted, report = fit_heads.fit_from_corpus(cfg, w, seqs, conds)
     report.update({"tokens_per_mesh": 512, "corpus_seed0": 5000})
@@ -204,11 +205,12 @@ def fitted_heads_arm(args, cfg, w, cond, T):
     out = {"k0": k0, "fitted_heads": fh}
     from paper_2507_23777_b200 import sweeps
     Ts = min(T, 2048)
+    k0_short = timed(cfg0, w0, Ts)["value"] if Ts < T else k0["value"]      # a step's time grows with the context: like with like
     # the paper's own acceptance rule, delta swept (Sec. 5.4), with the fitted heads
-    out["threshold_sweep"] = sweeps.threshold(cfg, fitted, cond, k0["value"], T=Ts)
+    out["threshold_sweep"] = sweeps.threshold(cfg, fitted, cond, k0_short, T=Ts)
     if args.head_sweep:
         out["head_sweep"] = sweeps.heads(cfg, lambda K: inputs.make_weights(dict(cfg, n_draft=K, seed=args.config)), cond, seqs, conds,
-                                         k0["value"], T=Ts)
+                                         k0_short, T=Ts)
     return out
 
 
