@@ -322,6 +322,10 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
         if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return bail(e, "cudaEventCreate");
     memset(ctx->pinned, 0, 64);
 
+    // The state starts at zero as well: a step behind a prefill that was captured and has not run yet finds positions, pages and
+    // tokens that exist, and ends in XSM_ERR_CAPACITY (the pool is empty).
+    if ((e = cudaMemsetAsync(ctx->ws + L.len, 0, L.xa - L.len, ctx->stream)) != cudaSuccess) return bail(e, "memset");
+
     // constant tables
     // cos and sin of position * theta^(-2i/dh) for every position a window row can take
     const int half = cfg->d_head / 2, n_pos = cfg->max_seq_len + cfg->n_draft + 2;

@@ -136,3 +136,33 @@ def test_parameters_that_were_only_captured_count_as_not_stored(binding, dtype):
         capture(ctx, stream, ctx.xsm_spec_step)
         assert ctx.xsm_kernel_launches() - before == 2 * direct + 1
         ctx.xsm_destroy()
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+def test_a_step_behind_a_prefill_that_was_only_captured_ends_in_an_error(binding, dtype, monkeypatch):
+    """The workspace is full of ones.  A prefill is captured and not run; a direct step then finds the state that xsm_create
+    left (no pages in the pool: XSM_ERR_CAPACITY).  Replayed, the prefill begins a request as always."""
+    import torch
+    cfg = gpu_cfg(dtype=dtype, n_draft=2, sigma=0.05)
+    w = inputs.make_weights(cfg, random_gains=True)
+    cond = inputs.make_cond(cfg, 2)
+    dc = binding.decode_config(cfg)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        other = binding.Context(cfg, w, max_batch=2)
+        other.prefill(cond, [0, 5], dc)
+        want, _, _ = other.generate(24)
+        other.xsm_destroy()
+        with monkeypatch.context() as m:
+            m.setattr(torch, "empty", lambda n, **kw: torch.full((n,), 255, **kw))
+            ctx = binding.Context(cfg, w, max_batch=2)
+        d_cond, d_prompt = ctx.cond_to_device(cond), torch.tensor([[0, 5]] * 2, dtype=torch.int32, device="cuda")
+        g = capture(ctx, stream, lambda: ctx.xsm_prefill(d_cond, d_prompt, 2, dc))
+        ctx.xsm_spec_step()
+        with pytest.raises(binding.XsmError) as e:
+            ctx.xsm_debug_get_state()
+        assert e.value.status == binding.XSM_ERR_CAPACITY
+        g.replay()
+        toks, lens, _ = ctx.generate(24)
+        assert (lens == 24).all() and np.array_equal(toks, want)
+        ctx.xsm_destroy()
