@@ -152,6 +152,8 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.tt = planes * T;
     const int tile_rows = std::min(rows, A.tok);
     A.tps = ((tile_rows + 3) / 4 + S - 1) / S * 4;
+    A.inv_s = 65536 / S + 1;
+    A.inv_q = 65536 / (A.tps / 4) + 1;
     const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
     // more tiles than SMs: two CTAs to an SM
     const int room = (tiles * A.tt * S > sms_ ? kProjSmemMax / 2 : kProjSmemMax) - 1024 - (S > 1 ? sums : 0);

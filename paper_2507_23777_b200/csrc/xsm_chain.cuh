@@ -40,6 +40,7 @@ struct ProjArgs {
     int tt, tok, qp;                  // tiles of tok token rows (parts of one plane set, or one for each); rows of the planes of queries
     int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
     int S, tps;                       // CTAs per cluster (cuts of the columns), token rows each of them finishes
+    uint32_t inv_s, inv_q;            // 65536 / S + 1, 65536 / (tps / 4) + 1: small numbers are divided by multiplying
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns
     int norm, ss_parts;               // the input is an RMSNorm input; shares of its sums of squares (0: not needed)
     int z_jobs, x_jobs;               // group 0 has one matrix per decoding head; the activations too

@@ -30,6 +30,19 @@ template <typename T> __device__ __forceinline__ void settle(T *&p) { asm volati
 __device__ __forceinline__ void settle(int &v) { asm volatile("" : "+r"(v)); }
 __device__ __forceinline__ void settle(uint32_t &v) { asm volatile("" : "+r"(v)); }
 __device__ __forceinline__ void settle(float &v) { asm volatile("" : "+f"(v)); }
+// sixteen bits that no kernel writes, requested here and not later (and, unlike with settle, not waited for)
+__device__ __forceinline__ uint32_t ld_early_u16(const void *p) {
+    uint16_t v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+
+// true in one lane of the warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 
 // ------------------------------------------------------------------------- shared memory, barriers
 
@@ -92,6 +105,11 @@ __device__ __forceinline__ void trace_mark(const Dev &D, int row) {
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_index() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %clusterid.x;" : "=r"(r));
     return r;
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }

@@ -21,16 +21,21 @@
 
 namespace xsm {
 
-constexpr int kProjThreads = 512;
+// CL: a tile's columns are cut over a cluster.  384 threads of at most 80 registers, so that the SM has room for the next kernel's
+// CTA as well (with 512 of 67 to 103 the next kernel's barriers, tensor memory and first copies came after this one's end: 20
+// token rows of width 1024 961 -> 908 us a step, 80 rows 1391 -> 1397).  Without a cluster two CTAs of 512 to an SM.
+constexpr int kClusterThreads = 384, kTileThreads = 512;
 constexpr int kBlockK = 64;                        // columns of one operand block (128 bytes: one swizzled row)
 constexpr int kABytes = 128 * kBlockK * 2;         // weight block
 
 struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate), group 1 (or up)
 
-// CL: a tile's columns are cut over a cluster.  Without it 64 registers a thread, so that two CTAs share an SM; with it 64 cost
-// 1 to 2 % of a step.
+// Where a kernel starts late (its shared memory does not fit beside its predecessor's), everything up to the wait is on the step's
+// way: barriers by the lanes of two warps, one cluster barrier and none of the CTA, weights requested at once, no divisions, no
+// load waited for.  20 token rows of width 1024 908 -> 766 us a step, 80 rows 1397 -> 1274, 28 rows of width 2048 2453 -> 2071 (with
+// the products issued by an elected lane and six shuffles for the sums of squares of four rows).
 template <int EPI0, int EPI1, bool CL>
-__global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
+__global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
     extern __shared__ char smem_raw[];
     char *const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);      // (swizzled tiles: 1024-byte boundaries)
     __shared__ __align__(8) uint64_t bars[4 * kProjRing + 1];      // A full, A empty, B full, B empty, done
@@ -39,14 +44,21 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
     __shared__ float s_inv[kTokenTile];
     __shared__ RowInfo s_row[kTokenTile];
     constexpr bool TWO = EPI0 == PE_GATEUP;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int kThreads = CL ? kClusterThreads : kTileThreads;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp's number: uniform, also to the compiler)
     const int S = CL ? A.S : 1, rank = CL ? (int)cluster_rank() : 0, Mp = A.Mp;
     // sequences that still run: looked at just before the wait, when the weights are on their way
     const int active = A.pos0 < 0 && !A.late_go ? __ldcg(D.n_active) : 1;
     // a tile of weight rows and a tile of token rows: neighbours share the weights
-    const int token_tile = A.tt > 1 ? (int)(blockIdx.x / S) % A.tt : 0, mb = token_tile * A.tok, rows = min(A.tok, A.rows - mb);
-    const int plane = mb / Mp, pm = mb - plane * Mp, Nt = min(A.tok, Mp - pm);      // where they are: plane set, first row; rows with padding
-    int tile = blockIdx.x / S / A.tt, job = 0, z = A.layer, grp = 0;
+    // (divisions only where there is something to divide: 90 cycles each, on the way of a kernel that starts late)
+    int tile = CL ? (int)cluster_index() : (int)blockIdx.x, token_tile = 0, plane = 0, job = 0, z = A.layer, grp = 0;
+    if (A.tt > 1) {
+        const int t = tile / A.tt;
+        token_tile = tile - t * A.tt;
+        tile = t;
+        plane = token_tile * A.tok / Mp;
+    }
+    const int mb = token_tile * A.tok, rows = min(A.tok, A.rows - mb), pm = mb - plane * Mp, Nt = min(A.tok, Mp - pm);      // plane set, first row there; rows with padding
     if (EPI1 >= 0 && tile >= A.g[0].tiles) {
         tile -= A.g[0].tiles;
         grp = 1;
@@ -57,7 +69,7 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
         tile -= job * G.job_tiles;
     }
     const int u0 = tile * (TWO ? 64 : 128);
-    const int nblk = A.kdim / kBlockK, k_lo = rank * nblk / S, n = (rank + 1) * nblk / S - k_lo;
+    const int nblk = A.kdim / kBlockK, k_lo = (int)((uint32_t)(rank * nblk) * A.inv_s >> 16), n = (int)((uint32_t)((rank + 1) * nblk) * A.inv_s >> 16) - k_lo;
     const int na = A.na, nb = A.nb;
     const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
     const uint32_t b_bytes = (uint32_t)(2 * Nt) * kBlockK * 2u, b_pitch = (uint32_t)(2 * A.tok) * kBlockK * 2u;
@@ -66,25 +78,6 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
     float *recv = reinterpret_cast<float *>(smem + (srecv - sa));
     auto bar = [&](int kind, int i) { return smem_u32(&bars[kind * kProjRing + i]); };
     const uint32_t done = smem_u32(&bars[4 * kProjRing]);
-    if (tid == 0) {
-        for (int i = 0; i < na; ++i) { mbar_init(bar(0, i), 1u); mbar_init(bar(1, i), 1u); }
-        for (int i = 0; i < nb; ++i) { mbar_init(bar(2, i), 1u); mbar_init(bar(3, i), 1u); }
-        mbar_init(done, 1u);
-        mbar_init(smem_u32(&recv_bar), 1u);
-        mbar_init_fence();
-        if (CL && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
-    }
-    if (warp == 2) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tcgen05_before_sync();
-    __syncthreads();
-    tcgen05_after_sync();
-    // (the tensor memory is taken before the next kernel may start: kernels further down the chain can then never hold
-    // columns that this one still waits for)
-    if (!A.late_go) chain_go();
-    if (CL) cluster_arrive();          // "this CTA runs": peers may write to its shared memory after cluster_wait
     const void *wmap = grp == 1 ? &T.w1 : &T.w0;
     auto load_a = [&](int i, int slot) {
         const uint32_t dst = sa + (uint32_t)slot * kABytes, b = bar(0, slot);
@@ -97,43 +90,69 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
             tma_box(dst, wmap, x, u0, z, b);
         }
     };
-    if (tid == 0)
+    // Barriers by the lanes of two warps, tensor memory by a third.  (The tensor memory is taken before the next kernel may start:
+    // kernels further down the chain can then never hold columns that this one still waits for.)
+    if (warp == 0) {
+        if (lane < na) { mbar_init(bar(0, lane), 1u); mbar_init(bar(1, lane), 1u); }
+        mbar_init_fence();
+    } else if (warp == 1) {
+        if (lane < nb) { mbar_init(bar(2, lane), 1u); mbar_init(bar(3, lane), 1u); }
+        if (lane == 31) {
+            mbar_init(done, 1u);
+            mbar_init(smem_u32(&recv_bar), 1u);
+        }
+        mbar_init_fence();
+        if (CL && lane == 31 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
+    } else if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (!A.late_go) chain_go();
+    }
+    __syncwarp();
+    // "this CTA runs": what it has set up is there, and peers may write to its shared memory, after cluster_wait
+    if (CL) cluster_arrive();
+    if (warp == 0 && elect_one())      // the weights' way is the longest: it begins as early as that
         for (int i = 0; i < min(n, na); ++i) load_a(i, i);
+    __syncwarp();
     if (A.stage == 0) trace_mark(D, 0);
     const bf16 *x = A.x + (size_t)(A.x_jobs ? job : plane) * 2 * Mp * A.kdim;
     const bf16 *xb = x + (size_t)k_lo * (128 * Mp) + (size_t)pm * 128;      // this CTA's blocks of the activations
-    const uint32_t idesc = umma_idesc(128, 2 * Nt), tmem = tmem_slot, full_a = bar(0, 0), full_b = bar(2, 0);
+    const uint32_t idesc = umma_idesc(128, 2 * Nt), full_a = bar(0, 0), full_b = bar(2, 0);
     settle(xb);
-    constexpr int ROWS = TWO ? 64 : 128, SIDES = kProjThreads / ROWS;
+    constexpr int ROWS = TWO ? 64 : 128, SIDES = kThreads / ROWS;
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
     const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
     const bool live_row = u_row < G.units;
-    float gain = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? to_f(__ldg(reinterpret_cast<const bf16 *>(A.gain) + u_row)) : 0.f;
+    const uint32_t gain_bits = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? ld_early_u16(reinterpret_cast<const bf16 *>(A.gain) + u_row) : 0u;
     // where this thread's weight row goes
-    const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col / D.dh : 0;
+    const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col >> (31 - __clz(D.dh)) : 0;      // (d_head is 32, 64 or 128)
     __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
     bf16 *xrow = G.out + (size_t)(job + plane) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (size_t)pm * 128 + (u_row & 7);
     const int xchunk = (u_row >> 3) & 7;
     float *lrow = G.logits + ((size_t)job * D.M + mb) * G.ld + u_row;
     __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
-    settle(gain); settle(qrow); settle(xrow); settle(lrow); settle(crow);
+    settle(qrow); settle(xrow); settle(lrow); settle(crow);
     // Accumulator -> the CTA that finishes the token rows: [sender][quad][weight row][4].  This thread's lane of the accumulator
     // is its weight row; eight token rows at a time, from c0 on.
-    const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = warp >> 2, qinv = 65536 / qps + 1;
+    const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = warp >> 2;
     const uint32_t recv_b = smem_u32(&recv_bar);
     uint32_t dst[2], dst_bar[2];
     auto where = [&](int c) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int quad = 2 * c + q, owner = (quad * qinv) >> 16, place = rank * qps + quad - owner * qps;      // (quad / qps: both are below 33)
+            const int quad = 2 * c + q, owner = (int)((uint32_t)quad * A.inv_q >> 16), place = rank * qps + quad - owner * qps;      // (quad / qps: both are below 33)
             dst[q] = CL ? map_rank(srecv + (uint32_t)(place * 128 + arow) * 16u, (uint32_t)min(owner, S - 1)) : (uint32_t)(quad * 128 + arow) * 16u;
             dst_bar[q] = CL ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;
         }
     };
     where(c0);
     settle(dst[0]); settle(dst[1]); settle(dst_bar[0]); settle(dst_bar[1]);
+    tcgen05_before_sync();
     if (CL) cluster_wait();            // the peers run: their barriers and shared memory are there
-    if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kProjThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
+    else __syncthreads();
+    tcgen05_after_sync();
+    const uint32_t tmem = tmem_slot;
+    if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (active == 0) {      // every sequence has ended in an earlier step
         if (tid == 0)
@@ -144,41 +163,58 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
     }
     if (A.late_go) chain_go();
     trace_mark(D, 1 + 2 * A.stage);
-    if (tid == 0) {
+    if (warp == 0) {
         // (written by ordinary stores of an earlier kernel, which has completed: nothing to order)
-        int slot = 0, a_slot = 0;
-        uint32_t par = 1u, a_par = 0u;
-        for (int i = 0; i < n; ++i) {
-            if (i >= nb) mbar_wait(bar(3, slot), par, D.mbar_limit, D.status);
-            mbar_arrive_expect_tx(full_b + 8u * (uint32_t)slot, b_bytes);
-            bulk_g2s(sb + (uint32_t)slot * b_pitch, xb + (size_t)i * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)slot);
-            if (++slot == nb) { slot = 0; par ^= 1u; }
-            if (i >= na) {
-                mbar_wait(bar(1, a_slot), a_par, D.mbar_limit, D.status);
-                load_a(i, a_slot);
-                if (++a_slot == na) { a_slot = 0; a_par ^= 1u; }
+        if (lane < min(n, nb)) {
+            mbar_arrive_expect_tx(full_b + 8u * (uint32_t)lane, b_bytes);
+            bulk_g2s(sb + (uint32_t)lane * b_pitch, xb + (size_t)lane * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)lane);
+        }
+        __syncwarp();
+        if (elect_one()) {
+            int slot = 0, a_slot = 0;
+            uint32_t par = 0u, a_par = 0u;
+            for (int i = min(na, nb); i < n; ++i) {
+                if (i >= nb) {
+                    mbar_wait(bar(3, slot), par, D.mbar_limit, D.status);
+                    mbar_arrive_expect_tx(full_b + 8u * (uint32_t)slot, b_bytes);
+                    bulk_g2s(sb + (uint32_t)slot * b_pitch, xb + (size_t)i * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)slot);
+                    if (++slot == nb) { slot = 0; par ^= 1u; }
+                }
+                if (i >= na) {
+                    mbar_wait(bar(1, a_slot), a_par, D.mbar_limit, D.status);
+                    load_a(i, a_slot);
+                    if (++a_slot == na) { a_slot = 0; a_par ^= 1u; }
+                }
             }
         }
-    } else if (tid == 32) {
+        __syncwarp();
+    } else if (warp == 1) {
+        // (the whole warp waits and one elected lane issues: a branch on the thread's number would keep the descriptors out of the
+        // uniform registers that the instruction takes them from)
+        const bool leader = elect_one();
         int ia = 0, ib = 0;
         uint32_t pa = 0u, pb = 0u;
         for (int i = 0; i < n; ++i) {
             mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
             mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
             tcgen05_after_sync();
+            if (leader) {
             const uint64_t da = umma_desc_sw128(sa + (uint32_t)ia * kABytes), db = umma_desc_sw128(sb + (uint32_t)ib * b_pitch);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, da + 2 * ks, db + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
             if (i + na < n) umma_commit(bar(1, ia));
             if (i + nb < n) umma_commit(bar(3, ib));
+            }
+            __syncwarp();
             if (++ia == na) { ia = 0; pa ^= 1u; }
             if (++ib == nb) { ib = 0; pb ^= 1u; }
         }
-        umma_commit(done);
+        if (leader) umma_commit(done);
+        __syncwarp();
     }
     // meanwhile: what the epilogue needs to know of the token rows that this CTA finishes
     if (warp >= 2) {
-        for (int i = tid - 64; i < nm; i += kProjThreads - 64) {
+        for (int i = tid - 64; i < nm; i += kThreads - 64) {
             const int m = m0 + i;
             float inv = 1.f;
             if (A.ss_parts > 0) {
@@ -214,13 +250,13 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
             if (EPI0 == PE_QKV && i < nm) csn[q] = __ldcg(D.row_cs + (size_t)(mb + m0 + i) * half + (e < half ? e : e - half));
         }
     };
-    __syncwarp();
+    const float gain = __uint_as_float(gain_bits << 16);
     request(side);
     __syncthreads();      // (what the epilogue needs is in shared memory; the last products are under way)
     const bool done_ok = mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
     tcgen05_after_sync();
-    for (int c = c0; c < (Nt >> 3); c += kProjThreads / 128) {      // hi and lo parts added
+    for (int c = c0; c < (Nt >> 3); c += kThreads / 128) {      // hi and lo parts added
         uint32_t v[16];
         tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
         if (c != c0) where(c);
@@ -276,20 +312,37 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
         total(quad, row, sum);
         if (TWO) total(quad, row + 64, other);
         if (EPI0 == PE_QKV) total(quad, e < half ? row + half : row - half, other);
+        if (EPI0 == PE_ADD) {
+            float o[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = 4 * quad + q, m = m0 + i;
+                o[q] = live_row && i < nm ? h[q] + sum[q] : 0.f;
+                if (live_row && i < nm) {
+                    D.h[(size_t)(mb + m) * D.d + u_row] = o[q];
+                    put_x(m, o[q] * gain);
+                }
+                o[q] *= o[q];
+            }
+            // the warp's sums of the four rows: a lane keeps two of them after the first exchange, one after the second (six
+            // shuffles instead of twenty, 38 cycles each); lane 8 r has row r
+            const bool up = lane & 16, mid = lane & 8;
+            float a = up ? o[2] : o[0], b = up ? o[3] : o[1];
+            a += __shfl_xor_sync(0xffffffffu, up ? o[0] : o[2], 16);
+            b += __shfl_xor_sync(0xffffffffu, up ? o[1] : o[3], 16);
+            float v = mid ? b : a;
+            v += __shfl_xor_sync(0xffffffffu, mid ? a : b, 8);
+#pragma unroll
+            for (int k = 4; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
+            const int i = 4 * quad + (lane >> 3);
+            if ((lane & 7) == 0 && i < nm) D.ss[(size_t)(mb + m0 + i) * kShareLd + tile * 4 + (row >> 5)] = v;
+        } else
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = 4 * quad + q, m = m0 + i;
             if (i >= nm) break;
             const float v = sum[q];
-            if (EPI0 == PE_ADD) {
-                const float o = live_row ? h[q] + v : 0.f;
-                if (live_row) {
-                    D.h[(size_t)(mb + m) * D.d + u_row] = o;
-                    put_x(m, o * gain);
-                }
-                const float ssq = warp_sum(o * o);
-                if (lane == 0) D.ss[(size_t)(mb + m) * kShareLd + tile * 4 + (row >> 5)] = ssq;
-            } else if (live_row) {
+            if (live_row) {
                 const float inv = s_inv[i], x1 = v * inv;
                 if (EPI0 == PE_QKV) {
                     const float x2 = other[q] * inv, o = sec == 2 ? x1 : e < half ? x1 * cs[q].x - x2 * cs[q].y : x1 * cs[q].x + x2 * cs[q].y;
@@ -315,9 +368,9 @@ __global__ void __launch_bounds__(kProjThreads, CL ? 1 : 2) proj_umma_kernel(con
     }
     // (every warp has read its part of the accumulator)
     if (warp != 2) {
-        asm volatile("bar.arrive 2, %0;" :: "n"(kProjThreads) : "memory");
+        asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
     } else {
-        asm volatile("bar.sync 2, %0;" :: "n"(kProjThreads) : "memory");
+        asm volatile("bar.sync 2, %0;" :: "n"(kThreads) : "memory");
         tcgen05_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
     }
@@ -329,7 +382,7 @@ static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMa
     cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
-    return L.launch(dim3(tiles * A.tt * A.S), dim3(kProjThreads), smem, A.S, (const void *)fn, D, A, T);
+    return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? kClusterThreads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
 }
 
 // (asked for once per device: the answer does not change, and asking takes longer than the rest of a context's creation)
@@ -347,7 +400,7 @@ int resident_clusters(int size) {
     at.val.clusterDim.x = (unsigned)size;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     c.gridDim = dim3(size);
-    c.blockDim = dim3(kProjThreads);
+    c.blockDim = dim3(kClusterThreads);
     c.dynamicSmemBytes = smem;
     c.attrs = &at;
     c.numAttrs = 1;
