@@ -8,8 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxsm.so")
-SOURCES = ["xsm_api.cu", "xsm_kernels.cu", "xsm_chain.cu", "xsm_proj_few_a.cu", "xsm_proj_few_b.cu", "xsm_proj_few_c.cu",
-           "xsm_proj_few_d.cu", "xsm_proj_umma.cu", "xsm_attn.cu", "xsm_f32.cu", "xsm_cond.cu", "xsm_tail.cu"]
+SOURCES = ["xsm_api.cu", "xsm_kernels.cu", "xsm_chain.cu", "xsm_proj_few.cu", "xsm_proj_umma.cu", "xsm_attn.cu", "xsm_f32.cu", "xsm_cond.cu", "xsm_tail.cu"]
 HEADERS = ["xsm_internal.h", "xsm_host.h", "xsm_common.cuh", "xsm_chain.cuh", "xsm_proj.cuh", "xsm_proj_few.cuh",
            os.path.join("..", "..", "include", "xsm.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

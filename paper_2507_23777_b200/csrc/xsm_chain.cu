@@ -125,15 +125,14 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.Mp = Mp;
     const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
     // How a tile of weight rows is cut: its columns over a cluster of S CTAs, as many as fit into the GPCs at a time (of six CTAs
-    // 22 clusters, of eight 15; a cluster more is a second wave).  More than 96 token rows in one plane: these into T parts too,
+    // 22 clusters, of eight 15; a cluster more is a second wave).  More than 48 token rows in one plane: these into T parts too,
     // each with the weights for itself, which leaves less to exchange and to finish in a CTA.  There the stage's time after the
     // wait in cycles, as measured, chooses among S and T: a product 47, or N / 2 where the token rows (hi and lo) bound it;
     // activations, and weights that do not fit the ring, 59 bytes a cycle; 45 for every token row that is sent, 250 for every
-    // one that is finished.  125 rows of width 1024: 2079 -> 1834 us a step.  Up to 96 rows T is 1 and the largest S that fits is
-    // taken, without weighing: the CTAs of more parts keep the next stage's weights out of shared memory for longer than they
-    // save (90 rows of width 768 703 -> 716, 80 rows 1494 -> 1498, 40 rows 1221 -> 1273).
+    // one that is finished.  Eight layers of width 1024: 90 rows 480 -> 425 us a step, 80 rows 444 -> 414, 60 rows 409 -> 375; 40
+    // rows 354 -> 356, 30 rows 304 -> 331, so up to 48 rows T is 1 and the largest S that fits is taken, without weighing.
     int S = 1, T = 1;
-    const bool parts = A.tt == 1 && rows > 96;
+    const bool parts = A.tt == 1 && rows > 48;
     double best = 1e30;
     for (int t = 1; t <= (parts ? Mp / 8 : 1); ++t) {
         const int nt = parts ? (Mp / 8 + t - 1) / t * 8 : std::min(Mp, kTokenTile);
@@ -150,14 +149,19 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int planes = A.tt;
     A.tok = planes > 1 ? Mp : (Mp / 8 + T - 1) / T * 8;
     A.tt = planes * T;
-    const int tile_rows = std::min(rows, A.tok);
-    A.tps = ((tile_rows + 3) / 4 + S - 1) / S * 4;
+    // Token rows are dealt out to the CTAs that finish them one by one where there are few (in fours, two of eight CTAs finished
+    // five rows, four by each thread: 763 -> 683 us a step at width 1024, 20 rows 771 -> 748); 28 rows at width 2048, five to a
+    // CTA, are finished faster in fours, read as 16 bytes (2085 against 2129).
+    const int tile_rows = std::min(rows, A.tok), G = S > 1 && rows <= 24 ? 1 : 4;
+    A.group = G;
+    A.tps = ((tile_rows + G - 1) / G + S - 1) / S * G;
     A.inv_s = 65536 / S + 1;
-    A.inv_q = 65536 / (A.tps / 4) + 1;
+    A.inv_q = 65536 / (A.tps / G) + 1;
     const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
     // more tiles than SMs: two CTAs to an SM
+    // (the activations' share of the ring: from the L2, but all of them after the wait)
     const int room = (tiles * A.tt * S > sms_ ? kProjSmemMax / 2 : kProjSmemMax) - 1024 - (S > 1 ? sums : 0);
-    A.nb = std::min(n, std::max(2, std::min(kProjRing, (room / 3) / b_bytes)));
+    A.nb = std::min(n, std::max(2, std::min(kProjRing, (rows > 32 ? room * 9 / 20 : room / 3) / b_bytes)));
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
     A.tmem_cols = 32;
@@ -167,18 +171,24 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
 }
 
 // The projections over few token rows: how the units are dealt out, passes over the columns, shared memory.  False: the
-// shape does not fit, or there are more token rows than the path serves.
+// shape does not fit, or the tensor cores of the 5th generation do better.  Whole steps, us, this path and that one, without
+// decoding heads:
+//   token rows        1            2            3            4
+//   width 768      280 285      283 291      287 296      304 294
+//   width 1024     593 574      612 582      659 604      684 623
+//   width 2048    1531 1520    1601 1602    1689 1655        -
+// (A CTA reads all activations here and a slice of them there, which tells as soon as they are more than a few KB.)
 bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
     ProjArgs &A = op.proj;
-    if (rows > kFewRows) return false;
+    if (rows > kFewRows || c_.d_model > kFewWidth) return false;
     const bool pairs = A.epi0 == PE_QKV || A.epi0 == PE_GATEUP;
     const int units = A.epi0 == PE_QKV ? A.g[0].units / 2 : A.g[0].units + (A.epi1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
     const int share = A.x_jobs ? std::max(1, sms_ / A.g[0].jobs) : sms_;      // CTAs for `units`
     A.upc = (units + share - 1) / share;
     A.ctas = (units + A.upc - 1) / A.upc;
-    const FewShape f = few_shape(rows, kdim);
+    const FewShape f = few_shape(kdim);
     const int n_rows = A.upc * (pairs ? 2 : 1), tiles = (n_rows + 15) / 16;
-    const int red = tiles * f.warps * 16 * (f.nt * 8 + 1) * 4;
+    const int red = tiles * f.warps * 16 * 9 * 4;
     A.slot_rows = tiles == 1 ? (n_rows + 7) / 8 * 8 : 16;
     // passes no wider than the registers hold, and narrow enough for two of them in flight
     int slots = 0;

@@ -39,8 +39,8 @@ struct ProjArgs {
     int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8, at most kTokenTile)
     int tt, tok, qp;                  // tiles of tok token rows (parts of one plane set, or one for each); rows of the planes of queries
     int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
-    int S, tps;                       // CTAs per cluster (cuts of the columns), token rows each of them finishes
-    uint32_t inv_s, inv_q;            // 65536 / S + 1, 65536 / (tps / 4) + 1: small numbers are divided by multiplying
+    int S, tps, group;                // CTAs per cluster (cuts of the columns), token rows each of them finishes, dealt out in groups of so many
+    uint32_t inv_s, inv_q;            // 65536 / S + 1, 65536 / (tps / group) + 1: small numbers are divided by multiplying
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns
     int norm, ss_parts;               // the input is an RMSNorm input; shares of its sums of squares (0: not needed)
     int z_jobs, x_jobs;               // group 0 has one matrix per decoding head; the activations too
@@ -107,16 +107,14 @@ struct ChainLaunch {
 // opens a kernel for `smem` bytes of dynamic shared memory (and for clusters of more than eight CTAs) on the current device
 cudaError_t open_kernel(const void *fn, int smem, bool large_cluster);
 
-// Instance of the projection over few token rows that serves `rows` token rows and rows of kdim weights: warps that
-// multiply, tiles of eight token rows, columns of one pass
-struct FewShape { int warps, nt, blocks, pass; bool pack; };
-constexpr int kFewRows = 16;
-inline FewShape few_shape(int rows, int kdim) {
+// Instance of the projection over few token rows that serves rows of kdim weights: warps that multiply, blocks of 32 columns
+// that each holds in registers, columns of one pass
+struct FewShape { int warps, blocks, pass; };
+constexpr int kFewRows = 3, kFewWidth = 768;      // most token rows, largest d_model
+inline FewShape few_shape(int kdim) {
     FewShape f;
-    f.pack = rows <= 4;
-    f.nt = rows <= 8 ? 1 : 2;
     f.warps = kdim > 2048 ? 15 : 8;
-    f.blocks = kdim > 2048 ? (f.nt == 1 ? 9 : 4) : kdim > 1024 ? 8 : 4;
+    f.blocks = kdim > 2048 ? 9 : kdim > 1024 ? 8 : 4;
     f.pass = f.warps * f.blocks * 32;
     return f;
 }

@@ -1,10 +1,10 @@
-// Projections over few token rows (at most 16) of bf16 models, as kernels of the launch chain.
+// Projections over few token rows (at most three, of narrow bf16 models), as kernels of the launch chain.
 //
 // A CTA owns a run of weight rows at full width.  Its rows are on their way to shared memory before the kernel waits for
 // its predecessor (bulk copies by a producer warp, tiles of 16 rows x one pass of columns).  Then every warp fetches the
 // activations of its own blocks of 32 columns straight into operand registers (one round trip to L2, nothing is staged),
-// multiplies all tiles with mma.sync.m16n8k16 (weight rows on M, token rows on N; hi and lo parts of the activations as
-// separate products), and parks its partial sums; after one barrier the sums over the warps are finished and stored.
+// multiplies all tiles with mma.sync.m16n8k16 (weight rows on M; on N the hi parts of four token rows and their lo parts
+// beside them), and parks its partial sums; after one barrier the sums over the warps are finished and stored.
 // Latency is all that counts here (a step has some 200 of these kernels in a row, 2 to 17 MB of weights each): no
 // cluster, because a cluster barrier with remote stores behind it costs 1 us, twice the products.
 #pragma once
@@ -12,14 +12,13 @@
 
 namespace xsm {
 
-// NW: multiplying warps; NT: tiles of 8 token rows; PACK: at most four token rows, hi and lo parts side by side in one
-// product; MAXB: blocks of 32 columns that a warp holds in registers (a pass is NW * MAXB blocks at most)
-template <int NW, int NT, bool PACK, int MAXB, int EPI0, int EPI1>
-__global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || MAXB == 4) ? 2 : 1) proj_few_kernel(const Dev D, const ProjArgs A) {
+// NW: multiplying warps; MAXB: blocks of 32 columns that a warp holds in registers (a pass is NW * MAXB blocks at most)
+template <int NW, int MAXB, int EPI0, int EPI1>
+__global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kernel(const Dev D, const ProjArgs A) {
     extern __shared__ __align__(128) char smem[];
     __shared__ __align__(8) uint64_t full[kProjRing], empty[kProjRing];
-    __shared__ float s_inv[16];
-    constexpr int kOutThreads = NW * 32, LDM = NT * 8 + 1;      // (odd pitch: neighbouring rows in other banks)
+    __shared__ float s_inv[8];
+    constexpr int kOutThreads = NW * 32, LDM = 9;      // (odd pitch: neighbouring rows in other banks)
     constexpr bool PAIRS = EPI0 == PE_QKV || EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (!A.late_go) chain_go();
@@ -78,7 +77,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     // Everything that does not depend on the step is worked out before the wait, so that little is left to issue after it (a
     // warp gets an instruction off every 8 cycles here): this thread's first output and where it goes, the places of the
     // warp's activations.
-    constexpr int MP = NT * 8;                     // rows of a plane
+    constexpr int MP = 8;                          // rows of a plane
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
     int lpt = 8;                                   // PE_ADD: lanes per token row
     if (EPI0 == PE_ADD)
@@ -137,21 +136,19 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     const bool has = warp < NW && tid < M * per_m && o1.r < n_units;
     if (EPI0 == PE_QKV && has && !A.late_go) position(o1);
     const int g = lane >> 2, t4 = lane & 3;
-    // the warp's blocks are warp + NW i.  Lanes past the last token row read another row of their tile (what they multiply goes
-    // nowhere): x_last for the last tile of token rows, x_full for those before it.
-    const bf16 *x_full[2], *x_last[2];
+    // the warp's blocks are warp + NW i.  Lanes 0..15: hi parts of token rows g & 3, the others lo parts; past the last token row
+    // the first one again (what they multiply goes nowhere)
+    const bf16 *x0[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {      // (odd NW: the blocks of a warp alternate between the halves of a 64-column block)
-        const int blk = warp + NW * q, tail = PACK ? ((g & 3) < M ? g & 3 : 0) : ((NT - 1) * 8 + g < M ? g : 0), chunk8 = (blk & 1) * 4 + t4;
-        const bf16 *base = A.x + (A.x_jobs ? (size_t)job * 2 * MP * kdim : 0) + (size_t)(blk >> 1) * (128 * MP);
-        x_full[q] = base + g * 64 + ((chunk8 ^ g) << 3);
-        x_last[q] = base + (NT - 1) * 1024 + tail * 64 + ((chunk8 ^ tail) << 3) + (PACK ? (g >> 2) * kLo : 0);
+        const int blk = warp + NW * q, m = (g & 3) < M ? g & 3 : 0, chunk8 = (blk & 1) * 4 + t4;
+        x0[q] = A.x + (A.x_jobs ? (size_t)job * 2 * MP * kdim : 0) + (size_t)(blk >> 1) * (128 * MP) + m * 64 + ((chunk8 ^ m) << 3) + (g >> 2) * kLo;
     }
     const uint32_t full0 = smem_u32(&full[0]);
     const char *w0 = smem + (size_t)g * pitch + t4 * 16 + warp * 64;
     float *dst0 = red + (size_t)(warp * 16 + g) * LDM + 2 * t4;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) { settle(x_full[q]); settle(x_last[q]); }
+    for (int q = 0; q < 2; ++q) settle(x0[q]);
     settle(o1.sum); settle(o1.p); settle(o1.h); settle(w0); settle(dst0);
     if (EPI0 == PE_ADD || HEAD) settle(o1.gain);
     if (warp < NW) bar_sync<NW * 32>(1);           // (warps that come to the wait together leave it sooner: 0.3 us a kernel)
@@ -168,31 +165,14 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     trace_mark(D, 1 + 2 * A.stage);
 
     float h_old = 0.f;
-    // one k-block of a tile: a, c: eight columns of weight rows g and g + 8
-    auto multiply = [&](float (&ah)[NT][4], float (&al)[NT][4], const uint4 &a, const uint4 &c, const uint4 (&h)[NT], const uint4 (&l)[NT]) {
+    auto park = [&](float *dst, const float (&c0)[4], const float (&c1)[4], bool first) {
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            mma16816_bf16(ah[nt], a.x, c.x, a.y, c.y, h[nt].x, h[nt].y);
-            if (PACK) {
-                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, h[nt].z, h[nt].w);
-            } else {
-                mma16816_bf16(al[nt], a.x, c.x, a.y, c.y, l[nt].x, l[nt].y);
-                mma16816_bf16(ah[nt], a.z, c.z, a.w, c.w, h[nt].z, h[nt].w);
-                mma16816_bf16(al[nt], a.z, c.z, a.w, c.w, l[nt].z, l[nt].w);
-            }
-        }
-    };
-    auto park = [&](float *dst, const float (&ah)[NT][4], const float (&al)[NT][4], bool first) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                float v = ah[nt][q] + al[nt][q];
-                if (PACK) v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
-                if (!PACK || t4 < 2) {
-                    float *o = dst + (q >> 1) * 8 * LDM + nt * 8 + (q & 1);
-                    *o = first ? v : *o + v;
-                }
+        for (int q = 0; q < 4; ++q) {
+            float v = c0[q] + c1[q];
+            v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
+            if (t4 < 2) {
+                float *o = dst + (q >> 1) * 8 * LDM + (q & 1);
+                *o = first ? v : *o + v;
             }
         }
     };
@@ -202,37 +182,28 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         for (int pass = 0; pass < passes; ++pass) {
             const int nb = min(chunk, kdim - pass * chunk) >> 5;      // blocks of 32 columns
             const size_t xp = (size_t)(pass * (chunk >> 6)) * (128 * MP);
-            uint4 xh[MAXB][NT], xl[MAXB][NT];
+            uint4 x[MAXB];
 #pragma unroll
-            for (int i = 0; i < MAXB; ++i) {
+            for (int i = 0; i < MAXB; ++i)
                 if (warp + NW * i < nb) {
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        const int q = (NW & 1) ? i & 1 : 0;
-                        const bf16 *p = (nt < NT - 1 ? x_full[q] + nt * 1024 : x_last[q]) + xp + (size_t)((NW & 1) ? (i >> 1) * NW : i * (NW / 2)) * (128 * MP);
-                        xh[i][nt] = __ldcg(reinterpret_cast<const uint4 *>(p));
-                        if (!PACK) xl[i][nt] = __ldcg(reinterpret_cast<const uint4 *>(p + kLo));
-                    }
+                    const int q = (NW & 1) ? i & 1 : 0;
+                    x[i] = __ldcg(reinterpret_cast<const uint4 *>(x0[q] + xp + (size_t)((NW & 1) ? (i >> 1) * NW : i * (NW / 2)) * (128 * MP)));
                 }
-            }
             if ((EPI0 == PE_ADD || HEAD) && pass == 0 && has) h_old = __ldcg(o1.h);
             float *dst = dst0;
             for (int tile = 0; tile < tiles; ++tile) {
                 const bool two = n_rows - tile * 16 > 8;
                 mbar_wait(full0 + 8u * (uint32_t)sl, par, D.mbar_limit, D.status);
                 const char *ws = w0 + (size_t)sl * slot_bytes;
-                float ah[NT][4], al[NT][4];
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) ah[nt][q] = al[nt][q] = 0.f;
+                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};      // even and odd steps of 16 columns
 #pragma unroll
                 for (int i = 0; i < MAXB; ++i) {
                     if (warp + NW * i < nb) {
                         const uint4 a = *reinterpret_cast<const uint4 *>(ws + NW * i * 64);
                         uint4 c = make_uint4(0u, 0u, 0u, 0u);
                         if (two) c = *reinterpret_cast<const uint4 *>(ws + 8 * pitch + NW * i * 64);
-                        multiply(ah, al, a, c, xh[i], xl[i]);
+                        mma16816_bf16(c0, a.x, c.x, a.y, c.y, x[i].x, x[i].y);
+                        mma16816_bf16(c1, a.z, c.z, a.w, c.w, x[i].z, x[i].w);
                     }
                 }
                 if (A.slots < tiles * passes) {
@@ -240,17 +211,14 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
                     if (lane == 0) mbar_arrive(smem_u32(&empty[sl]));
                 }
                 if (++sl == A.slots) { sl = 0; par ^= 1u; }
-                park(dst, ah, al, pass == 0);
+                park(dst, c0, c1, pass == 0);
                 dst += NW * 16 * LDM;
             }
         }
     } else {
         // the producer warp adds up the shares of the sums of squares: four lanes per token row, every fourth quad each
         if (A.ss_parts > 0) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            const int m = nt * 8 + g;
-            const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)min(m, M - 1) * kShareLd) + t4;
+            const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)min(g, M - 1) * kShareLd) + t4;
             float4 v[kShareLd / 16];
 #pragma unroll
             for (int q = 0; q < kShareLd / 16; ++q) v[q] = 16 * q + 4 * t4 < A.ss_parts ? __ldcg(sh + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -262,8 +230,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
             }
             ss += __shfl_xor_sync(0xffffffffu, ss, 1);
             ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-            if (t4 == 0) s_inv[m] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
-        }
+            if (t4 == 0) s_inv[g] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
         }
         // then the rest of the weights, as their slots become free
         int sl = 0;
@@ -299,7 +266,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         reinterpret_cast<__half *>(p)[0] = hi;
         reinterpret_cast<__half *>(p)[(size_t)MP * D.d] = lo_;
     };
-    for (int e = tid; e < M * per_m; e += kOutThreads) {
+    const int outputs = EPI0 == PE_ADD ? (M * per_m + 31) & ~31 : M * per_m;      // (PE_ADD: whole warps, which shuffle)
+    for (int e = tid; e < outputs; e += kOutThreads) {
         if (e != tid) {
             locate(e, o1);
             if (EPI0 == PE_QKV) position(o1);
@@ -308,14 +276,14 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
         const float inv = A.ss_parts > 0 ? s_inv[o1.m] : 1.f;
         if (EPI0 == PE_ADD) {
             float h = 0.f;
-            if (o1.r < n_units) {
+            if (o1.r < n_units && o1.m < M) {
                 h = h_old + total(o1.sum);
                 *const_cast<float *>(o1.h) = h;
                 put_bf16(o1.p, h * o1.gain);
             }
             float ssq = h * h;
             for (int k = lpt >> 1; k > 0; k >>= 1) ssq += __shfl_xor_sync(0xffffffffu, ssq, k);
-            if (o1.r == 0) D.ss[(size_t)o1.m * kShareLd + cta] = ssq;
+            if (o1.r == 0 && o1.m < M) D.ss[(size_t)o1.m * kShareLd + cta] = ssq;
         } else if (EPI0 == PE_QKV) {
             const float v = total(o1.sum) * inv, v2 = total(o1.sum + LDM) * inv;
             if (o1.sec == 0) {
@@ -343,17 +311,17 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || 
     trace_mark(D, 2 + 2 * A.stage);
 }
 
-template <int NW, int NT, bool PACK, int MAXB, int EPI0, int EPI1>
+template <int NW, int MAXB, int EPI0, int EPI1>
 static cudaError_t launch_few_instance(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
-    void (*fn)(const Dev, const ProjArgs) = proj_few_kernel<NW, NT, PACK, MAXB, EPI0, EPI1>;
+    void (*fn)(const Dev, const ProjArgs) = proj_few_kernel<NW, MAXB, EPI0, EPI1>;
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     return L.launch(dim3(A.x_jobs ? A.ctas * A.g[0].jobs : A.ctas), dim3((NW + 1) * 32), smem, 1, (const void *)fn, D, A);
 }
 
-template <int NW, int NT, bool PACK, int MAXB>
+template <int NW, int MAXB>
 static cudaError_t launch_few(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
-#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_few_instance<NW, NT, PACK, MAXB, a, b>(D, A, smem, L)
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_few_instance<NW, MAXB, a, b>(D, A, smem, L)
     XSM_EPI(PE_ADD, -1);
     if constexpr (NW == 8) {
         XSM_EPI(PE_QUERY, -1);

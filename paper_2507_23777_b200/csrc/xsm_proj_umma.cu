@@ -6,8 +6,8 @@
 // nothing of the activations is lost and a weight tile serves all token rows in one pass.  A tile's columns are cut over
 // the S CTAs of a cluster (a step has at most 128 token rows, so the row tiles alone would leave most of the chip idle).
 // Each of them hands the partial sums of a share of the token rows to the CTA that finishes those rows, straight from the
-// accumulator (asynchronous 16-byte stores that count on the receiver's barrier), and they are added in rank order:
-// results do not depend on timing.
+// accumulator (asynchronous stores that count on the receiver's barrier), and they are added in rank order: results do not
+// depend on timing.
 //
 // A chunk of a prompt has more token rows: tiles of 128 of them, two CTAs to an SM, so that one's products run under the
 // other's epilogue.
@@ -34,7 +34,12 @@ struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate)
 // way: barriers by the lanes of two warps, one cluster barrier and none of the CTA, weights requested at once, no divisions, no
 // load waited for.  20 token rows of width 1024 908 -> 766 us a step, 80 rows 1397 -> 1274, 28 rows of width 2048 2453 -> 2071 (with
 // the products issued by an elected lane and six shuffles for the sums of squares of four rows).
-template <int EPI0, int EPI1, bool CL>
+//
+// A chain of instructions bounds it at few token rows (nine cycles each): where every operand block has a place of its own, the
+// activations count on one barrier and the issuing warp adds to two descriptors; with a barrier and two commits a block, a block
+// took 0.28 us, eight of them more than the weights' way from memory (5 rows of width 1024 683 -> 631 us a step).
+// G: token rows of a group that is sent and finished together (plan_proj).
+template <int EPI0, int EPI1, bool CL, int G>
 __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
     extern __shared__ char smem_raw[];
     char *const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);      // (swizzled tiles: 1024-byte boundaries)
@@ -63,15 +68,16 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         tile -= A.g[0].tiles;
         grp = 1;
     }
-    const ProjGroup &G = A.g[grp];
+    const ProjGroup &W = A.g[grp];
     if (EPI1 >= 0 || A.z_jobs) {          // the matrices of a group (one per decoding head) share its map, one behind the other
-        z = job = grp == 1 || A.z_jobs ? tile / G.job_tiles : 0;
-        tile -= job * G.job_tiles;
+        z = job = grp == 1 || A.z_jobs ? tile / W.job_tiles : 0;
+        tile -= job * W.job_tiles;
     }
     const int u0 = tile * (TWO ? 64 : 128);
     const int nblk = A.kdim / kBlockK, k_lo = (int)((uint32_t)(rank * nblk) * A.inv_s >> 16), n = (int)((uint32_t)((rank + 1) * nblk) * A.inv_s >> 16) - k_lo;
     const int na = A.na, nb = A.nb;
-    const int qps = A.tps >> 2, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
+    const bool flat = na >= n && nb >= n;      // every block has a place of its own: the activations count on one barrier, nothing is given back
+    const int qps = A.tps / G, m0 = rank * A.tps, nm = min(A.tps, rows - m0);      // token rows that this CTA finishes (nm may be <= 0)
     const uint32_t b_bytes = (uint32_t)(2 * Nt) * kBlockK * 2u, b_pitch = (uint32_t)(2 * A.tok) * kBlockK * 2u;
     // operand rings; behind them (one CTA to a tile: in their place, when the products are done) the partial sums
     const uint32_t sa = smem_u32(smem), sb = sa + (uint32_t)na * kABytes, srecv = CL ? sb + (uint32_t)nb * b_pitch : sa;
@@ -98,11 +104,11 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     } else if (warp == 1) {
         if (lane < nb) { mbar_init(bar(2, lane), 1u); mbar_init(bar(3, lane), 1u); }
         if (lane == 31) {
-            mbar_init(done, 1u);
+            mbar_init(done, kThreads / 32 - 1);      // the last products, and what the epilogue needs to know (warps 2 and up)
             mbar_init(smem_u32(&recv_bar), 1u);
         }
         mbar_init_fence();
-        if (CL && lane == 31 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + 3) >> 2)) * 2048u);
+        if (CL && lane == 31 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + G - 1) / G)) * (512u * G));
     } else if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -122,31 +128,33 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     constexpr int ROWS = TWO ? 64 : 128, SIDES = kThreads / ROWS;
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
     const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
-    const bool live_row = u_row < G.units;
+    const bool live_row = u_row < W.units;
     const uint32_t gain_bits = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? ld_early_u16(reinterpret_cast<const bf16 *>(A.gain) + u_row) : 0u;
     // where this thread's weight row goes
     const int sec = EPI0 == PE_QKV ? (u_row >= D.d ? (u_row >= 2 * D.d ? 2 : 1) : 0) : 0, col = u_row - sec * D.d, head = EPI0 == PE_QKV ? col >> (31 - __clz(D.dh)) : 0;      // (d_head is 32, 64 or 128)
     __half *qrow = A.q + ((size_t)job * 2 * A.qp + mb) * D.d + (EPI0 == PE_QKV ? col : u_row);
-    bf16 *xrow = G.out + (size_t)(job + plane) * 2 * Mp * G.ld + (size_t)(u_row >> 6) * (128 * Mp) + (size_t)pm * 128 + (u_row & 7);
+    bf16 *xrow = W.out + (size_t)(job + plane) * 2 * Mp * W.ld + (size_t)(u_row >> 6) * (128 * Mp) + (size_t)pm * 128 + (u_row & 7);
     const int xchunk = (u_row >> 3) & 7;
-    float *lrow = G.logits + ((size_t)job * D.M + mb) * G.ld + u_row;
+    float *lrow = W.logits + ((size_t)job * D.M + mb) * W.ld + u_row;
     __half *crow = reinterpret_cast<__half *>(D.kv_pool) + ((size_t)(A.layer * 2 + (sec == 2 ? 1 : 0)) * D.n_pages * D.H + head) * (size_t)D.P * D.dh + (e & 7);
     settle(qrow); settle(xrow); settle(lrow); settle(crow);
-    // Accumulator -> the CTA that finishes the token rows: [sender][quad][weight row][4].  This thread's lane of the accumulator
+    // Accumulator -> the CTA that finishes the token rows: [sender][group][weight row][G].  This thread's lane of the accumulator
     // is its weight row; eight token rows at a time, from c0 on.
+    constexpr int GROUPS = 8 / G;
     const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = warp >> 2;
     const uint32_t recv_b = smem_u32(&recv_bar);
-    uint32_t dst[2], dst_bar[2];
+    uint32_t dst[GROUPS], dst_bar[GROUPS];
     auto where = [&](int c) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int quad = 2 * c + q, owner = (int)((uint32_t)quad * A.inv_q >> 16), place = rank * qps + quad - owner * qps;      // (quad / qps: both are below 33)
-            dst[q] = CL ? map_rank(srecv + (uint32_t)(place * 128 + arow) * 16u, (uint32_t)min(owner, S - 1)) : (uint32_t)(quad * 128 + arow) * 16u;
+        for (int q = 0; q < GROUPS; ++q) {
+            const int group = GROUPS * c + q, owner = (int)((uint32_t)group * A.inv_q >> 16), place = rank * qps + group - owner * qps;      // (group / qps: both are below 33)
+            dst[q] = CL ? map_rank(srecv + (uint32_t)(place * 128 + arow) * (4u * G), (uint32_t)min(owner, S - 1)) : (uint32_t)(group * 128 + arow) * (4u * G);
             dst_bar[q] = CL ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;
         }
     };
     where(c0);
-    settle(dst[0]); settle(dst[1]); settle(dst_bar[0]); settle(dst_bar[1]);
+#pragma unroll
+    for (int q = 0; q < GROUPS; ++q) { settle(dst[q]); settle(dst_bar[q]); }
     tcgen05_before_sync();
     if (CL) cluster_wait();            // the peers run: their barriers and shared memory are there
     else __syncthreads();
@@ -165,15 +173,20 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     trace_mark(D, 1 + 2 * A.stage);
     if (warp == 0) {
         // (written by ordinary stores of an earlier kernel, which has completed: nothing to order)
+        if (flat) {
+            if (lane == 0) mbar_arrive_expect_tx(full_b, (uint32_t)n * b_bytes);
+            __syncwarp();
+        }
         if (lane < min(n, nb)) {
-            mbar_arrive_expect_tx(full_b + 8u * (uint32_t)lane, b_bytes);
-            bulk_g2s(sb + (uint32_t)lane * b_pitch, xb + (size_t)lane * (128 * Mp), b_bytes, full_b + 8u * (uint32_t)lane);
+            const uint32_t f = flat ? full_b : full_b + 8u * (uint32_t)lane;
+            if (!flat) mbar_arrive_expect_tx(f, b_bytes);
+            bulk_g2s(sb + (uint32_t)lane * b_pitch, xb + (size_t)lane * (128 * Mp), b_bytes, f);
         }
         __syncwarp();
         if (elect_one()) {
             int slot = 0, a_slot = 0;
             uint32_t par = 0u, a_par = 0u;
-            for (int i = min(na, nb); i < n; ++i) {
+            for (int i = flat ? n : min(na, nb); i < n; ++i) {
                 if (i >= nb) {
                     mbar_wait(bar(3, slot), par, D.mbar_limit, D.status);
                     mbar_arrive_expect_tx(full_b + 8u * (uint32_t)slot, b_bytes);
@@ -192,22 +205,35 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         // (the whole warp waits and one elected lane issues: a branch on the thread's number would keep the descriptors out of the
         // uniform registers that the instruction takes them from)
         const bool leader = elect_one();
-        int ia = 0, ib = 0;
-        uint32_t pa = 0u, pb = 0u;
-        for (int i = 0; i < n; ++i) {
-            mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
-            mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
-            tcgen05_after_sync();
-            if (leader) {
-            const uint64_t da = umma_desc_sw128(sa + (uint32_t)ia * kABytes), db = umma_desc_sw128(sb + (uint32_t)ib * b_pitch);
+        const uint64_t da = umma_desc_sw128(sa), db = umma_desc_sw128(sb);
+        auto products = [&](int i, int ia, int ib) {
+            const uint64_t a = da + (uint64_t)(ia * (kABytes >> 4)), b = db + (uint64_t)((uint32_t)ib * (b_pitch >> 4));
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, da + 2 * ks, db + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
-            if (i + na < n) umma_commit(bar(1, ia));
-            if (i + nb < n) umma_commit(bar(3, ib));
+            for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, a + 2 * ks, b + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
+        };
+        if (flat) {
+            mbar_wait(full_b, 0u, D.mbar_limit, D.status);
+            for (int i = 0; i < n; ++i) {
+                mbar_wait(full_a + 8u * (uint32_t)i, 0u, D.mbar_limit, D.status);
+                tcgen05_after_sync();
+                if (leader) products(i, i, i);
             }
-            __syncwarp();
-            if (++ia == na) { ia = 0; pa ^= 1u; }
-            if (++ib == nb) { ib = 0; pb ^= 1u; }
+        } else {
+            const uint32_t empty_a = bar(1, 0), empty_b = bar(3, 0);
+            int ia = 0, ib = 0;
+            uint32_t pa = 0u, pb = 0u;
+            for (int i = 0; i < n; ++i) {
+                mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
+                mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
+                tcgen05_after_sync();
+                if (leader) {
+                    products(i, ia, ib);
+                    if (i + na < n) umma_commit(empty_a + 8u * (uint32_t)ia);
+                    if (i + nb < n) umma_commit(empty_b + 8u * (uint32_t)ib);
+                }
+                if (++ia == na) { ia = 0; pa ^= 1u; }
+                if (++ib == nb) { ib = 0; pb ^= 1u; }
+            }
         }
         if (leader) umma_commit(done);
         __syncwarp();
@@ -240,19 +266,20 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     // of four, which lie side by side in shared memory (one 16-byte load for each sender; four single ones met four-way bank
     // conflicts, half of an epilogue's time at 80 token rows); what it reads from memory is requested before the products
     // are waited for, or a round ahead.
-    float hn[4];
-    float2 csn[4];
-    auto request = [&](int quad) {
+    float hn[G];
+    float2 csn[G];
+    auto request = [&](int group) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = 4 * quad + q;
+        for (int q = 0; q < G; ++q) {
+            const int i = G * group + q;
             if ((EPI0 == PE_ADD || HEAD) && i < nm && live_row && u_row < D.d) hn[q] = __ldcg(D.h + (size_t)(mb + m0 + i) * D.d + u_row);
             if (EPI0 == PE_QKV && i < nm) csn[q] = __ldcg(D.row_cs + (size_t)(mb + m0 + i) * half + (e < half ? e : e - half));
         }
     };
+    __syncwarp();
+    if (warp >= 2 && lane == 0) mbar_arrive(done);
     const float gain = __uint_as_float(gain_bits << 16);
     request(side);
-    __syncthreads();      // (what the epilogue needs is in shared memory; the last products are under way)
     const bool done_ok = mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
     tcgen05_after_sync();
@@ -262,13 +289,17 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         if (c != c0) where(c);
         tmem_wait_ld();
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if ((2 * c + q) * 4 < rows) {
-                float f[4];
+        for (int q = 0; q < GROUPS; ++q) {
+            if ((GROUPS * c + q) * G < rows) {
+                float f[G];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) f[j] = __uint_as_float(v[4 * q + j]) + __uint_as_float(v[8 + 4 * q + j]);
-                if (!CL) *reinterpret_cast<float4 *>(smem + (srecv - sa) + dst[q]) = make_float4(f[0], f[1], f[2], f[3]);
-                else if (done_ok) st_async_v4(dst[q], f, dst_bar[q]);      // (a peer that gave up waiting may have left)
+                for (int j = 0; j < G; ++j) f[j] = __uint_as_float(v[G * q + j]) + __uint_as_float(v[8 + G * q + j]);
+                if constexpr (G == 1) {
+                    if (done_ok) st_async_f32(dst[q], f[0], dst_bar[q]);      // (a peer that gave up waiting may have left)
+                } else {
+                    if (!CL) *reinterpret_cast<float4 *>(smem + (srecv - sa) + dst[q]) = make_float4(f[0], f[1], f[2], f[3]);
+                    else if (done_ok) st_async_v4(dst[q], f, dst_bar[q]);
+                }
             }
         }
     }
@@ -279,15 +310,25 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     else if (nm > 0 && !mbar_wait(recv_b, 0u, D.mbar_limit, D.status)) mbar_wait(recv_b, 0u, D.mbar_limit, D.status);
     __syncwarp();
     // sums over the cluster in rank order, epilogue
-    auto total = [&](int quad, int r, float (&v)[4]) {
-        const float4 *p = reinterpret_cast<const float4 *>(recv) + quad * 128 + r;
+    auto total = [&](int group, int r, float (&v)[G]) {
         constexpr int kMost = CL ? 8 : 1;
-        float4 part[kMost];
+        if constexpr (G == 1) {
+            const float *p = recv + group * 128 + r;
+            float part[kMost];
 #pragma unroll
-        for (int s = 0; s < kMost; ++s) part[s] = s < S ? p[s * qps * 128] : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int s = 0; s < kMost; ++s) part[s] = s < S ? p[s * qps * 128] : 0.f;
+            v[0] = part[0];
 #pragma unroll
-        for (int s = 1; s < kMost; ++s) { part[0].x += part[s].x; part[0].y += part[s].y; part[0].z += part[s].z; part[0].w += part[s].w; }
-        v[0] = part[0].x; v[1] = part[0].y; v[2] = part[0].z; v[3] = part[0].w;
+            for (int s = 1; s < kMost; ++s) v[0] += part[s];
+        } else {
+            const float4 *p = reinterpret_cast<const float4 *>(recv) + group * 128 + r;
+            float4 part[kMost];
+#pragma unroll
+            for (int s = 0; s < kMost; ++s) part[s] = s < S ? p[s * qps * 128] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int s = 1; s < kMost; ++s) { part[0].x += part[s].x; part[0].y += part[s].y; part[0].z += part[s].z; part[0].w += part[s].w; }
+            v[0] = part[0].x; v[1] = part[0].y; v[2] = part[0].z; v[3] = part[0].w;
+        }
     };
     auto put_x = [&](int m, float v) {
         bf16 hi, lo;
@@ -302,21 +343,21 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         qrow[(size_t)m * D.d] = hi;
         qrow[(size_t)(A.qp + m) * D.d] = lo;
     };
-    for (int quad = side; 4 * quad < nm; quad += SIDES) {
-        float h[4];
-        float2 cs[4];
+    for (int group = side; G * group < nm; group += SIDES) {
+        float h[G];
+        float2 cs[G];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
-        request(quad + SIDES);
-        float sum[4], other[4];      // other: the rotation partner's, or up's
-        total(quad, row, sum);
-        if (TWO) total(quad, row + 64, other);
-        if (EPI0 == PE_QKV) total(quad, e < half ? row + half : row - half, other);
+        for (int q = 0; q < G; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
+        request(group + SIDES);
+        float sum[G], other[G];      // other: the rotation partner's, or up's
+        total(group, row, sum);
+        if (TWO) total(group, row + 64, other);
+        if (EPI0 == PE_QKV) total(group, e < half ? row + half : row - half, other);
         if (EPI0 == PE_ADD) {
-            float o[4];
+            float o[G];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = 4 * quad + q, m = m0 + i;
+            for (int q = 0; q < G; ++q) {
+                const int i = G * group + q, m = m0 + i;
                 o[q] = live_row && i < nm ? h[q] + sum[q] : 0.f;
                 if (live_row && i < nm) {
                     D.h[(size_t)(mb + m) * D.d + u_row] = o[q];
@@ -324,22 +365,27 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
                 }
                 o[q] *= o[q];
             }
-            // the warp's sums of the four rows: a lane keeps two of them after the first exchange, one after the second (six
-            // shuffles instead of twenty, 38 cycles each); lane 8 r has row r
-            const bool up = lane & 16, mid = lane & 8;
-            float a = up ? o[2] : o[0], b = up ? o[3] : o[1];
-            a += __shfl_xor_sync(0xffffffffu, up ? o[0] : o[2], 16);
-            b += __shfl_xor_sync(0xffffffffu, up ? o[1] : o[3], 16);
-            float v = mid ? b : a;
-            v += __shfl_xor_sync(0xffffffffu, mid ? a : b, 8);
+            if constexpr (G == 1) {
+                const float v = warp_sum(o[0]);
+                if (lane == 0) D.ss[(size_t)(mb + m0 + group) * kShareLd + tile * 4 + (row >> 5)] = v;
+            } else {
+                // the warp's sums of the four rows: a lane keeps two of them after the first exchange, one after the second (six
+                // shuffles instead of twenty, 38 cycles each); lane 8 r has row r
+                const bool up = lane & 16, mid = lane & 8;
+                float a = up ? o[2] : o[0], b = up ? o[3] : o[1];
+                a += __shfl_xor_sync(0xffffffffu, up ? o[0] : o[2], 16);
+                b += __shfl_xor_sync(0xffffffffu, up ? o[1] : o[3], 16);
+                float v = mid ? b : a;
+                v += __shfl_xor_sync(0xffffffffu, mid ? a : b, 8);
 #pragma unroll
-            for (int k = 4; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
-            const int i = 4 * quad + (lane >> 3);
-            if ((lane & 7) == 0 && i < nm) D.ss[(size_t)(mb + m0 + i) * kShareLd + tile * 4 + (row >> 5)] = v;
+                for (int k = 4; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
+                const int i = G * group + (lane >> 3);
+                if ((lane & 7) == 0 && i < nm) D.ss[(size_t)(mb + m0 + i) * kShareLd + tile * 4 + (row >> 5)] = v;
+            }
         } else
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = 4 * quad + q, m = m0 + i;
+        for (int q = 0; q < G; ++q) {
+            const int i = G * group + q, m = m0 + i;
             if (i >= nm) break;
             const float v = sum[q];
             if (live_row) {
@@ -357,7 +403,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
                 } else if (EPI1 == PE_HEADY && grp == 1) {
                     put_x(m, h[q] * inv * gain + silu_f(x1));
                 } else {
-                    lrow[(size_t)m * G.ld] = A.norm ? x1 : v;
+                    lrow[(size_t)m * W.ld] = A.norm ? x1 : v;
                 }
             }
         }
@@ -376,13 +422,19 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     }
 }
 
-template <int EPI0, int EPI1, bool CL>
+template <int EPI0, int EPI1, bool CL, int G>
 static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
-    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL>;
+    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL, G>;
     cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
     return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? kClusterThreads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
+}
+
+template <int EPI0, int EPI1>
+static cudaError_t launch_cut(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
+    if (A.S == 1) return launch_instance<EPI0, EPI1, false, 4>(D, A, T, smem, L);
+    return A.group == 1 ? launch_instance<EPI0, EPI1, true, 1>(D, A, T, smem, L) : launch_instance<EPI0, EPI1, true, 4>(D, A, T, smem, L);
 }
 
 // (asked for once per device: the answer does not change, and asking takes longer than the rest of a context's creation)
@@ -391,7 +443,7 @@ int resident_clusters(int size) {
     int dev = 0;
     if (size < 2 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
     if (const int k = known[dev][size].load()) return k - 1;
-    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1, true>;
+    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1, true, 4>;
     constexpr int smem = 200 * 1024;
     int n = 0;
     cudaLaunchConfig_t c = {};
@@ -414,7 +466,7 @@ int resident_clusters(int size) {
 
 cudaError_t launch_proj_umma(const Dev &D, const ProjArgs &A, const void *maps, int smem, const ChainLaunch &L) {
     const ProjMaps &T = *reinterpret_cast<const ProjMaps *>(maps);
-#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return A.S > 1 ? launch_instance<a, b, true>(D, A, T, smem, L) : launch_instance<a, b, false>(D, A, T, smem, L)
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_cut<a, b>(D, A, T, smem, L)
     XSM_EPI(PE_QKV, -1);
     XSM_EPI(PE_ADD, -1);
     XSM_EPI(PE_QUERY, -1);
