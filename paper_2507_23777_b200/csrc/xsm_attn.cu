@@ -177,6 +177,43 @@ __device__ __forceinline__ void rows_unit(const unsigned (&qh)[DH / 16][4], cons
     }
 }
 
+// n partial results of a row, `step` floats apart, as one: columns c and c + 1 of [columns .., maximum, sum].  Eight at a time,
+// all their loads together (one by one, each behind the last one's: large model, batch 1 1680 -> 1648 us a step).
+__device__ __forceinline__ void merge_states(const float *src, int dh, int c, int n, int step, float &m, float &l, float &o0, float &o1) {
+    m = kNegBig;
+    l = o0 = o1 = 0.f;
+#pragma unroll 1
+    for (; n > 0; n -= 8, src += 8 * step) {
+        float mv[8], lv[8];
+        float2 ov[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            mv[w] = kNegBig;
+            lv[w] = 0.f;
+            ov[w] = make_float2(0.f, 0.f);
+            if (w < n) {
+                const float2 ml = *reinterpret_cast<const float2 *>(src + w * step + dh);
+                mv[w] = ml.x;
+                lv[w] = ml.y;
+                ov[w] = *reinterpret_cast<const float2 *>(src + w * step + c);
+            }
+        }
+        const float before = m;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) m = fmaxf(m, mv[w]);
+        const float f0 = ex2(before - m);
+        l *= f0; o0 *= f0; o1 *= f0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+            if (w < n) {
+                const float f = ex2(mv[w] - m);
+                o0 += f * ov[w].x;
+                o1 += f * ov[w].y;
+                l += f * lv[w];
+            }
+    }
+}
+
 // ------------------------------------------------------------------------------------------- kernel
 
 __device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(reinterpret_cast<const unsigned *>(p)); }
@@ -297,32 +334,32 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
         };
         bool scaled = !QP;
-        if (lane == 0 || QP) {
-            const int n_old = cross ? np : page_of(D, first);         // pages that nobody writes in this step
-            bool waited = false;
-            for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
-                const int sl = all_in ? i : i % slots, rows = all_in && pg == p_hi - 1 ? last_rows : P;
-                const uint32_t part = (uint32_t)rows * RB;
-                if (QP && !all_in && i == slots) {      // (due before a slot is free again)
-                    scales();
-                    scaled = true;
-                }
-                if (QP && lane != 0) continue;
-                if (!all_in && i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
-                const int page = cross ? b * D.cpages + pg : __ldcg(D.block_table + (size_t)b * D.max_blocks + pg);
-                const int pool_pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
-                const __half *kt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 0, page, h);
-                const __half *vt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 1, page, h);
-                uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
-                mbar_arrive_expect_tx(f, 2u * part);
-                if (!waited && pg >= n_old) {
-                    settle(kt); settle(vt); settle(f); settle(dst);
-                    chain_wait();
-                    waited = true;
-                }
-                bulk_g2s(dst, kt, part, f);
-                bulk_g2s(dst + part, vt, part, f);
+        const int n_old = cross ? np : page_of(D, first);         // pages that nobody writes in this step
+        bool waited = false;
+        int looked_up = 0;      // page p_lo + i with i % 32 == lane (one after the other the look-ups took 0.4 us each)
+        for (int i = 0, pg = p_lo; pg < p_hi; ++pg, ++i) {
+            if (!cross && (i & 31) == 0) looked_up = pg + lane < p_hi ? __ldcg(D.block_table + (size_t)b * D.max_blocks + pg + lane) : 0;
+            const int page = cross ? b * D.cpages + pg : __shfl_sync(0xffffffffu, looked_up, i & 31);
+            const int sl = all_in ? i : i % slots, rows = all_in && pg == p_hi - 1 ? last_rows : P;
+            const uint32_t part = (uint32_t)rows * RB;
+            if (QP && !all_in && i == slots) {      // (due before a slot is free again)
+                scales();
+                scaled = true;
             }
+            if (lane != 0) continue;
+            if (!all_in && i >= slots) mbar_wait(smem_u32(&empty[sl]), (uint32_t)((i / slots - 1) & 1), D.mbar_limit, D.status);
+            const int pool_pages = cross ? D.B * D.cpages : D.n_pages, lay = cross && A.sets > 1 ? set : A.layer;
+            const __half *kt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 0, page, h);
+            const __half *vt = kv_tile<__half>(D, const_cast<void *>(A.pool), pool_pages, lay, 1, page, h);
+            uint32_t f = smem_u32(&full[sl]), dst = ring + (uint32_t)sl * 2u * tile_bytes;
+            mbar_arrive_expect_tx(f, 2u * part);
+            if (!waited && pg >= n_old) {
+                settle(kt); settle(vt); settle(f); settle(dst);
+                chain_wait();
+                waited = true;
+            }
+            bulk_g2s(dst, kt, part, f);
+            bulk_g2s(dst + part, vt, part, f);
         }
         __syncwarp();
         if (!scaled) scales();
@@ -524,16 +561,8 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
     };
     for (int e = tid; e < n_pairs; e += kThreads) {
         const int r = e / (DH / 2), c = (e - r * (DH / 2)) * 2;
-        const float *src = st + r * LD;                   // (row r of a row tile: the tiles of the first kg follow each other)
-        float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
-        for (int w = 0; w < states; ++w) m = fmaxf(m, src[w * step + DH]);
-        for (int w = 0; w < states; ++w) {
-            const float f = ex2(src[w * step + DH] - m);
-            const float2 o = *reinterpret_cast<const float2 *>(src + w * step + c);
-            o0 += f * o.x;
-            o1 += f * o.y;
-            l += f * src[w * step + DH + 1];
-        }
+        float m, o0, o1, l;
+        merge_states(st + r * LD, DH, c, states, step, m, l, o0, o1);      // (row r of a row tile: the tiles of the first kg follow each other)
         if (!CL || S == 1) {
             const float inv = 1.f / l;
             store(r, c, o0 * inv, o1 * inv);
@@ -553,17 +582,8 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
         __syncwarp();
         for (int e = tid; e < my_rows * (DH / 2); e += kThreads) {
             const int i = e / (DH / 2), c = (e - i * (DH / 2)) * 2;
-            const float *src = recv + i * LD;
-            float m = kNegBig, o0 = 0.f, o1 = 0.f, l = 0.f;
-            for (int s = 0; s < S; ++s) m = fmaxf(m, src[s * my_rows * LD + DH]);
-            for (int s = 0; s < S; ++s) {
-                const float *p = src + s * my_rows * LD;
-                const float f = ex2(p[DH] - m);
-                const float2 o = *reinterpret_cast<const float2 *>(p + c);
-                o0 += f * o.x;
-                o1 += f * o.y;
-                l += f * p[DH + 1];
-            }
+            float m, o0, o1, l;
+            merge_states(recv + i * LD, DH, c, S, my_rows * LD, m, l, o0, o1);
             const float inv = 1.f / l;
             store(rank + i * S, c, o0 * inv, o1 * inv);
         }
