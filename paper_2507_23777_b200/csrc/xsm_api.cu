@@ -32,6 +32,9 @@ struct Layout {
 
 size_t esize(const xsm_model_config &c) { return c.dtype == 1 ? 2 : 4; }
 
+// elements from one row of logits to the next (the tail copies rows in 16-byte pieces)
+size_t logits_ld(const xsm_model_config &c) { return ((size_t)c.vocab + 3) / 4 * 4; }
+
 size_t take(size_t &cur, size_t bytes) {
     size_t o = cur;
     cur = (cur + bytes + 255) / 256 * 256;
@@ -40,8 +43,8 @@ size_t take(size_t &cur, size_t bytes) {
 
 // workspace_bytes == 0: size the pool for max_batch full sequences
 bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
-    const size_t B = c.max_batch, K1 = c.n_draft + 1, M = B * K1, d = c.d_model, V = c.vocab, f = c.d_ff;
-    const size_t P = c.page_size, H = c.n_heads, dh = c.d_head;
+    const size_t B = c.max_batch, K1 = c.n_draft + 1, M = B * K1, d = c.d_model, f = c.d_ff;
+    const size_t P = c.page_size, H = c.n_heads, dh = c.d_head, ldv = logits_ld(c);
     L.max_blocks = (int)((c.max_seq_len + K1 + P - 1) / P);
     L.cpages = (int)((c.n_cond + P - 1) / P);
     L.tok_ld = c.max_seq_len + (int)K1;
@@ -82,8 +85,8 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.hq = take(cur, step_row * d * nh);
     L.ha = take(cur, step_row * d * nh);
     L.ss = take(cur, row * kShareLd);
-    L.logits0 = take(cur, 4 * M * V);
-    L.hlogits = take(cur, 4 * M * V * (c.n_draft > 0 ? c.n_draft : 1));
+    L.logits0 = take(cur, 4 * M * ldv);
+    L.hlogits = take(cur, 4 * M * ldv * (c.n_draft > 0 ? c.n_draft : 1));
     L.stage_cond = take(cur, esize(c) * B * c.n_cond * c.d_cond);
     L.stage_kv = take(cur, 4 * 2 * (size_t)kKvStagePositions * d);
     L.stage_tok = take(cur, 4 * B * (c.max_seq_len + 1));
@@ -356,7 +359,7 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     Dev &D = ctx->dev;
     memset(&D, 0, sizeof(D));
     D.L = cfg->n_layers; D.d = cfg->d_model; D.H = cfg->n_heads; D.dh = cfg->d_head; D.f = cfg->d_ff;
-    D.V = cfg->vocab; D.C = cfg->n_cond; D.dc = cfg->d_cond; D.K = cfg->n_draft; D.K1 = cfg->n_draft + 1;
+    D.V = cfg->vocab; D.ldv = (int)logits_ld(*cfg); D.C = cfg->n_cond; D.dc = cfg->d_cond; D.K = cfg->n_draft; D.K1 = cfg->n_draft + 1;
     D.P = cfg->page_size; D.max_blocks = L.max_blocks; D.n_pages = L.n_pages; D.cpages = L.cpages;
     D.p_shift = -1;
     for (int sh = 0; sh < 30; ++sh)
@@ -382,7 +385,6 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
     D.row_info = at<RowInfo>(ctx, L.row_info); D.row_cs = at<float2>(ctx, L.row_cs);
     D.xa_ = ctx->ws + L.xa; D.qp_ = ctx->ws + L.qp; D.aa_ = ctx->ws + L.aa; D.actp_ = ctx->ws + L.actp;
     D.yp_ = ctx->ws + L.yp; D.hq_ = ctx->ws + L.hq; D.ha_ = ctx->ws + L.ha; D.ss = at<float>(ctx, L.ss);
-    D.tail_row_bytes = 160 * 1024;
     D.logits0 = at<float>(ctx, L.logits0); D.hlogits = at<float>(ctx, L.hlogits);
     D.kv_pool = ctx->ws + L.kv_pool; D.ckv_pool = ctx->ws + L.ckv_pool; D.hckv_pool = ctx->ws + L.hckv_pool;
     *out = ctx;
@@ -578,9 +580,9 @@ xsm_status xsm_debug_get_logits(xsm_ctx *ctx, float *h_logits0, float *h_head_lo
     xsm_status st = check_device_status(ctx);
     if (st != XSM_OK) return st;
     if (h_logits0)
-        XSM_CUDA(ctx, cudaMemcpy(h_logits0, D.logits0, sizeof(float) * (size_t)D.M * D.V, cudaMemcpyDeviceToHost));
+        XSM_CUDA(ctx, cudaMemcpy2D(h_logits0, sizeof(float) * D.V, D.logits0, sizeof(float) * D.ldv, sizeof(float) * D.V, D.M, cudaMemcpyDeviceToHost));
     if (h_head_logits && D.K > 0)
-        XSM_CUDA(ctx, cudaMemcpy(h_head_logits, D.hlogits, sizeof(float) * (size_t)D.K * D.M * D.V, cudaMemcpyDeviceToHost));
+        XSM_CUDA(ctx, cudaMemcpy2D(h_head_logits, sizeof(float) * D.V, D.hlogits, sizeof(float) * D.ldv, sizeof(float) * D.V, (size_t)D.K * D.M, cudaMemcpyDeviceToHost));
     return XSM_OK;
 }
 

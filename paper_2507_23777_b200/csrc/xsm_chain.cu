@@ -345,7 +345,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     {
         ChainOp &op = proj(PE_LOGITS, K == 0 ? -1 : ca ? PE_QUERY : PE_HEADY, 0, lm_, K > 0 ? &head_in_ : nullptr, w_.W0,
                             K == 0 ? 0 : ca ? w_.hq[0] : w_.W1[0], D.xa_);
-        group(op.proj.g[0], V, 128, 1, V, nullptr, D.logits0);
+        group(op.proj.g[0], V, 128, 1, D.ldv, nullptr, D.logits0);
         if (K > 0) group(op.proj.g[1], d, 128, K, d, D.yp_, nullptr);
         op.proj.gain = gain(w_.gf);
         op.proj.q = (__half *)D.hq_;
@@ -362,7 +362,7 @@ bool Chain::build(const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
     }
     if (K > 0) {
         ChainOp &op = proj(PE_LOGITS, -1, 0, head_out_, nullptr, w_.Wout[0], 0, D.yp_);
-        group(op.proj.g[0], V, 128, K, V, nullptr, D.hlogits);
+        group(op.proj.g[0], V, 128, K, D.ldv, nullptr, D.hlogits);
         op.proj.z_jobs = op.proj.x_jobs = 1;
         plan_proj(op, rows, Mp, d);
     }

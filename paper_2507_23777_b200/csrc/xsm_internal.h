@@ -36,6 +36,7 @@ struct __align__(16) RowInfo {
 struct Dev {
     // shape
     int L, d, H, dh, f, V, C, dc, K, K1, B, M, P;
+    int ldv;                       // V rounded up to four: rows of logits are copied in 16-byte pieces
     int max_blocks, n_pages, cpages, max_seq_len, tok_ld;
     int p_shift;                   // log2 of the page size P if that is a power of two, else -1
     int head_kind;
@@ -56,12 +57,12 @@ struct Dev {
     int *stage_word;               // single stages (inspection): stages of the current step that have run
     // activations: bf16 models as hi and lo planes of Mp rows (layout: xsm_proj.cuh), queries fp16 [2][Mp][d]; fp32 models
     // [row][column]
-    int Mp, tail_row_bytes;        // rows of a plane for a step of the batch; largest logits row that the tail keeps in shared memory
+    int Mp;                        // rows of a plane for a step of the batch
     void *xa_;                     // the residual stream times the gain of the RMSNorm that reads it next
     void *qp_, *aa_, *actp_, *yp_; // queries, attention rows, gated activations, decoding heads' hidden states (a set per head)
     void *hq_, *ha_;               // cross-attention heads: queries, attention rows (a set per head)
     float *ss;                     // [row][kShareLd] shares of the sums of squares of the rows of h
-    float *logits0, *hlogits;      // [M][V], [K][M][V]
+    float *logits0, *hlogits;      // [M][ldv], [K][M][ldv]
     float *h;                      // residual stream [row][d]
     RowInfo *row_info;             // [row]; with row_cs written when the row is embedded, so that nobody else looks up positions and pages
     float2 *row_cs;                // [row][dh/2] cos, sin of the row's position

@@ -4,7 +4,9 @@
 
 namespace xsm {
 
-constexpr int kTailThreads = 256, kTailWarps = kTailThreads / 32;
+constexpr int kTailThreads = 512, kTailWarps = kTailThreads / 32, kEmbedThreads = 256;
+constexpr int kTailSmem = 200 * 1024;          // logits rows that the tail keeps in shared memory, at most
+enum TailRows : int { kRowsAll = 0, kRowsOne = 1, kRowsNone = 2 };
 constexpr int kMaxCand = 64;
 
 __device__ __forceinline__ uint32_t rand24(const RunParams &R, int seq, uint32_t step, uint32_t slot, uint32_t purpose) {
@@ -22,53 +24,59 @@ static __device__ void place_row(const Dev &D, int m, int b, int pos, bool live)
     D.row_info[m] = r;
 }
 
-// Row m of the window, at position pos, <- the embedding of `tok`: the position's cosines and sines, master copy, the copy that the first projection reads (times the gain of the
-// first RMSNorm) and its sum of squares.  All threads of the block, 16 bytes of a row each.
-template <typename WT> static __device__ void embed_row(const Dev &D, int m, int Mp, int tok, int pos, float *sh) {
+// 16 bytes of a row's embedding `e`, from column c on: master copy, the copy that the first projection reads (times the gain g
+// of the first RMSNorm); returns their sum of squares
+template <typename WT> static __device__ float embed_chunk(const Dev &D, int m, int Mp, int c, const uint4 &e_raw, const uint4 &g_raw) {
     constexpr int N = 16 / (int)sizeof(WT);
-    const WT *E = reinterpret_cast<const WT *>(D.E), *gain = reinterpret_cast<const WT *>(D.gain_first);
     const int d = D.d;
+    const WT *e = reinterpret_cast<const WT *>(&e_raw), *g = reinterpret_cast<const WT *>(&g_raw);
+    float v[N], ssq = 0.f;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        v[q] = to_f(e[q]);
+        ssq += v[q] * v[q];
+    }
+#pragma unroll
+    for (int q = 0; q < N; q += 4) *reinterpret_cast<float4 *>(D.h + (size_t)m * d + c + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+    if constexpr (sizeof(WT) == 2) {
+        __align__(16) bf16 hi[N], lo[N];
+#pragma unroll
+        for (int q = 0; q < N; ++q) split_bf16(v[q] * to_f(g[q]), hi[q], lo[q]);
+        bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + (size_t)(m / kTokenTile) * 2 * Mp * d + plane_off(Mp, m % kTokenTile, c);
+        *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
+        *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
+    } else {
+        *reinterpret_cast<float4 *>(reinterpret_cast<float *>(D.xa_) + (size_t)m * d + c) =
+            make_float4(v[0] * to_f(g[0]), v[1] * to_f(g[1]), v[2] * to_f(g[2]), v[3] * to_f(g[3]));
+    }
+    return ssq;
+}
+// 16 bytes of the embedding of `tok`, or of the gain of the first RMSNorm
+template <typename WT> static __device__ uint4 embedding(const Dev &D, int tok, int c) {
+    return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const WT *>(D.E) + (size_t)min(max(tok, 0), D.V - 1) * D.d + c));
+}
+template <typename WT> static __device__ uint4 first_gain(const Dev &D, int c) {
+    return __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const WT *>(D.gain_first) + c));
+}
+// the position's cosines and sines (first threads of the block), and the row's sum of squares from the threads' shares
+static __device__ void embed_position(const Dev &D, int m, int pos) {
     const int half = D.dh >> 1;
     if ((int)threadIdx.x < half) D.row_cs[(size_t)m * half + threadIdx.x] = __ldg(D.rope_cs + (size_t)pos * half + threadIdx.x);
-    float ssq = 0.f;
-    tok = min(max(tok, 0), D.V - 1);
-    for (int c = threadIdx.x * N; c < d; c += kTailThreads * N) {
-        __align__(16) WT e[N], g[N];
-        *reinterpret_cast<uint4 *>(e) = __ldg(reinterpret_cast<const uint4 *>(E + (size_t)tok * d + c));
-        *reinterpret_cast<uint4 *>(g) = __ldg(reinterpret_cast<const uint4 *>(gain + c));
-        float v[N];
-#pragma unroll
-        for (int q = 0; q < N; ++q) {
-            v[q] = to_f(e[q]);
-            ssq += v[q] * v[q];
-        }
-#pragma unroll
-        for (int q = 0; q < N; q += 4) *reinterpret_cast<float4 *>(D.h + (size_t)m * d + c + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-        if constexpr (sizeof(WT) == 2) {
-            __align__(16) bf16 hi[N], lo[N];
-#pragma unroll
-            for (int q = 0; q < N; ++q) split_bf16(v[q] * to_f(g[q]), hi[q], lo[q]);
-            bf16 *x = reinterpret_cast<bf16 *>(D.xa_) + (size_t)(m / kTokenTile) * 2 * Mp * d + plane_off(Mp, m % kTokenTile, c);
-            *reinterpret_cast<uint4 *>(x) = *reinterpret_cast<const uint4 *>(hi);
-            *reinterpret_cast<uint4 *>(x + kLo) = *reinterpret_cast<const uint4 *>(lo);
-        } else {
-            *reinterpret_cast<float4 *>(reinterpret_cast<float *>(D.xa_) + (size_t)m * d + c) =
-                make_float4(v[0] * to_f(g[0]), v[1] * to_f(g[1]), v[2] * to_f(g[2]), v[3] * to_f(g[3]));
-        }
-    }
+}
+template <int THREADS> static __device__ void embed_sum(const Dev &D, int m, float ssq, float *sh) {
     ssq = warp_sum(ssq);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ssq;
     __syncthreads();
     if (threadIdx.x == 0) {
         float s = 0.f;
-        for (int w = 0; w < kTailWarps; ++w) s += sh[w];
+        for (int w = 0; w < THREADS / 32; ++w) s += sh[w];
         D.ss[(size_t)m * kShareLd] = s;      // the only share
     }
 }
 
-template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0, int pos_end) {
-    __shared__ float sh[kTailWarps];
+template <typename WT> __global__ void __launch_bounds__(kEmbedThreads) embed_rows_kernel(const Dev D, int t, int Mp, int pos0, int pos_end) {
+    __shared__ float sh[kEmbedThreads / 32];
     chain_wait();
     chain_go();      // (only now: kernels further down may read what earlier chunks wrote before they wait themselves)
     const int b = blockIdx.x / t, j = blockIdx.x - b * t;
@@ -85,12 +93,16 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) embed_row
         tok = __ldcg(D.window + b * t + j);
     }
     if (threadIdx.x == 0) place_row(D, blockIdx.x, b, pos, live);
-    embed_row<WT>(D, blockIdx.x, Mp, tok, pos, sh);
+    constexpr int N = 16 / (int)sizeof(WT);
+    embed_position(D, blockIdx.x, pos);
+    float ssq = 0.f;
+    for (int c = threadIdx.x * N; c < D.d; c += kEmbedThreads * N) ssq += embed_chunk<WT>(D, blockIdx.x, Mp, c, embedding<WT>(D, tok, c), first_gain<WT>(D, c));
+    embed_sum<kEmbedThreads>(D, blockIdx.x, ssq, sh);
 }
 cudaError_t launch_embed_rows(const Dev &D, int dtype, int t, int pos0, int pos_end, const ChainLaunch &L) {
     const void *fn = dtype == 1 ? (const void *)embed_rows_kernel<bf16> : (const void *)embed_rows_kernel<float>;
     const int Mp = D.B * t > kTokenTile ? kTokenTile : (D.B * t + 7) / 8 * 8;
-    return L.launch(dim3(D.B * t), dim3(kTailThreads), 0, 1, fn, D, t, Mp, pos0, pos_end);
+    return L.launch(dim3(D.B * t), dim3(kEmbedThreads), 0, 1, fn, D, t, Mp, pos0, pos_end);
 }
 
 // ------------------------------------------------------------------------------------ block reductions
@@ -118,10 +130,12 @@ static __device__ float block_max(float v, float *sh) {
 }
 // (logit, token) as one 64-bit key whose unsigned order is the ranking: larger logit first, then smaller token.
 // 0 is below every key ("no candidate").  -0.0 ranks with +0.0.
-__device__ __forceinline__ unsigned long long rank_key(float z, int idx) {
-    uint32_t u = __float_as_uint(z + 0.0f);
-    u ^= (u & 0x80000000u) ? 0xFFFFFFFFu : 0x80000000u;
-    return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)idx);
+__device__ __forceinline__ uint32_t rank_bits(float z) {
+    const uint32_t u = __float_as_uint(z + 0.0f);
+    return u ^ ((uint32_t)((int)u >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long rank_key(uint32_t bits, int idx) {
+    return ((unsigned long long)bits << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)idx);
 }
 __device__ __forceinline__ float key_logit(unsigned long long k) {
     uint32_t u = (uint32_t)(k >> 32);
@@ -143,45 +157,19 @@ struct TailShared {
     unsigned long long best[kTailWarps * kMaxCand];      // the warps' ranked candidates
     float cv[kMaxCand], cw[kMaxCand];   // candidates, ranked: logits, sampling weights
     int ci[kMaxCand];
-    int accepted;                       // of the draft behind this CTA's row
+    int accepted[kMaxDraft];            // of the drafts (each CTA writes its own to all)
     int tok;                            // this slot's candidate
-    int cand[kMaxDraft], win[kMaxDraft];
+    int cand[kMaxDraft], win[kMaxDraft];      // cand: of all slots (each CTA writes its own to all)
+    uint32_t r24;                       // this slot's random number
+    int count, n_cand;                  // tokens ranked above the draft; tokens that may be among the best
     int old_win[kMaxDraft];
     int state[8];                       // len, n_gen, step_idx, n_blocks; new len, finished
     float tree_p[8];                    // probability tree: this head's best tokens
     int tree_t[8];
     double m[kMaxDraft * 8];            // the tree's tables (slot 1)
     int tk[kMaxDraft * 8];
-    int path[kMaxDraft];
 };
-
-// copies a logits row into shared memory, eight loads of a thread in flight
-static __device__ void stage_row(const float *z, float *row, int V) {
-    constexpr int N = 8;
-    __syncthreads();
-    if ((V & 3) == 0) {
-        for (int i0 = threadIdx.x; i0 < (V >> 2); i0 += N * kTailThreads) {
-            float4 v[N];
-#pragma unroll
-            for (int q = 0; q < N; ++q)
-                if (i0 + q * kTailThreads < (V >> 2)) v[q] = __ldcg(reinterpret_cast<const float4 *>(z) + i0 + q * kTailThreads);
-#pragma unroll
-            for (int q = 0; q < N; ++q)
-                if (i0 + q * kTailThreads < (V >> 2)) reinterpret_cast<float4 *>(row)[i0 + q * kTailThreads] = v[q];
-        }
-    } else {
-        for (int i0 = threadIdx.x; i0 < V; i0 += 2 * N * kTailThreads) {
-            float v[2 * N];
-#pragma unroll
-            for (int q = 0; q < 2 * N; ++q)
-                if (i0 + q * kTailThreads < V) v[q] = __ldcg(z + i0 + q * kTailThreads);
-#pragma unroll
-            for (int q = 0; q < 2 * N; ++q)
-                if (i0 + q * kTailThreads < V) row[i0 + q * kTailThreads] = v[q];
-        }
-    }
-    __syncthreads();
-}
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" :: "r"(addr), "r"(v) : "memory"); }
 
 // acceptance of token x under backbone logits z, block-wide; every thread returns the same answer
 static __device__ bool accept_token(const Dev &D, const RunParams &R, const float *z, int x, TailShared &sh) {
@@ -197,29 +185,84 @@ static __device__ bool accept_token(const Dev &D, const RunParams &R, const floa
         return expf(z[x] - m) / sum > R.delta;
     }
     const int ka = R.verify_mode == 0 ? 1 : R.k_accept;
-    const unsigned long long kx = rank_key(z[x], x);
+    const uint32_t ux = rank_bits(z[x]);
     int cnt = 0;
-    for (int v = threadIdx.x; v < V; v += kTailThreads) cnt += rank_key(z[v], v) > kx ? 1 : 0;
-    return (int)block_sum((float)cnt, sh.red) < ka;
+#pragma unroll 8
+    for (int v = threadIdx.x; v < V; v += kTailThreads) {
+        const uint32_t u = rank_bits(z[v]);
+        cnt += u > ux || (u == ux && v < x) ? 1 : 0;
+    }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&sh.count, cnt);
+    __syncthreads();
+    return sh.count < ka;
 }
 
-// the k best (logit, token) pairs of z, ranked, left in sh.cv, sh.ci: every warp ranks the k best of its share, the first warp
-// merges the lists (a pick is two warp reductions; block-wide picks with two barriers each took a microsecond for two)
-static __device__ void top_candidates(const Dev &D, const float *z, int k, TailShared &sh) {
+// The k best (logit, token) pairs of z, ranked, left in sh.cv, sh.ci.  Three to sixteen (one for each warp): the k-th largest of the
+// warps' maxima bounds the k-th best of all from below; what is not below it, a dozen or two as a rule, is listed and ranked by
+// counting.  False: too many are not below it (equal logits).
+static __device__ bool best_by_bound(const Dev &D, const float *z, int k, TailShared &sh) {
     const int V = D.V, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the two best of this thread's elements below `limit`
-    auto scan = [&](unsigned long long limit, unsigned long long &first, unsigned long long &second) {
-        first = second = 0ull;
+    uint32_t top = 0u;
+#pragma unroll 8
+    for (int v = threadIdx.x; v < V; v += kTailThreads) top = max(top, rank_bits(z[v]));
+    const uint32_t best = __reduce_max_sync(0xffffffffu, top);
+    uint32_t *maxima = reinterpret_cast<uint32_t *>(sh.cw);
+    if (lane == 0) maxima[warp] = best;
+    __syncthreads();
+    const uint32_t mine = lane < kTailWarps ? maxima[lane] : 0u;
+    int above = 0;
+#pragma unroll
+    for (int w = 0; w < kTailWarps; ++w) {
+        const uint32_t o = maxima[w];
+        above += o > mine || (o == mine && w < lane) ? 1 : 0;
+    }
+    const unsigned at = __ballot_sync(0xffffffffu, lane < kTailWarps && above == k - 1);
+    const uint32_t bound = __shfl_sync(0xffffffffu, mine, __ffs(at) - 1);
+    if (top >= bound)
         for (int v = threadIdx.x; v < V; v += kTailThreads) {
-            const unsigned long long kv = rank_key(z[v], v);
-            if (kv < limit) {
-                if (kv > first) { second = first; first = kv; }
-                else if (kv > second) second = kv;
+            const uint32_t u = rank_bits(z[v]);
+            if (u >= bound) {
+                const int n = atomicAdd(&sh.n_cand, 1);
+                if (n < kTailThreads) sh.best[n] = rank_key(u, v);
             }
         }
+    __syncthreads();
+    const int n = sh.n_cand;
+    if (n > kTailThreads) return false;
+    if ((int)threadIdx.x < n) {
+        const unsigned long long key = sh.best[threadIdx.x];
+        int rank = 0;
+        for (int i = 0; i < n; ++i) rank += sh.best[i] > key ? 1 : 0;
+        if (rank < k) { sh.cv[rank] = key_logit(key); sh.ci[rank] = key_token(key); }
+    }
+    __syncthreads();
+    return true;
+}
+// Any k: every warp ranks the k best of its share, the first warp merges the lists (a pick is two warp reductions; block-wide picks
+// with two barriers each took a microsecond for two).
+static __device__ void top_candidates(const Dev &D, const float *z, int k, TailShared &sh) {
+    if (k > 2 && k <= kTailWarps && k <= D.V && best_by_bound(D, z, k, sh)) return;
+    const int V = D.V, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the two best of this thread's elements below `limit` (its elements come in ascending order: of equal ones the first stays)
+    auto scan = [&](unsigned long long limit, unsigned long long &first, unsigned long long &second) {
+        const uint32_t ul = (uint32_t)(limit >> 32);
+        const int il = key_token(limit);
+        uint32_t u1 = 0u, u2 = 0u;
+        int i1 = -1, i2 = -1;
+#pragma unroll 8
+        for (int v = threadIdx.x; v < V; v += kTailThreads) {
+            const uint32_t u = rank_bits(z[v]);
+            if (u < ul || (u == ul && v > il)) {
+                if (u > u1 || i1 < 0) { u2 = u1; i2 = i1; u1 = u; i1 = v; }
+                else if (u > u2 || i2 < 0) { u2 = u; i2 = v; }
+            }
+        }
+        first = i1 < 0 ? 0ull : rank_key(u1, i1);
+        second = i2 < 0 ? 0ull : rank_key(u2, i2);
     };
     unsigned long long mine, next;
-    scan(~0ull, mine, next);
+    scan(0xFFFFFFFF00000000ull, mine, next);      // (all are below)
     bool known = true;                   // next is what follows mine
     for (int j = 0; j < k; ++j) {
         const unsigned long long win = warp_best(mine);
@@ -231,15 +274,15 @@ static __device__ void top_candidates(const Dev &D, const float *z, int k, TailS
     }
     __syncthreads();
     if (warp == 0) {
-        // lane l reads list l / 4, every fourth entry from l % 4 on
-        const unsigned long long *list = sh.best + (lane >> 2) * kMaxCand;
-        int at = lane & 3;
+        // lane l reads list l / 2, every second entry from l % 2 on
+        const unsigned long long *list = sh.best + (lane >> 1) * kMaxCand;
+        int at = lane & 1;
         unsigned long long head = at < k ? list[at] : 0ull;
         for (int j = 0; j < k; ++j) {
             const unsigned long long win = warp_best(head);
             if (lane == 0) { sh.cv[j] = key_logit(win); sh.ci[j] = key_token(win); }
             if (win == head) {
-                at += 4;
+                at += 2;
                 head = at < k ? list[at] : 0ull;
             }
         }
@@ -265,24 +308,23 @@ static __device__ int pick_candidate(const RunParams &R, int k, uint32_t r24, co
 // K_s^K paths in lexicographic order of the heads' ranked candidates, a path weighs the product of its tokens'
 // full-vocabulary probabilities, paths whose product falls below 1e-5 are pruned, and the first leaf whose cumulative
 // weight exceeds u * total is drawn (the last surviving leaf if rounding keeps the sum below; the most probable token of
-// every head if no path survives).  One warp; m: [K][8] in shared memory.  Returns the leaf's index.
-static __device__ int tree_pick(int K, int ks, const double *m, double u) {
+// every head if no path survives).  m: [K][8] in shared memory.
+static __device__ double leaf_weight(int K, int ks, int n_leaves, const double *m, int idx) {
+    double w = 1.0;
+    int div = n_leaves;
+    for (int d = 0; d < K; ++d) {
+        div /= ks;
+        const int k = idx / div;
+        idx -= k * div;
+        w *= m[d * 8 + k];
+        if (w < 1e-5) return 0.0;
+    }
+    return w;
+}
+// One warp; `known`: the leaves' weights, or null.  Returns the leaf's index.
+static __device__ int tree_pick(int K, int ks, int n_leaves, const double *m, const double *known, double u) {
     const int lane = threadIdx.x & 31;
-    int n_leaves = 1;
-    for (int d = 0; d < K; ++d) n_leaves *= ks;
-    auto weight = [&](int idx) -> double {
-        if (idx >= n_leaves) return 0.0;
-        double w = 1.0;
-        int div = n_leaves;
-        for (int d = 0; d < K; ++d) {
-            div /= ks;
-            const int k = idx / div;
-            idx -= k * div;
-            w *= m[d * 8 + k];
-            if (w < 1e-5) return 0.0;
-        }
-        return w;
-    };
+    auto weight = [&](int idx) -> double { return idx >= n_leaves ? 0.0 : known != nullptr ? known[idx] : leaf_weight(K, ks, n_leaves, m, idx); };
     double total = 0.0;
     for (int base = 0; base < n_leaves; base += 32) total += weight(base + lane);
 #pragma unroll
@@ -335,53 +377,91 @@ static __device__ void reserve_pages(const Dev &D, int b, int len, int held) {
 // Algorithm 1 lines 7-12 for one sequence by a cluster of K + 1 CTAs, one per window row and slot: CTA j < K decides on
 // the draft behind row j; with the accept length a known to all, CTA i draws candidate i from row a of the backbone (i = 0)
 // or of head i; every CTA works out the commit, CTA 0 writes it down, and CTA i embeds row i of the next window.
-template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int stage) {
-    extern __shared__ __align__(16) float row_buf[];
+// A chain of short steps (copies, scans, two or three cluster barriers of 0.5 us, the embedding's way from memory): every row that
+// may become row a is copied to shared memory at once, so that the candidates' scan starts when a is known.  `rows`: all of them,
+// or, where they are too many, the two that are needed one after the other, or none.
+template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kernel(const Dev D, int stage, int rows) {
+    extern __shared__ __align__(128) float row_buf[];
     __shared__ TailShared sh;
-    const int K1 = D.K1, K = D.K, V = D.V, tid = threadIdx.x;
+    __shared__ __align__(8) uint64_t bars[2];                // the row to verify, the candidates' rows
+    const int K1 = D.K1, K = D.K, V = D.V, ld = D.ldv, tid = threadIdx.x;
     const int b = blockIdx.x / K1, slot = blockIdx.x - b * K1;
-    const bool staged = (size_t)V * 4 <= (size_t)D.tail_row_bytes;      // else the rows are read where they are
     chain_go();
     const RunParams &R = *D.rp;
-    if (__ldcg(D.finished + b)) {
-        chain_wait();
+    // (the kernel before it fills the SMs, so this one starts when that ends: everything is asked for at once)
+    if (K > 0) cluster_arrive();       // "this CTA runs": peers may write to its shared memory after cluster_wait
+    if (tid == 0) {
+        mbar_init(smem_u32(&bars[0]), 1u);
+        mbar_init(smem_u32(&bars[1]), 1u);
+        mbar_init_fence();
+        sh.count = 0;
+        sh.n_cand = 0;
+    }
+    if (tid == 32) sh.state[0] = __ldcg(D.len + b);
+    if (tid == 64) sh.state[1] = __ldcg(D.n_gen + b);
+    if (tid == 96) sh.state[2] = (int)__ldcg(D.step_idx + b);
+    if (tid == 128) sh.state[3] = __ldcg(D.n_blocks + b);
+    if (tid == 160) sh.state[4] = __ldcg(D.finished + b);
+    if (tid >= 192 && tid < 192 + K1) sh.old_win[tid - 192] = __ldcg(D.window + b * K1 + tid - 192);
+    __syncthreads();      // (warps that come to the wait together leave it sooner)
+    if (K > 0) cluster_wait();
+    chain_wait();
+    if (sh.state[4]) {
         if (slot == 0 && tid == 0) __stcg(D.step_n_new + b, 0);
         return;
     }
-    if (tid == 32) sh.state[0] = __ldcg(D.len + b);
-    if (tid == 33) sh.state[1] = __ldcg(D.n_gen + b);
-    if (tid == 34) sh.state[2] = (int)__ldcg(D.step_idx + b);
-    if (tid == 35) sh.state[3] = __ldcg(D.n_blocks + b);
-    if (tid >= 64 && tid < 64 + K1) sh.old_win[tid - 64] = __ldcg(D.window + b * K1 + tid - 64);
-    __syncthreads();      // (warps that come to the wait together leave it sooner)
-    chain_wait();
     trace_mark(D, 1 + 2 * stage);
-    __syncthreads();
+    const float *verify = D.logits0 + (size_t)(b * K1 + slot) * ld;
+    const float *cands = slot == 0 ? D.logits0 + (size_t)b * K1 * ld : D.hlogits + ((size_t)(slot - 1) * D.M + b * K1) * ld;
+    const uint32_t row_bytes = (uint32_t)ld * 4u, to_verify = smem_u32(&bars[0]), to_pick = smem_u32(&bars[1]), buf = smem_u32(row_buf);
+    auto wait_rows = [&](uint32_t bar) { mbar_wait(bar, 0u, D.mbar_limit, D.status); };
+    if (rows == kRowsAll && tid < 32) {
+        if (tid == 0) mbar_arrive_expect_tx(to_pick, (uint32_t)K1 * row_bytes);
+        __syncwarp();
+        if (tid == K1 && slot > 0 && slot < K) {
+            mbar_arrive_expect_tx(to_verify, row_bytes);
+            bulk_g2s(buf + (uint32_t)K1 * row_bytes, verify, row_bytes, to_verify);
+        }
+        if (tid < K1) bulk_g2s(buf + (uint32_t)tid * row_bytes, cands + (size_t)tid * ld, row_bytes, to_pick);
+    } else if (rows == kRowsOne && tid == 0 && slot < K) {
+        mbar_arrive_expect_tx(to_verify, row_bytes);
+        bulk_g2s(buf, verify, row_bytes, to_verify);
+    }
+    if (tid == kTailThreads - 32) sh.r24 = rand24(R, b, (uint32_t)sh.state[2], (uint32_t)slot, 0u);      // (while the rows come)
     // (requested here and looked at in the end: nothing waits for it)
     const int raised = slot == 0 && tid == kTailThreads - 1 ? __ldcg(D.status) : 0;
-    const float *z = D.logits0 + (size_t)(b * K1 + slot) * V;
     int a = 0;
     if (K > 0) {
         if (slot < K) {
-            const float *row = z;
-            if (staged) { stage_row(z, row_buf, V); row = row_buf; }
+            const float *row = verify;
+            if (rows != kRowsNone) {
+                wait_rows(rows == kRowsAll && slot == 0 ? to_pick : to_verify);
+                row = row_buf + (rows == kRowsAll && slot > 0 ? (size_t)K1 * ld : 0);
+            }
             const bool ok = accept_token(D, R, row, sh.old_win[slot + 1], sh);
-            if (tid == 0) sh.accepted = ok ? 1 : 0;
+            if (tid < K1) st_cluster(map_rank(smem_u32(&sh.accepted[slot]), (uint32_t)tid), ok ? 1 : 0);
         }
         __syncthreads();
         cluster_arrive();
         cluster_wait();
-        int flag = 1;
         const int lane = tid & 31;
-        if (lane < K) asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(flag) : "r"(map_rank(smem_u32(&sh.accepted), (uint32_t)lane)) : "memory");
-        const unsigned no = __ballot_sync(0xffffffffu, lane < K && flag == 0);
+        const unsigned no = __ballot_sync(0xffffffffu, lane < K && sh.accepted[min(lane, K - 1)] == 0);
         a = no ? __ffs(no) - 1 : K;
     }
     // candidate of this slot
-    if (slot == 0) z = D.logits0 + (size_t)(b * K1 + a) * V;
-    else z = D.hlogits + ((size_t)(slot - 1) * D.M + b * K1 + a) * V;
-    if (staged) {
-        if (!(slot == 0 && a == 0 && K > 0)) stage_row(z, row_buf, V);      // (slot 0 has row 0 already)
+    const float *z = cands + (size_t)a * ld;
+    if (rows == kRowsAll) {
+        wait_rows(to_pick);
+        z = row_buf + (size_t)a * ld;
+    } else if (rows == kRowsOne) {
+        // (every thread has read the row that was verified; slot 0 has row 0 already)
+        if (!(slot == 0 && a == 0 && K > 0)) {
+            if (tid == 0) {
+                mbar_arrive_expect_tx(to_pick, row_bytes);
+                bulk_g2s(buf, z, row_bytes, to_pick);
+            }
+            wait_rows(to_pick);
+        }
         z = row_buf;
     }
     const bool tree = R.sample_mode == 2 && slot > 0;
@@ -392,7 +472,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
             if (tid < k) sh.cw[tid] = expf((sh.cv[tid] - sh.cv[0]) / R.temperature);
             __syncthreads();
         }
-        if (tid == 0) sh.tok = pick_candidate(R, k, rand24(R, b, (uint32_t)sh.state[2], (uint32_t)slot, 0u), sh);
+        if (tid == 0) sh.tok = pick_candidate(R, k, sh.r24, sh);
     } else {
         // probability tree: this head's K_s best tokens and their probabilities, for slot 1, which draws one path for all heads
         const float mx = sh.cv[0];
@@ -415,104 +495,123 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
                 sh.m[d * 8 + j] = (double)ld_cluster_f32(map_rank(smem_u32(&sh.tree_p[j]), (uint32_t)(d + 1)));
                 asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(sh.tk[d * 8 + j]) : "r"(map_rank(smem_u32(&sh.tree_t[j]), (uint32_t)(d + 1))) : "memory");
             }
+            int n_leaves = 1;
+            for (int d = 0; d < K; ++d) n_leaves *= ks;
             __syncthreads();
+            // (the rows' place is free: the leaves' weights, by all threads)
+            double *known = rows != kRowsNone && (size_t)n_leaves * 8 <= (size_t)row_bytes ? reinterpret_cast<double *>(row_buf) : nullptr;
+            if (known != nullptr) {
+                for (int i = tid; i < n_leaves; i += kTailThreads) known[i] = leaf_weight(K, ks, n_leaves, sh.m, i);
+                __syncthreads();
+            }
             if (tid < 32) {
-                const double u = (double)rand24(R, b, (uint32_t)sh.state[2], 1u, 0u) * (1.0 / 16777216.0);
-                int leaf = tree_pick(K, ks, sh.m, u), div = 1;
-                for (int d = 0; d < K; ++d) div *= ks;
+                const double u = (double)sh.r24 * (1.0 / 16777216.0);
+                int leaf = tree_pick(K, ks, n_leaves, sh.m, known, u), div = n_leaves;
                 for (int d = 0; d < K; ++d) {
                     div /= ks;
                     const int kk = leaf / div;
                     leaf -= kk * div;
-                    if (tid == 0) sh.path[d] = sh.tk[d * 8 + kk];
+                    if (tid < K1) st_cluster(map_rank(smem_u32(&sh.cand[d + 1]), (uint32_t)tid), sh.tk[d * 8 + kk]);
                 }
             }
         }
     }
     __syncthreads();
-    if (K > 0) { cluster_arrive(); cluster_wait(); }
-    if (tid < K1) {
-        int v = sh.tok;
-        if (K > 0) {
-            const bool from_path = R.sample_mode == 2 && tid > 0;
-            const uint32_t src = from_path ? map_rank(smem_u32(&sh.path[tid - 1]), 1u) : map_rank(smem_u32(&sh.tok), (uint32_t)tid);
-            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(src) : "memory");
-        }
-        sh.cand[tid] = v;
+    if (K > 0) {
+        if (tid < K1 && (R.sample_mode != 2 || slot == 0)) st_cluster(map_rank(smem_u32(&sh.cand[slot]), (uint32_t)tid), sh.tok);
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        if (tid == 0) sh.cand[0] = sh.tok;
+        __syncthreads();
     }
-    __syncthreads();
-    if (K > 0) cluster_arrive();         // (this CTA has read its peers' candidates)
-    // commit x_{s+1..s*}, s <- s*, next window <- candidates: worked out by every CTA, written by CTA 0
-    if (tid == 0) {
+    // (the embedding is on its way while the commit is worked out, which changes it only where drafts are scripted)
+    constexpr int N = 16 / (int)sizeof(WT);
+    static_assert(kTailThreads * 4 >= 2048, "a thread embeds 16 bytes at most");
+    const int col = tid * N, guess = sh.cand[slot];
+    uint4 e_raw, g_raw;
+    if (col < D.d) {
+        e_raw = embedding<WT>(D, guess, col);
+        g_raw = first_gain<WT>(D, col);
+    }
+    // commit x_{s+1..s*}, s <- s*, next window <- candidates: worked out by every CTA, written by CTA 0 (one warp, a lane a token)
+    if (tid < 32) {
         const bool w = slot == 0;
-        const int len0 = sh.state[0], len = len0 + a + 1;
+        const int len = sh.state[0] + a + 1, n_gen = sh.state[1];
         // scripted drafts: the token at the first rejected position is the script's as well, so that a near-tie
         // of the backbone's two best logits cannot take the run off the script for good
-        if (R.script != nullptr && len < R.script_n) sh.cand[0] = R.script[(size_t)b * R.script_n + len];
-        int n_gen = sh.state[1], fin = 0, n_out = 0;
-        for (int j = 0; j <= a; ++j) {
-            const int tok = j < a ? sh.old_win[j + 1] : sh.cand[0];
-            if (n_gen >= R.max_new) break;
-            if (w) {
-                __stcg(D.tok_log + (size_t)b * D.tok_ld + n_gen, tok);
-                __stcg(D.step_tokens + b * K1 + n_out, tok);
-            }
-            ++n_gen; ++n_out;
-            if (D.eos >= 0 && tok == D.eos) { fin = 1; break; }
-        }
-        if (n_gen >= R.max_new || len > D.max_seq_len) fin = 1;
-        for (int j = 0; j < K1; ++j) sh.win[j] = sh.cand[j];
-        if (R.script != nullptr) {
+        const int first = R.script != nullptr && len < R.script_n ? R.script[(size_t)b * R.script_n + len] : sh.cand[0];
+        const int tok = tid < a ? sh.old_win[min(tid + 1, K)] : first;
+        int n_out = max(0, min(a + 1, R.max_new - n_gen));
+        const unsigned ends = __ballot_sync(0xffffffffu, D.eos >= 0 && tid < n_out && tok == D.eos);
+        if (ends) n_out = __ffs(ends);
+        const int fin = ends != 0u || n_gen + n_out >= R.max_new || len > D.max_seq_len ? 1 : 0;
+        int next = tid == 0 ? first : tid < K1 ? sh.cand[tid] : 0;
+        if (R.script != nullptr && tid > 0 && tid < K1) {
             // scripted drafts: the next window drafts the script's tokens; the first `keep` stay as they
             // are, the others are made wrong (a forced accept length for a backbone that reproduces the script)
             const long long t = (long long)sh.state[2] + 1;
-            const int keep = (int)((((t + 1) * R.script_acc) >> 10) - ((t * R.script_acc) >> 10));
-            const int *sc = R.script + (size_t)b * R.script_n;
-            for (int j = 1; j < K1; ++j) {
-                const int pos = len + j;
-                int tok = pos < R.script_n ? sc[pos] : 0;
-                if (j > keep) tok = tok + 1 < D.V ? tok + 1 : 0;
-                sh.win[j] = tok;
-            }
+            const int keep = (int)((((t + 1) * R.script_acc) >> 10) - ((t * R.script_acc) >> 10)), pos = len + tid;
+            next = pos < R.script_n ? R.script[(size_t)b * R.script_n + pos] : 0;
+            if (tid > keep) next = next + 1 < D.V ? next + 1 : 0;
         }
-        sh.state[5] = fin;
+        if (tid < K1) sh.win[tid] = next;
+        if (tid == 0) sh.state[5] = fin;
         if (w) {
-            for (int j = n_out; j < K1; ++j) __stcg(D.step_tokens + b * K1 + j, -1);
-            __stcg(D.step_n_new + b, n_out);
-            __stcg(D.n_gen + b, n_gen);
-            __stcg(D.step_idx + b, (uint32_t)sh.state[2] + 1u);
-            D.hist[(size_t)b * (kMaxDraft + 1) + a] += 1ull;
-            D.steps[b] += 1ull;
-            if (fin) {
-                __stcg(D.finished + b, 1);
-                if (atomicSub(D.n_active, 1) == 1) {      // the last one: tell the host that its call is done
-                    __threadfence_system();
-                    *reinterpret_cast<volatile int *>(D.host_done) = R.call;
-                }
-            } else {
-                reserve_pages(D, b, len, sh.state[3]);
+            if (tid < n_out) __stcg(D.tok_log + (size_t)b * D.tok_ld + n_gen + tid, tok);
+            if (tid < K1) {
+                __stcg(D.step_tokens + b * K1 + tid, tid < n_out ? tok : -1);
+                __stcg(D.window + b * K1 + tid, next);
             }
-            __stcg(D.len + b, len);
-            for (int j = 0; j < K1; ++j) __stcg(D.window + b * K1 + j, sh.win[j]);
+            if (tid == 0) {
+                __stcg(D.step_n_new + b, n_out);
+                __stcg(D.n_gen + b, n_gen + n_out);
+                __stcg(D.step_idx + b, (uint32_t)sh.state[2] + 1u);
+                D.hist[(size_t)b * (kMaxDraft + 1) + a] += 1ull;
+                D.steps[b] += 1ull;
+                __stcg(D.len + b, len);
+                if (!fin) reserve_pages(D, b, len, sh.state[3]);
+            }
+            if (fin) {
+                __threadfence_system();      // (every lane's tokens are out before the host is told)
+                __syncwarp();
+                if (tid == 0) {
+                    __stcg(D.finished + b, 1);
+                    if (atomicSub(D.n_active, 1) == 1) {      // the last one: tell the host that its call is done
+                        __threadfence_system();
+                        *reinterpret_cast<volatile int *>(D.host_done) = R.call;
+                    }
+                }
+            }
         }
     }
     __syncthreads();
     const int new_len = sh.state[0] + a + 1;
     if (slot == 0 && tid >= kTailThreads - 32 && tid - (kTailThreads - 32) < K1)      // (the last warp: the embedding needs the first ones)
         place_row(D, b * K1 + tid - (kTailThreads - 32), b, new_len + tid - (kTailThreads - 32), !sh.state[5]);
-    if (!sh.state[5]) embed_row<WT>(D, b * K1 + slot, D.Mp, sh.win[slot], new_len + slot, sh.red);
+    if (!sh.state[5]) {
+        embed_position(D, b * K1 + slot, new_len + slot);
+        float ssq = 0.f;
+        if (col < D.d) {
+            if (sh.win[slot] != guess) e_raw = embedding<WT>(D, sh.win[slot], col);
+            ssq = embed_chunk<WT>(D, b * K1 + slot, D.Mp, col, e_raw, g_raw);
+        }
+        embed_sum<kTailThreads>(D, b * K1 + slot, ssq, sh.red);
+    }
     // a wait of this request ran out, or its pages: more steps are of no use (the host reads the status word itself)
     if (raised != 0) *reinterpret_cast<volatile int *>(D.host_done) = R.call;
-    if (K > 0) cluster_wait();           // peers may still read this CTA's candidate
     trace_mark(D, 2 + 2 * stage);
 }
 
 cudaError_t launch_tail(const Dev &D, int dtype, int stage, const ChainLaunch &L) {
     const void *fn = dtype == 1 ? (const void *)tail_kernel<bf16> : (const void *)tail_kernel<float>;
-    const int smem = (size_t)D.V * 4 <= (size_t)D.tail_row_bytes ? (D.V * 4 + 15) / 16 * 16 : 16;
+    // All rows, where two CTAs' share an SM or there is one for every CTA: a cluster more would be a second wave.
+    const size_t row = (size_t)D.ldv * 4, all = row * (D.K > 0 ? D.K1 + 1 : 1);
+    const bool fits = all <= kTailSmem / 2 || (all <= kTailSmem && (D.K == 0 || (D.K1 <= 8 && D.B <= resident_clusters(D.K1))));
+    const int rows = fits ? kRowsAll : row <= kTailSmem ? kRowsOne : kRowsNone, smem = fits ? (int)all : row <= kTailSmem ? (int)row : 16;
     cudaError_t e = open_kernel(fn, smem, D.K1 > 8);
     if (e != cudaSuccess) return e;
-    return L.launch(dim3(D.B * D.K1), dim3(kTailThreads), smem, D.K1, fn, D, stage);
+    return L.launch(dim3(D.B * D.K1), dim3(kTailThreads), smem, D.K1, fn, D, stage, rows);
 }
 
 // --------------------------------------------------------------------------------- start of a request
