@@ -6,6 +6,28 @@ namespace xsm {
 
 constexpr int kF32Warps = 8, kF32Threads = kF32Warps * 32;
 
+// Folds N values of every lane over the warp (lanes that differ in bits of at least `last`): each exchange halves the values
+// that a lane keeps, so N values cost N - 1 + a few shuffles of 38 cycles instead of 5 N.  Lane l gets value l / (32 / N); the
+// order of a sum is that of warp_sum.
+template <int N, typename Op> __device__ __forceinline__ float fold(float (&v)[N], Op op, int last) {
+    const int lane = threadIdx.x & 31;
+    int k = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, k /= 2) {
+        const bool up = lane & k;
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i)
+            if (i < n) {
+                const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                v[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, k));
+            }
+    }
+    for (; k >= last; k /= 2) v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], k));
+    return v[0];
+}
+struct Add { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
+struct Max { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
+
 // ------------------------------------------------------------------------------------ projections
 
 // A warp owns units (a row, or a pair of rows: rotation partners, gate and up), its lanes the columns.  The weights of the
@@ -61,13 +83,6 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
     chain_wait();
     if (A.late_go) chain_go();
     trace_mark(D, 1 + 2 * A.stage);
-    if (A.ss_parts > 0)
-        for (int m = warp; m < M; m += kF32Warps) {
-            float ss = 0.f;
-            for (int p = lane; p < A.ss_parts; p += 32) ss += __ldcg(D.ss + (size_t)m * kShareLd + p);
-            ss = warp_sum(ss);
-            if (lane == 0) s_inv[m] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
-        }
     const float *x = reinterpret_cast<const float *>(A.x) + (A.x_jobs ? (size_t)job * M * K : 0);
     auto stage = [&](int k0) {      // columns [k0, k0 + chunk) of all token rows
         const int n4 = min(chunk, K - k0) >> 2;
@@ -78,8 +93,39 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
         }
         __syncthreads();
     };
-    if (chunk >= K) stage(0);
-    float ssq_mine = 0.f;      // PE_ADD: lane m sums the squares of its token row over the warp's units
+    // 1/rms of the token rows (their shares are requested before the activations, and added up behind them)
+    constexpr int SHARES = (kShareLd + 31) / 32, MINE = (MT + kF32Warps - 1) / kF32Warps;
+    float share[MINE][SHARES];
+#pragma unroll
+    for (int i = 0; i < MINE; ++i)
+#pragma unroll
+        for (int p = 0; p < SHARES; ++p) {
+            const int m = warp + i * kF32Warps;
+            share[i][p] = m < M && p * 32 + lane < A.ss_parts ? __ldcg(D.ss + (size_t)m * kShareLd + p * 32 + lane) : 0.f;
+        }
+    if (chunk >= K) {
+        const int n4 = K >> 2;
+        for (int i = tid; i < M * n4; i += kF32Threads) {
+            const int m = i / n4, c = i - m * n4;
+            reinterpret_cast<float4 *>(xs + m * chunk)[c] = __ldcg(reinterpret_cast<const float4 *>(x + (size_t)m * K) + c);
+        }
+    }
+    if (A.ss_parts > 0) {
+#pragma unroll
+        for (int i = 0; i < MINE; ++i) {
+            if (warp + i * kF32Warps >= M) break;
+            float ss = 0.f;
+#pragma unroll
+            for (int p = 0; p < SHARES; ++p) ss += share[i][p];
+            ss = warp_sum(ss);
+            if (lane == 0) s_inv[warp + i * kF32Warps] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+        }
+    }
+    __syncthreads();
+    constexpr int ROWS = MT < 8 ? MT : 8, WIDTH = 32 / (ROWS * R);      // token rows folded at a time, lanes that share a value
+    float ssq_mine[MT / ROWS];      // PE_ADD: the squares of a lane's token rows over the warp's units
+#pragma unroll
+    for (int c = 0; c < MT / ROWS; ++c) ssq_mine[c] = 0.f;
     for (int base = cta * kF32Warps; base < units; base += step) {      // (all warps of the CTA together: they share the staged columns)
         const int unit = base + warp;
         float acc[R][MT];
@@ -124,27 +170,24 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
             }
         }
         if (!mine) continue;
-        // sums over the lanes; lane m keeps token row m
-        float v = 0.f, v2 = 0.f;
+        // sums over the lanes, ROWS token rows (both rows of a pair) at a time
 #pragma unroll
-        for (int m = 0; m < MT; ++m) {
-            if (m < M) {
-                const float s = warp_sum(acc[0][m]);
-                if (lane == m) v = s;
-                if (PAIRS) {
-                    const float s2 = warp_sum(acc[R - 1][m]);
-                    if (lane == m) v2 = s2;
-                }
-            }
-        }
-        const int m = lane;
-        if (m >= M) continue;
+        for (int ch = 0; ch < MT / ROWS; ++ch) {
+        if (ch * ROWS >= M) break;
+        float part[ROWS * R];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+            for (int r = 0; r < R; ++r) part[i * R + r] = acc[r][ch * ROWS + i];
+        float v = fold(part, Add(), 1), v2 = PAIRS ? __shfl_xor_sync(0xffffffffu, v, WIDTH) : 0.f;
+        const int m = ch * ROWS + lane / (WIDTH * R);
+        if (lane % (WIDTH * R) != 0 || m >= M) continue;
         const float inv = A.ss_parts > 0 ? s_inv[m] : 1.f;
         if (EPI0 == PE_ADD) {
             const float h = __ldcg(D.h + (size_t)m * D.d + u) + v;
             D.h[(size_t)m * D.d + u] = h;
             reinterpret_cast<float *>(A.g[0].out)[(size_t)m * A.g[0].ld + u] = h * __ldg(reinterpret_cast<const float *>(A.gain) + u);
-            ssq_mine += h * h;
+            ssq_mine[ch] += h * h;
         } else if (EPI0 == PE_QKV) {
             v *= inv;
             v2 *= inv;
@@ -172,11 +215,14 @@ __global__ void __launch_bounds__(kF32Threads) proj_f32_kernel(const Dev D, cons
         } else {
             A.g[0].logits[((size_t)j * D.M + m) * A.g[0].ld + u] = A.norm ? v * inv : v;
         }
+        }
     }
     if (EPI0 == PE_ADD) {
         // the CTA's shares of the sums of squares
         __syncthreads();
-        if (lane < M) xs[warp * MT + lane] = ssq_mine;
+#pragma unroll
+        for (int ch = 0; ch < MT / ROWS; ++ch)
+            if (lane % WIDTH == 0) xs[warp * MT + ch * ROWS + lane / WIDTH] = ssq_mine[ch];
         __syncthreads();
         if (tid < M) {
             float s = 0.f;
@@ -251,14 +297,19 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
             }
         }
         // running maximum of every row, weights relative to it
+        constexpr int ROWS = T < 8 ? T : 8;
 #pragma unroll
         for (int r = 0; r < T; ++r) {
             s[r] += __shfl_xor_sync(0xffffffffu, s[r], 1);
             if (key >= n_keys || (!cross && key > start + r)) s[r] = -INFINITY;
-            float m = s[r];
+        }
 #pragma unroll
-            for (int k = 16; k > 1; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
-            if (lane == 0) red[warp * T + r] = m;
+        for (int r0 = 0; r0 < T; r0 += ROWS) {
+            float v[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) v[r] = s[r0 + r];
+            const float m = fold(v, Max(), 2);
+            if (lane % (32 / ROWS) == 0) red[warp * T + r0 + lane / (32 / ROWS)] = m;
         }
         __syncthreads();
         if (tid < T) {
@@ -269,11 +320,16 @@ __global__ void __launch_bounds__(kF32Threads) attn_f32_kernel(const Dev D, cons
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < T; ++r) {
-            const float e = exp2f(s[r] - m_run[r]);
-            if (part == 0) p[r * kF32Keys + (tid >> 1)] = e;
-            const float l = warp_sum(part == 0 ? e : 0.f);
-            if (lane == 0) red[warp * T + r] = l;
+        for (int r0 = 0; r0 < T; r0 += ROWS) {
+            float v[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const float e = exp2f(s[r0 + r] - m_run[r0 + r]);
+                if (part == 0) p[(r0 + r) * kF32Keys + (tid >> 1)] = e;
+                v[r] = part == 0 ? e : 0.f;
+            }
+            const float l = fold(v, Add(), 1);
+            if (lane % (32 / ROWS) == 0) red[warp * T + r0 + lane / (32 / ROWS)] = l;
         }
         __syncthreads();
         if (tid < T) {
