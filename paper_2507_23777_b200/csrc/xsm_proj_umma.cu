@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     auto where = [&](int c) {
 #pragma unroll
         for (int q = 0; q < GROUPS; ++q) {
+            if (CL && G > 1 && (GROUPS * c + q) * G >= rows) continue;      // (token rows one by one: the branch costs more than it saves)
             const int group = GROUPS * c + q, owner = (int)((uint32_t)group * A.inv_q >> 16), place = rank * qps + group - owner * qps;      // (group / qps: both are below 33)
             dst[q] = CL ? map_rank(srecv + (uint32_t)(place * 128 + arow) * (4u * G), (uint32_t)min(owner, S - 1)) : (uint32_t)(group * 128 + arow) * (4u * G);
             dst_bar[q] = CL ? map_rank(recv_b, (uint32_t)min(owner, S - 1)) : recv_b;

@@ -7,7 +7,8 @@ told otherwise), then eleven traced steps, and prints for the one in the middle 
 long the step spends in it (last CTA of the previous stage done -> last CTA of this stage done), how long after the
 previous stage's end a CTA is past the wait for it, and how long it takes from there to its end.  Every mark is a read of
 the GPU's global timer plus a store (a few hundred nanoseconds), so a traced step is slower than an untraced one; compare
-shares, not totals.
+shares, not totals.  A traced step is launched kernel by kernel: four ordinary steps are queued before it, so that the host is
+ahead of the device as it is when recordings are replayed (else a kernel starts when the host launches it, every 4 us).
 """
 from __future__ import annotations
 
@@ -75,7 +76,12 @@ def main():
     for _ in range(args.warm):
         ctx.xsm_spec_step()
     print(f"config {args.config} ({cfg['name']}), batch {args.batch}, context {int(ctx.xsm_debug_get_state()['len'][0])}")
-    steps = sorted((ctx.xsm_debug_trace_step() for _ in range(11)), key=lambda t: int(t[-1].max()) - int(t[0][t[0] > 0].min()))
+    steps = []
+    for _ in range(11):
+        for _ in range(4):
+            ctx.xsm_spec_step()
+        steps.append(ctx.xsm_debug_trace_step())
+    steps.sort(key=lambda t: int(t[-1].max()) - int(t[0][t[0] > 0].min()))
     print(table(cfg, steps[5]))
     ctx.xsm_destroy()
 
