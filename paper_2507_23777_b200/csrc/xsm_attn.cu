@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
     const int start = first + q0, n_keys = cross ? D.C : A.pos0 >= 0 ? min(start + t_rows, A.pos_end) : start + t_rows;
     const int S = CL ? min(A.S, (n_keys + A.split - 1) / A.split) : 1;           // CTAs that take part
     if (CL && rank >= S) {
-        cluster_arrive();
+        cluster_arrive_relaxed();
         cluster_wait();
         return;
     }
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
     }
     __syncthreads();
     chain_go();
-    if (CL) { cluster_arrive(); cluster_wait(); }      // the peers run: what is sent to them has a place
+    if (CL) { cluster_arrive_relaxed(); cluster_wait(); }      // the peers run: what is sent to them has a place
     const bool dead = A.pos0 < 0 && __ldcg(D.finished + b) != 0;
     if (dead) {
         chain_wait();

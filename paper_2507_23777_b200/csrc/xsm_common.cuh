@@ -115,6 +115,9 @@ __device__ __forceinline__ uint32_t cluster_index() {
     asm volatile("mov.u32 %0, %clusterid.x;" : "=r"(r));
     return r;
 }
+// For threads that have written nothing that others read, barriers made known by mbar_init_fence apart: a release waits for all
+// that the thread has under way, loads from memory among it.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // shared-memory address of the same variable in CTA `rank` of the cluster

@@ -389,7 +389,7 @@ template <typename WT> __global__ void __launch_bounds__(kTailThreads) tail_kern
     chain_go();
     const RunParams &R = *D.rp;
     // (the kernel before it fills the SMs, so this one starts when that ends: everything is asked for at once)
-    if (K > 0) cluster_arrive();       // "this CTA runs": peers may write to its shared memory after cluster_wait
+    if (K > 0) cluster_arrive_relaxed();      // "this CTA runs": peers may write to its shared memory after cluster_wait
     if (tid == 0) {
         mbar_init(smem_u32(&bars[0]), 1u);
         mbar_init(smem_u32(&bars[1]), 1u);
