@@ -220,10 +220,10 @@ __device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(rein
 
 // QP (cross-attention of a step, few rows): the kernel projects the queries of its head itself, from the normalised residual
 // stream (every warp multiplies all rows over its share of the columns, as in the projections over few token rows), instead
-// of a kernel of its own: 7.5 -> 5 us for both at width 1024.  The head's rows of the projection and the pages are requested
-// before the wait, but a CTA (544 threads of 96 registers) shares an SM with none of the out-projection before it (288 of 94
-// or 96).  Where that leaves SMs free, they have arrived when the wait is over; at width 1024 it holds 147 of 148, so all but
-// one of the sixteen CTAs of a sequence start when it ends, and fetch about 200 KB in full view: 4.4 to 4.9 us after the wait.
+// of a kernel of its own: 630 against 650 us a step at width 1024.  The head's rows of the projection and the pages are requested
+// before the wait; a CTA (544 threads of 96 registers) shares an SM with none of the projections, but the out-projection before it
+// holds 64 of 148, so the sixteen CTAs of a sequence start some 7 us before it ends.  4.0 us after the wait: 0.5 until the
+// activations come, 0.9 products (128 KB of weights through shared memory), 0.6 sums, 1.0 keys, 1.3 merge and output.
 constexpr int kQueryBlocks = 4;      // blocks of 32 columns per warp: d_model up to 1024
 //
 // NW: warps that attend, beside the producer.  A unit of 32 keys is some 300 dependent instructions, 1 us for a warp on its
