@@ -13,6 +13,7 @@ namespace xsm {
 static_assert(sizeof(TensorMap) == sizeof(CUtensorMap), "tensor map size");
 
 constexpr int kMaxPlans = 8;                      // batch sizes whose recordings are kept
+constexpr int kAccumulators = 256;                // columns of tensor memory of a CTA (an SM has 512, and may hold two CTAs)
 constexpr int kProjSmemMax = 224 * 1024;          // dynamic shared memory of a projection (a CTA may have 227 KB in all)
 
 cudaError_t open_kernel(const void *fn, int smem, bool large_cluster) {
@@ -131,8 +132,17 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     // activations, and weights that do not fit the ring, 59 bytes a cycle; 45 for every token row that is sent, 250 for every
     // one that is finished.  Eight layers of width 1024: 90 rows 480 -> 425 us a step, 80 rows 444 -> 414, 60 rows 409 -> 375; 40
     // rows 354 -> 356, 30 rows 304 -> 331, so up to 48 rows T is 1 and the largest S that fits is taken, without weighing.
-    int S = 1, T = 1;
+    //
+    // How many blocks an accumulator adds up: every instruction cuts off what lies below the accumulator's last bit, so the error of a
+    // sum grows with their number (projections alone, against 64 bits, in units of 1e-6 of the result: sums of 128 instructions at
+    // width 2048 7.9, of at most 16 6.9, as warps that share the columns have with mma.sync).  Up to 16 token rows four blocks, 16
+    // instructions; token rows in parts: as many as a CTA would have with the largest S of whole token rows.  From 17 to 48 rows
+    // one for all blocks (8.0 at width 2048, 7.2 at 1024): several cost 1 to 4 % of a step.
+    int S = 1, T = 1, whole = 1;      // whole: that largest S
     const bool parts = A.tt == 1 && rows > 48;
+    for (int s = 2; s <= std::min(8, nblk); ++s)
+        if (tiles * A.tt <= clusters_[s]) whole = s;
+    const int chain = parts ? (nblk + whole - 1) / whole : rows <= 16 ? 4 : nblk;
     double best = 1e30;
     for (int t = 1; t <= (parts ? Mp / 8 : 1); ++t) {
         const int nt = parts ? (Mp / 8 + t - 1) / t * 8 : std::min(Mp, kTokenTile);
@@ -140,6 +150,7 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
         for (int s = 1; s <= std::min(8, nblk); ++s) {
             const int n = (nblk + s - 1) / s;
             if (s > 1 ? tiles * A.tt * t > clusters_[s] : t > 1 && tiles * t > sms_) continue;
+            if (parts && (n + chain - 1) / chain * 2 * nt > kAccumulators) continue;
             const double late = std::max(0.0, n * 16384.0 - 160 * 1024), sent = s > 1 ? 600 + 45.0 * nt : 0;
             const double cost = n * 4 * std::max(47.0, nt * 1.0) + (n * 256.0 * nt + late) / 59 + sent + 250.0 * ((nt + 4 * s - 1) / (4 * s) * 4);
             if (!parts || cost < best) { best = cost; S = s; T = t; }
@@ -164,8 +175,11 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.nb = std::min(n, std::max(2, std::min(kProjRing, (rows > 32 ? room * 9 / 20 : room / 3) / b_bytes)));
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
+    const int sums_fit = kAccumulators / (2 * A.tok);
+    A.many = parts || rows <= 16;
+    A.chain = std::max(chain, (n + sums_fit - 1) / sums_fit);
     A.tmem_cols = 32;
-    while (A.tmem_cols < 2 * A.tok) A.tmem_cols *= 2;
+    while (A.tmem_cols < (n + A.chain - 1) / A.chain * 2 * A.tok) A.tmem_cols *= 2;
     const int rings = A.na * a_bytes + A.nb * b_bytes;
     op.smem = 1024 + (S > 1 ? rings + sums : std::max(rings, sums));
 }

@@ -42,6 +42,7 @@ struct ProjArgs {
     int S, tps, group;                // CTAs per cluster (cuts of the columns), token rows each of them finishes, dealt out in groups of so many
     uint32_t inv_s, inv_q;            // 65536 / S + 1, 65536 / (tps / group) + 1: small numbers are divided by multiplying
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns
+    int many, chain;                  // a CTA may have several accumulators; operand blocks that each adds up
     int norm, ss_parts;               // the input is an RMSNorm input; shares of its sums of squares (0: not needed)
     int z_jobs, x_jobs;               // group 0 has one matrix per decoding head; the activations too
     const bf16 *x;                    // planes of kdim columns (x_jobs: a set per decoding head)

@@ -39,7 +39,10 @@ struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate)
 // activations count on one barrier and the issuing warp adds to two descriptors; with a barrier and two commits a block, a block
 // took 0.28 us, eight of them more than the weights' way from memory (5 rows of width 1024 683 -> 631 us a step).
 // G: token rows of a group that is sent and finished together (plan_proj).
-template <int EPI0, int EPI1, bool CL, int G>
+// MANY: the CTA's blocks are added up in accumulators of A.chain blocks each, side by side in tensor memory, and these in fp32 here
+// (plan_proj).  The price is code more than work: 5 rows of width 1024 612 -> 622 us a step, 619 with one accumulator in the same
+// code.  Fetching one while the tensor core fills the next (631), two at a time (632), or sending each by itself (646) is slower.
+template <int EPI0, int EPI1, bool CL, int G, bool MANY>
 __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
     extern __shared__ char smem_raw[];
     char *const smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);      // (swizzled tiles: 1024-byte boundaries)
@@ -207,33 +210,47 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         // uniform registers that the instruction takes them from)
         const bool leader = elect_one();
         const uint64_t da = umma_desc_sw128(sa), db = umma_desc_sw128(sb);
-        auto products = [&](int i, int ia, int ib) {
+        auto products = [&](uint32_t sum, int ia, int ib, bool add) {
             const uint64_t a = da + (uint64_t)(ia * (kABytes >> 4)), b = db + (uint64_t)((uint32_t)ib * (b_pitch >> 4));
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) umma_mma(tmem, a + 2 * ks, b + 2 * ks, idesc, (i > 0 || ks > 0) ? 1u : 0u);
+            for (int ks = 0; ks < 4; ++ks) umma_mma(sum, a + 2 * ks, b + 2 * ks, idesc, (add || ks > 0) ? 1u : 0u);
         };
+        // an accumulator after the other: blocks [i0, i1)
+        uint32_t sum = tmem;
         if (flat) {
             mbar_wait(full_b, 0u, D.mbar_limit, D.status);
-            for (int i = 0; i < n; ++i) {
-                mbar_wait(full_a + 8u * (uint32_t)i, 0u, D.mbar_limit, D.status);
-                tcgen05_after_sync();
-                if (leader) products(i, i, i);
+            for (int i0 = 0;;) {
+                const int i1 = MANY ? min(i0 + A.chain, n) : n;
+                for (int i = i0; i < i1; ++i) {
+                    mbar_wait(full_a + 8u * (uint32_t)i, 0u, D.mbar_limit, D.status);
+                    tcgen05_after_sync();
+                    if (leader) products(sum, i, i, i > i0);
+                }
+                if (!MANY || i1 == n) break;
+                i0 = i1;
+                sum += (uint32_t)(2 * Nt);
             }
         } else {
             const uint32_t empty_a = bar(1, 0), empty_b = bar(3, 0);
             int ia = 0, ib = 0;
             uint32_t pa = 0u, pb = 0u;
-            for (int i = 0; i < n; ++i) {
-                mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
-                mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
-                tcgen05_after_sync();
-                if (leader) {
-                    products(i, ia, ib);
-                    if (i + na < n) umma_commit(empty_a + 8u * (uint32_t)ia);
-                    if (i + nb < n) umma_commit(empty_b + 8u * (uint32_t)ib);
+            for (int i0 = 0;;) {
+                const int i1 = MANY ? min(i0 + A.chain, n) : n;
+                for (int i = i0; i < i1; ++i) {
+                    mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
+                    mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
+                    tcgen05_after_sync();
+                    if (leader) {
+                        products(sum, ia, ib, i > i0);
+                        if (i + na < n) umma_commit(empty_a + 8u * (uint32_t)ia);
+                        if (i + nb < n) umma_commit(empty_b + 8u * (uint32_t)ib);
+                    }
+                    if (++ia == na) { ia = 0; pa ^= 1u; }
+                    if (++ib == nb) { ib = 0; pb ^= 1u; }
                 }
-                if (++ia == na) { ia = 0; pa ^= 1u; }
-                if (++ib == nb) { ib = 0; pb ^= 1u; }
+                if (!MANY || i1 == n) break;
+                i0 = i1;
+                sum += (uint32_t)(2 * Nt);
             }
         }
         if (leader) umma_commit(done);
@@ -289,12 +306,26 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
         if (c != c0) where(c);
         tmem_wait_ld();
+        float sums[8];
+        if constexpr (MANY) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sums[j] = __uint_as_float(v[j]) + __uint_as_float(v[8 + j]);
+            uint32_t at = tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u;
+#pragma unroll 1
+            for (int k = A.chain; k < n; k += A.chain) {
+                at += (uint32_t)(2 * Nt);
+                tmem_ld16(v, at);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 8; ++j) sums[j] += __uint_as_float(v[j]) + __uint_as_float(v[8 + j]);
+            }
+        }
 #pragma unroll
         for (int q = 0; q < GROUPS; ++q) {
             if ((GROUPS * c + q) * G < rows) {
                 float f[G];
 #pragma unroll
-                for (int j = 0; j < G; ++j) f[j] = __uint_as_float(v[G * q + j]) + __uint_as_float(v[8 + G * q + j]);
+                for (int j = 0; j < G; ++j) f[j] = MANY ? sums[G * q + j] : __uint_as_float(v[G * q + j]) + __uint_as_float(v[8 + G * q + j]);
                 if constexpr (G == 1) {
                     if (done_ok) st_async_f32(dst[q], f[0], dst_bar[q]);      // (a peer that gave up waiting may have left)
                 } else {
@@ -423,19 +454,23 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     }
 }
 
-template <int EPI0, int EPI1, bool CL, int G>
+template <int EPI0, int EPI1, bool CL, int G, bool MANY>
 static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
-    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL, G>;
+    void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL, G, MANY>;
     cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
     return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? kClusterThreads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
 }
 
+template <int EPI0, int EPI1, bool MANY>
+static cudaError_t launch_sums(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
+    if (A.S == 1) return launch_instance<EPI0, EPI1, false, 4, MANY>(D, A, T, smem, L);
+    return A.group == 1 ? launch_instance<EPI0, EPI1, true, 1, MANY>(D, A, T, smem, L) : launch_instance<EPI0, EPI1, true, 4, MANY>(D, A, T, smem, L);
+}
 template <int EPI0, int EPI1>
 static cudaError_t launch_cut(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
-    if (A.S == 1) return launch_instance<EPI0, EPI1, false, 4>(D, A, T, smem, L);
-    return A.group == 1 ? launch_instance<EPI0, EPI1, true, 1>(D, A, T, smem, L) : launch_instance<EPI0, EPI1, true, 4>(D, A, T, smem, L);
+    return A.many ? launch_sums<EPI0, EPI1, true>(D, A, T, smem, L) : launch_sums<EPI0, EPI1, false>(D, A, T, smem, L);
 }
 
 // (asked for once per device: the answer does not change, and asking takes longer than the rest of a context's creation)
@@ -444,7 +479,7 @@ int resident_clusters(int size) {
     int dev = 0;
     if (size < 2 || size > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
     if (const int k = known[dev][size].load()) return k - 1;
-    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1, true, 4>;
+    const void *fn = (const void *)proj_umma_kernel<PE_ADD, -1, true, 4, false>;
     constexpr int smem = 200 * 1024;
     int n = 0;
     cudaLaunchConfig_t c = {};
