@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
                     }
                     if (++ia == na) { ia = 0; pa ^= 1u; }
                     if (++ib == nb) { ib = 0; pb ^= 1u; }
+                    __syncwarp();      // (a lane two fills of a slot behind the leader would wait for a phase that has gone by)
                 }
                 if (!MANY || i1 == n) break;
                 i0 = i1;

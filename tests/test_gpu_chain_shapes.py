@@ -31,6 +31,8 @@ SHAPES = {
     "prompt of 130": (_model(), 1, 130),
     "prompts of 90": (_model(), 3, 90),
     "prompt of 2100": (_model(256, 4, 64, 512), 1, 2100),
+    # (a ring of two slots of activations, refilled ten times in the down projection)
+    "prompt of 1100, 128 blocks of columns": (_model(256, 4, 64, 8192), 1, 1100),
     # queries projected by the cross-attention: one key tile, odd counts, keys cut over CTAs, keys that do not fit at once
     "16 condition latents": (_model(1024, 16, 64, 1024, C=16), 1, 1),
     "257 condition latents, three sequences": (_model(1024, 16, 64, 1024, K=2, C=257), 3, 1),
