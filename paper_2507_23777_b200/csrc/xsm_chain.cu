@@ -14,7 +14,6 @@ static_assert(sizeof(TensorMap) == sizeof(CUtensorMap), "tensor map size");
 
 constexpr int kMaxPlans = 8;                      // batch sizes whose recordings are kept
 constexpr int kAccumulators = 256;                // columns of tensor memory of a CTA (an SM has 512, and may hold two CTAs)
-constexpr int kProjSmemMax = 224 * 1024;          // dynamic shared memory of a projection (a CTA may have 227 KB in all)
 
 cudaError_t open_kernel(const void *fn, int smem, bool large_cluster) {
     static std::mutex mu;
@@ -171,7 +170,7 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
     // more tiles than SMs: two CTAs to an SM
     // (the activations' share of the ring: from the L2, but all of them after the wait)
-    const int room = (tiles * A.tt * S > sms_ ? kProjSmemMax / 2 : kProjSmemMax) - 1024 - (S > 1 ? sums : 0);
+    const int most = proj_smem_max(A.epi0), room = (tiles * A.tt * S > sms_ ? most / 2 : most) - 1024 - (S > 1 ? sums : 0);
     A.nb = std::min(n, std::max(2, std::min(kProjRing, (rows > 32 ? room * 9 / 20 : room / 3) / b_bytes)));
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
@@ -209,7 +208,7 @@ bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
     for (int passes = (kdim + f.pass - 1) / f.pass; passes <= 16; ++passes) {
         A.chunk = ((kdim + passes - 1) / passes + 63) / 64 * 64;
         const int pitch = A.chunk * 2 + 64, stages = tiles * ((kdim + A.chunk - 1) / A.chunk);
-        slots = std::min(std::min(stages, kProjRing), (kProjSmemMax - red) / (A.slot_rows * pitch));
+        slots = std::min(std::min(stages, kProjRing), (proj_smem_max(A.epi0) - red) / (A.slot_rows * pitch));
         if (slots >= std::min(stages, 2)) break;
         slots = 0;
     }
@@ -263,7 +262,7 @@ AttnArgs Chain::plan_attn(const Dev &D, bool cross, int sets, int t, int Mp) {
 bool Chain::own_queries(const Dev &D, AttnArgs &A) const {
     const int weights = attn_query_smem(D, A.t), pair = 2 * D.P * D.dh * 2;
     if (c_.dtype != 1 || weights == 0 || A.S * D.H * D.B > sms_ || (A.S > 1 && D.H * D.B > clusters_[A.S])) return false;
-    const int room = kProjSmemMax - weights - attn_recv(D, A.S, A.t), pages = (D.cpages + A.S - 1) / A.S;
+    const int room = proj_smem_max(PE_QUERY) - weights - attn_recv(D, A.S, A.t), pages = (D.cpages + A.S - 1) / A.S;
     const int all = A.S > 1 ? pages * pair : (pages - 1) * pair + ((D.C - (pages - 1) * D.P + 31) / 32 * 32) * D.dh * 4;
     A.ring = std::max(all <= room ? all : room / pair * pair, attn_park(D, A.t, 16));
     A.slots = std::min(16, A.ring / pair);

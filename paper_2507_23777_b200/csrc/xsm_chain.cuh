@@ -22,6 +22,9 @@ enum ProjEpilogue : int {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kTokenTile = 128;       // token rows that share a plane
 constexpr int kProjRing = 16;         // most operand blocks of one kind that a CTA keeps in shared memory
+constexpr int kCtaSmem = 227 * 1024;  // shared memory that a CTA may have
+// dynamic shared memory of a projection, at most (what a kernel declares comes on top: for q, k, v the token rows' places too)
+__host__ __device__ constexpr int proj_smem_max(int epi0) { return epi0 == PE_QKV ? 224 * 1024 - 128 : 224 * 1024; }
 
 // A group of weight matrices of one shape in a projection stage: one matrix, or one per decoding head.
 struct ProjGroup {

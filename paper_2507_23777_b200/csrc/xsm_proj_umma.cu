@@ -51,6 +51,8 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     __shared__ uint32_t tmem_slot;
     __shared__ float s_inv[kTokenTile];
     __shared__ RowInfo s_row[kTokenTile];
+    static_assert(sizeof(bars) + sizeof(recv_bar) + sizeof(s_inv) + (EPI0 == PE_QKV ? sizeof(s_row) : 0) + 64 + proj_smem_max(EPI0) <= kCtaSmem,
+                  "a ring that is as large as plan_proj allows has to fit");
     constexpr bool TWO = EPI0 == PE_GATEUP;
     constexpr int kThreads = CL ? kClusterThreads : kTileThreads;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp's number: uniform, also to the compiler)

@@ -26,6 +26,7 @@ SHAPES = {
     "three token rows, width 768": (_model(768, 12, f=3072, K=2), 1),
     "three token rows, width 896": (_model(896, 14, f=1024, K=2), 1),
     "four token rows, width 768": (_model(768, 12, f=3072, K=3), 1),
+    "five token rows, width 1792: rings that fill the shared memory of a CTA": (_model(1792, 28, f=4096, K=4), 1),
     "two token rows, width 2048": (_model(2048, 16, 128, 2048, K=1), 1),
     "five token rows over eight CTAs": (_model(1024, 16, f=4096, K=4), 1),
     "twenty-four token rows": (_model(512, 8, K=5), 4),
