@@ -85,12 +85,19 @@ bool make_layout(const xsm_model_config &c, size_t workspace_bytes, Layout &L) {
     L.hq = take(cur, step_row * d * nh);
     L.ha = take(cur, step_row * d * nh);
     L.ss = take(cur, row * kShareLd);
+    // The padding of the logits' rows (25 KB at most) adds nothing to the workspace, so that a size that held a batch of other
+    // vocabularies before there was padding still does: the timeline and the gathered keys, neither of which outlasts the call that
+    // returns it, share a place (47 and 256 KB at least), and what that leaves over stays unused.
+    const size_t heads = c.n_draft > 0 ? c.n_draft : 1, cond = esize(c) * B * c.n_cond * c.d_cond;
+    const size_t kv = 4 * 2 * (size_t)kKvStagePositions * d, trace = 8 * (size_t)(1 + 2 * L.n_stages) * kTraceCtas;
+    size_t unpadded = cur;
+    for (const size_t bytes : {4 * M * c.vocab, 4 * M * c.vocab * heads, cond, kv, 4 * B * (c.max_seq_len + 1), trace}) take(unpadded, bytes);
     L.logits0 = take(cur, 4 * M * ldv);
-    L.hlogits = take(cur, 4 * M * ldv * (c.n_draft > 0 ? c.n_draft : 1));
-    L.stage_cond = take(cur, esize(c) * B * c.n_cond * c.d_cond);
-    L.stage_kv = take(cur, 4 * 2 * (size_t)kKvStagePositions * d);
+    L.hlogits = take(cur, 4 * M * ldv * heads);
+    L.stage_cond = take(cur, cond);
     L.stage_tok = take(cur, 4 * B * (c.max_seq_len + 1));
-    L.trace = take(cur, 8 * (size_t)(1 + 2 * L.n_stages) * kTraceCtas);
+    L.stage_kv = L.trace = take(cur, kv > trace ? kv : trace);
+    cur = unpadded > cur ? unpadded : cur;
     L.ckv_pool = take(cur, esize(c) * (size_t)c.n_layers * 2 * B * L.cpages * H * P * dh);
     L.hckv_pool = take(cur, esize(c) * nh * 2 * B * L.cpages * H * P * dh);
     L.page_bytes = esize(c) * (size_t)c.n_layers * 2 * H * P * dh;

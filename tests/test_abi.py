@@ -43,6 +43,18 @@ def test_sizes_and_config_checks(lib):
     assert binding.xsm_workspace_bytes(binding.model_config(bad)) == 0
 
 
+def test_workspace_grows_evenly_with_the_vocabulary(lib):
+    """64 token rows: a token more takes 256 bytes for the backbone and for every head (one at least), whatever the rows of logits are padded to, so
+    a workspace that was enough before there was padding is enough."""
+    def size(vocab, **more):
+        return binding.xsm_workspace_bytes(binding.model_config(inputs.config(2, vocab=vocab, max_seq_len=300, **more)))
+    for more in (dict(n_draft=3, batch=16), dict(n_draft=15, batch=4, n_layers=1), dict(n_draft=0, batch=64, n_layers=2),
+                 dict(n_draft=7, batch=8, head_kind=1, d_model=128, n_heads=2, d_cond=128, d_ff=128, head_hidden=128, n_layers=1)):
+        assert size(4096, **more) > 0
+        for vocab in (4097, 4098, 4099, 4100, 4103):
+            assert size(vocab, **more) - size(4096, **more) == (vocab - 4096) * 256 * (1 + max(1, more["n_draft"])), (vocab, more)
+
+
 def test_null_arguments_are_rejected_on_the_host(lib):
     mc = binding.model_config(inputs.config(0))
     out = ctypes.c_void_p()
