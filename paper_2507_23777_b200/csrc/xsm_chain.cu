@@ -184,24 +184,30 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
 }
 
 // The projections over few token rows: how the units are dealt out, passes over the columns, shared memory.  False: the
-// shape does not fit, or the tensor cores of the 5th generation do better.  Whole steps, us, this path and that one, without
-// decoding heads:
-//   token rows        1            2            3            4
-//   width 768      280 285      283 291      287 296      304 294
-//   width 1024     593 574      612 582      659 604      684 623
-//   width 2048    1531 1520    1601 1602    1689 1655        -
-// (A CTA reads all activations here and a slice of them there, which tells as soon as they are more than a few KB.)
+// shape does not fit, or the tensor cores of the 5th generation do better: a CTA reads all activations here and a slice of them there,
+// which tells as soon as they are more than a few KB.  Whole steps of eight layers (four times as many gated as model columns, K
+// heads, vocabulary 2048), us, this path and that one:
+//   token rows         1, K 0     3, K 2     4, K 3     4, K 0     5, K 4     8, K 7     9, K 2    16, K 3
+//   width 128         132 154    138 165    140 167    138 159    147 169    154 180    166 182    173 199
+//   width 256         141 161    152 171    153 175    152 164    165 174    173 179    190 184    202 195
+//   width 384         156 170    166 180    168 182    164 177    186 187    198 189    220 184    239 199
+//   width 512         162 172    175 185    177 188    173 181    197 192    217 196    239 195    255 206
+//   width 640         176 182    191 193    194 195    185 190    208 198    228 207    252 204    266 217
+//   width 768         183 193    198 203    201 207    195 192    219 194    241 201    261 197    277 205
+// With eight times as many gated columns four rows lose in the down projection from 3072 columns on (width 384 191 against 179);
+// with a vocabulary of 8001 five rows of width 256 are even and eight lose (178 against 178, 195 against 184).
 bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
     ProjArgs &A = op.proj;
-    if (rows > kFewRows || c_.d_model > kFewWidth) return false;
+    const int width = rows <= 3 ? 768 : rows == 4 ? 640 : 128, columns = rows <= 3 ? 8192 : rows == 4 ? 2560 : 1024;      // most of each
+    if (rows > 16 || c_.d_model > width || kdim > columns) return false;
     const bool pairs = A.epi0 == PE_QKV || A.epi0 == PE_GATEUP;
     const int units = A.epi0 == PE_QKV ? A.g[0].units / 2 : A.g[0].units + (A.epi1 >= 0 ? A.g[1].units * A.g[1].jobs : 0);
     const int share = A.x_jobs ? std::max(1, sms_ / A.g[0].jobs) : sms_;      // CTAs for `units`
     A.upc = (units + share - 1) / share;
     A.ctas = (units + A.upc - 1) / A.upc;
-    const FewShape f = few_shape(kdim);
+    const FewShape f = few_shape(rows, kdim);
     const int n_rows = A.upc * (pairs ? 2 : 1), tiles = (n_rows + 15) / 16;
-    const int red = tiles * f.warps * 16 * 9 * 4;
+    const int red = tiles * f.warps * 16 * (f.nt * 8 + 1) * 4;
     A.slot_rows = tiles == 1 ? (n_rows + 7) / 8 * 8 : 16;
     // passes no wider than the registers hold, and narrow enough for two of them in flight
     int slots = 0;

@@ -111,12 +111,13 @@ struct ChainLaunch {
 // opens a kernel for `smem` bytes of dynamic shared memory (and for clusters of more than eight CTAs) on the current device
 cudaError_t open_kernel(const void *fn, int smem, bool large_cluster);
 
-// Instance of the projection over few token rows that serves rows of kdim weights: warps that multiply, blocks of 32 columns
-// that each holds in registers, columns of one pass
-struct FewShape { int warps, blocks, pass; };
-constexpr int kFewRows = 3, kFewWidth = 768;      // most token rows, largest d_model
-inline FewShape few_shape(int kdim) {
+// Instance of the projection over few token rows that serves `rows` token rows and rows of kdim weights: warps that multiply, tiles of
+// eight token rows, blocks of 32 columns that each holds in registers, columns of one pass, hi and lo parts in one product
+struct FewShape { int warps, nt, blocks, pass; bool pack; };
+inline FewShape few_shape(int rows, int kdim) {
     FewShape f;
+    f.pack = rows <= 4;
+    f.nt = rows <= 8 ? 1 : 2;
     f.warps = kdim > 2048 ? 15 : 8;
     f.blocks = kdim > 2048 ? 9 : kdim > 1024 ? 8 : 4;
     f.pass = f.warps * f.blocks * 32;

@@ -1,24 +1,25 @@
-// Projections over few token rows (at most three, of narrow bf16 models), as kernels of the launch chain.
+// Projections over few token rows of narrow bf16 models (plan_few), as kernels of the launch chain.
 //
 // A CTA owns a run of weight rows at full width.  Its rows are on their way to shared memory before the kernel waits for
 // its predecessor (bulk copies by a producer warp, tiles of 16 rows x one pass of columns).  Then every warp fetches the
 // activations of its own blocks of 32 columns straight into operand registers (one round trip to L2, nothing is staged),
 // multiplies all tiles with mma.sync.m16n8k16 (weight rows on M; on N the hi parts of four token rows and their lo parts
-// beside them), and parks its partial sums; after one barrier the sums over the warps are finished and stored.
-// Latency is all that counts here (a step has some 200 of these kernels in a row, 2 to 17 MB of weights each): no
-// cluster, because a cluster barrier with remote stores behind it costs 1 us, twice the products.
+// beside them, or eight token rows and a product for each part), and parks its partial sums; after one barrier the sums over the
+// warps are finished and stored.  Latency is all that counts here (a step has about a hundred of these kernels in a row, 0.1 to 9 MB
+// of weights each): no cluster, no exchange.
 #pragma once
 #include "xsm_proj.cuh"
 
 namespace xsm {
 
-// NW: multiplying warps; MAXB: blocks of 32 columns that a warp holds in registers (a pass is NW * MAXB blocks at most)
-template <int NW, int MAXB, int EPI0, int EPI1>
-__global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kernel(const Dev D, const ProjArgs A) {
+// NW: multiplying warps; NT: tiles of eight token rows; PACK: at most four token rows, hi and lo parts side by side in one product,
+// else in products of their own; MAXB: blocks of 32 columns that a warp holds in registers (a pass is NW * MAXB blocks at most)
+template <int NW, int NT, bool PACK, int MAXB, int EPI0, int EPI1>
+__global__ void __launch_bounds__((NW + 1) * 32, NW == 8 && NT == 1 && (PACK || MAXB == 4) ? 2 : 1) proj_few_kernel(const Dev D, const ProjArgs A) {
     extern __shared__ __align__(128) char smem[];
     __shared__ __align__(8) uint64_t full[kProjRing], empty[kProjRing];
-    __shared__ float s_inv[8];
-    constexpr int kOutThreads = NW * 32, LDM = 9;      // (odd pitch: neighbouring rows in other banks)
+    __shared__ float s_inv[NT * 8];
+    constexpr int kOutThreads = NW * 32, LDM = NT * 8 + 1;      // (odd pitch: neighbouring rows in other banks)
     constexpr bool PAIRS = EPI0 == PE_QKV || EPI0 == PE_GATEUP;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (!A.late_go) chain_go();
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
     // Everything that does not depend on the step is worked out before the wait, so that little is left to issue after it (a
     // warp gets an instruction off every 8 cycles here): this thread's first output and where it goes, the places of the
     // warp's activations.
-    constexpr int MP = 8;                          // rows of a plane
+    constexpr int MP = NT * 8;                     // rows of a plane
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
     int lpt = 8;                                   // PE_ADD: lanes per token row
     if (EPI0 == PE_ADD)
@@ -136,19 +137,21 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
     const bool has = warp < NW && tid < M * per_m && o1.r < n_units;
     if (EPI0 == PE_QKV && has && !A.late_go) position(o1);
     const int g = lane >> 2, t4 = lane & 3;
-    // the warp's blocks are warp + NW i.  Lanes 0..15: hi parts of token rows g & 3, the others lo parts; past the last token row
-    // the first one again (what they multiply goes nowhere)
-    const bf16 *x0[2];
+    // the warp's blocks are warp + NW i.  PACK: lanes 0..15 hi parts of token rows g & 3, the others lo parts.  Lanes past the last
+    // token row read the first one of their tile again (what they multiply goes nowhere).
+    const bf16 *x0[2], *x_last[2];      // first (of two tiles) and last tile
 #pragma unroll
     for (int q = 0; q < 2; ++q) {      // (odd NW: the blocks of a warp alternate between the halves of a 64-column block)
-        const int blk = warp + NW * q, m = (g & 3) < M ? g & 3 : 0, chunk8 = (blk & 1) * 4 + t4;
-        x0[q] = A.x + (A.x_jobs ? (size_t)job * 2 * MP * kdim : 0) + (size_t)(blk >> 1) * (128 * MP) + m * 64 + ((chunk8 ^ m) << 3) + (g >> 2) * kLo;
+        const int blk = warp + NW * q, m = PACK ? ((g & 3) < M ? g & 3 : 0) : (NT - 1) * 8 + g < M ? g : 0, chunk8 = (blk & 1) * 4 + t4;
+        const bf16 *base = A.x + (A.x_jobs ? (size_t)job * 2 * MP * kdim : 0) + (size_t)(blk >> 1) * (128 * MP);
+        x0[q] = base + g * 64 + ((chunk8 ^ g) << 3);
+        x_last[q] = base + (NT - 1) * 1024 + m * 64 + ((chunk8 ^ m) << 3) + (PACK ? (g >> 2) * kLo : 0);
     }
     const uint32_t full0 = smem_u32(&full[0]);
     const char *w0 = smem + (size_t)g * pitch + t4 * 16 + warp * 64;
     float *dst0 = red + (size_t)(warp * 16 + g) * LDM + 2 * t4;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) settle(x0[q]);
+    for (int q = 0; q < 2; ++q) { if (NT > 1) settle(x0[q]); settle(x_last[q]); }
     settle(o1.sum); settle(o1.p); settle(o1.h); settle(w0); settle(dst0);
     if (EPI0 == PE_ADD || HEAD) settle(o1.gain);
     if (warp < NW) bar_sync<NW * 32>(1);           // (warps that come to the wait together leave it sooner: 0.3 us a kernel)
@@ -165,16 +168,18 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
     trace_mark(D, 1 + 2 * A.stage);
 
     float h_old = 0.f;
-    auto park = [&](float *dst, const float (&c0)[4], const float (&c1)[4], bool first) {
+    auto park = [&](float *dst, const float (&c0)[NT][4], const float (&c1)[NT][4], bool first) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float v = c0[q] + c1[q];
-            v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
-            if (t4 < 2) {
-                float *o = dst + (q >> 1) * 8 * LDM + (q & 1);
-                *o = first ? v : *o + v;
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float v = c0[nt][q] + c1[nt][q];
+                if (PACK) v += __shfl_xor_sync(0xffffffffu, v, 2);      // columns 0..3: hi parts, 4..7: lo parts of the same rows
+                if (!PACK || t4 < 2) {
+                    float *o = dst + (q >> 1) * 8 * LDM + nt * 8 + (q & 1);
+                    *o = first ? v : *o + v;
+                }
             }
-        }
     };
     if (warp < NW) {
         int sl = 0;
@@ -182,12 +187,17 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
         for (int pass = 0; pass < passes; ++pass) {
             const int nb = min(chunk, kdim - pass * chunk) >> 5;      // blocks of 32 columns
             const size_t xp = (size_t)(pass * (chunk >> 6)) * (128 * MP);
-            uint4 x[MAXB];
+            uint4 x[MAXB][NT], xl[MAXB][NT];      // PACK: both parts; else hi parts, lo parts
 #pragma unroll
             for (int i = 0; i < MAXB; ++i)
                 if (warp + NW * i < nb) {
-                    const int q = (NW & 1) ? i & 1 : 0;
-                    x[i] = __ldcg(reinterpret_cast<const uint4 *>(x0[q] + xp + (size_t)((NW & 1) ? (i >> 1) * NW : i * (NW / 2)) * (128 * MP)));
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        const int q = (NW & 1) ? i & 1 : 0;
+                        const bf16 *p = (nt < NT - 1 ? x0[q] : x_last[q]) + xp + (size_t)((NW & 1) ? (i >> 1) * NW : i * (NW / 2)) * (128 * MP);
+                        x[i][nt] = __ldcg(reinterpret_cast<const uint4 *>(p));
+                        if (!PACK) xl[i][nt] = __ldcg(reinterpret_cast<const uint4 *>(p + kLo));
+                    }
                 }
             if ((EPI0 == PE_ADD || HEAD) && pass == 0 && has) h_old = __ldcg(o1.h);
             float *dst = dst0;
@@ -195,15 +205,28 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
                 const bool two = n_rows - tile * 16 > 8;
                 mbar_wait(full0 + 8u * (uint32_t)sl, par, D.mbar_limit, D.status);
                 const char *ws = w0 + (size_t)sl * slot_bytes;
-                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};      // even and odd steps of 16 columns
+                float c0[NT][4], c1[NT][4];      // PACK: even and odd steps of 16 columns; else hi parts, lo parts
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) c0[nt][q] = c1[nt][q] = 0.f;
 #pragma unroll
                 for (int i = 0; i < MAXB; ++i) {
                     if (warp + NW * i < nb) {
                         const uint4 a = *reinterpret_cast<const uint4 *>(ws + NW * i * 64);
                         uint4 c = make_uint4(0u, 0u, 0u, 0u);
                         if (two) c = *reinterpret_cast<const uint4 *>(ws + 8 * pitch + NW * i * 64);
-                        mma16816_bf16(c0, a.x, c.x, a.y, c.y, x[i].x, x[i].y);
-                        mma16816_bf16(c1, a.z, c.z, a.w, c.w, x[i].z, x[i].w);
+#pragma unroll
+                        for (int nt = 0; nt < NT; ++nt) {
+                            mma16816_bf16(c0[nt], a.x, c.x, a.y, c.y, x[i][nt].x, x[i][nt].y);
+                            if (PACK) {
+                                mma16816_bf16(c1[nt], a.z, c.z, a.w, c.w, x[i][nt].z, x[i][nt].w);
+                            } else {
+                                mma16816_bf16(c1[nt], a.x, c.x, a.y, c.y, xl[i][nt].x, xl[i][nt].y);
+                                mma16816_bf16(c0[nt], a.z, c.z, a.w, c.w, x[i][nt].z, x[i][nt].w);
+                                mma16816_bf16(c1[nt], a.z, c.z, a.w, c.w, xl[i][nt].z, xl[i][nt].w);
+                            }
+                        }
                     }
                 }
                 if (A.slots < tiles * passes) {
@@ -218,7 +241,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
     } else {
         // the producer warp adds up the shares of the sums of squares: four lanes per token row, every fourth quad each
         if (A.ss_parts > 0) {
-            const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)min(g, M - 1) * kShareLd) + t4;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            const float4 *sh = reinterpret_cast<const float4 *>(D.ss + (size_t)min(nt * 8 + g, M - 1) * kShareLd) + t4;
             float4 v[kShareLd / 16];
 #pragma unroll
             for (int q = 0; q < kShareLd / 16; ++q) v[q] = 16 * q + 4 * t4 < A.ss_parts ? __ldcg(sh + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -230,7 +255,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
             }
             ss += __shfl_xor_sync(0xffffffffu, ss, 1);
             ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-            if (t4 == 0) s_inv[g] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+            if (t4 == 0) s_inv[nt * 8 + g] = 1.0f / sqrtf(ss / (float)D.d + D.eps);
+        }
         }
         // then the rest of the weights, as their slots become free
         int sl = 0;
@@ -311,19 +337,19 @@ __global__ void __launch_bounds__((NW + 1) * 32, NW == 8 ? 2 : 1) proj_few_kerne
     trace_mark(D, 2 + 2 * A.stage);
 }
 
-template <int NW, int MAXB, int EPI0, int EPI1>
+template <int NW, int NT, bool PACK, int MAXB, int EPI0, int EPI1>
 static cudaError_t launch_few_instance(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
-    void (*fn)(const Dev, const ProjArgs) = proj_few_kernel<NW, MAXB, EPI0, EPI1>;
+    void (*fn)(const Dev, const ProjArgs) = proj_few_kernel<NW, NT, PACK, MAXB, EPI0, EPI1>;
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     return L.launch(dim3(A.x_jobs ? A.ctas * A.g[0].jobs : A.ctas), dim3((NW + 1) * 32), smem, 1, (const void *)fn, D, A);
 }
 
-template <int NW, int MAXB>
+template <int NW, int NT, bool PACK, int MAXB>
 static cudaError_t launch_few(const Dev &D, const ProjArgs &A, int smem, const ChainLaunch &L) {
-#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_few_instance<NW, MAXB, a, b>(D, A, smem, L)
+#define XSM_EPI(a, b) if (A.epi0 == a && A.epi1 == b) return launch_few_instance<NW, NT, PACK, MAXB, a, b>(D, A, smem, L)
     XSM_EPI(PE_ADD, -1);
-    if constexpr (NW == 8) {
+    if constexpr (NW == 8 && MAXB == 4) {      // (rows of more than 1024 columns: the down projection's only)
         XSM_EPI(PE_QUERY, -1);
         XSM_EPI(PE_QKV, -1);
         XSM_EPI(PE_GATEUP, -1);

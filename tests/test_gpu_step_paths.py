@@ -27,6 +27,15 @@ SHAPES = {
     "three token rows, width 896": (_model(896, 14, f=1024, K=2), 1),
     "four token rows, width 768": (_model(768, 12, f=3072, K=3), 1),
     "five token rows, width 1792: rings that fill the shared memory of a CTA": (_model(1792, 28, f=4096, K=4), 1),
+    "four token rows, width 640": (_model(640, 10, f=2560, K=3), 1),
+    "four token rows, width 512, tcgen05 for the down projection": (_model(512, 8, f=4096, K=3), 1),
+    "five token rows, width 128": (_model(128, 2, K=4), 1),
+    "eight token rows, width 128, tcgen05 for the down projection": (_model(128, 4, 32, 2048, K=7), 1),
+    "nine token rows, width 128": (_model(128, 4, 32, 1024, K=2), 3),
+    "sixteen token rows, width 128": (_model(128, 2, K=3), 4),
+    "seventeen token rows, width 128": (_model(128, 2, K=0), 17),
+    "five token rows, width 128, cross-attention heads": (_model(128, 2, K=4, head_kind=1), 1),
+    "fifteen token rows, width 128, cross-attention heads": (_model(128, 2, K=4, head_kind=1), 3),
     "two token rows, width 2048": (_model(2048, 16, 128, 2048, K=1), 1),
     "five token rows over eight CTAs": (_model(1024, 16, f=4096, K=4), 1),
     "twenty-four token rows": (_model(512, 8, K=5), 4),
