@@ -175,8 +175,10 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.na = std::min(n, std::min(kProjRing, (room - A.nb * b_bytes) / a_bytes));
     A.nb = std::min(n, std::min(kProjRing, (room - A.na * a_bytes) / b_bytes));
     const int sums_fit = kAccumulators / (2 * A.tok);
-    A.many = parts || rows <= 16;
     A.chain = std::max(chain, (n + sums_fit - 1) / sums_fit);
+    // (the residual projections of a step share a kernel: with one for out and one for down, each evicts the other's code, and five
+    // rows of width 768 take 299 us a step instead of 292; with several accumulators in all kernels 295)
+    A.many = n > A.chain || (A.epi0 == PE_ADD && (parts || rows <= 16));
     A.tmem_cols = 32;
     while (A.tmem_cols < (n + A.chain - 1) / A.chain * 2 * A.tok) A.tmem_cols *= 2;
     const int rings = A.na * a_bytes + A.nb * b_bytes;

@@ -40,7 +40,7 @@ struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate)
 // took 0.28 us, eight of them more than the weights' way from memory (5 rows of width 1024 683 -> 631 us a step).
 // G: token rows of a group that is sent and finished together (plan_proj).
 // MANY: the CTA's blocks are added up in accumulators of A.chain blocks each, side by side in tensor memory, and these in fp32 here
-// (plan_proj).  The price is code more than work: 5 rows of width 1024 612 -> 622 us a step, 619 with one accumulator in the same
+// (plan_proj).  The price is code more than work: 5 rows of width 1024 609 -> 621 us a step, 617 with one accumulator in the same
 // code.  Fetching one while the tensor core fills the next (631), two at a time (632), or sending each by itself (646) is slower.
 template <int EPI0, int EPI1, bool CL, int G, bool MANY>
 __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
