@@ -220,6 +220,7 @@ bool Chain::plan_few(ChainOp &op, int rows, int Mp, int kdim) {
         if (slots >= std::min(stages, 2)) break;
         slots = 0;
     }
+    // (a residual projection folds a token row over 32 lanes at most: enough on 24 SMs and more)
     if (slots == 0 || (A.upc > 32 && A.epi0 == PE_ADD) || A.ctas > kShareLd) return false;
     A.kdim = kdim;
     A.rows = rows;

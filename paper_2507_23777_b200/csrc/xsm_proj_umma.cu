@@ -283,10 +283,10 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
             if (EPI0 == PE_QKV) *reinterpret_cast<int4 *>(&s_row[i]) = __ldcg(reinterpret_cast<const int4 *>(D.row_info + mb + m));
         }
     }
-    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row in groups
-    // of four, which lie side by side in shared memory (one 16-byte load for each sender; four single ones met four-way bank
-    // conflicts, half of an epilogue's time at 80 token rows); what it reads from memory is requested before the products
-    // are waited for, or a round ahead.
+    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row in groups of
+    // G, which lie side by side in shared memory: up to 24 rows one by one, else four (one 16-byte load for each sender; four single
+    // ones met four-way bank conflicts, half of an epilogue's time at 80 token rows); what it reads from memory is requested before
+    // the products are waited for, or a round ahead.
     float hn[G];
     float2 csn[G];
     auto request = [&](int group) {
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
 template <int EPI0, int EPI1, bool CL, int G, bool MANY>
 static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMaps &T, int smem, const ChainLaunch &L) {
     void (*fn)(const Dev, const ProjArgs, const ProjMaps) = proj_umma_kernel<EPI0, EPI1, CL, G, MANY>;
-    cudaError_t e = open_kernel((const void *)fn, smem, A.S > 8);
+    cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
     return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? kClusterThreads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
