@@ -17,8 +17,8 @@ def _model(d=512, H=8, dh=64, f=1024, K=4, L=1, V=777, C=40, **kw):
 
 # model, sequences, tokens of the prompt
 SHAPES = {
-    # projections: few token rows (one and two tiles of eight, packed hi and lo parts), tensor cores from 17 rows on, token rows
-    # in parts from 97
+    # projections: mma.sync up to four token rows at this width, tensor cores from five on; accumulators of four blocks up to sixteen
+    # rows, of all blocks behind; tiles and remainders of token rows, these cut into parts from 49 on
     "one token row": (_model(K=0), 1, 1),
     "four token rows": (_model(K=3), 1, 1),
     "nine token rows": (_model(K=2), 3, 1),
