@@ -40,8 +40,8 @@ struct __align__(64) ProjMaps { CUtensorMap w0, w1; };      // group 0 (or gate)
 // took 0.28 us, eight of them more than the weights' way from memory (5 rows of width 1024 683 -> 631 us a step).
 // G: token rows of a group that is sent and finished together (plan_proj).
 // MANY: the CTA's blocks are added up in accumulators of A.chain blocks each, side by side in tensor memory, and these in fp32 here
-// (plan_proj).  The price is code more than work: 5 rows of width 1024 609 -> 621 us a step, 617 with one accumulator in the same
-// code.  Fetching one while the tensor core fills the next (631), two at a time (632), or sending each by itself (646) is slower.
+// (plan_proj).  The price is code as much as work: 5 rows of width 1024 611 -> 615 us a step, 7 of width 2048 1647 -> 1691.  Fetching
+// one while the tensor core fills the next, two at a time, or sending each by itself is 1.5 to 4 % slower.
 template <int EPI0, int EPI1, bool CL, int G, bool MANY>
 __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_umma_kernel(const Dev D, const ProjArgs A, const __grid_constant__ ProjMaps T) {
     extern __shared__ char smem_raw[];
@@ -217,43 +217,38 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) umma_mma(sum, a + 2 * ks, b + 2 * ks, idesc, (add || ks > 0) ? 1u : 0u);
         };
-        // an accumulator after the other: blocks [i0, i1)
+        // (one loop with a counter: a loop for each accumulator around one for its blocks costs 2 % of a step where rings are refilled)
         uint32_t sum = tmem;
+        int held = 0;      // blocks in the accumulator
+        auto next_sum = [&]() {
+            if (!MANY) held = 1;
+            else if (++held == A.chain) { held = 0; sum += (uint32_t)(2 * Nt); }
+        };
         if (flat) {
             mbar_wait(full_b, 0u, D.mbar_limit, D.status);
-            for (int i0 = 0;;) {
-                const int i1 = MANY ? min(i0 + A.chain, n) : n;
-                for (int i = i0; i < i1; ++i) {
-                    mbar_wait(full_a + 8u * (uint32_t)i, 0u, D.mbar_limit, D.status);
-                    tcgen05_after_sync();
-                    if (leader) products(sum, i, i, i > i0);
-                }
-                if (!MANY || i1 == n) break;
-                i0 = i1;
-                sum += (uint32_t)(2 * Nt);
+            for (int i = 0; i < n; ++i) {
+                mbar_wait(full_a + 8u * (uint32_t)i, 0u, D.mbar_limit, D.status);
+                tcgen05_after_sync();
+                if (leader) products(sum, i, i, held > 0);
+                next_sum();
             }
         } else {
             const uint32_t empty_a = bar(1, 0), empty_b = bar(3, 0);
             int ia = 0, ib = 0;
             uint32_t pa = 0u, pb = 0u;
-            for (int i0 = 0;;) {
-                const int i1 = MANY ? min(i0 + A.chain, n) : n;
-                for (int i = i0; i < i1; ++i) {
-                    mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
-                    mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
-                    tcgen05_after_sync();
-                    if (leader) {
-                        products(sum, ia, ib, i > i0);
-                        if (i + na < n) umma_commit(empty_a + 8u * (uint32_t)ia);
-                        if (i + nb < n) umma_commit(empty_b + 8u * (uint32_t)ib);
-                    }
-                    if (++ia == na) { ia = 0; pa ^= 1u; }
-                    if (++ib == nb) { ib = 0; pb ^= 1u; }
-                    __syncwarp();      // (a lane two fills of a slot behind the leader would wait for a phase that has gone by)
+            for (int i = 0; i < n; ++i) {
+                mbar_wait(full_a + 8u * (uint32_t)ia, pa, D.mbar_limit, D.status);
+                mbar_wait(full_b + 8u * (uint32_t)ib, pb, D.mbar_limit, D.status);
+                tcgen05_after_sync();
+                if (leader) {
+                    products(sum, ia, ib, held > 0);
+                    if (i + na < n) umma_commit(empty_a + 8u * (uint32_t)ia);
+                    if (i + nb < n) umma_commit(empty_b + 8u * (uint32_t)ib);
                 }
-                if (!MANY || i1 == n) break;
-                i0 = i1;
-                sum += (uint32_t)(2 * Nt);
+                next_sum();
+                if (++ia == na) { ia = 0; pa ^= 1u; }
+                if (++ib == nb) { ib = 0; pb ^= 1u; }
+                __syncwarp();      // (a lane two fills of a slot behind the leader would wait for a phase that has gone by)
             }
         }
         if (leader) umma_commit(done);
