@@ -222,8 +222,8 @@ __device__ __forceinline__ unsigned ldcg_u32(const void *p) { return __ldcg(rein
 // stream (every warp multiplies all rows over its share of the columns, as in the projections over few token rows), instead
 // of a kernel of its own: 630 against 650 us a step at width 1024.  The head's rows of the projection and the pages are requested
 // before the wait; a CTA (544 threads of 96 registers) shares an SM with none of the projections, but the out-projection before it
-// holds 64 of 148, so the sixteen CTAs of a sequence start some 7 us before it ends.  4.0 us after the wait: 0.5 until the
-// activations come, 0.9 products (128 KB of weights through shared memory), 0.6 sums, 1.0 keys, 1.3 merge and output.
+// holds 64 of 148, so the sixteen CTAs of a sequence start some 7 us before it ends.  4.0 us after the wait: 0.6 until the
+// activations come, 1.3 products (128 KB of weights through shared memory), 0.4 sums, 1.1 keys, 0.6 merge and output.
 constexpr int kQueryBlocks = 4;      // blocks of 32 columns per warp: d_model up to 1024
 //
 // NW: warps that attend, beside the producer.  A unit of 32 keys is some 300 dependent instructions, 1 us for a warp on its

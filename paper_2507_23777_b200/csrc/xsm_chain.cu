@@ -124,13 +124,14 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     A.rows = rows;
     A.Mp = Mp;
     const int tiles = A.g[0].tiles + (A.epi1 >= 0 ? A.g[1].tiles : 0), nblk = kdim / 64;
-    // How a tile of weight rows is cut: its columns over a cluster of S CTAs, as many as fit into the GPCs at a time (of six CTAs
-    // 22 clusters, of eight 15; a cluster more is a second wave).  More than 48 token rows in one plane: these into T parts too,
+    // How a tile of weight rows is cut: its columns over a cluster of S CTAs, as many as fit into the GPCs at a time, an SM to each
+    // CTA (of six CTAs 22 clusters, of eight 15; where two CTAs fit an SM more would run, which has not been tried).  More than 48 token rows in one plane: these into T parts too,
     // each with the weights for itself, which leaves less to exchange and to finish in a CTA.  There the stage's time after the
     // wait in cycles, as measured, chooses among S and T: a product 47, or N / 2 where the token rows (hi and lo) bound it;
     // activations, and weights that do not fit the ring, 59 bytes a cycle; 45 for every token row that is sent, 250 for every
-    // one that is finished.  Eight layers of width 1024: 90 rows 480 -> 425 us a step, 80 rows 444 -> 414, 60 rows 409 -> 375; 40
-    // rows 354 -> 356, 30 rows 304 -> 331, so up to 48 rows T is 1 and the largest S that fits is taken, without weighing.
+    // one that is finished.  Eight layers of width 1024, whole rows and parts: 112 rows 565 and 459 us a step, 90 rows 470 and 424, 80
+    // rows 433 and 411, 60 rows 401 and 369, 50 rows 373 and 361; with one accumulator 40 rows 354 and 356, 30 rows 304 and 331, so
+    // up to 48 rows T is 1 and the largest S that fits is taken, without weighing.
     //
     // How many blocks an accumulator adds up: every instruction cuts off what lies below the accumulator's last bit, so the error of a
     // sum grows with their number (projections alone, against 64 bits, in units of 1e-6 of the result: sums of 128 instructions at
