@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     static_assert(sizeof(bars) + sizeof(recv_bar) + sizeof(s_inv) + (EPI0 == PE_QKV ? sizeof(s_row) : 0) + 64 + proj_smem_max(EPI0) <= kCtaSmem,
                   "a ring that is as large as plan_proj allows has to fit");
     constexpr bool TWO = EPI0 == PE_GATEUP;
-    constexpr int kThreads = CL ? kClusterThreads : kTileThreads;
+    constexpr int kThreads = CL ? kClusterThreads : kTileThreads, kTmemWarp = kThreads / 32 - 1;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp's number: uniform, also to the compiler)
     const int S = CL ? A.S : 1, rank = CL ? (int)cluster_rank() : 0, Mp = A.Mp;
     // sequences that still run: looked at just before the wait, when the weights are on their way
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         }
         mbar_init_fence();
         if (CL && lane == 31 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + G - 1) / G)) * (512u * G));
-    } else if (warp == 2) {
+    } else if (warp == kTmemWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         if (!A.late_go) chain_go();
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         if (tid == 0)
             for (int i = 0; i < min(n, na); ++i) mbar_wait(bar(0, i), 0u, D.mbar_limit, D.status);
         __syncthreads();
-        if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
+        if (warp == kTmemWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
         return;
     }
     if (A.late_go) chain_go();
@@ -334,6 +334,16 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         }
     }
     tcgen05_before_sync();
+    // The tensor memory goes back while the shares are on their way, by the last warp, which has token rows of its own only where there
+    // are many (at the kernel's end it kept the next one waiting: 5 rows of width 768 35.7 -> 34.6 ms a request, of width 1024 59.3 ->
+    // 58.1, 20 rows 40.1 -> 39.0, 7 rows of width 2048 59.9 -> 59.7).
+    if (warp != kTmemWarp) {
+        asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
+    } else {
+        asm volatile("bar.sync 2, %0;" :: "n"(kThreads) : "memory");
+        tcgen05_after_sync();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
+    }
     // One CTA to a tile: a barrier.  In a cluster every CTA waits for all shares of its rows, its own among them, so none leaves
     // before what is sent to it has come: no barrier at the end, whose wait for all stores took 1600 to 2400 cycles.
     if (!CL) __syncthreads();
@@ -441,14 +451,6 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     if (D.trace != nullptr) {
         __syncthreads();
         trace_mark(D, 2 + 2 * A.stage);
-    }
-    // (every warp has read its part of the accumulator)
-    if (warp != 2) {
-        asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
-    } else {
-        asm volatile("bar.sync 2, %0;" :: "n"(kThreads) : "memory");
-        tcgen05_after_sync();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
     }
 }
 
