@@ -120,8 +120,11 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         if (!A.late_go) chain_go();
     }
     __syncwarp();
-    // "this CTA runs": what it has set up is there, and peers may write to its shared memory, after cluster_wait
-    if (CL) cluster_arrive();
+    // "this CTA runs": its barriers are there (mbar_init_fence), and peers may write to its shared memory, after cluster_wait.  A release
+    // would wait for the load above, and hold back the weights' copies, which a kernel that starts late waits for: 5 rows of width 768
+    // 37.6 -> 37.2 ms a request, of width 1024 61.1 -> 60.6, 20 rows 38.8 -> 37.4, 7 rows of width 2048 59.4 -> 58.8 (all of them with
+    // a thread for every weight row and no more, where one token row is finished).
+    if (CL) cluster_arrive_relaxed();
     if (warp == 0 && elect_one())      // the weights' way is the longest: it begins as early as that
         for (int i = 0; i < min(n, na); ++i) load_a(i, i);
     __syncwarp();
@@ -165,7 +168,6 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     if (CL) cluster_wait();            // the peers run: their barriers and shared memory are there
     else __syncthreads();
     tcgen05_after_sync();
-    const uint32_t tmem = tmem_slot;
     if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (active == 0) {      // every sequence has ended in an earlier step
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
             for (int ks = 0; ks < 4; ++ks) umma_mma(sum, a + 2 * ks, b + 2 * ks, idesc, (add || ks > 0) ? 1u : 0u);
         };
         // (one loop with a counter: a loop for each accumulator around one for its blocks costs 2 % of a step where rings are refilled)
-        uint32_t sum = tmem;
+        uint32_t sum = tmem_slot;
         int held = 0;      // blocks in the accumulator
         auto next_sum = [&]() {
             if (!MANY) held = 1;
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     const bool done_ok = mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
     tcgen05_after_sync();
+    const uint32_t tmem = tmem_slot;      // (its warp has arrived at `done`)
     for (int c = c0; c < (Nt >> 3); c += kThreads / 128) {      // hi and lo parts added
         uint32_t v[16];
         tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
