@@ -166,6 +166,10 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int tile_rows = std::min(rows, A.tok), G = S > 1 && rows <= 24 ? 1 : 4;
     A.group = G;
     A.tps = ((tile_rows + G - 1) / G + S - 1) / S * G;
+    // Four warps more than finish token rows (they are those that also fetch and multiply), or as many as the accumulator's columns
+    // keep busy: 256 against 384 threads, 5 rows of width 768 34.56 -> 34.15 ms a request, of width 1024 58.24 -> 57.09, one row 54.49
+    // -> 53.91 (with the start without a release); 128, the same warps for all of it, 37.6 and 61.1.
+    A.threads = G == 1 ? 128 * std::min(kClusterThreads / 128, std::max(1 + (A.epi0 == PE_GATEUP ? (A.tps + 1) / 2 : A.tps), A.tok / 8)) : kClusterThreads;
     A.inv_s = 65536 / S + 1;
     A.inv_q = 65536 / (A.tps / G) + 1;
     const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;

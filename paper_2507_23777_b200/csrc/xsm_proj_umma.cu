@@ -21,10 +21,10 @@
 
 namespace xsm {
 
-// CL: a tile's columns are cut over a cluster.  384 threads of at most 80 registers, so that the SM has room for the next kernel's
+// CL: a tile's columns are cut over a cluster.  256 or 384 threads (plan_proj) of at most 80 registers, so that the SM has room for the next kernel's
 // CTA as well (with 512 of 67 to 103 the next kernel's barriers, tensor memory and first copies came after this one's end: 20
 // token rows of width 1024 961 -> 908 us a step, 80 rows 1391 -> 1397).  Without a cluster two CTAs of 512 to an SM.
-constexpr int kClusterThreads = 384, kTileThreads = 512;
+constexpr int kTileThreads = 512;
 constexpr int kBlockK = 64;                        // columns of one operand block (128 bytes: one swizzled row)
 constexpr int kABytes = 128 * kBlockK * 2;         // weight block
 
@@ -54,7 +54,10 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     static_assert(sizeof(bars) + sizeof(recv_bar) + sizeof(s_inv) + (EPI0 == PE_QKV ? sizeof(s_row) : 0) + 64 + proj_smem_max(EPI0) <= kCtaSmem,
                   "a ring that is as large as plan_proj allows has to fit");
     constexpr bool TWO = EPI0 == PE_GATEUP;
-    constexpr int kThreads = CL ? kClusterThreads : kTileThreads, kTmemWarp = kThreads / 32 - 1;
+    const int threads = CL && G == 1 ? (int)blockDim.x : CL ? kClusterThreads : kTileThreads;
+    // Of eight warps the first four fetch, multiply and set up, the others take the accumulator and the first token rows.
+    const bool apart = CL && G == 1 && threads == 256;
+    const int tmem_warp = apart ? 3 : (threads >> 5) - 1;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp's number: uniform, also to the compiler)
     const int S = CL ? A.S : 1, rank = CL ? (int)cluster_rank() : 0, Mp = A.Mp;
     // sequences that still run: looked at just before the wait, when the weights are on their way
@@ -109,12 +112,12 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     } else if (warp == 1) {
         if (lane < nb) { mbar_init(bar(2, lane), 1u); mbar_init(bar(3, lane), 1u); }
         if (lane == 31) {
-            mbar_init(done, kThreads / 32 - 1);      // the last products, and what the epilogue needs to know (warps 2 and up)
+            mbar_init(done, (uint32_t)(threads >> 5) - 1u);      // the last products, and what the epilogue needs to know (warps 2 and up)
             mbar_init(smem_u32(&recv_bar), 1u);
         }
         mbar_init_fence();
         if (CL && lane == 31 && nm > 0) mbar_arrive_expect_tx(smem_u32(&recv_bar), (uint32_t)(S * ((nm + G - 1) / G)) * (512u * G));
-    } else if (warp == kTmemWarp) {
+    } else if (warp == tmem_warp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tmem_slot)), "r"(A.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         if (!A.late_go) chain_go();
@@ -133,9 +136,11 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     const bf16 *xb = x + (size_t)k_lo * (128 * Mp) + (size_t)pm * 128;      // this CTA's blocks of the activations
     const uint32_t idesc = umma_idesc(128, 2 * Nt), full_a = bar(0, 0), full_b = bar(2, 0);
     settle(xb);
-    constexpr int ROWS = TWO ? 64 : 128, SIDES = kThreads / ROWS;
+    constexpr int ROWS = TWO ? 64 : 128;
+    const int sides = threads / ROWS;
     constexpr bool HEAD = EPI0 == PE_HEADADD || EPI1 == PE_HEADY;
-    const int row = tid & (ROWS - 1), side = tid / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
+    const int place = apart ? tid ^ 128 : tid;
+    const int row = tid & (ROWS - 1), side = place / ROWS, u_row = u0 + row, half = D.dh >> 1, e = row & (D.dh - 1);
     const bool live_row = u_row < W.units;
     const uint32_t gain_bits = (EPI0 == PE_ADD || HEAD) && u_row < D.d ? ld_early_u16(reinterpret_cast<const bf16 *>(A.gain) + u_row) : 0u;
     // where this thread's weight row goes
@@ -149,7 +154,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     // Accumulator -> the CTA that finishes the token rows: [sender][group][weight row][G].  This thread's lane of the accumulator
     // is its weight row; eight token rows at a time, from c0 on.
     constexpr int GROUPS = 8 / G;
-    const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = warp >> 2;
+    const int lanes = warp & 3, arow = lanes * 32 + lane, c0 = place >> 7;
     const uint32_t recv_b = smem_u32(&recv_bar);
     uint32_t dst[GROUPS], dst_bar[GROUPS];
     auto where = [&](int c) {
@@ -168,13 +173,13 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     if (CL) cluster_wait();            // the peers run: their barriers and shared memory are there
     else __syncthreads();
     tcgen05_after_sync();
-    if (warp > 0) asm volatile("bar.sync 1, %0;" :: "n"(kThreads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
+    if (warp > 0) asm volatile("bar.sync 1, %0;" :: "r"(threads - 32) : "memory");      // (warps that come to the wait together leave it sooner)
     chain_wait();
     if (active == 0) {      // every sequence has ended in an earlier step
         if (tid == 0)
             for (int i = 0; i < min(n, na); ++i) mbar_wait(bar(0, i), 0u, D.mbar_limit, D.status);
         __syncthreads();
-        if (warp == kTmemWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
+        if (warp == tmem_warp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_slot), "r"(A.tmem_cols) : "memory");
         return;
     }
     if (A.late_go) chain_go();
@@ -258,7 +263,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     }
     // meanwhile: what the epilogue needs to know of the token rows that this CTA finishes
     if (warp >= 2) {
-        for (int i = tid - 64; i < nm; i += kThreads - 64) {
+        for (int i = tid - 64; i < nm; i += threads - 64) {
             const int m = m0 + i;
             float inv = 1.f;
             if (A.ss_parts > 0) {
@@ -280,7 +285,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
             if (EPI0 == PE_QKV) *reinterpret_cast<int4 *>(&s_row[i]) = __ldcg(reinterpret_cast<const int4 *>(D.row_info + mb + m));
         }
     }
-    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the SIDES threads of a weight row in groups of
+    // The epilogue: thread = weight row, the token rows of this CTA are dealt out to the `sides` threads of a weight row in groups of
     // G, which lie side by side in shared memory: up to 24 rows one by one, else four (one 16-byte load for each sender; four single
     // ones met four-way bank conflicts, half of an epilogue's time at 80 token rows); what it reads from memory is requested before
     // the products are waited for, or a round ahead.
@@ -302,7 +307,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     __syncwarp();
     tcgen05_after_sync();
     const uint32_t tmem = tmem_slot;      // (its warp has arrived at `done`)
-    for (int c = c0; c < (Nt >> 3); c += kThreads / 128) {      // hi and lo parts added
+    for (int c = c0; c < (Nt >> 3); c += threads >> 7) {      // hi and lo parts added
         uint32_t v[16];
         tmem_ld16(v, tmem + ((uint32_t)(lanes * 32) << 16) + (uint32_t)c * 16u);
         if (c != c0) where(c);
@@ -340,10 +345,10 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     // The tensor memory goes back while the shares are on their way, by the last warp, which has token rows of its own only where there
     // are many (at the kernel's end it kept the next one waiting: 5 rows of width 768 35.7 -> 34.6 ms a request, of width 1024 59.3 ->
     // 58.1, 20 rows 40.1 -> 39.0, 7 rows of width 2048 59.9 -> 59.7).
-    if (warp != kTmemWarp) {
-        asm volatile("bar.arrive 2, %0;" :: "n"(kThreads) : "memory");
+    if (warp != tmem_warp) {
+        asm volatile("bar.arrive 2, %0;" :: "r"(threads) : "memory");
     } else {
-        asm volatile("bar.sync 2, %0;" :: "n"(kThreads) : "memory");
+        asm volatile("bar.sync 2, %0;" :: "r"(threads) : "memory");
         tcgen05_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
     }
@@ -386,12 +391,12 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         qrow[(size_t)m * D.d] = hi;
         qrow[(size_t)(A.qp + m) * D.d] = lo;
     };
-    for (int group = side; G * group < nm; group += SIDES) {
+    for (int group = side; G * group < nm; group += sides) {
         float h[G];
         float2 cs[G];
 #pragma unroll
         for (int q = 0; q < G; ++q) { h[q] = hn[q]; cs[q] = csn[q]; }
-        request(group + SIDES);
+        request(group + sides);
         float sum[G], other[G];      // other: the rotation partner's, or up's
         total(group, row, sum);
         if (TWO) total(group, row + 64, other);
@@ -463,7 +468,7 @@ static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMa
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
-    return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? kClusterThreads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
+    return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? A.threads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
 }
 
 template <int EPI0, int EPI1, bool MANY>
