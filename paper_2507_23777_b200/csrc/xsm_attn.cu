@@ -382,6 +382,9 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             trace_mark(D, 1 + 2 * A.stage);
         }
         if (FEW) {
+            // Warps without keys neither fetch queries nor leave a state: 5 rows of width 768 34.15 -> 33.77 ms a request, of width
+            // 1024 57.09 -> 56.84, 20 rows 37.50 -> 37.10, 7 rows of width 2048 58.82 -> 58.09.
+            const bool busy = !all_in || warp < n_units;
             unsigned qh[DH / 8], ql[DH / 8];
             if constexpr (QP) {
                 constexpr int TILES = DH / 32;       // row tiles of a warp: eight warps share the columns, two such groups the rows
@@ -441,8 +444,8 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             } else
 #pragma unroll
             for (int c = 0; c < DH / 8; ++c) {
-                qh[c] = g < t_rows ? ldcg_u32(qhi + 8 * c) : 0u;
-                ql[c] = g < t_rows ? ldcg_u32(qlo + 8 * c) : 0u;
+                qh[c] = g < t_rows && busy ? ldcg_u32(qhi + 8 * c) : 0u;
+                ql[c] = g < t_rows && busy ? ldcg_u32(qlo + 8 * c) : 0u;
             }
             FewState<DH> ws;
 #pragma unroll
@@ -481,7 +484,7 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int r = 2 * t4 + c;
-                if (real && r < t_rows) {
+                if (real && busy && r < t_rows) {
                     float *dst = st + (warp * srows + r) * LD;
 #pragma unroll
                     for (int dp = 0; dp < DH / 16; ++dp) {
