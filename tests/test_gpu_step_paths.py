@@ -1,5 +1,5 @@
 """GPU parity on both sides of the lines at which a decoding step changes path: mma.sync or tcgen05 projections, several accumulators
-or one, token rows dealt out one by one or in fours and cut into parts, the tail's rows of logits and its choice of the best tokens, and the token
+or one, token rows dealt out one by one or in fours and cut into parts, warps of a projection, the tail's rows of logits and its choice of the best tokens, and the token
 rows that fp32 kernels fold together."""
 import numpy as np
 import pytest
@@ -40,6 +40,9 @@ SHAPES = {
     "five token rows over eight CTAs": (_model(1024, 16, f=4096, K=4), 1),
     "sixteen token rows, width 2048, eight accumulators": (_model(2048, 16, 128, 2048, K=3, V=1500), 4),
     "seventeen token rows, width 2048, one accumulator": (_model(2048, 16, 128, 2048, K=0, V=1500), 17),
+    "eight token rows, two to a CTA": (_model(1792, 28, f=2048, K=7), 1),
+    "sixteen token rows, two accumulator parts": (_model(1024, 16, f=4096, K=3), 4),
+    "two token rows, width 1024": (_model(1024, 16, f=4096, K=1), 1),
     "twenty-four token rows": (_model(512, 8, K=5), 4),
     "twenty-five token rows": (_model(512, 8, K=4), 5),
     "forty-eight token rows": (_model(512, 8, K=5), 8),
