@@ -216,6 +216,16 @@ XSM_API xsm_status xsm_debug_set_wait_limits(xsm_ctx *ctx, uint32_t polls, uint3
  * runs out; the status then shows at the next synchronising call, and xsm_prefill starts afresh. */
 XSM_API xsm_status xsm_debug_launch_stage(xsm_ctx *ctx, int stage);
 
+/* How one decoding step of `batch` sequences (prompt_positions 0), or a chunk of so many positions of each of their prompts, is cut over
+ * a chip of `sms` SMs on which clusters[s] clusters of s = 2..8 CTAs run at a time (HOST int32 [9]; NULL: the current device).  Nothing
+ * is launched, and with `clusters` no device is needed.  h_stages HOST int32 [capacity][8], a row for every kernel: its kind (0: tensor
+ * cores of the 5th generation; 1: mma.sync; 2: fp32; 3: attention; 4: tail; 5: embedding) and, for kind 0, what it does (0: q, k, v; 1:
+ * residual; 2: cross q; 3: gate/up; 4: logits; 6: head out-projection), threads, CTAs of a cluster, token rows of a tile, token rows that
+ * a CTA finishes, columns of tensor memory, bytes of shared memory that a CTA takes at least.  Returns the number of kernels, 0 where
+ * there is no such step. */
+XSM_API int xsm_debug_plan(const xsm_model_config *cfg, int batch, int prompt_positions, int sms, const int32_t *clusters,
+                           int32_t *h_stages, int capacity);
+
 /* Launches the stages of a step one after the other, without overlap, instead of as a recorded graph (1) or back (0). */
 XSM_API xsm_status xsm_debug_set_phase_launch(xsm_ctx *ctx, int on);
 

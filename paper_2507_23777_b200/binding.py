@@ -23,7 +23,7 @@ EXPORTS = [
     "xsm_generate_host", "xsm_destroy", "xsm_last_error", "xsm_kernel_launches", "xsm_debug_get_logits",
     "xsm_debug_get_kv", "xsm_debug_set_drafts", "xsm_debug_get_state", "xsm_debug_set_phase_launch",
     "xsm_debug_trace_step", "xsm_spec_step_static", "xsm_debug_set_wait_limits", "xsm_debug_launch_stage",
-    "xsm_debug_set_script",
+    "xsm_debug_set_script", "xsm_debug_plan",
 ]
 
 
@@ -86,6 +86,8 @@ def load(path: str | None = None):
     L.xsm_debug_set_phase_launch.argtypes = [vp, C.c_int]
     L.xsm_debug_set_script.argtypes = [vp, ip, C.c_int, C.c_float]
     L.xsm_debug_set_wait_limits.argtypes = [vp, C.c_uint32, C.c_uint32]
+    L.xsm_debug_plan.restype = C.c_int
+    L.xsm_debug_plan.argtypes = [C.POINTER(ModelConfig), C.c_int, C.c_int, C.c_int, vp, vp, C.c_int]
     L.xsm_debug_launch_stage.argtypes = [vp, C.c_int]
     L.xsm_debug_trace_step.argtypes = [vp, vp, C.c_size_t, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     if path is None:
@@ -111,6 +113,13 @@ def xsm_weights_bytes(mc: ModelConfig) -> int:
 
 def xsm_workspace_bytes(mc: ModelConfig) -> int:
     return load().xsm_workspace_bytes(C.byref(mc))
+
+
+def xsm_debug_plan(mc: ModelConfig, batch: int, prompt_positions: int = 0, sms: int = 0, clusters=None) -> np.ndarray:
+    """The kernels of a step, a row each (see include/xsm.h); clusters: how many of 0..8 CTAs run at a time (None: the current device)."""
+    own = None if clusters is None else np.ascontiguousarray(clusters, dtype=np.int32)
+    out = np.zeros((8 * mc.n_layers + 8, 8), dtype=np.int32)
+    return out[:load().xsm_debug_plan(C.byref(mc), batch, prompt_positions, sms, _np_ptr(own), _np_ptr(out), len(out))]
 
 
 def _np_ptr(a):

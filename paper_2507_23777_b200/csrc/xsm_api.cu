@@ -187,6 +187,16 @@ WeightOffsets weight_offsets(const xsm_model_config &c) {
     return w;
 }
 
+// what the launch chain goes by
+void set_shape(Dev &D, const xsm_model_config &c, const Layout &L) {
+    D.L = c.n_layers; D.d = c.d_model; D.H = c.n_heads; D.dh = c.d_head; D.f = c.d_ff;
+    D.V = c.vocab; D.ldv = (int)logits_ld(c); D.C = c.n_cond; D.dc = c.d_cond; D.K = c.n_draft; D.K1 = c.n_draft + 1;
+    D.P = c.page_size; D.max_blocks = L.max_blocks; D.n_pages = L.n_pages; D.cpages = L.cpages;
+    D.head_kind = c.head_kind;
+    D.scale = (float)(1.0 / sqrt((double)c.d_head));
+}
+void set_batch(Dev &D, int batch) { D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8; }
+
 }  // namespace
 
 struct xsm_ctx {
@@ -365,17 +375,14 @@ xsm_status xsm_create(const xsm_model_config *cfg, const void *d_weights, void *
 
     Dev &D = ctx->dev;
     memset(&D, 0, sizeof(D));
-    D.L = cfg->n_layers; D.d = cfg->d_model; D.H = cfg->n_heads; D.dh = cfg->d_head; D.f = cfg->d_ff;
-    D.V = cfg->vocab; D.ldv = (int)logits_ld(*cfg); D.C = cfg->n_cond; D.dc = cfg->d_cond; D.K = cfg->n_draft; D.K1 = cfg->n_draft + 1;
-    D.P = cfg->page_size; D.max_blocks = L.max_blocks; D.n_pages = L.n_pages; D.cpages = L.cpages;
+    set_shape(D, *cfg, L);
     D.p_shift = -1;
     for (int sh = 0; sh < 30; ++sh)
         if ((1 << sh) == cfg->page_size) D.p_shift = sh;
     D.max_seq_len = cfg->max_seq_len; D.tok_ld = L.tok_ld;
-    D.eps = cfg->rms_eps; D.scale = (float)(1.0 / sqrt((double)cfg->d_head)); D.bos = cfg->bos_id; D.eos = cfg->eos_id;
+    D.eps = cfg->rms_eps; D.bos = cfg->bos_id; D.eos = cfg->eos_id;
     D.spin_limit = kSpinLimit; D.mbar_limit = kMbarSpinLimit;
     D.E = wptr(ctx, ctx->wo.E); D.gain_first = wptr(ctx, ctx->wo.g1[0]);
-    D.head_kind = cfg->head_kind;
     D.len = at<int>(ctx, L.len); D.window = at<int>(ctx, L.window);
     D.finished = at<int>(ctx, L.finished); D.n_gen = at<int>(ctx, L.n_gen);
     D.n_blocks = at<int>(ctx, L.n_blocks); D.block_table = at<int>(ctx, L.block_table);
@@ -424,7 +431,7 @@ xsm_status xsm_prefill(xsm_ctx *ctx, int batch, const void *d_cond, const int32_
     if (capture != XSM_OK) return capture;
     Dev &D = ctx->dev;
     if (c.dtype == 0 && batch * D.K1 > kF32Rows) return fail(ctx, XSM_ERR_CAPACITY, "fp32 models support at most 24 token rows per step");
-    D.B = batch; D.M = batch * D.K1; D.Mp = (D.M + 7) / 8 * 8;
+    set_batch(D, batch);
     if (!ctx->chain.select(D)) return fail(ctx, XSM_ERR_CUDA, "the tensor maps of the step could not be made");
     ctx->n_stages = ctx->chain.n_ops();
     RunParams r;
@@ -711,6 +718,38 @@ xsm_status xsm_debug_launch_stage(xsm_ctx *ctx, int stage) {
     XSM_CUDA(ctx, launch_stage_mark(ctx->dev, (stage + 1) % ctx->n_stages, ctx->stream));
     ctx->launches += 2;
     return XSM_OK;
+}
+
+int xsm_debug_plan(const xsm_model_config *cfg, int batch, int prompt_positions, int sms, const int32_t *clusters, int32_t *h_stages, int capacity) {
+    if (!cfg || !h_stages || check_config(*cfg) || cfg->n_layers > capacity || batch < 1 || batch > cfg->max_batch || prompt_positions < 0 || prompt_positions > cfg->max_seq_len) return 0;
+    if (prompt_positions > 0 && (long long)batch * prompt_positions > prompt_rows(*cfg)) return 0;
+    if (cfg->dtype == 0 && prompt_positions == 0 && batch * (cfg->n_draft + 1) > kF32Rows) return 0;
+    int own[9] = {};
+    if (!clusters) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        for (int s = 2; s <= 8; ++s) own[s] = resident_clusters(s);
+    }
+    if (sms < 1) return 0;
+    Layout L;
+    make_layout(*cfg, 0, L);
+    Dev D;
+    memset(&D, 0, sizeof(D));
+    set_shape(D, *cfg, L);
+    set_batch(D, batch);
+    Chain chain;
+    std::vector<ChainOp> ops;
+    if (!chain.plan(*cfg, weight_offsets(*cfg), sms, clusters ? clusters : own, D, prompt_positions ? prompt_positions : D.K1, prompt_positions > 0, ops)) return 0;
+    if ((int)ops.size() > capacity) return 0;
+    for (size_t i = 0; i < ops.size(); ++i) {
+        const ProjArgs &A = ops[i].proj;
+        const int32_t words[8] = {(int32_t)ops[i].kind, A.epi0, A.threads, A.S, A.tok, A.tps, A.tmem_cols, ops[i].smem + kProjDeclared + 1024};
+        for (int k = 0; k < 8; ++k) h_stages[8 * i + k] = k == 0 || ops[i].kind == ChainOp::PROJ ? words[k] : 0;
+    }
+    return (int)ops.size();
 }
 
 xsm_status xsm_debug_set_phase_launch(xsm_ctx *ctx, int on) {

@@ -13,7 +13,7 @@ namespace xsm {
 static_assert(sizeof(TensorMap) == sizeof(CUtensorMap), "tensor map size");
 
 constexpr int kMaxPlans = 8;                      // batch sizes whose recordings are kept
-constexpr int kAccumulators = 256;                // columns of tensor memory of a CTA (an SM has 512, and may hold two CTAs)
+constexpr int kAccumulators = 256;                // columns of tensor memory of a CTA, at most
 
 cudaError_t open_kernel(const void *fn, int smem, bool large_cluster) {
     static std::mutex mu;
@@ -169,7 +169,7 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     // Four warps more than finish token rows (they are those that also fetch and multiply), or as many as the accumulator's columns
     // keep busy: 256 against 384 threads, 5 rows of width 768 34.56 -> 34.15 ms a request, of width 1024 58.24 -> 57.09, one row 54.49
     // -> 53.91 (with the start without a release); 128, the same warps for all of it, 37.6 and 61.1.
-    A.threads = G == 1 ? 128 * std::min(kClusterThreads / 128, std::max(1 + (A.epi0 == PE_GATEUP ? (A.tps + 1) / 2 : A.tps), A.tok / 8)) : kClusterThreads;
+    A.threads = S == 1 ? kTileThreads : G == 1 ? 128 * std::min(kClusterThreads / 128, std::max(1 + (A.epi0 == PE_GATEUP ? (A.tps + 1) / 2 : A.tps), A.tok / 8)) : kClusterThreads;
     A.inv_s = 65536 / S + 1;
     A.inv_q = 65536 / (A.tps / G) + 1;
     const int n = (nblk + S - 1) / S, b_bytes = 2 * A.tok * 128, a_bytes = 128 * 128, sums = S * A.tps * 512;
@@ -188,6 +188,12 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     while (A.tmem_cols < (n + A.chain - 1) / A.chain * 2 * A.tok) A.tmem_cols *= 2;
     const int rings = A.na * a_bytes + A.nb * b_bytes;
     op.smem = 1024 + (S > 1 ? rings + sums : std::max(rings, sums));
+    // A CTA that asks for tensor memory waits until there is enough, and its cluster, which holds some, waits for it: two clusters of
+    // different streams must never wait for each other so.  CTAs of a cluster take at least the share of an SM's shared memory that
+    // their columns are of its tensor memory: what fits the one fits the other, whichever meet there and however few registers they
+    // have.  (Kernels without clusters wait for nobody who may be waiting so.  From 33 rows on, in narrow models and short cuts of the
+    // columns, there is something to add: 50 KB become 57, 103 become 114.)
+    if (S > 1) op.smem = std::max(op.smem, A.tmem_cols * (kSmSmem / kSmTmemCols) - 1024 - kProjDeclared);
 }
 
 // The projections over few token rows: how the units are dealt out, passes over the columns, shared memory.  False: the
@@ -418,6 +424,14 @@ cudaError_t Chain::run(const Dev &D, const ChainOp &op, int t, const ChainLaunch
         case ChainOp::EMBED: return launch_embed_rows(D, c_.dtype, t, op.attn.pos0, op.attn.pos_end, L);
     }
     return cudaErrorInvalidValue;
+}
+
+bool Chain::plan(const xsm_model_config &c, const WeightOffsets &w, int sms, const int *clusters, const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops) {
+    c_ = c;
+    w_ = w;
+    sms_ = sms;
+    for (int s = 2; s <= 8; ++s) clusters_[s] = clusters[s];
+    return build(D, t, prompt, ops);
 }
 
 bool Chain::select(const Dev &D) {

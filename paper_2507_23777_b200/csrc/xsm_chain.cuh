@@ -22,8 +22,11 @@ enum ProjEpilogue : int {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kTokenTile = 128;       // token rows that share a plane
 constexpr int kProjRing = 16;         // most operand blocks of one kind that a CTA keeps in shared memory
-constexpr int kClusterThreads = 384;   // most threads of a projection's CTA in a cluster
+constexpr int kClusterThreads = 384;  // most threads of a projection's CTA in a cluster
+constexpr int kTileThreads = 512;     // of one without
 constexpr int kCtaSmem = 227 * 1024;  // shared memory that a CTA may have
+constexpr int kSmSmem = 228 * 1024, kSmTmemCols = 512;      // of an SM: shared memory (1 KB of every CTA's is the system's), columns of tensor memory
+constexpr int kProjDeclared = (4 * kProjRing + 1) * 8 + kTokenTile * 4;      // shared memory that every tcgen05 projection declares, at least
 // dynamic shared memory of a projection, at most (what a kernel declares comes on top: for q, k, v the token rows' places too)
 __host__ __device__ constexpr int proj_smem_max(int epi0) { return epi0 == PE_QKV ? 224 * 1024 - 128 : 224 * 1024; }
 
@@ -43,7 +46,7 @@ struct ProjArgs {
     int layer, kdim, rows, Mp;        // rows: token rows; Mp: rows of a plane (a multiple of 8, at most kTokenTile)
     int tt, tok, qp;                  // tiles of tok token rows (parts of one plane set, or one for each); rows of the planes of queries
     int t, pos0, pos_end;             // token row m is position start + m % t of sequence m / t; start: pos0, or the sequence's length if pos0 < 0
-    int threads;                      // of a CTA of a cluster
+    int threads;                      // of a CTA
     int S, tps, group;                // CTAs per cluster (cuts of the columns), token rows each of them finishes, dealt out in groups of so many
     uint32_t inv_s, inv_q;            // 65536 / S + 1, 65536 / (tps / group) + 1: small numbers are divided by multiplying
     int na, nb, tmem_cols;            // operand blocks in shared memory (weights, activations), accumulator columns

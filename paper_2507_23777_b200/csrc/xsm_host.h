@@ -46,6 +46,8 @@ class Chain {
     bool init(const xsm_model_config &c, const WeightOffsets &w, const char *weights, int sm_count);
     // the kernels of a decoding step for the batch in D (D.B, D.M, D.Mp set); they are kept for later requests
     bool select(const Dev &D);
+    // the kernels alone, of a step or of a chunk of t positions of a prompt, on a chip of that many SMs and clusters: no device is needed
+    bool plan(const xsm_model_config &c, const WeightOffsets &w, int sms, const int *clusters, const Dev &D, int t, bool prompt, std::vector<ChainOp> &ops);
     void forget();                       // drops what is kept (a launch parameter has changed)
     int n_ops() const { return plan_ ? (int)plan_->ops.size() : 0; }
     // one decoding step; graph: replay the recording (made at the first call)

@@ -24,7 +24,6 @@ namespace xsm {
 // CL: a tile's columns are cut over a cluster.  256 or 384 threads (plan_proj) of at most 80 registers, so that the SM has room for the next kernel's
 // CTA as well (with 512 of 67 to 103 the next kernel's barriers, tensor memory and first copies came after this one's end: 20
 // token rows of width 1024 961 -> 908 us a step, 80 rows 1391 -> 1397).  Without a cluster two CTAs of 512 to an SM.
-constexpr int kTileThreads = 512;
 constexpr int kBlockK = 64;                        // columns of one operand block (128 bytes: one swizzled row)
 constexpr int kABytes = 128 * kBlockK * 2;         // weight block
 
@@ -51,6 +50,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     __shared__ uint32_t tmem_slot;
     __shared__ float s_inv[kTokenTile];
     __shared__ RowInfo s_row[kTokenTile];
+    static_assert(sizeof(bars) + sizeof(s_inv) >= kProjDeclared, "plan_proj counts on that much");
     static_assert(sizeof(bars) + sizeof(recv_bar) + sizeof(s_inv) + (EPI0 == PE_QKV ? sizeof(s_row) : 0) + 64 + proj_smem_max(EPI0) <= kCtaSmem,
                   "a ring that is as large as plan_proj allows has to fit");
     constexpr bool TWO = EPI0 == PE_GATEUP;
@@ -471,7 +471,7 @@ static cudaError_t launch_instance(const Dev &D, const ProjArgs &A, const ProjMa
     cudaError_t e = open_kernel((const void *)fn, smem, false);
     if (e != cudaSuccess) return e;
     const int tiles = A.g[0].tiles + (EPI1 >= 0 ? A.g[1].tiles : 0);
-    return L.launch(dim3(tiles * A.tt * A.S), dim3(CL ? A.threads : kTileThreads), smem, A.S, (const void *)fn, D, A, T);
+    return L.launch(dim3(tiles * A.tt * A.S), dim3(A.threads), smem, A.S, (const void *)fn, D, A, T);
 }
 
 template <int EPI0, int EPI1, bool MANY>

@@ -166,3 +166,42 @@ def test_a_step_behind_a_prefill_that_was_only_captured_ends_in_an_error(binding
         toks, lens, _ = ctx.generate(24)
         assert (lens == 24).all() and np.array_equal(toks, want)
         ctx.xsm_destroy()
+
+
+def test_contexts_on_streams_of_their_own_decode_as_they_do_alone(binding):
+    """Five contexts, each with its thread and stream, whose projections take 32 to 256 columns of an SM's 512 of tensor memory and meet
+    there."""
+    import threading
+
+    import torch
+    models = []
+    for d, H, f, K, batch in ((128, 2, 128, 7, 16), (256, 4, 512, 3, 1), (512, 8, 512, 0, 97), (128, 2, 256, 4, 6), (1280, 20, 512, 7, 15)):
+        cfg = inputs.config(2, d_model=d, n_heads=H, d_head=64, d_ff=f, d_cond=d, head_hidden=d, n_draft=K, n_layers=2, vocab=777, n_cond=40,
+                            sigma=0.02 * (1024 / d) ** 0.5, max_seq_len=96)
+        models.append((cfg, batch, inputs.make_weights(cfg), inputs.make_cond(cfg, batch)))
+
+    def request(model, stream, times):
+        cfg, batch, w, cond = model
+        out = []
+        with torch.cuda.stream(stream):
+            ctx = binding.Context(cfg, w, max_batch=batch, stream=stream)
+            for _ in range(times):
+                ctx.prefill(cond, [0, 3, 7], binding.decode_config(cfg))
+                out.append(ctx.generate(64)[0])
+            ctx.xsm_destroy()
+        return out
+
+    streams = [torch.cuda.Stream() for _ in models]
+    alone = [request(m, s, 1)[0] for m, s in zip(models, streams)]
+    got = [None] * len(models)
+
+    def work(i):
+        got[i] = request(models[i], streams[i], 8)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(models))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for i, want in enumerate(alone):
+        assert got[i] is not None and all(np.array_equal(g, want) for g in got[i]), i
