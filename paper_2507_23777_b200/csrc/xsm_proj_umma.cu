@@ -345,13 +345,16 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
         }
     }
     tcgen05_before_sync();
-    // The tensor memory goes back while the shares are on their way, by the last warp, which has token rows of its own only where there
-    // are many (at the kernel's end it kept the next one waiting: 5 rows of width 768 35.7 -> 34.6 ms a request, of width 1024 59.3 ->
-    // 58.1, 20 rows 40.1 -> 39.0, 7 rows of width 2048 59.9 -> 59.7).
+    // The tensor memory goes back while the shares are on their way (at the kernel's end it kept the next one waiting: 5 rows of width
+    // 768 35.7 -> 34.6 ms a request, of width 1024 59.3 -> 58.1, 20 rows 40.1 -> 39.0, 7 rows of width 2048 59.9 -> 59.7).  Behind the
+    // barrier every product has been issued.  This warp waits for them itself: it may not have done so before, and others may have
+    // given up waiting, and another CTA must not get columns that products are still added to.  (0 to 0.5 % of a request.)
     if (warp != tmem_warp) {
         asm volatile("bar.arrive 2, %0;" :: "r"(threads) : "memory");
     } else {
         asm volatile("bar.sync 2, %0;" :: "r"(threads) : "memory");
+        mbar_wait(done, 0u, D.mbar_limit, D.status);
+        __syncwarp();
         tcgen05_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
     }

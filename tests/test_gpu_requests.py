@@ -205,3 +205,45 @@ def test_contexts_on_streams_of_their_own_decode_as_they_do_alone(binding):
         t.join()
     for i, want in enumerate(alone):
         assert got[i] is not None and all(np.array_equal(g, want) for g in got[i]), i
+
+
+def test_a_request_that_gave_up_waiting_disturbs_no_other_context(binding):
+    """One context's stages are launched out of turn and give up; kernels of another, on a stream of its own, share the SMs (and their
+    tensor memory) with them all the while."""
+    import threading
+
+    import torch
+    cfg = inputs.config(2, d_model=512, n_heads=8, d_head=64, d_ff=512, d_cond=512, head_hidden=512, n_draft=3, n_layers=2, vocab=777, n_cond=40,
+                        max_seq_len=96)
+    w, cond, dc = inputs.make_weights(cfg), inputs.make_cond(cfg, 4), binding.decode_config(cfg)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    with torch.cuda.stream(streams[0]):
+        ctx = binding.Context(cfg, w, max_batch=4, stream=streams[0])
+        ctx.prefill(cond, [0], dc)
+        want = ctx.generate(64)[0]
+    got = []
+
+    def decode():
+        with torch.cuda.stream(streams[0]):
+            for _ in range(12):
+                ctx.prefill(cond, [0], dc)
+                got.append(ctx.generate(64)[0])
+
+    with torch.cuda.stream(streams[1]):
+        other = binding.Context(cfg, w, max_batch=4, stream=streams[1])
+        t = threading.Thread(target=decode)
+        t.start()
+        for stage in (2, 5, 6, 9):
+            other.prefill(cond, [0], dc)
+            other.xsm_debug_set_wait_limits(3000, 0)
+            other.xsm_debug_launch_stage(stage)
+            with pytest.raises(binding.XsmError) as e:
+                other.xsm_debug_get_state()
+            assert e.value.status == binding.XSM_ERR_TIMEOUT
+            other.xsm_debug_set_wait_limits(0, 0)
+        other.prefill(cond, [0], dc)
+        last = other.generate(64)[0]
+        t.join()
+        other.xsm_destroy()
+    assert len(got) == 12 and all(np.array_equal(g, want) for g in got) and np.array_equal(last, want)
+    ctx.xsm_destroy()
