@@ -38,10 +38,12 @@ SHAPES = {
     "fifteen token rows, width 128, cross-attention heads": (_model(128, 2, K=4, head_kind=1), 3),
     "two token rows, width 2048": (_model(2048, 16, 128, 2048, K=1), 1),
     "five token rows over eight CTAs": (_model(1024, 16, f=4096, K=4), 1),
-    "sixteen token rows, width 2048, eight accumulators": (_model(2048, 16, 128, 2048, K=3, V=1500), 4),
+    "sixteen token rows, width 2048, four accumulators": (_model(2048, 16, 128, 2048, K=3, V=1500), 4),
     "seventeen token rows, width 2048, one accumulator": (_model(2048, 16, 128, 2048, K=0, V=1500), 17),
     "eight token rows, two to a CTA": (_model(1792, 28, f=2048, K=7), 1),
-    "sixteen token rows, two accumulator parts": (_model(1024, 16, f=4096, K=3), 4),
+    "sixteen token rows over eight CTAs, two to a CTA": (_model(1024, 16, f=4096, K=3), 4),
+    "sixteen token rows, the accumulator in two parts, warps apart": (_model(512, 8, f=512, K=3), 4),
+    "sixteen token rows, width 2048, eight accumulators without a cluster": (_model(2048, 16, 128, 4864, K=3, V=1500), 4),
     "two token rows, width 1024": (_model(1024, 16, f=4096, K=1), 1),
     "twenty-four token rows": (_model(512, 8, K=5), 4),
     "twenty-five token rows": (_model(512, 8, K=4), 5),
@@ -62,6 +64,51 @@ SHAPES = {
 }
 
 
+MMA, UMMA, ANY = {1}, {0}, None
+QKV, RESIDUAL, CROSS_Q, GATE_UP, LOGITS = 0, 1, 2, 3, 4
+# What a shape is there for: kinds of its projections; (what one does, threads, token rows of a tile, token rows that a CTA finishes,
+# columns of tensor memory), on every chip of 148 SMs however its GPCs are cut
+SELECTS = {
+    "three token rows, width 768": (MMA,),
+    "three token rows, width 896": (UMMA,),
+    "four token rows, width 768": (UMMA,),
+    "four token rows, width 640": (MMA,),
+    "four token rows, width 512, tcgen05 for the down projection": (MMA | UMMA, (RESIDUAL, 256, 8, 1, 32)),
+    "eight token rows, width 128, tcgen05 for the down projection": (MMA | UMMA, (RESIDUAL, 256, 8, 1, 32)),
+    "nine token rows, width 128": (MMA,),
+    "sixteen token rows, width 128": (MMA,),
+    "seventeen token rows, width 128": (UMMA,),
+    "two token rows, width 2048": (UMMA, (QKV, 256, 8, 1, 64), (RESIDUAL, 256, 8, 1, 32), (CROSS_Q, 256, 8, 1, 32), (GATE_UP, 256, 8, 1, 32),
+                                   (LOGITS, 256, 8, 1, 32)),
+    "five token rows over eight CTAs": (UMMA, (RESIDUAL, 256, 8, 1, 32), (GATE_UP, 384, 8, 3, 32)),
+    "sixteen token rows, width 2048, four accumulators": (UMMA, (QKV, 384, 16, ANY, 128)),
+    "seventeen token rows, width 2048, one accumulator": (UMMA, (QKV, 384, 24, ANY, 64)),
+    "eight token rows, two to a CTA": (UMMA, (GATE_UP, 256, 8, 2, 32)),
+    "sixteen token rows over eight CTAs, two to a CTA": (UMMA, (RESIDUAL, 384, 16, 2, 32)),
+    "sixteen token rows, the accumulator in two parts, warps apart": (UMMA, (GATE_UP, 256, 16, 2, 32)),
+    "sixteen token rows, width 2048, eight accumulators without a cluster": (UMMA, (GATE_UP, 512, 16, 16, 256)),
+    "twenty-four token rows": (UMMA, (QKV, 384, 24, 3, 64)),
+    "twenty-five token rows": (UMMA, (QKV, 384, 32, 4, 64)),
+    "forty-eight token rows": (UMMA, (QKV, 384, 48, 8, 128)),
+    "forty-nine token rows": (UMMA, (RESIDUAL, 384, 8, 4, 32), (GATE_UP, 384, 16, 4, 64)),
+    "eighty token rows, width 1024": (UMMA, (RESIDUAL, 384, 24, 8, 128), (GATE_UP, 384, 40, 20, 256)),
+}
+
+
+def check_what_is_selected(shape, **chip):
+    """The plan of the step (of the current device, or of the chip that is told) has what the shape is there for."""
+    from paper_2507_23777_b200 import binding
+    over, batch = SHAPES[shape]
+    cfg = inputs.config(2, **over)
+    cfg["max_seq_len"] = 48
+    rows = [[int(v) for v in r] for r in binding.xsm_debug_plan(binding.model_config(cfg, batch), batch, **chip)]
+    kinds, *wanted = SELECTS[shape]
+    assert {r[0] for r in rows if r[0] < 3} == kinds
+    found = [(r[1], r[2], r[4], r[5], r[6]) for r in rows if r[0] == 0]
+    for w in wanted:
+        assert any(all(a in (ANY, b) for a, b in zip(w, f)) for f in found), (w, found)
+
+
 @pytest.mark.parametrize("shape", list(SHAPES))
 def test_step_against_the_oracle(shape):
     import torch
@@ -69,6 +116,8 @@ def test_step_against_the_oracle(shape):
     from paper_2507_23777_b200 import build
     build.build()
     import parity
+    if shape in SELECTS:
+        check_what_is_selected(shape)
     over, batch = SHAPES[shape]
     cfg = inputs.config(2, **over)
     cfg["max_seq_len"] = 48

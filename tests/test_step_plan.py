@@ -1,9 +1,10 @@
 """How a step is cut over the chip: plans alone, no GPU."""
 import pytest
 
+import test_gpu_step_paths as paths
 from paper_2507_23777_b200 import binding, build, inputs
 
-SMS, CLUSTERS = 148, [0, 0, 74, 48, 36, 28, 22, 18, 15]      # a B200's
+SMS, CLUSTERS = 148, [0, 0, 74, 45, 33, 26, 22, 15, 15]      # a B200's
 UMMA = 0
 KIND, DOES, THREADS, CTAS, TOK, ROWS, COLUMNS, SMEM = range(8)
 
@@ -50,3 +51,8 @@ def test_there_is_no_plan_for_what_is_refused():
     assert len(plan(128, 100, 4, 1)) == 0             # d_ff no multiple of 128
     assert len(plan(128, 128, 4, 1, 100000)) == 0     # a prompt beyond the room
     assert len(plan(128, 128, 4, 8, dtype=0)) == 0    # fp32: 40 token rows
+
+
+@pytest.mark.parametrize("shape", list(paths.SELECTS))
+def test_shapes_of_the_step_paths_select_what_they_are_named_for(shape):
+    paths.check_what_is_selected(shape, sms=SMS, clusters=CLUSTERS)
