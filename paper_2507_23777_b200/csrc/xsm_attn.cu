@@ -382,8 +382,9 @@ __global__ void __launch_bounds__(NW * 32 + 32, FEW && DH <= 64 && NW == 8 ? 2 :
             trace_mark(D, 1 + 2 * A.stage);
         }
         if (FEW) {
-            // Warps without keys neither fetch queries nor leave a state: 5 rows of width 768 34.15 -> 33.77 ms a request, of width
-            // 1024 57.09 -> 56.84, 20 rows 37.50 -> 37.10, 7 rows of width 2048 58.82 -> 58.09.
+            // Warps without keys leave no state, and fetch no queries (where the kernel projects them itself all warps take part in
+            // that): 5 rows of width 768 33.87 -> 33.57 ms a request, of width 1024 56.71 -> 56.48, 20 rows 37.37 -> 36.98, 7 rows of
+            // width 2048 58.72 -> 58.05.
             const bool busy = !all_in || warp < n_units;
             unsigned qh[DH / 8], ql[DH / 8];
             if constexpr (QP) {

@@ -166,9 +166,10 @@ void Chain::plan_proj(ChainOp &op, int rows, int Mp, int kdim) {
     const int tile_rows = std::min(rows, A.tok), G = S > 1 && rows <= 24 ? 1 : 4;
     A.group = G;
     A.tps = ((tile_rows + G - 1) / G + S - 1) / S * G;
-    // Four warps more than finish token rows (they are those that also fetch and multiply), or as many as the accumulator's columns
-    // keep busy: 256 against 384 threads, 5 rows of width 768 34.56 -> 34.15 ms a request, of width 1024 58.24 -> 57.09, one row 54.49
-    // -> 53.91 (with the start without a release); 128, the same warps for all of it, 37.6 and 61.1.
+    // Four warps more than finish token rows, or as many as the accumulator's columns keep busy, at most twelve.  Eight are enough where a
+    // CTA finishes one row (two in gate/up, whose rows take 64 threads each): the first four fetch and multiply, the others finish.
+    // Against twelve there too: 5 rows of width 768 33.83 -> 33.57 ms a request, of width 1024 57.45 -> 56.48, one row 54.90 -> 53.76.  Of
+    // twelve warps the first four do both, and those that are left over prepare the rows' scales and wait for nothing.
     A.threads = S == 1 ? kTileThreads : G == 1 ? 128 * std::min(kClusterThreads / 128, std::max(1 + (A.epi0 == PE_GATEUP ? (A.tps + 1) / 2 : A.tps), A.tok / 8)) : kClusterThreads;
     A.inv_s = 65536 / S + 1;
     A.inv_q = 65536 / (A.tps / G) + 1;

@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
                   "a ring that is as large as plan_proj allows has to fit");
     constexpr bool TWO = EPI0 == PE_GATEUP;
     const int threads = CL && G == 1 ? (int)blockDim.x : CL ? kClusterThreads : kTileThreads;
-    // Of eight warps the first four fetch, multiply and set up, the others take the accumulator and the first token rows.
+    // Of eight warps the first four fetch, multiply and set up (and take the second part of an accumulator of two, more than eight token
+    // rows); the others take its first part and the first token rows.  Of twelve the first four do both.
     const bool apart = CL && G == 1 && threads == 256;
     const int tmem_warp = apart ? 3 : (threads >> 5) - 1;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp's number: uniform, also to the compiler)
@@ -125,8 +126,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     __syncwarp();
     // "this CTA runs": its barriers are there (mbar_init_fence), and peers may write to its shared memory, after cluster_wait.  A release
     // would wait for the load above, and hold back the weights' copies, which a kernel that starts late waits for: 5 rows of width 768
-    // 37.6 -> 37.2 ms a request, of width 1024 61.1 -> 60.6, 20 rows 38.8 -> 37.4, 7 rows of width 2048 59.4 -> 58.8 (all of them with
-    // a thread for every weight row and no more, where one token row is finished).
+    // 33.91 -> 33.57 ms a request, of width 1024 57.23 -> 56.48, 20 rows 38.21 -> 36.98, 7 rows of width 2048 58.89 -> 58.05.
     if (CL) cluster_arrive_relaxed();
     if (warp == 0 && elect_one())      // the weights' way is the longest: it begins as early as that
         for (int i = 0; i < min(n, na); ++i) load_a(i, i);
@@ -303,8 +303,8 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     if (warp >= 2 && lane == 0) mbar_arrive(done);
     const float gain = __uint_as_float(gain_bits << 16);
     request(side);
-    // (warps with neither a part of the accumulator nor token rows wait for nothing more: 5 rows of width 768 33.82 -> 33.54 ms a request,
-    // of width 1024 56.88 -> 56.41, 20 rows 37.11 -> 36.87, 7 rows of width 2048 58.04 -> 57.65)
+    // (warps with neither a part of the accumulator nor token rows wait for nothing more: 5 rows of width 768 33.94 -> 33.57 ms a request,
+    // of width 1024 56.93 -> 56.48, 20 rows 37.23 -> 36.98, 7 rows of width 2048 58.42 -> 58.05)
     const bool part = !CL || (c0 << 3) < Nt || G * side < nm;
     const bool done_ok = !part || mbar_wait(done, 0u, D.mbar_limit, D.status);
     __syncwarp();
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     }
     tcgen05_before_sync();
     // The tensor memory goes back while the shares are on their way (at the kernel's end it kept the next one waiting: 5 rows of width
-    // 768 35.7 -> 34.6 ms a request, of width 1024 59.3 -> 58.1, 20 rows 40.1 -> 39.0, 7 rows of width 2048 59.9 -> 59.7).  Behind the
+    // 768 35.14 -> 33.57 ms a request, of width 1024 58.04 -> 56.48, 20 rows 38.24 -> 36.98, 7 rows of width 2048 58.95 -> 58.05).  Behind the
     // barrier every product has been issued.  This warp waits for them itself: it may not have done so before, and others may have
     // given up waiting, and another CTA must not get columns that products are still added to.  (0 to 0.5 % of a request.)
     if (warp != tmem_warp) {
