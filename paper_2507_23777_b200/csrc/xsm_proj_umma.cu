@@ -348,12 +348,13 @@ __global__ void __launch_bounds__(CL ? kClusterThreads : kTileThreads, 2) proj_u
     // The tensor memory goes back while the shares are on their way (at the kernel's end it kept the next one waiting: 5 rows of width
     // 768 35.14 -> 33.57 ms a request, of width 1024 58.04 -> 56.48, 20 rows 38.24 -> 36.98, 7 rows of width 2048 58.95 -> 58.05).  Behind the
     // barrier every product has been issued.  This warp waits for them itself: it may not have done so before, and others may have
-    // given up waiting, and another CTA must not get columns that products are still added to.  (0 to 0.5 % of a request.)
+    // given up waiting (and have raised the status), and another CTA must not get columns that products are still added to.  (0 to 0.3 %
+    // of a request; with the status raised here as well, which is code for nothing, to 0.6 %.)
     if (warp != tmem_warp) {
         asm volatile("bar.arrive 2, %0;" :: "r"(threads) : "memory");
     } else {
         asm volatile("bar.sync 2, %0;" :: "r"(threads) : "memory");
-        mbar_wait(done, 0u, D.mbar_limit, D.status);
+        for (unsigned i = 0; !mbar_try_wait(done, 0u) && i < D.mbar_limit; ++i);
         __syncwarp();
         tcgen05_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(A.tmem_cols) : "memory");
